@@ -1,6 +1,7 @@
 // api.cu -- host side of the C ABI declared in include/mba.h: problem creation
 // (one device pool sized up front), the solve driver that issues the LM
 // iterations without host round trips, and the inspection entry points.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <atomic>
@@ -64,6 +65,8 @@ struct mba_problem {
     cudaStream_t stream = nullptr;
     void *pool = nullptr;
     size_t pool_bytes = 0;
+    void *pool2 = nullptr;          // arrays whose layout depends on the sorted observations
+    size_t pool2_bytes = 0;
     int32_t *cfirst = nullptr;      // per camera first chunk (device)
     int32_t *orig_cam = nullptr, *orig_pt = nullptr;
     double2 *orig_uv = nullptr;
@@ -131,6 +134,7 @@ void mba_problem_destroy(mba_problem *pr) {
     if (!pr) return;
     if (pr->stream) cudaStreamSynchronize(pr->stream);
     if (pr->pool) cudaFree(pr->pool);
+    if (pr->pool2) cudaFree(pr->pool2);
     delete pr;
 }
 
@@ -164,6 +168,8 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
     P.np = np;
     P.n = n;
     P.npad = ((n + 63) / 64) * 64 + 64;
+    P.np_pad = (np + 63) / 64 * 64;
+    P.slot_cap = (sell_slot_bound(n, np) + 63) / 64 * 64;
     P.fp32 = o.precision == MBA_FP32_MIXED;
     P.loss = o.loss;
     P.delta = o.huber_delta;
@@ -182,6 +188,12 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
         pr->nb_chunk = sms * 4;
     }
     pr->nb_cost = cost_grid(P);
+    // block-owned products (own.cu) where the problem's shape suits them; the
+    // FP32 form falls back to the gathered product, the FP64 form keeps the stored
+    // Jacobian otherwise
+    P.own = !P.autodiff && own_wanted(P, sms) ? 1 : 0;
+    P.sorted = (P.fact || P.own) ? 1 : 0;
+    const bool stored = !P.fact && !P.own;  // the PCG reads a stored Jacobian
     const int red_len = 3 * 8192;
     const int64_t stage = n < kEvalSlice ? n : kEvalSlice;
 
@@ -192,27 +204,24 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
         P.pts = c.take<double>(3 * (size_t)np);
         P.pts_new = c.take<double>(3 * (size_t)np);
         P.pts0 = c.take<double>(3 * (size_t)np);
-        P.pm_cam = c.take<int32_t>(n + 64);  // slack for 16-byte-rounded bulk copies
+        P.pm_cam = c.take<int32_t>(n);
         P.pm_pt = c.take<int32_t>(n);
         P.pm_orig = c.take<int32_t>(n);
         P.pm_uv = c.take<double2>(n);
-        P.pt_ptr = c.take<int32_t>((size_t)np + 64);  // slack for 16-byte-rounded bulk copies
+        P.pt_ptr = c.take<int32_t>((size_t)np + 1);
         P.cm_pt = c.take<int32_t>(n);
         P.cm_orig = c.take<int32_t>(n);
         P.cm_uv = c.take<double2>(n);
         P.cam_ptr = c.take<int32_t>((size_t)nc + 1);
-        P.wchunk = c.take<int2>((size_t)np + 64);
-        P.tiles = c.take<int2>((size_t)np + 2);
-        P.tdesc = c.take<int4>(3 * ((size_t)np + 2));
-        P.long_chunks = c.take<int32_t>((size_t)np + 2);
+        P.wchunk = !stored ? nullptr : c.take<int2>((size_t)np + 1);
         P.cchunk_cam = c.take<int32_t>(cbound);
         P.cchunk_beg = c.take<int32_t>(cbound + 1);
         pr->cfirst = c.take<int32_t>((size_t)nc + 1);
         pr->orig_cam = c.take<int32_t>(n);
         pr->orig_pt = c.take<int32_t>(n);
         pr->orig_uv = c.take<double2>(n);
-        P.J = P.fact ? nullptr : c.take<char>(24 * (size_t)P.npad * w);
-        P.res = c.take<char>(2 * (size_t)P.npad * w);
+        P.J = !stored ? nullptr : c.take<char>(24 * (size_t)P.npad * w);
+        P.res = !stored ? nullptr : c.take<char>(2 * (size_t)P.npad * w);
         P.camtab = c.take<char>((size_t)nc * kCamTab * w);
         P.camtab64 = c.take<double>((size_t)nc * kCamTab);
         P.Hpp = c.take<double>(45 * (size_t)nc);
@@ -222,37 +231,52 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
         P.cpart = c.take<double>(54 * (size_t)cbound);
         P.Bd = c.take<double>(81 * (size_t)nc);
         P.Binv = c.take<double>(81 * (size_t)nc);
-        P.Cinv = c.take<char>((6 * (size_t)np + 64) * w);
+        P.Cinv = c.take<char>(6 * (size_t)P.np_pad * w);
         P.x = c.take<double>((size_t)nc * kVec);
         P.r = c.take<double>((size_t)nc * kVec);
         P.z = c.take<double>((size_t)nc * kVec);
         P.p = c.take<double>((size_t)nc * kVec);
         P.q = c.take<double>((size_t)nc * kVec);
         P.g = c.take<double>((size_t)nc * kVec);
-        P.pT = c.take<char>((size_t)nc * ((P.fp32 && !P.autodiff) ? kRow * 4 : kVec * w));
+        P.pT = c.take<char>((size_t)nc * (P.fact ? kRowG * 4 : kVec * w));
         P.p2 = c.take<double>((size_t)nc * kVec);
-        P.sbuf = c.take<char>(2 * (size_t)P.npad * w);
+        P.sbuf = !stored ? nullptr : c.take<char>(2 * (size_t)P.npad * w);
         P.cta_cam = c.take<int32_t>(4096 + 1);
-        P.pm2cm = c.take<int32_t>(n + 64);
-        P.pm_uv32 = P.fp32 ? c.take<float2>(n) : nullptr;
+        P.pm2cm = !stored ? nullptr : c.take<int32_t>(n);
+        P.pm_uv32 = (P.fp32 && !P.fact) ? c.take<float2>(n) : nullptr;
         P.cm_uv32 = P.fp32 ? c.take<float2>(n) : nullptr;
-        P.pts32 = P.fp32 ? c.take<float4>((size_t)np) : nullptr;
+        P.pts32 = (P.fp32 && !P.fact) ? c.take<float4>((size_t)np) : nullptr;
         P.cam_fixed = c.take<uint8_t>((size_t)nc);
         P.pt_fixed = c.take<uint8_t>((size_t)np);
         // copies for the PCG: the camera-major stored Jacobian (FP64, or FP32-mixed
         // with dual numbers), else the factored form's per-observation data
         const bool fact = P.fact != 0;
-        P.PXpm = fact ? c.take<float>(3 * (size_t)P.npad) : nullptr;
-        P.Jph = fact ? c.take<float>(6 * (size_t)P.npad) : nullptr;
-        P.RXcm = fact ? c.take<float>(4 * (size_t)P.npad) : nullptr;
-        P.swpm = (fact && o.loss != MBA_LOSS_NONE) ? c.take<float>((size_t)P.npad) : nullptr;
+        const size_t slots = P.sorted ? (size_t)P.slot_cap : 0;
+        const bool lossy = P.sorted && o.loss != MBA_LOSS_NONE;
+        P.slice = P.sorted ? c.take<int4>((size_t)sell_slice_bound(n, np)) : nullptr;
+        P.sp_pt = P.sorted ? c.take<int32_t>((size_t)np) : nullptr;
+        P.sl_cam = P.sorted ? c.take<int32_t>(slots) : nullptr;
+        P.cm_sp = P.sorted ? c.take<int32_t>((size_t)n) : nullptr;
+        P.sl_uv32 = fact ? c.take<float2>(slots) : nullptr;
+        P.sl_px = fact ? c.take<float4>(slots) : nullptr;
+        P.sl_w = fact && lossy ? c.take<float>(slots) : nullptr;
+        P.sp_X = fact ? c.take<float4>((size_t)np) : nullptr;
+        P.camstat = fact ? c.take<float>((size_t)kCamStat * nc) : nullptr;
+        P.ctr = fact ? c.take<float>((size_t)kCtr * nc) : nullptr;
+        const bool own64 = P.own && !P.fp32;
+        P.sl_uv = own64 ? c.take<double2>(slots) : nullptr;
+        P.sl_hg = own64 ? c.take<double2>(5 * slots) : nullptr;
+        P.sl_w64 = own64 && lossy ? c.take<double>(slots) : nullptr;
+        P.sp_X64 = own64 ? c.take<double>(4 * (size_t)np) : nullptr;
+        P.sp_b64 = own64 ? c.take<double>(4 * (size_t)np) : nullptr;
+        P.ctr64 = own64 ? c.take<double>((size_t)kCtr * nc) : nullptr;
         P.camff = fact ? c.take<float2>(16 * (size_t)nc) : nullptr;
         P.uvff = fact ? c.take<float4>((size_t)n) : nullptr;
         P.ptsff = fact ? c.take<float2>(3 * (size_t)np) : nullptr;
-        // float copies of z and p (the factored form: their camera rows, kRow floats)
-        P.zT = P.fp32 ? c.take<float>((size_t)nc * (fact ? kRow : kVec)) : nullptr;
-        P.pT2 = c.take<char>((size_t)nc * (fact ? kRow * 4 : kVec * w));
-        P.Jcm = P.fp32 ? nullptr : c.take<double>(18 * (size_t)P.npad);
+        // float copies of z and p (the factored form: z's camera rows)
+        P.zT = P.fp32 || own64 ? c.take<char>((size_t)nc * kVec * w) : nullptr;
+        P.pT2 = fact ? nullptr : c.take<char>((size_t)nc * kVec * w);
+        P.Jcm = P.fp32 || P.own ? nullptr : c.take<double>(18 * (size_t)P.npad);
         P.JcmT = P.fp32 ? (P.autodiff ? (void *)c.take<float>(18 * (size_t)P.npad) : nullptr) : (void *)P.Jcm;
         P.dp = c.take<double>(3 * (size_t)np);
         P.red = c.take<double>(red_len);
@@ -267,10 +291,15 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
     layout(sizing);
     pr->pool_bytes = sizing.off;
     P.red_len = red_len;
-    const size_t sort_tmp = stable_sort_tmp_bytes(n, np > nc ? np : nc);
+    // scratch of the sorts; the sliced order reuses it once the observations are sorted
+    size_t sort_tmp = std::max(stable_sort_tmp_bytes(n, np > nc ? np : nc), sell_tmp_bytes(np));
+    if (P.own) sort_tmp = std::max(sort_tmp, own_tmp_bytes(P, 4 * (int64_t)sms));
+    sort_tmp = al(sort_tmp);  // the observations follow it
     const size_t setup_bytes = sort_tmp + al(sizeof(double) * 2 * (size_t)n) + 256;
-    if (mba::over_memory_limit(pr->pool_bytes + setup_bytes)) {
-        const size_t need = pr->pool_bytes + setup_bytes;
+    // the second pool's size is known after the sorts: about its share per observation here
+    const size_t later = P.own ? (P.fp32 ? 24 : 92) * (size_t)n : (P.fact ? 20 * (size_t)n + 16 * (size_t)np : 0);
+    if (mba::over_memory_limit(pr->pool_bytes + later + setup_bytes)) {
+        const size_t need = pr->pool_bytes + later + setup_bytes;
         delete pr;
         return fail(MBA_ERR_OOM, "device memory limit: creation needs " + std::to_string(need) + " bytes");
     }
@@ -326,7 +355,7 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
     CKC(gather_layout(P, obs_d, pr->orig_cam, pr->orig_pt, nullptr, flags, s));
     // point-major position -> camera-major position, via the inverse of the
     // camera-major permutation (set-up scratch): the point pass writes s there
-    CKC(build_pm2cm(P, (int32_t *)tmp, s));
+    if (P.pm2cm) CKC(build_pm2cm(P, (int32_t *)tmp, s));
     CKC(launch_split_observations(P, s));  // float-float pixels for the FP32-mixed solve's cost
     // keep the observations in input order too (for mba_evaluate)
     {
@@ -343,6 +372,35 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
     if (max_track > kMaxTrack)
         return cleanup_fail(MBA_ERR_INVALID_ARG,
                             "a point has " + std::to_string(max_track) + " observations; at most 1024 are supported");
+
+    if (P.sorted) CKC(build_slices(P, sms, max_track, tmp, sort_tmp, s));
+    // padding slots are never written: camera -1, all bits set
+    if (P.sl_px) CKC(cudaMemsetAsync(P.sl_px, 0xff, sizeof(float4) * (size_t)P.nslots, s));
+    if (!P.own && !P.fact && P.sorted) return cleanup_fail(MBA_ERR_INVALID_ARG, "internal: block-owned layout");
+    if (P.own) {
+        const cudaError_t e = build_own(P, tmp, sort_tmp, &pr->pool2, &pr->pool2_bytes, s);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            return cleanup_fail(MBA_ERR_OOM, "device memory for " + std::to_string(pr->pool2_bytes) + " bytes of run layout");
+        }
+        CKC(e);
+    } else if (P.fact) {  // the gathered product's arrays
+        const bool lossy = o.loss != MBA_LOSS_NONE;
+        auto layout2 = [&](Carve &c) {
+            P.RXcm = c.take<float4>((size_t)n);
+            P.sp_b = c.take<float4>((size_t)np);
+            P.cm_w = lossy ? c.take<float>((size_t)n) : nullptr;
+        };
+        Carve size2, real2;
+        layout2(size2);
+        pr->pool2_bytes = size2.off;
+        if (mba::over_memory_limit(pr->pool_bytes + size2.off) || cudaMalloc(&pr->pool2, size2.off) != cudaSuccess) {
+            cudaGetLastError();
+            return cleanup_fail(MBA_ERR_OOM, "device memory for " + std::to_string(size2.off) + " bytes");
+        }
+        real2.base = (char *)pr->pool2;
+        layout2(real2);
+    }
 
     // PCG camera partition: one group of whole cameras per CTA (one CTA per SM),
     // cut at the camera boundaries nearest to equal observation counts; then
@@ -378,6 +436,7 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
             chunk *= 2;
         }
         P.pcg_max_cta_chunks = max_chunks;
+        for (int k = 0; k < G; ++k) P.pcg_max_cta_cams = std::max(P.pcg_max_cta_cams, cta[k + 1] - cta[k]);
         std::vector<int32_t> ccam, cbeg, cfirst((size_t)nc + 1);
         for (int32_t i = 0; i < nc; ++i) {
             cfirst[i] = (int32_t)ccam.size();
@@ -397,9 +456,9 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
         CKC(cudaMemcpyAsync(P.cta_cam, cta.data(), sizeof(int32_t) * cta.size(), cudaMemcpyHostToDevice, s));
         CKC(cudaStreamSynchronize(s));  // host vectors go out of scope
     }
-    // warp chunks of the PCG point pass: greedy runs of whole points with at
-    // most 32 observations; a point with a longer track forms its own chunk
-    {
+    // warp chunks of the point-major passes over a stored Jacobian: greedy runs of
+    // whole points with at most 32 observations; a longer track forms its own chunk
+    if (P.wchunk) {
         std::vector<int32_t> pp((size_t)np + 1);
         CKC(cudaMemcpyAsync(pp.data(), P.pt_ptr, sizeof(int32_t) * pp.size(), cudaMemcpyDeviceToHost, s));
         CKC(cudaStreamSynchronize(s));
@@ -416,50 +475,6 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
         }
         wc.push_back(make_int2(np, (int32_t)n));
         P.n_wchunks = (int32_t)wc.size() - 1;
-        // tiles of the staged point pass: greedy runs of consecutive chunks with at
-        // most 32 observations each, within the stage capacity; a chunk of a longer
-        // track ends the run and is listed apart
-        std::vector<int2> tiles;
-        std::vector<int32_t> longs;
-        {
-            int32_t tb = -1, tobs = 0, tpts = 0;
-            auto close = [&](int32_t end) {
-                if (tb >= 0) tiles.push_back(make_int2(tb, end));
-                tb = -1;
-                tobs = tpts = 0;
-            };
-            for (int32_t k = 0; k < P.n_wchunks; ++k) {
-                const int32_t m = wc[k + 1].y - wc[k].y, npts = wc[k + 1].x - wc[k].x;
-                if (m > 32) {
-                    close(k);
-                    longs.push_back(k);
-                    continue;
-                }
-                if (tb >= 0 && (tobs + m > kTileObs || tpts + npts > kTilePts || k - tb + 1 > kTileChunks)) close(k);
-                if (tb < 0) tb = k;
-                tobs += m;
-                tpts += npts;
-            }
-            close(P.n_wchunks);
-        }
-        P.n_tiles = (int32_t)tiles.size();
-        P.n_long = (int32_t)longs.size();
-        // copy ranges of each tile, rounded to 16 bytes: observations [w0.y, w1.y),
-        // C~^-1 floats of points [w0.x, w1.x), CSR offsets pt_ptr[w0.x .. w1.x], chunk
-        // entries [cb, ce]
-        std::vector<int4> tdesc(3 * tiles.size());
-        for (size_t t = 0; t < tiles.size(); ++t) {
-            const int2 w0 = wc[tiles[t].x], w1 = wc[tiles[t].y];
-            tdesc[3 * t] = make_int4(w0.y & ~3, (w1.y + 3) & ~3, (6 * w0.x) & ~3, (6 * w1.x + 3) & ~3);
-            tdesc[3 * t + 1] = make_int4(w0.x & ~3, (w1.x + 4) & ~3, tiles[t].x & ~1, (tiles[t].y + 2) & ~1);
-            tdesc[3 * t + 2] = make_int4(tiles[t].x, tiles[t].y, 0, 0);
-        }
-        if (!tiles.empty()) {
-            CKC(cudaMemcpyAsync(P.tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, s));
-            CKC(cudaMemcpyAsync(P.tdesc, tdesc.data(), sizeof(int4) * tdesc.size(), cudaMemcpyHostToDevice, s));
-        }
-        if (!longs.empty())
-            CKC(cudaMemcpyAsync(P.long_chunks, longs.data(), sizeof(int32_t) * longs.size(), cudaMemcpyHostToDevice, s));
         CKC(cudaMemcpyAsync(P.wchunk, wc.data(), sizeof(int2) * wc.size(), cudaMemcpyHostToDevice, s));
         CKC(cudaStreamSynchronize(s));
     }
@@ -467,7 +482,7 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
     CKC(cudaMemcpyAsync(P.pts0, P.pts, sizeof(double) * 3 * (size_t)np, cudaMemcpyDeviceToDevice, s));
     CKC(cudaMemsetAsync(P.st, 0, sizeof(DevState), s));
     if (P.J) CKC(cudaMemsetAsync(P.J, 0, 24 * (size_t)P.npad * w, s));
-    CKC(cudaMemsetAsync(P.res, 0, 2 * (size_t)P.npad * w, s));
+    if (P.res) CKC(cudaMemsetAsync(P.res, 0, 2 * (size_t)P.npad * w, s));
     CKC(cudaStreamSynchronize(s));
     cudaFree(tmp);
 #undef CKC
@@ -492,7 +507,7 @@ mba_status mba_problem_info(const mba_problem *pr, int32_t *nc, int32_t *np, int
     if (nc) *nc = pr->P.nc;
     if (np) *np = pr->P.np;
     if (n) *n = pr->P.n;
-    if (bytes) *bytes = pr->pool_bytes;
+    if (bytes) *bytes = pr->pool_bytes + pr->pool2_bytes;
     return MBA_OK;
 }
 
@@ -756,10 +771,11 @@ mba_status mba_solve(mba_problem *pr, const mba_solver_options *opt, mba_summary
     CK(rec(ne > 0 ? ne - 1 : 0));
     // state_init, camera table, 2 cost kernels; per iteration: camera table, 3
     // linearisation, 2 damping, PCG, 3 back-substitution, camera table, 2 cost,
-    // LM update, accept; the factored form adds the camera rows of dc, the
+    // LM update, accept; the FP32 forms add their point copy and, where the
+    // factored form's camera rows do not fit in shared memory, the rows of dc, the
     // float-float cost its point copy before each cost, the Schur-Jacobi
     // preconditioner two damping kernels
-    const int fact = P.fact ? 1 : 0, ffc = ff ? 1 : 0;
+    const int fact = (P.fp32 ? 1 : 0) + (P.fact && P.nc * kRowS * 4 > 220 * 1024 ? 1 : 0), ffc = ff ? 1 : 0;
     const int launches =
         4 + ffc + (15 + fact + ffc + (o.preconditioner == MBA_PRECOND_SCHUR_JACOBI ? 2 : 0)) * o.max_iter;
     DevState hs;

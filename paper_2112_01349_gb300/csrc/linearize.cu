@@ -25,10 +25,64 @@ inline unsigned grid_for(int64_t n, int per = kBlock) {
     return (unsigned)(g < 1 ? 1 : g);
 }
 
+// Camera constants of the factored FP32 product, from the FP64 table row.
+// stat: f, k1, k2, sqrt(2) times the unit quaternion of R (half-angle form, so
+// that x + w c + v x c with c = v x x rotates x), t.  ctr: the 9 x 3 transform
+// between a camera vector (rotation, translation, intrinsics) and the three
+// triples a row holds: R M for the rotation, the identity for the translation,
+// (1, 0, 0; k1, f, 0; k2, 0, f)^T for f, k1, k2 (the Jacobian of f d(r^2) is
+// d, f r^2, f r^4 = the row (1, k1, k2) / (0, f, 0) / (0, 0, f) applied to
+// (1, r^2, r^4)).
+__device__ __forceinline__ void factored_camera(const double *row, float *stat, float *ctr) {
+    const double w0 = row[25], w1 = row[26], w2 = row[27];
+    const double th = sqrt(w0 * w0 + w1 * w1 + w2 * w2), root2 = 1.4142135623730951;
+    double sh = 0.0, ch = 1.0, k = 0.5;
+    if (row[24] == 0.0) {
+        sincos(0.5 * th, &sh, &ch);
+        k = sh / th;
+    }
+    stat[0] = (float)row[21];
+    stat[1] = (float)row[22];
+    stat[2] = (float)row[23];
+    stat[3] = (float)(root2 * ch);
+    stat[4] = (float)(root2 * k * w0);
+    stat[5] = (float)(root2 * k * w1);
+    stat[6] = (float)(root2 * k * w2);
+    stat[7] = (float)row[18];
+    stat[8] = (float)row[19];
+    stat[9] = (float)row[20];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            ctr[3 * a + b] = (float)(row[3 * b] * row[9 + a] + row[3 * b + 1] * row[12 + a] + row[3 * b + 2] * row[15 + a]);
+            ctr[9 + 3 * a + b] = a == b ? 1.f : 0.f;
+        }
+    const float in[9] = {1.f, stat[1], stat[2], 0.f, stat[0], 0.f, 0.f, 0.f, stat[0]};
+#pragma unroll
+    for (int q = 0; q < 9; ++q) ctr[18 + q] = in[q];
+}
+
+// The same transform of the block-owned FP64 product, whose rows are in the
+// world frame: M for the rotation, R for the translation.
+__device__ __forceinline__ void own_camera(const double *row, double *ctr) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            ctr[3 * a + b] = row[9 + 3 * b + a];
+            ctr[9 + 3 * a + b] = row[3 * a + b];
+        }
+    const double in[9] = {1.0, row[22], row[23], 0.0, row[21], 0.0, 0.0, 0.0, row[21]};
+#pragma unroll
+    for (int q = 0; q < 9; ++q) ctr[18 + q] = in[q];
+}
+
 template <typename T>
 __global__ void camera_table_kernel(const double *__restrict__ cams, int32_t nc, T *__restrict__ tab,
-                                    double *__restrict__ tab64, float2 *__restrict__ tabff, const DevState *st,
-                                    int gate) {
+                                    double *__restrict__ tab64, float2 *__restrict__ tabff,
+                                    float *__restrict__ stat, float *__restrict__ ctr, double *__restrict__ ctr64,
+                                    const DevState *st, int gate) {
     if (gate == 1 && (st->done || !st->relin)) return;
     if (gate == 2 && st->done) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
@@ -40,6 +94,8 @@ __global__ void camera_table_kernel(const double *__restrict__ cams, int32_t nc,
         if (tab64)
 #pragma unroll
             for (int q = 0; q < kCamTab; ++q) tab64[(int64_t)i * kCamTab + q] = row[q];
+        if (ctr64) own_camera(row, ctr64 + (int64_t)i * kCtr);
+        if (ctr) factored_camera(row, stat + (int64_t)i * kCamStat, ctr + (int64_t)i * kCtr);
         if (tabff) {  // R, t, f, k1, k2 as float-float
 #pragma unroll
             for (int q = 0; q < 9; ++q) {
@@ -72,14 +128,27 @@ __global__ void uv32_kernel(const double2 *__restrict__ uv, int64_t n, float2 *_
     }
 }
 
-// FP32 copy of the current points for the FP32-mixed linearisation, one float4
-// per point; runs where the linearisation runs (same gate).
-__global__ void point_table_kernel(const double *__restrict__ pts, int32_t np, float4 *__restrict__ out,
-                                   const DevState *st, int gate) {
+// FP32 copy of the current points for the FP32-mixed linearisation; runs where
+// the linearisation runs (same gate).  One float4 per
+// point, in sorted order in the factored form.
+__global__ void point_table_kernel(const double *__restrict__ pts, const int32_t *__restrict__ sp_pt, int32_t np,
+                                   float4 *__restrict__ out, const DevState *st, int gate) {
     if (gate && (st->done || !st->relin)) return;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < np; j += gridDim.x * blockDim.x)
-        out[j] = make_float4((float)pts[3 * (int64_t)j], (float)pts[3 * (int64_t)j + 1], (float)pts[3 * (int64_t)j + 2],
-                             0.f);
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < np; s += gridDim.x * blockDim.x) {
+        const int64_t j = sp_pt ? sp_pt[s] : s;
+        out[s] = make_float4((float)pts[3 * j], (float)pts[3 * j + 1], (float)pts[3 * j + 2], 0.f);
+    }
+}
+
+__global__ void point_table64_kernel(const double *__restrict__ pts, const int32_t *__restrict__ sp_pt, int32_t np,
+                                     double *__restrict__ out, const DevState *st, int gate) {
+    if (gate && (st->done || !st->relin)) return;
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < np; s += gridDim.x * blockDim.x) {
+        const int64_t j = sp_pt[s];
+        double2 *o = (double2 *)(out + 4 * (int64_t)s);
+        o[0] = make_double2(pts[3 * j], pts[3 * j + 1]);
+        o[1] = make_double2(pts[3 * j + 2], 0.0);
+    }
 }
 
 __global__ void split_uv_kernel(const double2 *__restrict__ uv, int64_t n, float4 *__restrict__ out) {
@@ -145,7 +214,6 @@ __global__ void __launch_bounds__(kBlock) cost_partial_ff_kernel(Prob P, double 
 // Jp~^T Jp~, then -Jp~^T e~).
 template <typename T, bool AD>
 __device__ __forceinline__ void lin_point_obs(const Prob &P, int64_t o, int cam, int pt, T *q) {
-    constexpr bool FACT = sizeof(T) == 4 && !AD;  // FP32-mixed analytic: no stored Jacobian
     const T *__restrict__ camtab = (const T *)P.camtab;
     T *__restrict__ J = (T *)P.J;
     T *__restrict__ res = (T *)P.res;
@@ -153,8 +221,8 @@ __device__ __forceinline__ void lin_point_obs(const Prob &P, int64_t o, int cam,
     T X0, X1, X2, u0, u1;
     load_point<T>(P, pt, X0, X1, X2);
     load_uv<T>(P.pm_uv, P.pm_uv32, o, u0, u1);
-    T e[2], Jc[18], Jp[6], pz[3];
-    edge_eval<T, AD>(camtab + (int64_t)cam * kCamTab, X0, X1, X2, u0, u1, e, Jc, Jp, FACT ? pz : nullptr);
+    T e[2], Jc[18], Jp[6];
+    edge_eval<T, AD>(camtab + (int64_t)cam * kCamTab, X0, X1, X2, u0, u1, e, Jc, Jp);
     zero_fixed_columns<T>(P, cam, pt, Jc, Jp);
     T rho, W;
     loss_weight<T>(P.loss, (T)P.delta, e[0] * e[0] + e[1] * e[1], &rho, &W);
@@ -163,18 +231,10 @@ __device__ __forceinline__ void lin_point_obs(const Prob &P, int64_t o, int cam,
     for (int k = 0; k < 18; ++k) Jc[k] *= sw;
 #pragma unroll
     for (int k = 0; k < 6; ++k) Jp[k] *= sw;
-    if (FACT) {  // factored form: (px, py, 1/Pz), W Jp and, with a loss, sqrt(W)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) P.PXpm[k * np_ + o] = (float)pz[k];
+    for (int k = 0; k < 18; ++k) J[k * np_ + o] = Jc[k];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) P.Jph[k * np_ + o] = (float)(sw * Jp[k]);
-        if (P.swpm) P.swpm[o] = (float)sw;
-    } else {
-#pragma unroll
-        for (int k = 0; k < 18; ++k) J[k * np_ + o] = Jc[k];
-#pragma unroll
-        for (int k = 0; k < 6; ++k) J[(18 + k) * np_ + o] = Jp[k];
-    }
+    for (int k = 0; k < 6; ++k) J[(18 + k) * np_ + o] = Jp[k];
     e[0] *= sw;
     e[1] *= sw;
     res[o] = e[0];
@@ -258,6 +318,126 @@ __global__ void __launch_bounds__(kBlock, 4) lin_point_kernel(Prob P, int force)
     }
 }
 
+// H = W Jp^T Jp, g = W Jp^T p and r2 of one observation (h = W Jp), as pairs.
+__device__ __forceinline__ void store_hg(double2 *o, int64_t st, const double *h, const double *Jp, const double *pz) {
+    o[0] = make_double2(h[0] * Jp[0] + h[3] * Jp[3], h[0] * Jp[1] + h[3] * Jp[4]);
+    o[st] = make_double2(h[0] * Jp[2] + h[3] * Jp[5], h[1] * Jp[1] + h[4] * Jp[4]);
+    o[2 * st] = make_double2(h[1] * Jp[2] + h[4] * Jp[5], h[2] * Jp[2] + h[5] * Jp[5]);
+    o[3 * st] = make_double2(h[0] * pz[0] + h[3] * pz[1], h[1] * pz[0] + h[4] * pz[1]);
+    o[4 * st] = make_double2(h[2] * pz[0] + h[5] * pz[1], pz[0] * pz[0] + pz[1] * pz[1]);
+}
+
+// Point-major linearisation of the factored form over slices: per observation
+// (px, py, 1/P_z) and, with a loss, W; per point C = sum W Jp^T Jp and w = -sum
+// W Jp^T e, summed in the point's lanes.
+// SMEM: the CTA first copies R, t, f, k1, k2 of every camera into shared memory
+// (stride kRowS), so that the per-observation camera read is four 16-byte
+// shared loads instead of a gather through L1.
+// FP64: H = W Jp^T Jp, g = W Jp^T p, r2 (and W) per observation for the
+// block-owned product; the table has 15 doubles per camera (odd: few conflicts).
+template <typename T, bool SMEM>
+__global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512, 1) lin_slices_kernel(Prob P, int force) {
+    if (!force && (P.st->done || !P.st->relin)) return;
+    constexpr int TS = sizeof(T) == 4 ? kRowS : 15;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    T *s_tab = (T *)s_raw;
+    const T *__restrict__ camtab = (const T *)P.camtab;
+    if (SMEM) {
+        for (int e = threadIdx.x; e < 16 * P.nc; e += blockDim.x) {
+            const int cam = e >> 4, q = e & 15;
+            if (q < 15) s_tab[cam * TS + q] = __ldg(camtab + (int64_t)cam * kCamTab + (q < 9 ? q : q + 9));
+        }
+        __syncthreads();
+    }
+    const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+    const unsigned full = 0xffffffffu;
+    const T delta = (T)P.delta;
+    for (int w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < P.n_slices; w += gridDim.x * nwarp) {
+        const int4 sl = __ldg(P.slice + w);
+        const int K = sl.w & 0xffff, lg = sl.w >> 16, in = lane >> lg;
+        const int count = sl.y & 0xff;
+        const int s = sl.x + (in < count ? in : 0);
+        T X0, X1, X2;
+        if constexpr (sizeof(T) == 4) {
+            const float4 X = __ldg(P.sp_X + s);
+            X0 = X.x, X1 = X.y, X2 = X.z;
+        } else {
+            X0 = __ldg(P.sp_X64 + 4 * (int64_t)s), X1 = __ldg(P.sp_X64 + 4 * (int64_t)s + 1);
+            X2 = __ldg(P.sp_X64 + 4 * (int64_t)s + 2);
+        }
+        T q[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) q[k] = T(0);
+        for (int k = 0; k < K; ++k) {
+            const int64_t slot = (int64_t)sl.z + 32 * k + lane;
+            const int cam = __ldg(P.sl_cam + slot);
+            if (cam < 0) continue;
+            T ct[kCamTab];
+            if constexpr (sizeof(T) == 8) {
+                const T *src = SMEM ? s_tab + cam * TS : camtab + (int64_t)cam * kCamTab;
+#pragma unroll
+                for (int r = 0; r < 9; ++r) ct[r] = src[r];
+#pragma unroll
+                for (int r = 0; r < 6; ++r) ct[18 + r] = src[(SMEM ? 9 : 18) + r];
+            } else {
+                const float4 *src = (const float4 *)(SMEM ? s_tab + cam * TS : camtab + (int64_t)cam * kCamTab);
+                const float4 a = src[0], b = src[1], c = src[2], d = src[SMEM ? 3 : 4];
+                ct[0] = a.x, ct[1] = a.y, ct[2] = a.z, ct[3] = a.w, ct[4] = b.x, ct[5] = b.y, ct[6] = b.z, ct[7] = b.w;
+                ct[8] = c.x;
+                if (SMEM) {
+                    ct[18] = c.y, ct[19] = c.z, ct[20] = c.w, ct[21] = d.x, ct[22] = d.y, ct[23] = d.z;
+                } else {
+                    const float4 f = src[5];
+                    ct[18] = d.z, ct[19] = d.w, ct[20] = f.x, ct[21] = f.y, ct[22] = f.z, ct[23] = f.w;
+                }
+            }
+            T u0, u1;
+            if constexpr (sizeof(T) == 4) {
+                const float2 uv = __ldg(P.sl_uv32 + slot);
+                u0 = uv.x, u1 = uv.y;
+            } else {
+                const double2 uv = __ldg(P.sl_uv + slot);
+                u0 = uv.x, u1 = uv.y;
+            }
+            T e[2], Jc[18], Jp[6], pz[3];
+            project<T, true>(ct, X0, X1, X2, u0, u1, e, Jc, Jp, pz);
+            T rho, W;
+            loss_weight<T>(P.loss, delta, e[0] * e[0] + e[1] * e[1], &rho, &W);
+            T h[6];
+#pragma unroll
+            for (int r = 0; r < 6; ++r) h[r] = W * Jp[r];
+            if constexpr (sizeof(T) == 4) {
+                P.sl_px[slot] = make_float4(__int_as_float(cam), pz[0], pz[1], pz[2]);
+                if (P.sl_w) P.sl_w[slot] = W;
+            } else {
+                store_hg(P.sl_hg + slot, P.slot_cap, h, Jp, pz);
+                if (P.sl_w64) P.sl_w64[slot] = W;
+            }
+            q[0] += h[0] * Jp[0] + h[3] * Jp[3];
+            q[1] += h[0] * Jp[1] + h[3] * Jp[4];
+            q[2] += h[0] * Jp[2] + h[3] * Jp[5];
+            q[3] += h[1] * Jp[1] + h[4] * Jp[4];
+            q[4] += h[1] * Jp[2] + h[4] * Jp[5];
+            q[5] += h[2] * Jp[2] + h[5] * Jp[5];
+            q[6] -= h[0] * e[0] + h[3] * e[1];
+            q[7] -= h[1] * e[0] + h[4] * e[1];
+            q[8] -= h[2] * e[0] + h[5] * e[1];
+        }
+        for (int d = 1; d < (1 << lg); d <<= 1) {
+#pragma unroll
+            for (int k = 0; k < 9; ++k) q[k] += __shfl_xor_sync(full, q[k], d);
+        }
+        if (in < count && (lane & ((1 << lg) - 1)) == 0) {
+            const int64_t pt = __ldg(P.sp_pt + s);
+            const bool fixed = P.has_fixed && P.pt_fixed[pt];  // its Jacobian columns are zero
+#pragma unroll
+            for (int k = 0; k < 6; ++k) P.Hll[6 * pt + k] = fixed ? 0.0 : (double)q[k];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) P.w[3 * pt + k] = fixed ? 0.0 : (double)q[6 + k];
+        }
+    }
+}
+
 // One warp per camera chunk: each lane accumulates the 54 block terms of its
 // observations, then one shuffle tree per chunk (a CTA-wide reduction per
 // chunk of a few hundred observations cost as much as the Jacobians).
@@ -283,26 +463,37 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) lin_camera_ker
         // two-deep pipeline over this lane's observations (the point index two
         // ahead, the point and pixels one ahead), so that the dependent point
         // gather is in flight while the previous observation is worked
+        // the factored form gathers X in sorted point order
+        constexpr bool FACT = sizeof(T) == 4 && !AD;
+        const int32_t *__restrict__ cmp = FACT ? P.cm_sp : P.cm_pt;
+        auto point = [&](int at, T &x0, T &x1, T &x2) {
+            if constexpr (FACT) {
+                const float4 v = __ldg(P.sp_X + at);
+                x0 = v.x, x1 = v.y, x2 = v.z;
+            } else {
+                load_point<T>(P, at, x0, x1, x2);
+            }
+        };
         int s = b0 + lane;
-        int pa = s < b1 ? P.cm_pt[s] : 0;
-        int pb = s + 32 < b1 ? P.cm_pt[s + 32] : 0;
+        int pa = s < b1 ? cmp[s] : 0;
+        int pb = s + 32 < b1 ? cmp[s + 32] : 0;
         T Xa0 = T(0), Xa1 = T(0), Xa2 = T(0), ua0 = T(0), ua1 = T(0);
         if (s < b1) {
-            load_point<T>(P, pa, Xa0, Xa1, Xa2);
+            point(pa, Xa0, Xa1, Xa2);
             load_uv<T>(P.cm_uv, P.cm_uv32, s, ua0, ua1);
         }
         for (; s < b1; s += 32) {
             const int pt = pa;
             const T X0 = Xa0, X1 = Xa1, X2 = Xa2, u0 = ua0, u1 = ua1;
-            const int pc = s + 64 < b1 ? P.cm_pt[s + 64] : 0;
+            const int pc = s + 64 < b1 ? cmp[s + 64] : 0;
             if (s + 32 < b1) {
-                load_point<T>(P, pb, Xa0, Xa1, Xa2);
+                point(pb, Xa0, Xa1, Xa2);
                 load_uv<T>(P.cm_uv, P.cm_uv32, s + 32, ua0, ua1);
             }
             pa = pb;
             pb = pc;
             T e[2], Jc[18], Jp[6], pz[3];
-            edge_eval<T, AD, true, false>(ctab, X0, X1, X2, u0, u1, e, Jc, Jp, (sizeof(T) == 4 && !AD) ? pz : nullptr);
+            edge_eval<T, AD, true, false>(ctab, X0, X1, X2, u0, u1, e, Jc, Jp, AD ? nullptr : pz);
             zero_fixed_columns<T>(P, cam, pt, Jc, (T *)nullptr);
             T rho, W;
             loss_weight<T>(P.loss, delta, e[0] * e[0] + e[1] * e[1], &rho, &W);
@@ -313,15 +504,25 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) lin_camera_ker
             e[1] *= sw;
             // what the PCG camera pass reads in camera-major order: the stored
             // Jacobian (FP64, or any dual-number Jacobian), else the factored
-            // form's (R X, 1/Pz)
+            // form's (R X, 1 / P_z) and IRLS weight
             if ((sizeof(T) == 8 || AD) && P.JcmT) {
 #pragma unroll
                 for (int q = 0; q < 18; ++q) ((T *)P.JcmT)[(int64_t)q * P.npad + s] = Jc[q];
             }
-            if (sizeof(T) == 4 && !AD && P.fact) {
-                ((float4 *)P.RXcm)[s] = make_float4((float)(ctab[0] * X0 + ctab[1] * X1 + ctab[2] * X2),
-                                                    (float)(ctab[3] * X0 + ctab[4] * X1 + ctab[5] * X2),
-                                                    (float)(ctab[6] * X0 + ctab[7] * X1 + ctab[8] * X2), (float)pz[2]);
+            if constexpr (FACT) {
+                const float4 rx = make_float4(ctab[0] * X0 + ctab[1] * X1 + ctab[2] * X2, ctab[3] * X0 + ctab[4] * X1 + ctab[5] * X2,
+                                              ctab[6] * X0 + ctab[7] * X1 + ctab[8] * X2, pz[2]);
+                const int64_t o = P.own ? (int64_t)P.cm2r[s] : (int64_t)s;
+                (P.own ? P.r_rx : P.RXcm)[o] = rx;
+                if (P.loss != MBA_LOSS_NONE) (P.own ? P.r_w : P.cm_w)[o] = W;
+            }
+            if constexpr (sizeof(T) == 8 && !AD) {
+                if (P.own) {
+                    T h[6];
+#pragma unroll
+                    for (int r = 0; r < 6; ++r) h[r] = W * Jp[r];
+                    store_hg(P.r_hg + P.cm2r[s], P.rslot_cap, h, Jp, pz);
+                }
             }
             int idx = 0;
 #pragma unroll
@@ -424,11 +625,14 @@ cudaError_t launch_camera_tables(const Prob &P, const double *cams, bool for_lin
     const unsigned g = grid_for(P.nc, 128);
     if (for_lin) {
         if (P.fp32)
-            camera_table_kernel<float><<<g, 128, 0, s>>>(cams, P.nc, (float *)P.camtab, nullptr, nullptr, P.st, 1);
+            camera_table_kernel<float><<<g, 128, 0, s>>>(cams, P.nc, (float *)P.camtab, nullptr, nullptr, P.camstat,
+                                                         P.ctr, nullptr, P.st, 1);
         else
-            camera_table_kernel<double><<<g, 128, 0, s>>>(cams, P.nc, (double *)P.camtab, nullptr, nullptr, P.st, 1);
+            camera_table_kernel<double><<<g, 128, 0, s>>>(cams, P.nc, (double *)P.camtab, nullptr, nullptr, nullptr,
+                                                          nullptr, P.ctr64, P.st, 1);
     } else {
-        camera_table_kernel<double><<<g, 128, 0, s>>>(cams, P.nc, nullptr, P.camtab64, P.camff, P.st, 2);
+        camera_table_kernel<double><<<g, 128, 0, s>>>(cams, P.nc, nullptr, P.camtab64, P.camff, nullptr, nullptr,
+                                                      nullptr, P.st, 2);
     }
     return cudaGetLastError();
 }
@@ -436,9 +640,11 @@ cudaError_t launch_camera_tables(const Prob &P, const double *cams, bool for_lin
 cudaError_t launch_camera_tables_forced(const Prob &P, const double *cams, cudaStream_t s) {
     const unsigned g = grid_for(P.nc, 128);
     if (P.fp32)
-        camera_table_kernel<float><<<g, 128, 0, s>>>(cams, P.nc, (float *)P.camtab, P.camtab64, P.camff, P.st, 0);
+        camera_table_kernel<float><<<g, 128, 0, s>>>(cams, P.nc, (float *)P.camtab, P.camtab64, P.camff, P.camstat,
+                                                     P.ctr, nullptr, P.st, 0);
     else
-        camera_table_kernel<double><<<g, 128, 0, s>>>(cams, P.nc, (double *)P.camtab, P.camtab64, nullptr, P.st, 0);
+        camera_table_kernel<double><<<g, 128, 0, s>>>(cams, P.nc, (double *)P.camtab, P.camtab64, nullptr, nullptr,
+                                                      nullptr, P.ctr64, P.st, 0);
     return cudaGetLastError();
 }
 
@@ -451,9 +657,21 @@ cudaError_t launch_split_observations(const Prob &P, cudaStream_t s) {
 
 template <typename T, bool AD>
 static void launch_lin_pair(const Prob &P, int force, cudaStream_t s) {
-    int nbp = (P.n_wchunks + kWarps - 1) / kWarps;
-    if (nbp > 152 * 16) nbp = 152 * 16;
-    lin_point_kernel<T, AD><<<nbp < 1 ? 1 : nbp, kBlock, 0, s>>>(P, force);
+    if (!AD && P.n_slices > 0) {
+        // one CTA per SM, with as many warps as there are slices for it
+        const int smem = P.nc * (sizeof(T) == 4 ? kRowS * 4 : 15 * 8);
+        const SliceGrid g = slice_grid(P, sizeof(T) == 4 ? 1024 : 512);
+        if (smem <= 220 * 1024) {
+            cudaFuncSetAttribute(lin_slices_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            lin_slices_kernel<T, true><<<g.ctas, g.threads, smem, s>>>(P, force);
+        } else {
+            lin_slices_kernel<T, false><<<g.ctas, g.threads, 0, s>>>(P, force);
+        }
+    } else {
+        int nbp = (P.n_wchunks + kWarps - 1) / kWarps;
+        if (nbp > 152 * 16) nbp = 152 * 16;
+        lin_point_kernel<T, AD><<<nbp < 1 ? 1 : nbp, kBlock, 0, s>>>(P, force);
+    }
     int nbc = (P.n_cchunks + kWarps - 1) / kWarps;
     if (nbc > 152 * 16) nbc = 152 * 16;
     lin_camera_kernel<T, AD><<<nbc < 1 ? 1 : nbc, kBlock, 0, s>>>(P, force);
@@ -461,10 +679,13 @@ static void launch_lin_pair(const Prob &P, int force, cudaStream_t s) {
 
 cudaError_t launch_linearize_impl(const Prob &P, const int32_t *cfirst, int force, cudaStream_t s) {
     if (P.fp32) {
-        point_table_kernel<<<grid_for(P.np), kBlock, 0, s>>>(P.pts, P.np, P.pts32, P.st, force ? 0 : 1);
+        point_table_kernel<<<grid_for(P.np), kBlock, 0, s>>>(P.pts, P.fact ? P.sp_pt : nullptr, P.np,
+                                                             P.fact ? P.sp_X : P.pts32, P.st, force ? 0 : 1);
         if (P.autodiff) launch_lin_pair<float, true>(P, force, s);
         else launch_lin_pair<float, false>(P, force, s);
     } else {
+        if (P.own)
+            point_table64_kernel<<<grid_for(P.np), kBlock, 0, s>>>(P.pts, P.sp_pt, P.np, P.sp_X64, P.st, force ? 0 : 1);
         if (P.autodiff) launch_lin_pair<double, true>(P, force, s);
         else launch_lin_pair<double, false>(P, force, s);
     }

@@ -17,21 +17,15 @@ constexpr int kBlock = 256;          // threads per CTA for every kernel
 constexpr int kWarps = kBlock / 32;
 constexpr int kCamTab = 28;          // values per camera in the camera table
 constexpr int kVec = 12;             // padded stride of 9-vectors per camera (16-B aligned rows)
-constexpr int kRow = 12;             // floats per camera row of the factored FP32 Schur product
-// Staged point pass of the factored FP32 PCG: tiles of whole warp chunks copied
-// into shared memory by 1-D bulk copies.  A tile holds at most kTileObs
-// observations, kTilePts points and kTileChunks chunks; a stage holds one tile:
-// per observation the camera index, the camera-major position of s, W Jp (6) and
-// (px, py, 1/Pz) (3), each row with 8 words of slack for 16-byte rounding, then
-// the points' C~^-1 (6 floats each), their CSR offsets and the chunk table.
-constexpr int kTileObs = 1024, kTilePts = 384, kTileChunks = 31, kMaxStages = 4;
-constexpr int kTileRow = kTileObs + 8;
-constexpr int kStwSo = kTileRow, kStwJh = 2 * kTileRow, kStwPx = 8 * kTileRow, kStwCinv = 11 * kTileRow;
-constexpr int kStwPtp = kStwCinv + 6 * kTilePts + 8, kStwWch = kStwPtp + kTilePts + 8;
-constexpr int kStageWords = kStwWch + 2 * (kTileChunks + 4);
-constexpr int kStageBytes = (kStageWords * 4 + 127) & ~127;
-static_assert(kTileRow % 4 == 0 && kStwCinv % 4 == 0 && kStwPtp % 4 == 0 && kStwWch % 4 == 0,
-              "16-byte aligned stage rows");
+constexpr int kRowG = 16;            // floats per camera row of the factored FP32 Schur product in global memory
+constexpr int kRowS = 20;            // the same in shared memory: 80-byte rows put eight lanes' 16-byte loads of
+                                     // random rows into eight different bank groups (a 64-byte stride has two)
+constexpr int kRowD = 10;            // doubles per camera row of the block-owned FP64 product (m, a', v_f, v_a, v_b, flag)
+constexpr int kPartF = 12, kPartD = 10;  // stride of a camera's nine partial sums (FP32, FP64), for 16-byte stores
+constexpr int kOwnSmem = 218 * 1024; // dynamic shared memory the block-owned PCG kernel may use
+constexpr int kMaxParts = 16;        // parts a camera's run may be split into
+constexpr int kCtr = 28;             // stride of a camera's 9 x 3 row transform (27 values)
+constexpr int kCamStat = 12;         // per camera: f, k1, k2, the quaternion of R times sqrt 2 (w, x, y, z), t (3), pad
 constexpr int kCamChunk = 256;       // observations per camera-major chunk (at least)
 constexpr int kMaxTrack = 1024;      // longest supported point track
 
@@ -98,28 +92,62 @@ struct Prob {
     // the FP32 kernels convert nothing per observation (on GB300 a conversion from
     // FP64 runs on the FP64 pipe); null in FP64 problems
     float2 *pm_uv32, *cm_uv32;
-    float4 *pts32;
+    float4 *pts32;          // dual-number FP32 problems; the factored form reads X from sp_X
     // nodes held constant (mba_set_fixed): nonzero bytes mark fixed cameras and
     // points; has_fixed = 0 while none is fixed, so no kernel reads the masks
     uint8_t *cam_fixed, *pt_fixed;
     int32_t has_fixed;
-    // staged point pass (factored FP32 form): tiles (first chunk, end chunk) of
-    // whole warp chunks with <= 32 observations, tile t worked by CTA t mod grid;
-    // chunks of longer tracks are listed apart and read from global memory
-    int2 *tiles;
-    int4 *tdesc;            // per tile: (oa, ob, ca, cz), (pa, pz, wa, wz), (first chunk, end chunk, 0, 0):
-                            // the 16-byte-rounded copy ranges of its observation rows, C~^-1 floats,
-                            // CSR offsets and chunk entries
-    int32_t n_tiles;
-    int32_t *long_chunks;
-    int32_t n_long;
-    int32_t pcg_stages;     // stages of the staged point pass (0: not staged)
-    int32_t pcg_stage_off;  // byte offset of the stages in the PCG kernel's dynamic shared memory
+    // sliced point order (sell.cu): points sorted by decreasing track length, in
+    // slices of one warp.  A slice holds 32 / G points of one length class, G lanes
+    // per point, K = ceil(length / G) rounds; round k of a slice is the 32
+    // consecutive slots base + 32 k + lane, so lane-private sums replace the
+    // segmented scans and every stream over the slots is coalesced.
+    int32_t n_slices;
+    int64_t nslots;         // slots in use (a multiple of 32); the arrays hold `slot_cap`
+    int64_t slot_cap;
+    int4 *slice;            // (first sorted point, points | index of the first in its block << 8, first slot,
+                            //  K | log2 G << 16)
+    int32_t *sp_pt;         // sorted point -> point
+    int32_t *sl_cam;        // [slots] camera, -1 in padding (read by the linearisation and the FP64 form)
+    float2 *sl_uv32;        // [slots] pixels
+    float *sl_w;            // [slots] IRLS weight (null without a loss)
+    float4 *sl_px;          // [slots] (camera index as bits, px, py, 1 / P_z)
+    int32_t *cm_sp;         // camera-major: sorted point of each observation
+    float *cm_w;            // camera-major IRLS weight (null without a loss)
+    float4 *sp_X;           // sorted point order: X of the linearisation
+    float4 *sp_b;           // sorted point order: b = C~^-1 E^T p of the current product
+    float4 *RXcm;           // camera-major (R X, 1 / P_z)
+    float *camstat;         // [nc][kCamStat]
+    float *ctr;             // [nc][kCtr] row transform: row = ctr^T v (per group of three), c = ctr raw
+    int32_t np_pad;         // stride of the structure-of-arrays Cinv (sorted order)
+    int32_t sorted;         // 1: Cinv is [6][np_pad] in sorted point order, else [np][6]
+    // block-owned product (own.cu; analytic Jacobian, where own = 1)
+    int32_t own, nblk, n_vblk;  // blocks; rows of partial sums (blocks x parts)
+    int32_t own_pb;         // points of a block, at most (the stride of b in shared memory)
+    int32_t own_off_b, own_off_dots;  // byte offsets in the kernel's dynamic shared memory
+    int32_t r_lg;           // log2 of the lanes per run
+    int64_t rslot_cap;
+    int2 *rslice;           // per run slice: (first slot, rounds)
+    int2 *rlane;            // [run slices][32]: (camera or -1, row of the partial sums)
+    int32_t *blk_rslice;    // nblk + 1
+    int32_t *cm2r;          // camera-major position -> run slot
+    float4 *r_rx;           // FP32: [run slots] (R X, 1 / P_z)
+    uint16_t *r_pt16;       // FP32: the point's index in its block, 0xffff in padding
+    float *r_w;             // FP32: IRLS weight (null without a loss)
+    int32_t *r_pt;          // FP64: sorted point, -1 in padding
+    double2 *r_hg;          // FP64: [5][rslot_cap] pairs of H00 H01 H02 H11 H12 H22 g0 g1 g2 r2
+    double2 *sl_hg;         // FP64: [5][slot_cap] the same in slice order
+    double *sl_w64;         // FP64: [slot_cap] IRLS weight (null without a loss)
+    double2 *sl_uv;         // FP64: [slot_cap] pixels
+    double *sp_X64, *sp_b64;  // FP64: [np][4] sorted point order
+    double *ctr64;          // FP64: [nc][kCtr] row transform
+    void *c_part;           // [n_vblk][nc][kPartF / kPartD] T
     // chunk tables
     int32_t *cchunk_cam, *cchunk_beg;  // n_cchunks, n_cchunks + 1
     int32_t *cfirst;               // nc + 1: first camera chunk of each camera
     int32_t *cta_cam;              // grid + 1: cameras owned by each PCG CTA (balanced by observations)
     int32_t pcg_max_cta_chunks;    // most camera chunks any PCG CTA owns
+    int32_t pcg_max_cta_cams;      // most cameras any PCG CTA owns
     int32_t pcg_ps_bytes;          // shared-memory bytes of the search-direction copy
 
     // per-linearisation data (T = float in FP32-mixed, double otherwise)
@@ -132,17 +160,9 @@ struct Prob {
     double *Hll;    // [np][6] packed upper triangle of C
     double *w;      // [np][3]
     double *cpart;  // [n_cchunks][54] camera-chunk partial sums (the PCG reuses [n_cchunks][9])
-    void *zT;       // FP32-mixed: [nc][kVec] float copy of z
+    void *zT;       // FP32-mixed: [nc][kVec] float copy of z (factored form: its camera rows, without constants)
     void *pT2;      // FP32-mixed: second float search-direction buffer (alternate iterations)
     double *Jcm;    // FP64: [18][npad] sqrt(W)-scaled camera Jacobian, camera-major
-    // FP32-mixed analytic (factored) form: per observation the normalised point
-    // and 1 / P_z (point-major), the point rotated into the camera frame, R X,
-    // with 1 / P_z (camera-major), and the W-scaled point Jacobian, from which
-    // the PCG re-derives Jc p and Jc^T s with per-camera constants
-    float *PXpm;    // [3][npad] (px, py, 1/Pz), point-major
-    float *Jph;     // [6][npad] W Jp, point-major
-    float *RXcm;    // [npad] float4 (R X, 1/Pz), camera-major
-    float *swpm;    // [npad] sqrt(W), point-major (factored form with a robust loss; else null)
     // float-float copies for the FP32-mixed solve's cost (ff.cuh; else null)
     float2 *camff;  // [nc][16] R (9), t (3), f, k1, k2 of the cost's camera table
     float4 *uvff;   // [n] observations, point-major (u hi, u lo, v hi, v lo)
@@ -154,7 +174,7 @@ struct Prob {
     // per-solve data
     double *Bd;     // [nc][81] damped B~
     double *Binv;   // [nc][81] inverse of B~ (block-Jacobi preconditioner)
-    void *Cinv;     // [np][6] packed inverse of damped C~, T
+    void *Cinv;     // packed inverse of damped C~, T: [np][6]; factored form: [6][np_pad] in sorted point order
     // PCG vectors, [nc][kVec] FP64
     double *x, *r, *z, *p, *p2, *q, *g;  // p, p2: search directions of alternate iterations
     void *pT;       // [nc][kVec] search direction in T (point pass gathers when not in shared memory)
@@ -392,6 +412,11 @@ __device__ __forceinline__ void loss_weight(int loss, T delta, T s, T *rho, T *w
 template <typename T> __device__ __forceinline__ T ldcg(const T *p) { return __ldcg(p); }
 template <typename T> __device__ __forceinline__ void stcg(T *p, T v) { __stcg(p, v); }
 
+// Brings a line of a stream into L2 ahead of its load: the streams of a PCG
+// iteration exceed L2, and a warp's registers hold one round of them, too little
+// to cover the latency of HBM.
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Block-wide sum of one double per thread in a fixed tree order (shuffles in
 // each warp, then across the warp sums in warp 0); result valid in thread 0.
 // sbuf holds one double per warp (up to 32).
@@ -416,43 +441,6 @@ __device__ __forceinline__ double block_sum(double v, double *sbuf) {
 // acquire load sees k * gridDim.x.  A CTA that polls more than `limit` times, or sees the error
 // flag raised, records MBA_ERR_TIMEOUT and returns false; the caller must
 // then leave the kernel.  Returns true when every CTA has arrived.
-// ---------------------------------------------------------------------------
-// mbarrier and 1-D bulk copy (cp.async.bulk) helpers for shared-memory staging.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-// one arrival that also expects `bytes` of bulk-copy completions in this phase
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-// wait for the phase of the given parity to complete; false after `limit` polls
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, long long limit) {
-    for (long long i = 0; i < limit; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
-// global -> shared copy of `bytes` (a multiple of 16; both addresses 16-byte
-// aligned) completing on `bar`
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
-}
-
 __device__ __forceinline__ bool grid_barrier(DevState *st, uint32_t &epoch, long long limit) {
     __shared__ int s_ok;
     __syncthreads();
@@ -499,6 +487,28 @@ cudaError_t validate_inputs(const double *cams, int32_t nc, const double *pts, i
 cudaError_t gather_layout(Prob &P, const double *obs_in, const int32_t *ci, const int32_t *pi, int32_t *max_track,
                           int32_t *tmp_i, cudaStream_t s);
 cudaError_t build_pm2cm(Prob &P, int32_t *tmp_n, cudaStream_t s);
+
+// sell.cu: the sliced point order
+int64_t sell_slot_bound(int64_t n, int32_t np);
+int64_t sell_slice_bound(int64_t n, int32_t np);
+size_t sell_tmp_bytes(int32_t np);
+// own.cu: the block-owned layout
+bool own_wanted(const Prob &P, int grid);
+size_t own_tmp_bytes(const Prob &P, int64_t nblk);
+cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void **pool, size_t *pool_bytes, cudaStream_t s);
+// launch shape of a kernel that works whole slices per warp, one CTA per SM
+struct SliceGrid {
+    int ctas, threads;
+};
+inline SliceGrid slice_grid(const Prob &P, int most = 1024) {
+    int warps = (P.n_slices + 151) / 152;
+    if (warps < 2) warps = 2;
+    if (warps > most / 32) warps = most / 32;
+    const int need = (P.n_slices + warps - 1) / warps;
+    return SliceGrid{need < 152 ? (need < 1 ? 1 : need) : 152, 32 * warps};
+}
+cudaError_t build_slices(Prob &P, int grid, int max_track, void *tmp, size_t tmp_bytes, cudaStream_t s);
+bool over_memory_limit(size_t bytes);
 
 // linearize.cu
 cudaError_t launch_camera_tables(const Prob &P, const double *cams, bool for_lin, cudaStream_t s);

@@ -1,0 +1,231 @@
+// own.cu -- block-owned layout of the analytic Schur product (pcg_own_kernel).
+//
+// The sliced point order (sell.cu) is dealt to blocks, one per CTA of the PCG
+// kernel: slice i belongs to block i mod nblk.  A block owns its points, so
+// b_j = C~_j^-1 sum u never leaves the CTA, and the camera side of the product
+// runs over the block's own observations, grouped by camera: a run is the
+// observations of one camera in one block.  Runs are laid out like the point
+// slices, sorted by decreasing length, G lanes per run: round k of a run slice
+// is 32 consecutive slots, a run's nine sums stay in its lanes, and each run
+// ends in one store to the block's row of the partial sums, which the camera's
+// owner adds in block order.  Cameras with long runs (few cameras) are split
+// into parts, each with its own row.
+#include <algorithm>
+#include <vector>
+
+#include "mba_internal.cuh"
+
+namespace mba {
+
+namespace {
+
+__global__ void point_blocks_kernel(const int4 *__restrict__ slice, int32_t n_slices, int32_t nblk,
+                                    int2 *__restrict__ sp_bl) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_slices; i += gridDim.x * blockDim.x) {
+        const int4 s = slice[i];
+        const int count = s.y & 0xff, base = s.y >> 8;
+        for (int p = 0; p < count; ++p) sp_bl[s.x + p] = make_int2(i % nblk, base + p);
+    }
+}
+
+__global__ void obs_block_kernel(const int32_t *__restrict__ cm_sp, const int2 *__restrict__ sp_bl, int64_t n,
+                                 int32_t *__restrict__ key) {
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x)
+        key[s] = sp_bl[cm_sp[s]].x;
+}
+
+// run index block * nc + camera of every observation, in (block, camera) order
+__global__ void run_key_kernel(const int32_t *__restrict__ ord, const int32_t *__restrict__ key,
+                               const int32_t *__restrict__ cam_ptr, int32_t nc, int64_t n, int32_t *__restrict__ run,
+                               int32_t *__restrict__ count) {
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+        const int s = ord[t];
+        int lo = 0, hi = nc - 1;  // last camera with cam_ptr <= s
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (cam_ptr[mid] <= s) lo = mid;
+            else hi = mid - 1;
+        }
+        const int r = key[s] * nc + lo;
+        run[t] = r;
+        atomicAdd(count + r, 1);
+    }
+}
+
+__global__ void fill_runs_kernel(Prob P, const int32_t *__restrict__ ord, const int32_t *__restrict__ run,
+                                 const int32_t *__restrict__ run_ptr, const int32_t *__restrict__ base, int parts, int lg,
+                                 const int2 *__restrict__ sp_bl) {
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < P.n; t += (int64_t)gridDim.x * blockDim.x) {
+        const int s = ord[t], r = run[t], k = (int)(t - run_ptr[r]);
+        const int part = k % parts, kk = k / parts;
+        const int slot = base[(int64_t)r * parts + part] + 32 * (kk >> lg) + (kk & ((1 << lg) - 1));
+        P.cm2r[s] = slot;
+        const int sp = P.cm_sp[s];
+        if (P.r_pt16) P.r_pt16[slot] = (uint16_t)sp_bl[sp].y;
+        else P.r_pt[slot] = sp;
+    }
+}
+
+inline unsigned grid_for(int64_t n) {
+    int64_t g = (n + kBlock - 1) / kBlock;
+    if (g > 152 * 16) g = 152 * 16;
+    return (unsigned)(g < 1 ? 1 : g);
+}
+
+size_t al256(size_t v) { return (v + 255) & ~size_t(255); }
+
+}  // namespace
+
+// The block-owned product is used where the camera rows leave room in shared
+// memory and where the runs are long enough that the partial sums (written and
+// read once per product) cost less than the gathers of b they replace: at least
+// kMinRun observations on average, or partial sums of a few MB, which stay in L2.
+constexpr double kMinRun = 4.0;
+constexpr int64_t kSmallParts = 16 << 20;
+bool own_wanted(const Prob &P, int grid) {
+    const int64_t rows = (int64_t)P.nc * (P.fp32 ? kRowS * 4 : kRowD * 8);
+    const int64_t parts = (int64_t)grid * P.nc * (P.fp32 ? kPartF * 4 : kPartD * 8);
+    return rows + 40 * 1024 <= kOwnSmem && ((double)P.n >= kMinRun * (double)grid * P.nc || parts <= kSmallParts);
+}
+
+size_t own_tmp_bytes(const Prob &P, int64_t nblk) {
+    return al256(8 * (size_t)P.np) + 3 * al256(4 * (size_t)P.n) + 2 * al256(4 * ((size_t)nblk * P.nc + 2)) +
+           al256(4 * (size_t)nblk * P.nc * (P.nc < 128 ? kMaxParts : 1)) + 4 * (size_t)exclusive_scan_tmp_ints(nblk * P.nc + 2) + 1024 +
+           stable_sort_tmp_bytes(P.n, (int32_t)nblk + 1);
+}
+
+// Builds the run layout; allocates its arrays (OwnArrays, freed with the problem).
+cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void **pool, size_t *pool_bytes, cudaStream_t s) {
+    const int64_t nblk = P.nblk, nruns = nblk * P.nc;
+    if (tmp_bytes < own_tmp_bytes(P, nblk)) return cudaErrorInvalidValue;
+    char *t = (char *)tmp;
+    auto take = [&](size_t bytes) {
+        char *p = t;
+        t += al256(bytes);
+        return p;
+    };
+    int2 *sp_bl = (int2 *)take(8 * (size_t)P.np);
+    int32_t *key = (int32_t *)take(4 * (size_t)P.n), *ord = (int32_t *)take(4 * (size_t)P.n),
+            *run = (int32_t *)take(4 * (size_t)P.n);
+    int32_t *count = (int32_t *)take(4 * ((size_t)nruns + 2)), *run_ptr = (int32_t *)take(4 * ((size_t)nruns + 2));
+    int32_t *base_d = (int32_t *)take(4 * (size_t)nruns * (P.nc < 128 ? kMaxParts : 1));
+    int32_t *scan_tmp = (int32_t *)take(4 * (size_t)exclusive_scan_tmp_ints(nruns + 2));
+    const size_t sort_bytes = stable_sort_tmp_bytes(P.n, (int32_t)nblk + 1);
+
+    point_blocks_kernel<<<grid_for(P.n_slices), kBlock, 0, s>>>(P.slice, P.n_slices, P.nblk, sp_bl);
+    obs_block_kernel<<<grid_for(P.n), kBlock, 0, s>>>(P.cm_sp, sp_bl, P.n, key);
+    cudaError_t e = stable_sort_by_key(key, P.n, (int32_t)nblk, ord, run_ptr, t, sort_bytes, s);  // run_ptr: unused here
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(count, 0, 4 * ((size_t)nruns + 2), s);
+    if (e != cudaSuccess) return e;
+    run_key_kernel<<<grid_for(P.n), kBlock, 0, s>>>(ord, key, P.cam_ptr, P.nc, P.n, run, count);
+    e = exclusive_scan_i32(count, run_ptr, nruns + 1, scan_tmp, s);
+    if (e != cudaSuccess) return e;
+    std::vector<int32_t> len((size_t)nruns);
+    e = cudaMemcpyAsync(len.data(), count, 4 * (size_t)nruns, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return e;
+
+    // few cameras: split their runs until a block has work for a few hundred lanes
+    const double mean = (double)P.n / (double)nruns;
+    int parts = 1;
+    while (parts < kMaxParts && (int64_t)P.nc * parts < 128 && mean / parts > 16.0) parts *= 2;
+    P.n_vblk = (int32_t)(nblk * parts);
+    // shared memory: camera rows, b of a block's points (FP32) or the owner's
+    // group sums over them, dot products
+    // lanes per run, no more than the mean run fills.  FP32: a few rounds of the
+    // CTA's warps.  FP64: two where the runs then still fit its 512 lanes twice,
+    // more only to give the FP64 pipe a handful of warps (the reduction of nine
+    // values over a run's lanes takes a third of a round's pipe time per level)
+    int lg = 0;
+    const int64_t items_blk = (int64_t)P.nc * parts;
+    while (lg < 3 && (2 << lg) <= mean / parts &&
+           (items_blk << (lg + 1)) <= (P.fp32 ? 4096 : (lg == 0 ? 1024 : 256)))
+        ++lg;
+    const int G = 1 << lg, per = 32 / G;
+
+    std::vector<int32_t> base((size_t)nruns * parts, 0), blk((size_t)nblk + 1);
+    std::vector<int2> rs, lanes;
+    int64_t slots = 0;
+    std::vector<int32_t> order, bucket;
+    for (int64_t b = 0; b < nblk; ++b) {
+        blk[b] = (int32_t)rs.size();
+        // the block's (camera, part) pairs by decreasing length: counting sort
+        const int32_t *l = len.data() + b * P.nc;
+        const int64_t items = (int64_t)P.nc * parts;
+        auto part_len = [&](int64_t it) { return (int32_t)((l[it / parts] + parts - 1 - it % parts) / parts); };
+        int32_t longest = 0;
+        for (int32_t c = 0; c < P.nc; ++c) longest = std::max(longest, (l[c] + parts - 1) / parts);
+        bucket.assign((size_t)longest + 2, 0);
+        for (int64_t it = 0; it < items; ++it) bucket[(size_t)(longest - part_len(it)) + 1]++;
+        for (size_t k = 1; k < bucket.size(); ++k) bucket[k] += bucket[k - 1];
+        const int32_t used = bucket[(size_t)longest];  // those of length >= 1
+        order.resize((size_t)items);
+        for (int64_t it = 0; it < items; ++it) order[(size_t)bucket[(size_t)(longest - part_len(it))]++] = (int32_t)it;
+        for (int32_t q0 = 0; q0 < used; q0 += per) {
+            const int K = (part_len(order[q0]) + G - 1) >> lg;
+            rs.push_back(make_int2((int32_t)slots, K));
+            for (int j = 0; j < per; ++j) {
+                const int32_t q = q0 + j;
+                int2 ln = make_int2(-1, 0);
+                if (q < used) {
+                    const int64_t it = order[q], cam = it / parts, part = it % parts;
+                    base[(size_t)((b * P.nc + cam) * parts + part)] = (int32_t)slots + j * G;
+                    ln = make_int2((int32_t)cam, (int32_t)(b * parts + part));
+                }
+                for (int g = 0; g < G; ++g) lanes.push_back(ln);
+            }
+            slots += 32 * (int64_t)K;
+        }
+        if (slots > 2000000000ll) return cudaErrorInvalidValue;
+    }
+    blk[nblk] = (int32_t)rs.size();
+    P.r_lg = lg;
+    P.rslot_cap = (slots + 31) / 32 * 32;
+
+    // arrays
+    const bool loss = P.loss != MBA_LOSS_NONE;
+    const size_t ns = (size_t)P.rslot_cap, part_vals = (size_t)P.n_vblk * P.nc * (P.fp32 ? kPartF : kPartD);
+    for (int pass = 0; pass < 2; ++pass) {
+        char *q = (char *)*pool;
+        size_t off = 0;
+        auto arr = [&](size_t bytes) -> void * {
+            void *p = pass ? q + off : nullptr;
+            off += al256(bytes ? bytes : 1);
+            return p;
+        };
+        P.rslice = (int2 *)arr(8 * rs.size());
+        P.rlane = (int2 *)arr(8 * lanes.size());
+        P.blk_rslice = (int32_t *)arr(4 * blk.size());
+        P.cm2r = (int32_t *)arr(4 * (size_t)P.n);
+        P.c_part = arr(part_vals * (P.fp32 ? 4 : 8));
+        if (P.fp32) {
+            P.r_rx = (float4 *)arr(16 * ns);
+            P.r_pt16 = (uint16_t *)arr(2 * ns);
+            P.r_w = loss ? (float *)arr(4 * ns) : nullptr;
+        } else {
+            P.r_pt = (int32_t *)arr(4 * ns);
+            P.r_hg = (double2 *)arr(80 * ns);
+        }
+        if (pass == 0) {
+            *pool_bytes = off;
+            if (over_memory_limit(off)) return cudaErrorMemoryAllocation;
+            e = cudaMalloc(pool, off);
+            if (e != cudaSuccess) return e;
+        }
+    }
+    e = cudaMemcpyAsync(P.rslice, rs.data(), 8 * rs.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(P.rlane, lanes.data(), 8 * lanes.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(P.blk_rslice, blk.data(), 4 * blk.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(base_d, base.data(), 4 * base.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(P.c_part, 0, part_vals * (P.fp32 ? 4 : 8), s);
+    if (e == cudaSuccess)
+        e = P.fp32 ? cudaMemsetAsync(P.r_pt16, 0xff, 2 * ns, s) : cudaMemsetAsync(P.r_pt, 0xff, 4 * ns, s);
+    if (e != cudaSuccess) return e;
+    fill_runs_kernel<<<grid_for(P.n), kBlock, 0, s>>>(P, ord, run, run_ptr, base_d, parts, lg, sp_bl);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host vectors go out of scope
+    return e;
+}
+
+}  // namespace mba

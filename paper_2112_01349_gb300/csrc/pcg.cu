@@ -2,15 +2,16 @@
 // camera system (Alg. 2) with the implicit Schur product (Alg. 3), and the
 // point back-substitution (Sec. 3 Eq. 4) with the linear model decrease.
 //
-// Implicit product S p = B~ p - E C~^-1 E^T p, one pass over the point-major
-// observation stream per PCG iteration:
+// Implicit product S p = B~ p - E C~^-1 E^T p, a point pass and a camera pass
+// per PCG iteration:
 //   per observation  t_k = Jc~_k p_i(k),  u_k = Jp~_k^T t_k        (E^T p)
 //   per point        b_j = C~_j^-1 sum_k u_k                       (C~^-1)
 //   per observation  y_k = Jc~_k^T (Jp~_k b_j) added into camera i(k) (E b)
-// so the 24 Jacobian values of each observation are read once per iteration.
 // The camera-side work (B~ p, the preconditioner B~^-1 r, dot products,
 // axpys) is FP64 in both precisions, spread over all CTAs, three cameras per
 // warp, with bounded grid barriers between the phases.
+#include <type_traits>
+
 #include "mba_internal.cuh"
 
 namespace mba {
@@ -125,7 +126,10 @@ __global__ void damp_points_kernel(Prob P, int damping) {
     if (st->done) return;
     const double mu = current_mu(st);
     T *Ci = (T *)P.Cinv;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < P.np; j += (int64_t)gridDim.x * blockDim.x) {
+    const bool sorted = P.sorted != 0;  // [6][np_pad] in sorted point order, else [np][6]
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < P.np; s += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = sorted ? __ldg(P.sp_pt + s) : s;
+        const int64_t base = sorted ? s : 6 * j, step = sorted ? P.np_pad : 1;
         const double *h = P.Hll + 6 * j;
         const double a00 = h[0] + mu * damp_term(damping, h[0]), a01 = h[1], a02 = h[2];
         const double a11 = h[3] + mu * damp_term(damping, h[3]), a12 = h[4];
@@ -137,12 +141,12 @@ __global__ void damp_points_kernel(Prob P, int damping) {
             continue;
         }
         const double id = 1.0 / det;
-        Ci[6 * j + 0] = (T)(c00 * id);
-        Ci[6 * j + 1] = (T)(c01 * id);
-        Ci[6 * j + 2] = (T)(c02 * id);
-        Ci[6 * j + 3] = (T)((a00 * a22 - a02 * a02) * id);
-        Ci[6 * j + 4] = (T)((a02 * a01 - a00 * a12) * id);
-        Ci[6 * j + 5] = (T)((a00 * a11 - a01 * a01) * id);
+        Ci[base] = (T)(c00 * id);
+        Ci[base + step] = (T)(c01 * id);
+        Ci[base + 2 * step] = (T)(c02 * id);
+        Ci[base + 3 * step] = (T)((a00 * a22 - a02 * a02) * id);
+        Ci[base + 4 * step] = (T)((a02 * a01 - a00 * a12) * id);
+        Ci[base + 5 * step] = (T)((a00 * a11 - a01 * a01) * id);
     }
 }
 
@@ -174,18 +178,25 @@ __global__ void __launch_bounds__(kBlock) sj_camera_kernel(Prob P) {
 #pragma unroll
         for (int q = 0; q < 45; ++q) acc[q] = T(0);
         for (int s = b0 + threadIdx.x; s < b1; s += kBlock) {
+            constexpr bool FACT = sizeof(T) == 4 && !AD;
             const int pt = P.cm_pt[s];
-            T X0, X1, X2, u0, u1;
-            load_point<T>(P, pt, X0, X1, X2);
+            T X0, X1, X2, u0, u1, c6[6];
+            const int64_t sp = P.sorted ? P.cm_sp[s] : 0;
+            if constexpr (FACT) {
+                const float4 X = P.sp_X[sp];
+                X0 = X.x, X1 = X.y, X2 = X.z;
+            } else {
+                load_point<T>(P, pt, X0, X1, X2);
+            }
+#pragma unroll
+            for (int q = 0; q < 6; ++q) c6[q] = P.sorted ? Ci[q * P.np_pad + sp] : Ci[6 * (int64_t)pt + q];
             load_uv<T>(P.cm_uv, P.cm_uv32, s, u0, u1);
             T e[2], Jc[18], Jp[6];
             edge_eval<T, AD>(ctab, X0, X1, X2, u0, u1, e, Jc, Jp);
             zero_fixed_columns<T>(P, cam, pt, Jc, Jp);
             T rho, W;
             loss_weight<T>(P.loss, delta, e[0] * e[0] + e[1] * e[1], &rho, &W);
-            T c6[6], q0[3], q1[3];
-#pragma unroll
-            for (int q = 0; q < 6; ++q) c6[q] = Ci[6 * (int64_t)pt + q];
+            T q0[3], q1[3];
             // Q = Jp C~^-1 (rows), G = W^2 Q Jp^T
             q0[0] = c6[0] * Jp[0] + c6[1] * Jp[1] + c6[2] * Jp[2];
             q0[1] = c6[1] * Jp[0] + c6[3] * Jp[1] + c6[4] * Jp[2];
@@ -482,478 +493,241 @@ __device__ void point_pass(const Prob &P, const T *ps, const T *pT, typename V2<
 // (M: the rotation factor of the camera table).  Because R (a x b) = R a x R b,
 // the two products the PCG needs reduce to per-observation data and
 // per-camera constants:
-//   Jc v = D (n x (P - t) + v_t) + p (d v_f + f r2 v_k1 + f r2^2 v_k2),   n = R M v_w,
-//   sum_k Jc_k^T s_k = [ (R M)^T sum_k RX_k x D_k^T s_k ; sum_k D_k^T s_k ;
-//                        (sum_k d p.s, f sum_k r2 p.s, f sum_k r2^2 p.s) ],
-// RX = R X = P - t.  The point pass streams (px, py, 1/P_z) and W Jp, 36 bytes
-// per observation instead of the 96-byte Jacobian, and forms
+//   Jc v = D (n x (P - t) + v_t) + p (v_f + r2 (v_a + r2 v_b)),
+//          n = R M v_w,  v_a = k1 v_f + f v_k1,  v_b = k2 v_f + f v_k2;
+//   sum_k Jc_k^T s_k = [ (R M)^T sum_k RX_k x y_k ; sum_k y_k ;
+//                        (S0 + k1 S1 + k2 S2, f S1, f S2) ],
+//          y_k = D_k^T s_k,  S_m = sum_k r2^m p.s,  RX = R X = P - t.
+// The two triples of camera transforms are transposes of each other (P.ctr).
+//
+// Point pass (sliced order, sell.cu): per observation the camera index and
+// (px, py, 1/P_z), 16 bytes, and the camera's row from shared memory;
+// u = Jp^T t = R^T D^T t, R from its quaternion (two cross products), so that a
+// row is 16 floats, four 16-byte shared loads, which bound the pass.  It forms
 // (n x (P - t) + v_t) / P_z = n x (-px, -py, 1) + h / P_z with the camera
 // constant h = v_t - n x t: one cancellation of order |t| / |RX| per
-// observation.  The camera pass reads (RX, 1/P_z) as one float4 and recomputes
-// p from P = RX + t, so its cross products, summed over a chunk of hundreds of
-// observations, use RX itself: forming them as P_z q - t instead would cancel
-// after the sum, and that loss broke the PCG near mu ~ 1e-7.
+// observation.
+// Camera pass: per observation (RX, 1/P_z), the point index and one 16-byte
+// gather of b_j; the camera is uniform in the warp, so s = Jp b and Jc^T s are
+// formed in registers.  Gathering (X, b) as one 32-byte record and recomputing
+// the projection took 35.1 against 33.4 us on the Venice-shaped problem and 264
+// against 225 on the Final-shaped one: the pass is bound by the gathers, which an
+// SM issues at about one per two cycles.  The cross products,
+// summed over hundreds of observations, use RX itself: forming them from P and t
+// instead would cancel after the sum, and that loss broke the PCG near mu ~ 1e-7.
+// Against the form that streamed (px, py, 1/P_z) and W Jp point-major, scattered
+// s = Jp b into camera-major order and streamed it back with (RX, 1/P_z), 76
+// bytes per observation and a segmented shuffle scan per chunk: see the figures
+// at pcg_kernel.
 // (In the first-order rotation branch, |w|^2 <= 2.2e-16, both apply
 // R = I + [w]x where the Jacobian has I: a relative difference of at most |w|,
 // below FP32 rounding.)
 //
-// Per-camera row of kRow = 12 floats for a vector v = (v_w, v_t, v_f, v_k1, v_k2):
-//   n = R M v_w, h = v_t - n x t, e = (v_f, f v_k1, f v_k2), then (f, k1, k2)
-//   (consts) or zeros.  The row is linear in v apart from the constants, so
-//   row(z) + beta row(p) with the constants carried by row(z) alone is the row
-//   of z + beta p.
+// Camera row of a vector v: n (3), h (3), v_f, v_a, v_b; in shared memory and in
+// the global copy followed by f, k1, k2 and the quaternion (P.camstat).  The
+// first nine are linear in v, so row(z) + beta row(p) is the row of z + beta p.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void fact_row(const float *__restrict__ ct, const float *v, bool consts, float *r) {
-    const float m0 = ct[9] * v[0] + ct[10] * v[1] + ct[11] * v[2];
-    const float m1 = ct[12] * v[0] + ct[13] * v[1] + ct[14] * v[2];
-    const float m2 = ct[15] * v[0] + ct[16] * v[1] + ct[17] * v[2];
-    const float n0 = ct[0] * m0 + ct[1] * m1 + ct[2] * m2;
-    const float n1 = ct[3] * m0 + ct[4] * m1 + ct[5] * m2;
-    const float n2 = ct[6] * m0 + ct[7] * m1 + ct[8] * m2;
-    const float t0 = ct[18], t1 = ct[19], t2 = ct[20], f = ct[21];
-    r[0] = n0;
-    r[1] = n1;
-    r[2] = n2;
-    r[3] = v[3] - (n1 * t2 - n2 * t1);
-    r[4] = v[4] - (n2 * t0 - n0 * t2);
-    r[5] = v[5] - (n0 * t1 - n1 * t0);
-    r[6] = v[6];
-    r[7] = f * v[7];
-    r[8] = f * v[8];
-    r[9] = consts ? f : 0.f;
-    r[10] = consts ? ct[22] : 0.f;
-    r[11] = consts ? ct[23] : 0.f;
-}
 
 // Warp-collective (all 32 lanes call it): lanes 9s..9s+8 hold the nine
-// components of camera `cam` (lane s of the three-camera group); each active
-// lane writes its element of the camera's row to dst[cam][kRow] (lanes of rows
-// 0..2 also the elements 9..11).
-__device__ __forceinline__ void fact_row_store(const Prob &P, float *dst, int cam, bool act, double val, int sub,
-                                               int row, bool consts) {
-    const float fv = (float)val;
-    float v[9];
-#pragma unroll
-    for (int j = 0; j < 9; ++j) v[j] = __shfl_sync(0xffffffffu, fv, (9 * sub + j) & 31);
-    if (!act) return;
-    float r[kRow];
-    fact_row((const float *)P.camtab + (int64_t)cam * kCamTab, v, consts, r);
-    float mine = r[0], pad = r[9];
-#pragma unroll
-    for (int j = 1; j < 9; ++j)
-        if (row == j) mine = r[j];
-    if (row == 1) pad = r[10];
-    if (row == 2) pad = r[11];
-    stcg(dst + (int64_t)cam * kRow + row, mine);
-    if (row < 3) stcg(dst + (int64_t)cam * kRow + 9 + row, pad);
-}
-
-// The camera's row: shared memory (ps, [nc][kRow]) or the global copy.
-__device__ __forceinline__ void gather_row(const float *ps, const float *pT, int cam, float *r) {
-    float4 q[kRow / 4];
-    if (ps) {
-        const float4 *src = (const float4 *)(ps + cam * kRow);
-#pragma unroll
-        for (int i = 0; i < kRow / 4; ++i) q[i] = src[i];
-    } else {
-        const float4 *src = (const float4 *)(pT + (int64_t)cam * kRow);
-#pragma unroll
-        for (int i = 0; i < kRow / 4; ++i) q[i] = __ldcg(src + i);
-    }
-#pragma unroll
-    for (int i = 0; i < kRow / 4; ++i) {
-        r[4 * i] = q[i].x;
-        r[4 * i + 1] = q[i].y;
-        r[4 * i + 2] = q[i].z;
-        r[4 * i + 3] = q[i].w;
-    }
-}
-
-// t = Jc v (unscaled) for one observation from (px, py, 1/Pz) and the camera's row.
-__device__ __forceinline__ void fact_jc_v(float px, float py, float iz, const float *r, float *t) {
-    const float f = r[9], k1 = r[10], k2 = r[11];
-    const float r2 = px * px + py * py;
-    const float d = 1.f + k1 * r2 + k2 * r2 * r2;
-    const float dd = 2.f * k1 + 4.f * k2 * r2;
-    const float a00 = f * (d + dd * px * px), a01 = f * dd * px * py, a11 = f * (d + dd * py * py);
-    // (n x (P - t) + v_t) / P_z = n x (-px, -py, 1) + h / P_z
-    const float w0 = r[1] + r[2] * py + iz * r[3];
-    const float w1 = -r[0] - r[2] * px + iz * r[4];
-    const float w2 = r[1] * px - r[0] * py + iz * r[5];
-    const float z0 = w0 + px * w2, z1 = w1 + py * w2;
-    const float ei = r[6] * d + r2 * (r[7] + r2 * r[8]);
-    t[0] = -(a00 * z0 + a01 * z1) + px * ei;
-    t[1] = -(a01 * z0 + a11 * z1) + py * ei;
-}
-
-// One point with a long track (more than 32 observations, one warp): two
-// sweeps over 32-observation slices, reading global memory.
-template <bool RHS>
-__device__ void long_chunk_fact(const Prob &P, const float *ps, const float *pT, float2 *sbuf, int pt, int o0, int m) {
-    const float *__restrict__ Jh = P.Jph;
-    const float *__restrict__ PX = P.PXpm;
-    const int64_t npad = P.npad;
-    const int lane = threadIdx.x & 31;
+// components of camera `cam` (lane s of the three-camera group); returns the
+// lane's component of the camera's row.
+__device__ __forceinline__ float fact_row_lane(const Prob &P, int cam, double val, int sub, int row) {
     const unsigned full = 0xffffffffu;
-    float ci[6], b[3];
-    load_sym3((const float *)P.Cinv + 6 * (int64_t)pt, ci);
-    if (RHS) {
-        apply_sym3(ci, (float)P.w[3 * (int64_t)pt], (float)P.w[3 * (int64_t)pt + 1], (float)P.w[3 * (int64_t)pt + 2],
-                   b);
-    } else {
-        float a[3] = {0.f, 0.f, 0.f};
-        for (int base = 0; base < m; base += 32) {
-            if (base + lane < m) {
-                const int64_t o = (int64_t)o0 + base + lane;
-                float r[kRow], t[2];
-                gather_row(ps, pT, __ldcs(P.pm_cam + o), r);
-                fact_jc_v(__ldcs(PX + o), __ldcs(PX + npad + o), __ldcs(PX + 2 * npad + o), r, t);
+    const float v = (float)val;
+    const int g0 = row < 3 ? 0 : (row < 6 ? 3 : 6), b = row - g0, at = 9 * sub + g0;
+    const float *ct = P.ctr + (int64_t)cam * kCtr + 3 * g0 + b;
+    float r = 0.f;
 #pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    a[q] += __ldcs(Jh + q * npad + o) * t[0] + __ldcs(Jh + (3 + q) * npad + o) * t[1];
-            }
-        }
-#pragma unroll
-        for (int dl = 16; dl > 0; dl >>= 1) {
-            a[0] += __shfl_xor_sync(full, a[0], dl);
-            a[1] += __shfl_xor_sync(full, a[1], dl);
-            a[2] += __shfl_xor_sync(full, a[2], dl);
-        }
-        apply_sym3(ci, a[0], a[1], a[2], b);
+    for (int i = 0; i < 3; ++i) r = fmaf(__ldg(ct + 3 * i), __shfl_sync(full, v, (at + i) & 31), r);
+    // h = v_t - n x t
+    const int b1 = b == 2 ? 0 : b + 1, b2 = b == 0 ? 2 : b - 1;
+    const float n1 = __shfl_sync(full, r, (9 * sub + b1) & 31), n2 = __shfl_sync(full, r, (9 * sub + b2) & 31);
+    if (g0 == 3) {
+        const float *t = P.camstat + (int64_t)cam * kCamStat + 7;
+        r -= n1 * __ldg(t + b2) - n2 * __ldg(t + b1);
     }
-    for (int base = 0; base < m; base += 32) {
-        if (base + lane < m) {
-            const int64_t o = (int64_t)o0 + base + lane;
-            float jh[6];
-#pragma unroll
-            for (int q = 0; q < 6; ++q) jh[q] = __ldcs(Jh + q * npad + o);
-            store_s<float>(sbuf, __ldcs(P.pm2cm + o), jh, b);
-        }
-    }
+    return r;
 }
 
-// Point pass of the factored form: as point_pass, with u = (W Jp)^T (Jc p)
-// and s = (W Jp) b, so the camera pass forms sum Jc^T s with unscaled Jc.
-template <bool RHS>
-__device__ void point_pass_fact(const Prob &P, const float *ps, const float *pT, float2 *sbuf) {
-    const float *__restrict__ Jh = P.Jph;
-    const float *__restrict__ PX = P.PXpm;
-    const float *__restrict__ Cinv = (const float *)P.Cinv;
-    const int64_t npad = P.npad;
-    const int lane = threadIdx.x & 31;
-    const int nwarp = blockDim.x >> 5;
-    const unsigned full = 0xffffffffu;
-    const int gstride = gridDim.x * nwarp;
-    int w = blockIdx.x * nwarp + (threadIdx.x >> 5);
-    int2 c0 = make_int2(0, 0), c1 = make_int2(0, 0);
-    if (w < P.n_wchunks) {
-        c0 = P.wchunk[w];
-        c1 = P.wchunk[w + 1];
-    }
-    for (; w < P.n_wchunks; w += gstride) {
-        const int wn = w + gstride;
-        int2 n0 = c0, n1 = c1;
-        if (wn < P.n_wchunks) {
-            n0 = P.wchunk[wn];
-            n1 = P.wchunk[wn + 1];
+// The whole row of one camera by one thread.
+__device__ __forceinline__ void fact_row(const Prob &P, int cam, const float *v, float *r) {
+    const float *ct = P.ctr + (int64_t)cam * kCtr, *st = P.camstat + (int64_t)cam * kCamStat;
+#pragma unroll
+    for (int g = 0; g < 3; ++g)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            float x = 0.f;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) x = fmaf(__ldg(ct + 9 * g + 3 * i + b), v[3 * g + i], x);
+            r[3 * g + b] = x;
         }
-        const int o0 = c0.y, m = c1.y - c0.y;
-        if (m <= 32) {
-            const bool act = lane < m;
-            const int64_t o = (int64_t)o0 + (act ? lane : 0);
-            // point of each lane from the chunk's point starts (whole points, <= 32 observations)
-            const int npts = c1.x - c0.x;
-            const int rs = lane < npts ? __ldg(P.pt_ptr + c0.x + lane) - o0 : 32;
-            const unsigned starts = __reduce_or_sync(full, rs < 32 ? (1u << rs) : 0u);
-            const int pt = act ? c0.x + __popc(starts & (0xffffffffu >> (31 - lane))) - 1 : -1 - lane;
-            const int cam = act ? __ldcs(P.pm_cam + o) : 0;
-            const int so = act ? __ldcs(P.pm2cm + o) : 0;  // where the camera pass reads s
-            float jh[6], ci[6];
+    const float t0 = st[7], t1 = st[8], t2 = st[9];
+    r[3] -= r[1] * t2 - r[2] * t1;
+    r[4] -= r[2] * t0 - r[0] * t2;
+    r[5] -= r[0] * t1 - r[1] * t0;
 #pragma unroll
-            for (int q = 0; q < 6; ++q) jh[q] = ci[q] = 0.f;
-            float px = 0.f, py = 0.f, iz = 0.f;
-            if (act) {
-#pragma unroll
-                for (int q = 0; q < 6; ++q) jh[q] = __ldcs(Jh + q * npad + o);
-                if (!RHS) {
-                    px = __ldcs(PX + o);
-                    py = __ldcs(PX + npad + o);
-                    iz = __ldcs(PX + 2 * npad + o);
-                }
-                load_sym3(Cinv + 6 * (int64_t)pt, ci);
-            }
-            float b[3] = {0.f, 0.f, 0.f};
-            if (RHS) {
-                if (act)
-                    apply_sym3(ci, (float)P.w[3 * (int64_t)pt], (float)P.w[3 * (int64_t)pt + 1],
-                               (float)P.w[3 * (int64_t)pt + 2], b);
-            } else {
-                float u[3] = {0.f, 0.f, 0.f};
-                if (act) {
-                    float r[kRow], t[2];
-                    gather_row(ps, pT, cam, r);
-                    fact_jc_v(px, py, iz, r, t);
-                    u[0] = jh[0] * t[0] + jh[3] * t[1];
-                    u[1] = jh[1] * t[0] + jh[4] * t[1];
-                    u[2] = jh[2] * t[0] + jh[5] * t[1];
-                }
-                // inclusive segmented scan keyed by point (segments are contiguous)
-#pragma unroll
-                for (int dl = 1; dl < 32; dl <<= 1) {
-                    const int kp = __shfl_up_sync(full, pt, dl);
-                    const float v0 = __shfl_up_sync(full, u[0], dl), v1 = __shfl_up_sync(full, u[1], dl),
-                                v2 = __shfl_up_sync(full, u[2], dl);
-                    if (lane >= dl && kp == pt) {
-                        u[0] += v0;
-                        u[1] += v1;
-                        u[2] += v2;
-                    }
-                }
-                const int nxt = __shfl_down_sync(full, pt, 1);
-                const bool tail = act && (lane == 31 || lane == m - 1 || nxt != pt);
-                const unsigned tails = __ballot_sync(full, tail);
-                float bt[3];
-                apply_sym3(ci, u[0], u[1], u[2], bt);
-                const unsigned mine = tails & (0xffffffffu << lane);
-                const int src = mine ? __ffs(mine) - 1 : lane;
-                b[0] = __shfl_sync(full, bt[0], src);
-                b[1] = __shfl_sync(full, bt[1], src);
-                b[2] = __shfl_sync(full, bt[2], src);
-            }
-            if (act) store_s<float>(sbuf, so, jh, b);
-        } else {
-            long_chunk_fact<RHS>(P, ps, pT, sbuf, c0.x, o0, m);
-        }
-        c0 = n0;
-        c1 = n1;
-    }
+    for (int q = 0; q < 7; ++q) r[9 + q] = st[q];
 }
 
-// ---------------------------------------------------------------------------
-// Staged point pass of the factored form (iterations and the single product;
-// the right-hand-side pass keeps point_pass_fact).  A producer/consumer
-// pipeline in shared memory: the CTA's last warp copies the CTA's tiles (tile t
-// belongs to CTA t mod grid) into S stages with 1-D bulk copies, each stage
-// completing on its "full" mbarrier; the other warps wait for a stage, work on
-// it from shared memory (one warp chunk each), and release it on its "empty"
-// mbarrier, which the producer waits on before refilling the stage.  There is no
-// CTA-wide barrier between tiles, so warps drift across tiles and the copies run
-// up to S tiles ahead of the slowest consumer.  The per-observation streams do
-// not change within a launch, so the producer also runs ahead into the next
-// pass, across the camera pass and the grid barriers.  Use index u of the CTA
-// (counted over the whole launch) lives in stage u mod S; its full phase has
-// parity (u / S) mod 2, and so has the empty phase that releases it.
-// ---------------------------------------------------------------------------
-struct StageOrg {
-    int32_t oa, ca, pa, wa;  // first index copied of the observation rows, C~^-1 floats, pt_ptr, chunk table
-    int32_t cb, ce;          // the tile's chunks [cb, ce)
-    int32_t ok, pad;         // 0: the tile did not fit its stage (not copied)
+// A point's b: written inside the PCG launch by other CTAs before a grid
+// barrier, so an ordinary load, not the read-only path.
+__device__ __forceinline__ float4 load_b(const float4 *at) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(at));
+    return v;
+}
+// 32 bytes by one load; ordinary coherent loads, for rows that other CTAs of
+// the same launch wrote before a grid barrier.
+__device__ __forceinline__ void load8(const float *at, float4 &x, float4 &y) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w), "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w)
+                 : "l"(at));
+}
+
+struct CamRow {
+    float n0, n1, n2, h0, h1, h2, vf, va, vb, f, k1, k2, q0, q1, q2, q3;
 };
-constexpr long long kStageSpin = 1ll << 20;  // polls of a stage barrier before giving up
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// Producer warp (all lanes): the copies of use `use` into stage use mod S, one
-// array per lane; d0..d2 is the tile's descriptor (in every lane).
-__device__ void stage_issue(const Prob &P, unsigned char *stages, uint64_t *full, StageOrg *org, int S, uint32_t use,
-                            int4 d0, int4 d1, int4 d2) {
-    const int lane = threadIdx.x & 31;
-    const int sidx = (int)(use % (uint32_t)S);
-    const int oa = d0.x, ob = d0.y, ca = d0.z, cz = d0.w, pa = d1.x, pz = d1.y, wa = d1.z, wz = d1.w;
-    const bool fits = d2.y > d2.x && ob - oa <= kTileRow && cz - ca <= 6 * kTilePts + 8 && pz - pa <= kTilePts + 8 &&
-                      wz - wa <= kTileChunks + 4 && d2.y - d2.x <= kTileChunks;
-    const uint32_t bo = 4u * (uint32_t)(ob - oa);
-    uint64_t *bar = full + sidx;
-    float *st = (float *)(stages + (size_t)sidx * kStageBytes);
-    if (lane == 0) {
-        org[sidx] = StageOrg{oa, ca, pa, wa, d2.x, d2.y, fits ? 1 : 0, 0};
-        const uint32_t total = 11u * bo + 4u * (uint32_t)(cz - ca) + 4u * (uint32_t)(pz - pa) + 8u * (uint32_t)(wz - wa);
-        mbar_arrive_expect_tx(bar, fits ? total : 0u);
-    }
-    __syncwarp();
-    if (!fits || lane >= 14) return;
-    const void *src;
-    void *dst;
-    uint32_t bytes = bo;
-    if (lane == 0) {
-        src = P.pm_cam + oa;
-        dst = st;
-    } else if (lane == 1) {
-        src = P.pm2cm + oa;
-        dst = st + kStwSo;
-    } else if (lane < 8) {
-        src = P.Jph + (int64_t)(lane - 2) * P.npad + oa;
-        dst = st + kStwJh + (lane - 2) * kTileRow;
-    } else if (lane < 11) {
-        src = P.PXpm + (int64_t)(lane - 8) * P.npad + oa;
-        dst = st + kStwPx + (lane - 8) * kTileRow;
-    } else if (lane == 11) {
-        src = (const float *)P.Cinv + ca;
-        dst = st + kStwCinv;
-        bytes = 4u * (uint32_t)(cz - ca);
-    } else if (lane == 12) {
-        src = P.pt_ptr + pa;
-        dst = st + kStwPtp;
-        bytes = 4u * (uint32_t)(pz - pa);
+// ps: shared memory (stride kRowS); otherwise the global rows (stride kRowG),
+// written by other CTAs before the last grid barrier, whose acquire orders
+// these loads after the writes.
+__device__ __forceinline__ CamRow load_row(const float *ps, const float *rows, int cam) {
+    float4 a, b, c, d;
+    if (ps) {
+        const float4 *src = (const float4 *)(ps + cam * kRowS);
+        a = src[0], b = src[1], c = src[2], d = src[3];
     } else {
-        src = P.wchunk + wa;
-        dst = st + kStwWch;
-        bytes = 8u * (uint32_t)(wz - wa);
+        load8(rows + (int64_t)cam * kRowG, a, b);
+        load8(rows + (int64_t)cam * kRowG + 8, c, d);
     }
-    bulk_g2s(dst, src, bytes, bar);
+    return CamRow{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, d.x, d.y, d.z, d.w};
 }
 
-// The arithmetic of one warp chunk (at most 32 observations) once its inputs
-// are in registers: t = Jc p from the camera row, u = (W Jp)^T t, the
-// segmented scan by point, b = C~^-1 u at each point's last lane, and
-// s = (W Jp) b written to the camera-major position so.
-__device__ __forceinline__ void chunk_tail(const float *ps, const float *pT, float2 *sbuf, bool act, int m, int pt,
-                                           int cam, int so, const float *jh, const float *ci, float px, float py,
-                                           float iz) {
+// A and the scaled camera-frame vector w of one observation, then t = Jc v.
+struct FactObs {
+    float a00, a01, a11, w0, w1, w2, ei;
+};
+__device__ __forceinline__ FactObs fact_obs(float px, float py, float iz, const CamRow &r) {
+    FactObs o;
+    const float r2 = px * px + py * py;
+    const float d = 1.f + r2 * (r.k1 + r.k2 * r2);
+    const float fd = r.f * d, fdd = r.f * (2.f * r.k1 + 4.f * r.k2 * r2);
+    const float gx = fdd * px;
+    o.a00 = fd + gx * px;
+    o.a01 = gx * py;
+    o.a11 = fd + fdd * py * py;
+    // (n x (P - t) + v_t) / P_z = n x (-px, -py, 1) + h / P_z
+    o.w0 = r.n1 + r.n2 * py + iz * r.h0;
+    o.w1 = -r.n0 - r.n2 * px + iz * r.h1;
+    o.w2 = r.n1 * px - r.n0 * py + iz * r.h2;
+    o.ei = r.vf + r2 * (r.va + r2 * r.vb);
+    return o;
+}
+__device__ __forceinline__ void fact_t(const FactObs &o, float px, float py, float &t0, float &t1) {
+    const float z0 = o.w0 + px * o.w2, z1 = o.w1 + py * o.w2;
+    t0 = px * o.ei - (o.a00 * z0 + o.a01 * z1);
+    t1 = py * o.ei - (o.a01 * z0 + o.a11 * z1);
+}
+// u += W Jp^T t = W R^T D^T t
+__device__ __forceinline__ void fact_jpt(const FactObs &o, const CamRow &r, float px, float py, float wiz, float t0,
+                                         float t1, float *u) {
+    const float y0 = -wiz * (o.a00 * t0 + o.a01 * t1), y1 = -wiz * (o.a01 * t0 + o.a11 * t1), y2 = px * y0 + py * y1;
+    const float c0 = r.q2 * y2 - r.q3 * y1, c1 = r.q3 * y0 - r.q1 * y2, c2 = r.q1 * y1 - r.q2 * y0;
+    u[0] += y0 - r.q0 * c0 + (r.q2 * c2 - r.q3 * c1);
+    u[1] += y1 - r.q0 * c1 + (r.q3 * c0 - r.q1 * c2);
+    u[2] += y2 - r.q0 * c2 + (r.q1 * c1 - r.q2 * c0);
+}
+
+struct FactStream {
+    int cam;
+    float px, py, iz, W;
+};
+__device__ __forceinline__ FactStream load_stream(const Prob &P, int64_t slot) {
+    const float4 v = __ldg(P.sl_px + slot);
+    return FactStream{__float_as_int(v.x), v.y, v.z, v.w, P.sl_w ? __ldg(P.sl_w + slot) : 1.f};
+}
+
+// The sum of W Jp^T Jc v over the lane's observations of one slice.
+__device__ __forceinline__ void fact_slice_sum(const Prob &P, const float *ps, const float *rows, int64_t slot, int K,
+                                               float *a) {
+    a[0] = a[1] = a[2] = 0.f;
+#pragma unroll 2
+    for (int k = 0; k < K; ++k, slot += 32) {
+        const FactStream c = load_stream(P, slot);
+        if (c.cam < 0) continue;
+        const CamRow r = load_row(ps, rows, c.cam);
+        const FactObs o = fact_obs(c.px, c.py, c.iz, r);
+        float t0, t1;
+        fact_t(o, c.px, c.py, t0, t1);
+        fact_jpt(o, r, c.px, c.py, c.W * c.iz, t0, t1, a);
+    }
+}
+
+// Point pass over this warp's slices: b_j = C~_j^-1 sum_k u_k into the record.
+// The stream of the next round (of this slice or the next one, whose
+// descriptor is read a slice ahead) is in flight while a round is worked.
+__device__ void point_pass_fact(const Prob &P, const float *ps, const float *rows) {
+    const float *__restrict__ Ci = (const float *)P.Cinv;
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    float u[3] = {0.f, 0.f, 0.f};
-    if (act) {
-        float r[kRow], t[2];
-        gather_row(ps, pT, cam, r);
-        fact_jc_v(px, py, iz, r, t);
-        u[0] = jh[0] * t[0] + jh[3] * t[1];
-        u[1] = jh[1] * t[0] + jh[4] * t[1];
-        u[2] = jh[2] * t[0] + jh[5] * t[1];
-    }
-    // inclusive segmented scan keyed by point (segments are contiguous)
-#pragma unroll
-    for (int dl = 1; dl < 32; dl <<= 1) {
-        const int kp = __shfl_up_sync(full, pt, dl);
-        const float v0 = __shfl_up_sync(full, u[0], dl), v1 = __shfl_up_sync(full, u[1], dl),
-                    v2 = __shfl_up_sync(full, u[2], dl);
-        if (lane >= dl && kp == pt) {
-            u[0] += v0;
-            u[1] += v1;
-            u[2] += v2;
+    const int gstride = gridDim.x * (blockDim.x >> 5);
+    int w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    if (w >= P.n_slices) return;
+    int4 sl = __ldg(P.slice + w);
+    FactStream cur = load_stream(P, (int64_t)sl.z + lane);
+    for (;;) {
+        const int wn = w + gstride;
+        const int4 nx = wn < P.n_slices ? __ldg(P.slice + wn) : sl;
+        const int K = sl.w & 0xffff, lg = sl.w >> 16, in = lane >> lg;
+        const int count = sl.y & 0xff;
+        const int s = sl.x + (in < count ? in : 0);
+        float a[3] = {0.f, 0.f, 0.f};
+        for (int k = 1; k <= K; ++k) {
+            const FactStream c = cur;
+            cur = load_stream(P, (int64_t)(k < K ? sl.z + 32 * k : nx.z) + lane);
+            prefetch_l2(P.sl_px + nx.z + 32 * (k < (nx.w & 0xffff) ? k : 0) + lane);
+            if (c.cam >= 0) {
+                const CamRow r = load_row(ps, rows, c.cam);
+                const FactObs o = fact_obs(c.px, c.py, c.iz, r);
+                float t0, t1;
+                fact_t(o, c.px, c.py, t0, t1);
+                fact_jpt(o, r, c.px, c.py, c.W * c.iz, t0, t1, a);
+            }
         }
+        float ci[6], b[3];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) ci[q] = __ldg(Ci + (int64_t)q * P.np_pad + s);
+        for (int d = 1; d < (1 << lg); d <<= 1) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) a[q] += __shfl_xor_sync(full, a[q], d);
+        }
+        if (in < count && (lane & ((1 << lg) - 1)) == 0) {
+            if (P.has_fixed && P.pt_fixed[P.sp_pt[s]]) a[0] = a[1] = a[2] = 0.f;
+            apply_sym3(ci, a[0], a[1], a[2], b);
+            P.sp_b[s] = make_float4(b[0], b[1], b[2], 0.f);
+        }
+        if (wn >= P.n_slices) return;
+        w = wn;
+        sl = nx;
     }
-    const int nxt = __shfl_down_sync(full, pt, 1);
-    const bool tail = act && (lane == 31 || lane == m - 1 || nxt != pt);
-    const unsigned tails = __ballot_sync(full, tail);
-    float bt[3], b[3];
-    apply_sym3(ci, u[0], u[1], u[2], bt);
-    const unsigned mine = tails & (0xffffffffu << lane);
-    const int src = mine ? __ffs(mine) - 1 : lane;
-    b[0] = __shfl_sync(full, bt[0], src);
-    b[1] = __shfl_sync(full, bt[1], src);
-    b[2] = __shfl_sync(full, bt[2], src);
-    if (act) store_s<float>(sbuf, so, jh, b);
 }
 
-// One warp chunk of a stage (at most 32 observations), as point_pass_fact with
-// every per-observation and per-point input read from the stage.
-__device__ __forceinline__ void staged_chunk(const float *ps, const float *pT, float2 *sbuf, const float *st,
-                                             const StageOrg &o, int k) {
-    const int lane = threadIdx.x & 31;
-    const unsigned full = 0xffffffffu;
-    const int *s_cam = (const int *)st, *s_so = (const int *)(st + kStwSo);
-    const float *s_jh = st + kStwJh, *s_px = st + kStwPx, *s_ci = st + kStwCinv;
-    const int *s_ptp = (const int *)(st + kStwPtp);
-    const int2 *s_wch = (const int2 *)(st + kStwWch);
-    const int2 c0 = s_wch[k - o.wa], c1 = s_wch[k + 1 - o.wa];
-    const int o0 = c0.y, m = c1.y - c0.y;  // at most 32: longer tracks are not in tiles
-    const bool act = lane < m;
-    const int li = o0 - o.oa + (act ? lane : 0);
-    const int npts = c1.x - c0.x;
-    const int rs = lane < npts ? s_ptp[c0.x + lane - o.pa] - o0 : 32;
-    const unsigned starts = __reduce_or_sync(full, rs < 32 ? (1u << rs) : 0u);
-    const int pt = act ? c0.x + __popc(starts & (0xffffffffu >> (31 - lane))) - 1 : -1 - lane;
-    float jh[6], ci[6], px = 0.f, py = 0.f, iz = 0.f;
-    int so = 0, cam = 0;
+// Right-hand side: b_j = C~_j^-1 w_j.
+__device__ void point_pass_fact_rhs(const Prob &P) {
+    const float *__restrict__ Ci = (const float *)P.Cinv;
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < P.np; s += gridDim.x * blockDim.x) {
+        const int64_t pt = __ldg(P.sp_pt + s);
+        float ci[6], b[3];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) jh[q] = ci[q] = 0.f;
-    if (act) {
-        so = s_so[li];
-        cam = s_cam[li];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) jh[q] = s_jh[q * kTileRow + li];
-        // C~^-1 of the point, from the stage (plain shared-memory loads)
-#pragma unroll
-        for (int q = 0; q < 6; ++q) ci[q] = s_ci[6 * pt - o.ca + q];
-        px = s_px[li];
-        py = s_px[kTileRow + li];
-        iz = s_px[2 * kTileRow + li];
+        for (int q = 0; q < 6; ++q) ci[q] = __ldg(Ci + (int64_t)q * P.np_pad + s);
+        apply_sym3(ci, (float)P.w[3 * pt], (float)P.w[3 * pt + 1], (float)P.w[3 * pt + 2], b);
+        P.sp_b[s] = make_float4(b[0], b[1], b[2], 0.f);
     }
-    chunk_tail(ps, pT, sbuf, act, m, pt, cam, so, jh, ci, px, py, iz);
-}
-
-// The staged pass.  `base` counts the uses consumed before this pass (the same
-// in every thread); `issued` the uses issued so far (the producer warp's).
-// Returns false in every thread if a stage barrier gave up (the error is recorded).
-__device__ bool point_pass_fact_staged(const Prob &P, const float *ps, const float *pT, float2 *sbuf,
-                                       unsigned char *stages, uint64_t *full, uint64_t *empty, StageOrg *org, int S,
-                                       int my_nt, uint32_t &base, uint32_t &issued) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    const uint32_t Su = (uint32_t)S;
-    bool ok = true;
-    if (wid == nwarp - 1) {
-        // producer: through the first S uses of the next pass, each after the
-        // consumers released its stage (the tile's descriptor is read first, so
-        // its latency overlaps the wait)
-        const uint32_t target = my_nt > 0 ? base + (uint32_t)my_nt + Su : 0u;
-        while (issued < target) {
-            const uint32_t u = issued;
-            const int t = (int)blockIdx.x + (int)(u % (uint32_t)my_nt) * (int)gridDim.x;
-            int4 d = make_int4(0, 0, 0, 0);
-            if (lane < 3) d = __ldg(P.tdesc + 3 * (int64_t)t + lane);
-            if (u >= Su && !mbar_wait(empty + u % Su, (u / Su - 1u) & 1u, kStageSpin)) {
-                if (lane == 0) atomicCAS(&P.st->err, 0, (int)MBA_ERR_TIMEOUT);
-                ok = false;
-                break;
-            }
-            int4 d0, d1, d2;
-            d0.x = __shfl_sync(0xffffffffu, d.x, 0), d0.y = __shfl_sync(0xffffffffu, d.y, 0);
-            d0.z = __shfl_sync(0xffffffffu, d.z, 0), d0.w = __shfl_sync(0xffffffffu, d.w, 0);
-            d1.x = __shfl_sync(0xffffffffu, d.x, 1), d1.y = __shfl_sync(0xffffffffu, d.y, 1);
-            d1.z = __shfl_sync(0xffffffffu, d.z, 1), d1.w = __shfl_sync(0xffffffffu, d.w, 1);
-            d2.x = __shfl_sync(0xffffffffu, d.x, 2), d2.y = __shfl_sync(0xffffffffu, d.y, 2);
-            d2.z = 0, d2.w = 0;
-            stage_issue(P, stages, full, org, S, u, d0, d1, d2);
-            ++issued;
-        }
-    } else {
-        // consumers: warp w works chunk w of every tile, then releases the stage
-        for (int j = 0; j < my_nt; ++j) {
-            const uint32_t u = base + (uint32_t)j;
-            const int sidx = (int)(u % Su);
-            if (!mbar_wait(full + sidx, (u / Su) & 1u, kStageSpin)) {
-                if (lane == 0) atomicCAS(&P.st->err, 0, (int)MBA_ERR_TIMEOUT);
-                ok = false;
-                break;
-            }
-            const StageOrg o = org[sidx];
-            if (o.ok) {
-                const int k = o.cb + wid;
-                if (k < o.ce) staged_chunk(ps, pT, sbuf, (const float *)(stages + (size_t)sidx * kStageBytes), o, k);
-            } else if (wid == 0 && lane == 0) {
-                atomicCAS(&P.st->err, 0, (int)MBA_ERR_INVALID_ARG);
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(empty + sidx);
-        }
-    }
-    base += (uint32_t)my_nt;
-    // chunks of tracks longer than 32 observations, over every warp of the grid
-    if (ok)
-        for (int i = (int)blockIdx.x * nwarp + wid; i < P.n_long; i += (int)gridDim.x * nwarp) {
-            const int k = P.long_chunks[i];
-            const int2 c0 = P.wchunk[k], c1 = P.wchunk[k + 1];
-            long_chunk_fact<false>(P, ps, pT, sbuf, c0.x, c0.y, c1.y - c0.y);
-        }
-    return __syncthreads_or(ok ? 0 : 1) == 0;
 }
 
 template <typename T, bool RHS, bool FACT>
 __device__ __forceinline__ void point_pass_any(const Prob &P, const T *ps, const T *pT, typename V2<T>::type *sbuf) {
-    if constexpr (FACT) point_pass_fact<RHS>(P, (const float *)ps, (const float *)pT, (float2 *)sbuf);
+    if constexpr (FACT && RHS) point_pass_fact_rhs(P);
+    else if constexpr (FACT) point_pass_fact(P, (const float *)ps, (const float *)pT);
     else point_pass<T, RHS>(P, ps, pT, sbuf);
 }
 
@@ -973,11 +747,74 @@ __device__ __forceinline__ double2 cta_sum2(double x, double y, bool warp_data, 
 __device__ __forceinline__ double3 cta_sum3(double x, double y, double z, bool warp_data, double *sb);
 
 
+// Sums of 9 values over the warp's lanes by exchanging halves: 14 shuffles
+// where nine butterflies take 45.  Lane l with l mod 4 == 0 returns the sum of
+// value 4 bit4(l) + 2 bit3(l) + bit2(l); `last` is the sum of v[8] in every lane.
+__device__ __forceinline__ float reduce9(float *v, float &last) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    float w = v[8];
+#pragma unroll
+    for (int h = 4; h >= 1; h >>= 1) {
+        const bool up = lane & (h << 2);
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float send = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(full, send, h << 2);
+        }
+        w += __shfl_xor_sync(full, w, h << 2);
+    }
+    float r = v[0];
+    r += __shfl_xor_sync(full, r, 2);
+    w += __shfl_xor_sync(full, w, 2);
+    r += __shfl_xor_sync(full, r, 1);
+    w += __shfl_xor_sync(full, w, 1);
+    last = w;
+    return r;
+}
+
+// gathers of b in flight per lane (Venice-shaped camera pass: 33.4 us with one,
+// 34.8 with two, 41.5 with three, which spill)
+constexpr int kCamDepth = 1;
+// One observation of the factored camera pass: the raw sums RX x y (0..2), y
+// (3..5), p.s (1, r2, r2^2) (6..8); X = (R X, 1 / P_z).  R b is formed from the
+// same quaternion as the point pass's R^T y: with a rounded matrix here the two
+// passes would apply rotations that differ by a fixed rounding per camera, an
+// asymmetry of the product that PCG sees in every iteration.
+struct CamConst {
+    float q0, q1, q2, q3, t0, t1, f, k1, k2;
+};
+__device__ __forceinline__ void fact_camera_obs(const CamConst &ct, const float4 X, const float4 b, float W, float *acc) {
+    const float e0 = ct.q2 * b.z - ct.q3 * b.y, e1 = ct.q3 * b.x - ct.q1 * b.z, e2 = ct.q1 * b.y - ct.q2 * b.x;
+    const float b0 = b.x + ct.q0 * e0 + (ct.q2 * e2 - ct.q3 * e1), b1 = b.y + ct.q0 * e1 + (ct.q3 * e0 - ct.q1 * e2),
+                b2 = b.z + ct.q0 * e2 + (ct.q1 * e1 - ct.q2 * e0);
+    const float iz = X.w;
+    const float x = -(X.x + ct.t0) * iz, y = -(X.y + ct.t1) * iz;
+    const float r2 = x * x + y * y, f = ct.f, k1 = ct.k1, k2 = ct.k2;
+    const float d = 1.f + r2 * (k1 + k2 * r2);
+    const float fd = f * d, fdd = f * (2.f * k1 + 4.f * k2 * r2), gx = fdd * x;
+    const float a00 = fd + gx * x, a01 = gx * y, a11 = fd + fdd * y * y;
+    // s = W Jp b = -(W / P_z) A (Rb_xy + p Rb_z)
+    const float c0 = b0 + x * b2, c1 = b1 + y * b2, wz = -W * iz;
+    const float s0 = wz * (a00 * c0 + a01 * c1), s1 = wz * (a01 * c0 + a11 * c1);
+    const float y0 = -iz * (a00 * s0 + a01 * s1), y1 = -iz * (a01 * s0 + a11 * s1), y2 = x * y0 + y * y1;
+    acc[0] += X.y * y2 - X.z * y1;
+    acc[1] += X.z * y0 - X.x * y2;
+    acc[2] += X.x * y1 - X.y * y0;
+    acc[3] += y0;
+    acc[4] += y1;
+    acc[5] += y2;
+    const float ps = x * s0 + y * s1, qs = r2 * ps;
+    acc[6] += ps;
+    acc[7] += qs;
+    acc[8] += r2 * qs;
+}
+
 // Camera pass.  Each CTA owns a contiguous run of whole cameras
 // [cta_cam[b], cta_cam[b+1]), balanced by observation count at creation; its
-// warps reduce the run's camera chunks into shared-memory slots, then, after a
-// block barrier, each camera's chunk sums are added in chunk order and the
-// camera is finalised.  No global atomics or fences; results do not depend on
+// warps reduce parts of the cameras (the stored form: camera chunks) into
+// shared-memory slots, then, after a block barrier, each camera's slots are
+// added in observation order and the camera is finalised.  No global atomics or fences; results do not depend on
 // timing.  CAM_RHS: g = v - c, x = 0, r = g, z = B~^-1 g; returns this CTA's
 // (r.r, r.z).  CAM_ITER: p = z + beta p_prev (p = z first), q = B~ p - c;
 // returns (p.q, 0).  CAM_MATVEC: q = B~ p - c with p given.  CAM_SR (the
@@ -985,129 +822,127 @@ __device__ __forceinline__ double3 cta_sum3(double x, double y, double z, bool w
 // r.u) and w.u in *third.
 template <typename T, int MODE, bool JS>
 __device__ double2 camera_pass(const Prob &P, const typename V2<T>::type *sbuf, const double *p_prev, double *p_cur,
-                               T *pT_cur, double beta, bool first, double *cslot, double *sb,
-                               double *third = nullptr) {
+                               double beta, bool first, double *cslot, double *sb, double *third = nullptr) {
     using T2 = typename V2<T>::type;
     constexpr int U = 4;
     constexpr bool FACT = sizeof(T) == 4 && !JS;
-    __shared__ T cts[32][kCamTab];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nwarp = blockDim.x >> 5;
     const unsigned full = 0xffffffffu;
-    const T *camtab = (const T *)P.camtab;
-    T *ct = cts[wid];
-    __shared__ int next_chunk;
     const int cb = P.cta_cam[blockIdx.x], ce = P.cta_cam[blockIdx.x + 1];
-    const int k0 = P.cfirst[cb], k1 = P.cfirst[ce];
-    if (threadIdx.x == 0) next_chunk = k0 + nwarp;
-    __syncthreads();
-    int loaded = -1;
-    // warps claim chunks dynamically; each chunk's sum goes to its own slot, so
-    // the result does not depend on which warp took it
-    for (int k = k0 + wid; k < k1;) {
-        const int cam = P.cchunk_cam[k];
-        const int b0 = P.cchunk_beg[k], b1 = P.cchunk_beg[k + 1];
-        if (sizeof(T) == 4 && !JS && cam != loaded) {
-            __syncwarp();
-            if (lane < kCamTab) ct[lane] = __ldg(camtab + (int64_t)cam * kCamTab + lane);
-            __syncwarp();
-            loaded = cam;
-        }
-        T acc[9];
-#pragma unroll
-        for (int a = 0; a < 9; ++a) acc[a] = T(0);
-        // factored form: the camera's t_x, t_y, f, k1, k2 for every observation of the chunk
-        float ct0 = 0.f, ct1 = 0.f, cf = 0.f, ck1 = 0.f, ck2 = 0.f;
-        if (FACT) {
-            ct0 = (float)ct[18];
-            ct1 = (float)ct[19];
-            cf = (float)ct[21];
-            ck1 = (float)ct[22];
-            ck2 = (float)ct[23];
-        }
-        for (int s0 = b0; s0 < b1; s0 += 32 * U) {
-            // s arrives in camera-major order (the point pass scattered it), so
-            // every load of the batch is a coalesced stream
-            bool in[U];
-            float rx0[U], rx1[U], rx2[U], rz[U];  // R X and 1 / P_z
-            T2 sv[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int s = s0 + u * 32 + lane;
-                in[u] = s < b1;
-                if (in[u]) sv[u] = ldcg(sbuf + s);
-                if (FACT) {
-                    const float4 v = in[u] ? __ldcs((const float4 *)P.RXcm + s) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    rx0[u] = v.x;
-                    rx1[u] = v.y;
-                    rx2[u] = v.z;
-                    rz[u] = v.w;
-                }
+    int k0 = 0, per = 32, o0 = 0;
+    if constexpr (FACT) {
+        // each warp takes an equal run of the CTA's observations (a multiple of 32)
+        // and flushes its sums at every camera boundary; warp w's part of camera i
+        // has the slot w + i - cb, which increases along the run, so a camera's
+        // parts are consecutive slots in observation order
+        o0 = __ldg(P.cam_ptr + cb);
+        const int total = __ldg(P.cam_ptr + ce) - o0;
+        per = ((total + nwarp - 1) / nwarp + 31) & ~31;
+        if (per < 32) per = 32;
+        int s0 = o0 + wid * per;
+        const int s1 = min(o0 + total, s0 + per);
+        int cam = cb;
+        if (s0 < s1) {  // the camera of the first observation: last i in [cb, ce) with cam_ptr[i] <= s0
+            int hi = ce - 1;
+            while (cam < hi) {
+                const int mid = (cam + hi + 1) >> 1;
+                if (__ldg(P.cam_ptr + mid) <= s0) cam = mid;
+                else hi = mid - 1;
             }
+        }
+        for (; s0 < s1; ++cam) {
+            const int e = min(s1, __ldg(P.cam_ptr + cam + 1));
+            CamConst ct;
+            {
+                const float *st = P.camstat + (int64_t)cam * kCamStat;
+                ct.f = __ldg(st), ct.k1 = __ldg(st + 1), ct.k2 = __ldg(st + 2);
+                ct.q0 = __ldg(st + 3), ct.q1 = __ldg(st + 4), ct.q2 = __ldg(st + 5), ct.q3 = __ldg(st + 6);
+                ct.t0 = __ldg(st + 7), ct.t1 = __ldg(st + 8);
+            }
+            float acc[9];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (in[u]) {
-                    if (FACT) {
-                        // y_t = D^T s = -(1/Pz) (g0, g1, p.g) with g = A s; accumulate
-                        // y_t, RX x y_t, and p.s (d, r2, r2^2)
-                        const float X0 = rx0[u], X1 = rx1[u], X2 = rx2[u];
-                        const float s0v = (float)sv[u].x, s1v = (float)sv[u].y;
-                        const float iz = rz[u];
-                        const float x = -(X0 + ct0) * iz, y = -(X1 + ct1) * iz;
-                        const float r2 = x * x + y * y;
-                        const float d = 1.f + ck1 * r2 + ck2 * r2 * r2;
-                        const float dd = 2.f * ck1 + 4.f * ck2 * r2;
-                        const float a00 = cf * (d + dd * x * x), a01 = cf * dd * x * y, a11 = cf * (d + dd * y * y);
-                        const float g0 = a00 * s0v + a01 * s1v, g1 = a01 * s0v + a11 * s1v;
-                        const float y0 = -iz * g0, y1 = -iz * g1, y2 = x * y0 + y * y1;
-                        acc[0] += (T)y0;
-                        acc[1] += (T)y1;
-                        acc[2] += (T)y2;
-                        acc[3] += (T)(X1 * y2 - X2 * y1);
-                        acc[4] += (T)(X2 * y0 - X0 * y2);
-                        acc[5] += (T)(X0 * y1 - X1 * y0);
-                        const float pss = x * s0v + y * s1v;
-                        acc[6] += (T)(d * pss);
-                        acc[7] += (T)(r2 * pss);
-                        acc[8] += (T)(r2 * r2 * pss);
-                    } else {
-                        camera_acc_stored<T>(P, s0 + u * 32 + lane, (T)sv[u].x, (T)sv[u].y, acc);
+            for (int a = 0; a < 9; ++a) acc[a] = 0.f;
+            // kCamDepth observations' (R X, 1/P_z), b and the point index after them
+            // are in flight while one is worked; each is copied out of its
+            // registers before the next load into them is issued, so that no copy
+            // waits for a load in flight
+            constexpr int D = kCamDepth;
+            float4 X[D], v[D];
+            int id[D];
+            const int q0 = s0 + lane;
+#pragma unroll
+            for (int j = 0; j < D; ++j) {
+                X[j] = v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (q0 + 32 * j < e) {
+                    X[j] = __ldg(P.RXcm + q0 + 32 * j);
+                    v[j] = load_b(P.sp_b + __ldg(P.cm_sp + q0 + 32 * j));
+                }
+                id[j] = q0 + 32 * (j + D) < e ? __ldg(P.cm_sp + q0 + 32 * (j + D)) : 0;
+            }
+            for (int p = q0; p < e; p += 32 * D) {
+#pragma unroll
+                for (int j = 0; j < D; ++j) {
+                    const int o = p + 32 * j, on = o + 32 * D;
+                    const float4 Xc = X[j], vc = v[j];
+                    if (on < e) {
+                        X[j] = __ldg(P.RXcm + on);
+                        v[j] = load_b(P.sp_b + id[j]);
+                        if (on + 32 * D < e) id[j] = __ldg(P.cm_sp + on + 32 * D);
                     }
+                    if (o < e) fact_camera_obs(ct, Xc, vc, P.cm_w ? __ldg(P.cm_w + o) : 1.f, acc);
                 }
             }
+            __syncwarp();
+            float last;
+            const float mine = reduce9(acc, last);
+            const int q = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+            double *slot = cslot + 9 * (wid + cam - cb);
+            if ((lane & 3) == 0) slot[q] = (double)mine;
+            if (lane == 1) slot[8] = (double)last;
+            s0 = e;
         }
-        T mine = T(0);
+    } else {
+        __shared__ int next_chunk;
+        k0 = P.cfirst[cb];
+        const int k1 = P.cfirst[ce];
+        if (threadIdx.x == 0) next_chunk = k0 + nwarp;
+        __syncthreads();
+        // warps claim chunks dynamically; each chunk's sum goes to its own slot, so
+        // the result does not depend on which warp took it
+        for (int k = k0 + wid; k < k1;) {
+            const int b0 = P.cchunk_beg[k], b1 = P.cchunk_beg[k + 1];
+            T acc[9];
 #pragma unroll
-        for (int a = 0; a < 9; ++a) {
-            T v = acc[a];
+            for (int a = 0; a < 9; ++a) acc[a] = T(0);
+            for (int s0 = b0; s0 < b1; s0 += 32 * U) {
+                // s arrives in camera-major order (the point pass scattered it), so
+                // every load of the batch is a coalesced stream
+                bool in[U];
+                T2 sv[U];
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(full, v, d);
-            if (FACT) acc[a] = v;  // every lane holds every sum
-            else if (lane == a) mine = v;
+                for (int u = 0; u < U; ++u) {
+                    const int s = s0 + u * 32 + lane;
+                    in[u] = s < b1;
+                    if (in[u]) sv[u] = ldcg(sbuf + s);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (in[u]) camera_acc_stored<T>(P, s0 + u * 32 + lane, (T)sv[u].x, (T)sv[u].y, acc);
+            }
+            T mine = T(0);
+#pragma unroll
+            for (int a = 0; a < 9; ++a) {
+                T v = acc[a];
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(full, v, d);
+                if (lane == a) mine = v;
+            }
+            if (lane < 9) cslot[(k - k0) * 9 + lane] = (double)mine;  // one conversion per lane
+            int nk = 0;
+            if (lane == 0) nk = atomicAdd(&next_chunk, 1);
+            k = __shfl_sync(full, nk, 0);
         }
-        if (FACT) {
-            // Jc^T s of the chunk: rotation (R M)^T sum RX x y_t, translation
-            // sum y_t, intrinsics (sum d p.s, f sum r2 p.s, f sum r2^2 p.s)
-            const float Y0 = (float)acc[0], Y1 = (float)acc[1], Y2 = (float)acc[2];
-            const float c0 = (float)acc[3], c1 = (float)acc[4], c2 = (float)acc[5];
-            const float q0 = ct[0] * c0 + ct[3] * c1 + ct[6] * c2;  // R^T c
-            const float q1 = ct[1] * c0 + ct[4] * c1 + ct[7] * c2;
-            const float q2 = ct[2] * c0 + ct[5] * c1 + ct[8] * c2;
-            const int a = lane < 3 ? lane : 0;
-            const float yr = ct[9 + a] * q0 + ct[12 + a] * q1 + ct[15 + a] * q2;  // (M^T q)_a
-            float mv = yr;
-            if (lane == 3) mv = Y0;
-            if (lane == 4) mv = Y1;
-            if (lane == 5) mv = Y2;
-            if (lane == 6) mv = (float)acc[6];
-            if (lane == 7) mv = cf * (float)acc[7];
-            if (lane == 8) mv = cf * (float)acc[8];
-            mine = (T)mv;
-        }
-        if (lane < 9) cslot[(k - k0) * 9 + lane] = (double)mine;  // one conversion per lane
-        int nk = 0;
-        if (lane == 0) nk = atomicAdd(&next_chunk, 1);
-        k = __shfl_sync(full, nk, 0);
     }
     __syncthreads();
     // finalise this CTA's cameras, three per warp (lanes 9s..9s+8 hold rows of
@@ -1131,8 +966,23 @@ __device__ double2 camera_pass(const Prob &P, const typename V2<T>::type *sbuf, 
 #pragma unroll
         for (int b = 0; b < 9; ++b) brow[b] = (kEarly && act) ? __ldg(Mrow + b) : 0.0;
         double cs = 0.0;
-        if (act)
-            for (int k = P.cfirst[cm]; k < P.cfirst[cm + 1]; ++k) cs += cslot[(k - k0) * 9 + a];
+        if (act) {
+            if constexpr (FACT) {
+                const int w0 = (__ldg(P.cam_ptr + cm) - o0) / per, w1 = (__ldg(P.cam_ptr + cm + 1) - 1 - o0) / per;
+                for (int k = w0 + cm - cb; k <= w1 + cm - cb; ++k) cs += cslot[k * 9 + a];
+            } else {
+                for (int k = P.cfirst[cm]; k < P.cfirst[cm + 1]; ++k) cs += cslot[(k - k0) * 9 + a];
+            }
+        }
+        if constexpr (FACT) {  // c = ctr raw, three terms of the lane's group
+            const int g0 = a < 3 ? 0 : (a < 6 ? 3 : 6);
+            const float *ct = P.ctr + (int64_t)cm * kCtr + 3 * a;
+            double c = 0.0;
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+                c = fma((double)__ldg(ct + b), __shfl_sync(full, cs, (9 * sub + g0 + b) & 31), c);
+            cs = c;
+        }
         // a fixed camera has no Schur coupling (its Jacobian columns are zero; the
         // factored product forms Jc^T s from the geometry, so it is masked here)
         if (P.has_fixed && act && P.cam_fixed[cm]) cs = 0.0;
@@ -1154,7 +1004,10 @@ __device__ double2 camera_pass(const Prob &P, const typename V2<T>::type *sbuf, 
                 v1 = g * g;
                 v2 = g * z;
             }
-            if (FACT) fact_row_store(P, (float *)P.zT, cm, act, z, sub, row, true);
+            if constexpr (FACT) {
+                const float rv = fact_row_lane(P, cm, act ? z : 0.0, sub, row);
+                if (act) stcg((float *)P.zT + vo, rv);
+            }
         } else {
             double p = 0.0;
             if (act) {
@@ -1173,7 +1026,7 @@ __device__ double2 camera_pass(const Prob &P, const typename V2<T>::type *sbuf, 
                 stcg(P.q + vo, q);
                 if (MODE == CAM_ITER) {
                     stcg(p_cur + vo, p);
-                    if (pT_cur && !FACT) stcg(pT_cur + vo, (T)p);
+                    if (sizeof(T) == 4 && !FACT && P.pcg_use_ps) stcg((T *)(p_cur == P.p ? P.pT : P.pT2) + vo, (T)p);
                 }
                 if (MODE == CAM_SR) {
                     const double rv = ldcg(P.r + vo);
@@ -1184,7 +1037,6 @@ __device__ double2 camera_pass(const Prob &P, const typename V2<T>::type *sbuf, 
                     v1 = p * q;
                 }
             }
-            if (FACT && MODE == CAM_ITER && pT_cur) fact_row_store(P, (float *)pT_cur, cm, act, p, sub, row, false);
         }
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) {
@@ -1210,36 +1062,44 @@ __device__ double2 camera_pass(const Prob &P, const typename V2<T>::type *sbuf, 
 // (p = z on the first iteration), or the given FP64 p (src_given).  The FP32
 // form builds it from float copies of z and p_prev with float4 loads; the FP64
 // form from the FP64 vectors, as the camera pass does.
-// Factored form: the camera rows ([nc][kRow] floats) instead: row(z) + beta
-// row(p_prev) from the float row copies, or the rows of the given FP64 p.
+// Factored form: the camera rows instead (stride kRowS): the constants once
+// (first), the nine linear entries as row(z) + beta times the row of the
+// previous iteration that is still in shared memory, or the rows of the given
+// FP64 p.
 template <typename T, bool FACT>
 __device__ void stage_p(const Prob &P, T *ps, const double *p_prev, const T *pT_prev, double beta, bool first,
                         const double *src_given) {
     if constexpr (FACT) {
-        float4 *dst = (float4 *)ps;
         if (!src_given) {
-            const float4 *z4 = (const float4 *)P.zT, *p4 = (const float4 *)pT_prev;
+            const float4 *z4 = (const float4 *)P.zT;
             const float fb = (float)beta;
-            const int nq = P.nc * (kRow / 4);  // float4 per camera row
+            const int nq = P.nc * 3;  // three float4 per camera: n, h, (v_f, v_a, v_b)
             for (int e = threadIdx.x; e < nq; e += blockDim.x) {
-                const float4 zv = __ldcg(z4 + e);
-                float4 v = zv;
+                const int cam = e / 3, part = e - 3 * cam;
+                const float4 z = __ldcg(z4 + e);
+                float4 *dst = (float4 *)(ps + cam * kRowS) + part;
+                float4 v = z;
                 if (!first) {
-                    const float4 pv = __ldcg(p4 + e);
-                    v = make_float4(fmaf(fb, pv.x, zv.x), fmaf(fb, pv.y, zv.y), fmaf(fb, pv.z, zv.z),
-                                    fmaf(fb, pv.w, zv.w));
+                    const float4 o = *dst;
+                    v = make_float4(fmaf(fb, o.x, z.x), fmaf(fb, o.y, z.y), fmaf(fb, o.z, z.z), fmaf(fb, o.w, z.w));
+                    if (part == 2) v.y = o.y, v.z = o.z, v.w = o.w;
+                } else if (part == 2) {
+                    const float *st = P.camstat + (int64_t)cam * kCamStat;
+                    v.y = __ldg(st), v.z = __ldg(st + 1), v.w = __ldg(st + 2);
+                    dst[1] = make_float4(__ldg(st + 3), __ldg(st + 4), __ldg(st + 5), __ldg(st + 6));
                 }
-                dst[e] = v;
+                *dst = v;
             }
         } else {
             for (int cam = threadIdx.x; cam < P.nc; cam += blockDim.x) {
-                float v[9], r[kRow];
+                float v[9], r[kRowG];
+                const bool fixed = P.has_fixed && P.cam_fixed[cam];  // its Jacobian columns are zero
 #pragma unroll
-                for (int j = 0; j < 9; ++j) v[j] = (float)src_given[(int64_t)cam * kVec + j];
-                fact_row((const float *)P.camtab + (int64_t)cam * kCamTab, v, true, r);
+                for (int j = 0; j < 9; ++j) v[j] = fixed ? 0.f : (float)src_given[(int64_t)cam * kVec + j];
+                fact_row(P, cam, v, r);
+                float4 *dst = (float4 *)(ps + cam * kRowS);
 #pragma unroll
-                for (int i = 0; i < kRow / 4; ++i)
-                    dst[(kRow / 4) * cam + i] = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+                for (int i = 0; i < kRowG / 4; ++i) dst[i] = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
             }
         }
         __syncthreads();
@@ -1328,21 +1188,34 @@ __device__ __forceinline__ double2 cta_sum2(double x, double y, bool warp_data, 
 }
 
 
-// Two sums of n per-CTA partials (n <= blockDim.x: one load per thread, then
-// shuffle trees only in the warps that hold partials); every thread of every
-// CTA gets the same values.
-__device__ __forceinline__ double2 sum_parts2(const double *a, const double *b, int n, double *sb) {
+// Two sums of n per-CTA partials in warp 0: each lane adds its partials in
+// order (the loads in flight together), then one shuffle tree; valid in thread
+// 0, which runs the scalar recurrences that use them.  (All warps adding the
+// partials through cta_sum2 costs a second tree and three CTA barriers.)
+__device__ __forceinline__ double2 sum_parts2(const double *a, const double *b, int n) {
     double x = 0.0, y = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        x += ldcg(a + i);
-        y += b ? ldcg(b + i) : 0.0;
+    if (threadIdx.x < 32) {
+        for (int i0 = threadIdx.x; i0 < n; i0 += 160) {
+            double u[5], v[5];
+#pragma unroll
+            for (int j = 0; j < 5; ++j) {
+                const int i = i0 + 32 * j;
+                u[j] = i < n ? ldcg(a + i) : 0.0;
+                v[j] = (b && i < n) ? ldcg(b + i) : 0.0;
+            }
+            x += (u[0] + u[1]) + (u[2] + u[3]) + u[4];
+            if (b) y += (v[0] + v[1]) + (v[2] + v[3]) + v[4];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            x += __shfl_down_sync(0xffffffffu, x, o);
+            if (b) y += __shfl_down_sync(0xffffffffu, y, o);
+        }
     }
-    return cta_sum2(x, y, (int)(threadIdx.x & ~31u) < n, sb);
+    return make_double2(x, y);
 }
 
-__device__ __forceinline__ double sum_parts(const double *parts, int n, double *sb) {
-    return sum_parts2(parts, nullptr, n, sb).x;
-}
+__device__ __forceinline__ double sum_parts(const double *parts, int n) { return sum_parts2(parts, nullptr, n).x; }
 
 // Three-value forms of cta_sum2 / sum_parts2 (the single-reduction PCG); sb
 // holds 96 doubles.
@@ -1394,10 +1267,8 @@ __device__ __forceinline__ double3 sum_parts3(const double *a, const double *b, 
 // ---------------------------------------------------------------------------
 // JS: the camera pass reads the stored camera-major Jacobian (always in FP64;
 // in FP32-mixed when the Jacobian comes from dual numbers).
-// STG: the staged point pass (factored form only, a separate instantiation so
-// that its code does not weigh on the direct pass's registers).
 // SR: the single-reduction recurrence (mba_pcg_variant), also its own instance.
-template <typename T, bool JS, bool STG, bool SR>
+template <typename T, bool JS, bool SR>
 __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
     pcg_kernel(Prob P, int mode, int max_iter, double tol, long long spin, int forcing) {
     using T2 = typename V2<T>::type;
@@ -1425,45 +1296,19 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
     double *cslot = (double *)(smem_raw + P.pcg_ps_bytes);
     bool ok = true;
     auto barrier = [&]() -> bool { return grid_barrier(st, epoch, spin); };
-    // staged point pass (factored form): stage barriers, use counters, and the
-    // drain that waits for copies still in flight before the CTA leaves
-    __shared__ __align__(8) uint64_t s_full[kMaxStages], s_empty[kMaxStages];
-    __shared__ StageOrg s_org[kMaxStages];
-    const int S = (FACT && STG) ? P.pcg_stages : 0;
-    const uint32_t Su = S > 0 ? (uint32_t)S : 1u;
-    unsigned char *stages = smem_raw + P.pcg_stage_off;
-    const int my_nt = (S && P.n_tiles > (int)blockIdx.x) ? (P.n_tiles - 1 - (int)blockIdx.x) / G + 1 : 0;
-    uint32_t use = 0, issued = 0;
-    if (STG && S) {
-        if (threadIdx.x == 0) {
-            for (int i = 0; i < S; ++i) {
-                mbar_init(s_full + i, 1);
-                mbar_init(s_empty + i, (uint32_t)(nwarp - 1));
-            }
-            mbar_init_fence();
-        }
-        __syncthreads();
-    }
-    // the producer warp's first lane waits for the copies it issued beyond the
-    // last consumed use before the CTA leaves
-    auto drain = [&]() {
-        if (STG && S && threadIdx.x == (unsigned)(nwarp - 1) * 32)
-            for (uint32_t u = use; u < issued; ++u)
-                if (!mbar_wait(s_full + u % Su, (u / Su) & 1u, kStageSpin)) {
-                    atomicCAS(&st->err, 0, (int)MBA_ERR_TIMEOUT);
-                    break;
-                }
-    };
     // the point pass of one product; rows: the search rows in global memory
     // (read where they are not in shared memory)
-    auto point_pass_iter = [&](const T *rows) -> bool {
-        if constexpr (FACT && STG) {
-            if (S)
-                return point_pass_fact_staged(P, (const float *)ps, (const float *)rows, (float2 *)sbuf, stages,
-                                              s_full, s_empty, s_org, S, my_nt, use, issued);
+    auto point_pass_iter = [&](const T *rows) { point_pass_any<T, false, FACT>(P, ps, rows, sbuf); };
+    // owner's copy of a vector's camera row (factored form): the nine linear
+    // entries (zT), or the whole row where the point pass reads it from global memory
+    auto store_row = [&](int cam, bool act, double val, float *lin, float *whole) {
+        const float r = fact_row_lane(P, cam, act ? val : 0.0, my_sub, row);
+        if (!act) return;
+        if (lin) stcg(lin + (int64_t)cam * kVec + row, r);
+        if (whole) {
+            stcg(whole + (int64_t)cam * kRowG + row, r);
+            if (row < 7) stcg(whole + (int64_t)cam * kRowG + 9 + row, P.camstat[(int64_t)cam * kCamStat + row]);
         }
-        point_pass_any<T, false, FACT>(P, ps, rows, sbuf);
-        return true;
     };
     // owner phase: p = z + beta p_prev written in FP64 and, for the gathers, as
     // T (or, in the factored form, as the camera's row)
@@ -1478,7 +1323,10 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
                 if (!given) stcg(p_cur + vo, pn);
                 if (!FACT) stcg(pT + vo, (T)pn);
             }
-            if (FACT) fact_row_store(P, (float *)pT, act ? cam : 0, act, pn, my_sub, row, true);
+            if constexpr (FACT) {
+                const bool fixed = given && act && P.has_fixed && P.cam_fixed[cam];
+                store_row(act ? cam : 0, act, fixed ? 0.0 : pn, nullptr, (float *)pT);
+            }
         }
     };
 
@@ -1490,9 +1338,8 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
             phase_p(nullptr, nullptr, 0.0, true, P.p);
             if (!(ok = barrier())) return;
         }
-        const bool pok = point_pass_iter(pT);
-        if (pok && barrier()) camera_pass<T, CAM_MATVEC, JS>(P, sbuf, nullptr, nullptr, nullptr, 0.0, true, cslot, sb);
-        drain();
+        point_pass_iter(pT);
+        if (barrier()) camera_pass<T, CAM_MATVEC, JS>(P, sbuf, nullptr, nullptr, 0.0, true, cslot, sb);
         return;
     }
 
@@ -1500,7 +1347,7 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
     point_pass_any<T, true, FACT>(P, nullptr, nullptr, sbuf);
     ok = barrier();
     if (ok) {
-        const double2 d = camera_pass<T, CAM_RHS, JS>(P, sbuf, nullptr, nullptr, nullptr, 0.0, true, cslot, sb);
+        const double2 d = camera_pass<T, CAM_RHS, JS>(P, sbuf, nullptr, nullptr, 0.0, true, cslot, sb);
         if (mode == PCG_RHS_ONLY) return;
         if (threadIdx.x == 0) {
             stcg(part_rr + blockIdx.x, d.x);
@@ -1528,16 +1375,20 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
         __shared__ double s_alpha, s_beta, s_r0, s_rn, s_stop2, s_gprev, s_aprev;
         __shared__ int s_go;
         // where the point pass finds u's rows when they are not in shared memory
-        const T *rows_u = sizeof(T) == 8 ? (const T *)P.z : (const T *)P.zT;
+        const T *rows_u = FACT ? (const T *)P.pT : (sizeof(T) == 8 ? (const T *)P.z : (const T *)P.zT);
+        if (FACT && !ps) {  // u_0's rows, published by a barrier of their own
+            phase_p(nullptr, P.p, 0.0, true, nullptr);
+            ok = barrier();
+        }
         int n = 0;
         while (ok && (n == 0 || n < max_iter)) {
             if (ps) stage_p<T, FACT>(P, ps, nullptr, nullptr, 0.0, true, nullptr);
-            if (!(ok = point_pass_iter(rows_u))) break;
+            point_pass_iter(rows_u);
             if (!(ok = barrier())) break;
             {
                 double wu = 0.0;
                 const double2 d =
-                    camera_pass<T, CAM_SR, JS>(P, sbuf, nullptr, nullptr, nullptr, 0.0, false, cslot, sb, &wu);
+                    camera_pass<T, CAM_SR, JS>(P, sbuf, nullptr, nullptr, 0.0, false, cslot, sb, &wu);
                 if (threadIdx.x == 0) {
                     stcg(part_rr + blockIdx.x, d.x);
                     stcg(part_rho + blockIdx.x, d.y);
@@ -1606,7 +1457,8 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
                         const double rc = __shfl_sync(full, rv, my_sub * 9 + c);
                         if (act) z = fma(__ldg(P.Binv + 81 * (int64_t)cam + row * 9 + c), rc, z);
                     }
-                    if (FACT) fact_row_store(P, (float *)P.zT, act ? cam : c0, act, z, my_sub, row, true);
+                    if constexpr (FACT)
+                        store_row(act ? cam : c0, act, z, ps ? (float *)P.zT : nullptr, ps ? nullptr : (float *)pT);
                     if (act) {
                         stcg(P.z + vo, z);
                         if (sizeof(T) == 4 && !FACT) stcg((float *)P.zT + vo, (float)z);
@@ -1622,14 +1474,13 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
             ++n;
             if (last) {
                 if (!(ok = barrier())) break;
-                const double rrn = sum_parts(P.red + 3 * G, G, sb);
+                const double rrn = sum_parts(P.red + 3 * G, G);
                 if (threadIdx.x == 0) s_rn = sqrt(rrn);
                 __syncthreads();
                 break;
             }
             if (!(ok = barrier())) break;
         }
-        drain();
         if (!ok) atomicCAS(&st->err, 0, (int)MBA_ERR_TIMEOUT);
         if (ok && blockIdx.x == 0 && threadIdx.x == 0) {
             st->pcg_iters = n;
@@ -1650,7 +1501,7 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
     __shared__ int s_go;
     int n = 0;
     if (ok) {
-        const double2 s0 = sum_parts2(part_rr, part_rho, G, sb);
+        const double2 s0 = sum_parts2(part_rr, part_rho, G);
         if (threadIdx.x == 0) {
             const double r0 = sqrt(s0.x);
             double t = tol;
@@ -1672,7 +1523,6 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
             const double beta = s_beta;
             double *p_cur = (n & 1) ? P.p2 : P.p;
             const double *p_prev = (n & 1) ? P.p : P.p2;
-            T *pT_cur = (n & 1) ? (T *)P.pT2 : pT;
             const T *pT_prev = (n & 1) ? pT : (T *)P.pT2;
             if (ps) {
                 stage_p<T, FACT>(P, ps, p_prev, pT_prev, beta, n == 0, nullptr);
@@ -1680,16 +1530,14 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
                 phase_p(p_prev, p_cur, beta, n == 0, nullptr);
                 if (!(ok = barrier())) break;
             }
-            if (!(ok = point_pass_iter(pT))) break;
+            point_pass_iter(pT);
             if (!(ok = barrier())) break;
             {
-                const double2 d = camera_pass<T, CAM_ITER, JS>(P, sbuf, p_prev, p_cur,
-                                                               (sizeof(T) == 4 && ps) ? pT_cur : nullptr,
-                                                           beta, n == 0, cslot, sb);
+                const double2 d = camera_pass<T, CAM_ITER, JS>(P, sbuf, p_prev, p_cur, beta, n == 0, cslot, sb);
                 if (threadIdx.x == 0) stcg(part_pq + blockIdx.x, d.x);
             }
             if (!(ok = barrier())) break;
-            const double pq = sum_parts(part_pq, G, sb);
+            const double pq = sum_parts(part_pq, G);
             if (threadIdx.x == 0) {
                 const bool go = (pq > 0.0) && isfinite(pq);
                 s_go = go ? 1 : 0;
@@ -1723,7 +1571,9 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
                         const double rc = __shfl_sync(full, rv, my_sub * 9 + c);
                         z = fma(bi[c], rc, z);
                     }
-                    if (FACT) fact_row_store(P, (float *)P.zT, act ? cam : c0, act, z, my_sub, row, true);
+                    if constexpr (FACT) {
+                        if (ps) store_row(act ? cam : c0, act, z, (float *)P.zT, nullptr);
+                    }
                     if (act) {
                         stcg(P.z + vo, z);
                         if (sizeof(T) == 4 && !FACT) stcg((float *)P.zT + vo, (float)z);
@@ -1740,7 +1590,7 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
             }
             if (!(ok = barrier())) break;
             ++n;
-            const double2 sums = sum_parts2(part_rho, part_rr, G, sb);
+            const double2 sums = sum_parts2(part_rho, part_rr, G);
             if (threadIdx.x == 0) {
                 const double rho_prev = s_rho, rho = sums.x, rn = sqrt(sums.y);
                 s_rho = rho;
@@ -1753,7 +1603,6 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
             if (!s_go) break;
         }
     }
-    drain();
     if (!ok) atomicCAS(&st->err, 0, (int)MBA_ERR_TIMEOUT);
     if (ok && blockIdx.x == 0 && threadIdx.x == 0) {
         st->pcg_iters = n;
@@ -1762,50 +1611,34 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
     }
 }
 
+#include "pcg_own.cuh"
+
 // ---------------------------------------------------------------------------
 // back-substitution dp_j = C~_j^-1 (w_j - sum_k Jp~_k^T Jc~_k dc_i(k)) (Eq. 4),
 // candidate points, and the model decrease sum_k (-e~_k.d_k - |d_k|^2/2)
 // with d_k = Jc~_k dc + Jp~_k dp.
 // ---------------------------------------------------------------------------
-// Per observation: t = Jc dc (sqrt(W)-scaled in the stored form, unscaled in
-// FACT) and the point-side Jacobian (Jp~, or W Jp in FACT), so that
-// u = jp^T t is this observation's term of Jp~^T Jc~ dc.
-template <typename T, bool FACT>
+// Per observation: t = Jc~ dc and Jp~, so that u = jp^T t is this observation's
+// term of Jp~^T Jc~ dc.
+template <typename T>
 __device__ __forceinline__ void backsub_obs(const Prob &P, int64_t o, int cam, T *t, T *jp) {
-    const int64_t npad = P.npad;
-    if constexpr (FACT) {
-        float r[kRow];
-        gather_row(nullptr, (const float *)P.pT, cam, r);
-        fact_jc_v(__ldcs(P.PXpm + o), __ldcs(P.PXpm + npad + o), __ldcs(P.PXpm + 2 * npad + o), r, t);
+    T Jc[18];
+    load_jac_stream((const T *)P.J, P.npad, o, Jc, jp);
+    const double *xc = P.x + (int64_t)cam * kVec;
+    t[0] = t[1] = T(0);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) jp[k] = __ldcs(P.Jph + k * npad + o);
-    } else {
-        T Jc[18];
-        load_jac_stream((const T *)P.J, npad, o, Jc, jp);
-        const double *xc = P.x + (int64_t)cam * kVec;
-        t[0] = t[1] = T(0);
-#pragma unroll
-        for (int a = 0; a < 9; ++a) {
-            const T xa = (T)xc[a];
-            t[0] += Jc[a] * xa;
-            t[1] += Jc[9 + a] * xa;
-        }
+    for (int a = 0; a < 9; ++a) {
+        const T xa = (T)xc[a];
+        t[0] += Jc[a] * xa;
+        t[1] += Jc[9 + a] * xa;
     }
 }
 // Model-decrease term of one observation given its point step: d~ = J~_k (dc, dp),
-// -e~.d~ - |d~|^2 / 2 (FACT: d~ = sqrt(W) t + (W Jp) dp / sqrt(W)).
-template <typename T, bool FACT>
+// -e~.d~ - |d~|^2 / 2.
+template <typename T>
 __device__ __forceinline__ double backsub_dec(const Prob &P, int64_t o, const T *t, const T *jp, const T *dp) {
-    T d0 = jp[0] * dp[0] + jp[1] * dp[1] + jp[2] * dp[2];
-    T d1 = jp[3] * dp[0] + jp[4] * dp[1] + jp[5] * dp[2];
-    if constexpr (FACT) {
-        const float sw = P.swpm ? __ldg(P.swpm + o) : 1.f, isw = 1.f / sw;
-        d0 = sw * t[0] + isw * d0;
-        d1 = sw * t[1] + isw * d1;
-    } else {
-        d0 += t[0];
-        d1 += t[1];
-    }
+    const T d0 = jp[0] * dp[0] + jp[1] * dp[1] + jp[2] * dp[2] + t[0];
+    const T d1 = jp[3] * dp[0] + jp[4] * dp[1] + jp[5] * dp[2] + t[1];
     const T *res = (const T *)P.res;
     const double e0 = (double)__ldcs(res + o), e1 = (double)__ldcs(res + P.npad + o);
     const double dd0 = (double)d0, dd1 = (double)d1;
@@ -1829,11 +1662,9 @@ __device__ __forceinline__ void backsub_point(const Prob &P, int pt, const T *a,
 // candidate points, and the model decrease sum_k (-e~_k.d_k - |d_k|^2/2)
 // with d_k = Jc~_k dc + Jp~_k dp, in one sweep over point-major warp chunks:
 // a segmented scan gives each point's sum, its last lane forms dp and the
-// point's lanes take it by a shuffle.  FACT (FP32-mixed analytic): t = Jc dc
-// from the camera rows of dc (fact_rows_kernel, into the free search-direction
-// buffer) and (px, py, 1/Pz).
+// point's lanes take it by a shuffle.
 // ---------------------------------------------------------------------------
-template <typename T, bool FACT>
+template <typename T>
 __global__ void __launch_bounds__(kBlock) backsub_kernel(Prob P, double *partial) {
     __shared__ double sb[kWarps];
     if (P.st->done) return;
@@ -1853,7 +1684,7 @@ __global__ void __launch_bounds__(kBlock) backsub_kernel(Prob P, double *partial
             T t[2] = {T(0), T(0)}, jp[6], u[3];
 #pragma unroll
             for (int k = 0; k < 6; ++k) jp[k] = T(0);
-            if (act) backsub_obs<T, FACT>(P, o, __ldg(P.pm_cam + o), t, jp);
+            if (act) backsub_obs<T>(P, o, __ldg(P.pm_cam + o), t, jp);
             u[0] = jp[0] * t[0] + jp[3] * t[1];
             u[1] = jp[1] * t[0] + jp[4] * t[1];
             u[2] = jp[2] * t[0] + jp[5] * t[1];
@@ -1878,7 +1709,7 @@ __global__ void __launch_bounds__(kBlock) backsub_kernel(Prob P, double *partial
             T dq[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) dq[k] = __shfl_sync(full, dp[k], src);
-            if (act) ldec += backsub_dec<T, FACT>(P, o, t, jp, dq);
+            if (act) ldec += backsub_dec<T>(P, o, t, jp, dq);
         } else {
             // one point with a long track: the sum over 32-observation slices, then
             // a second sweep for the model decrease
@@ -1888,7 +1719,7 @@ __global__ void __launch_bounds__(kBlock) backsub_kernel(Prob P, double *partial
                 if (base + lane < m) {
                     const int64_t o = (int64_t)o0 + base + lane;
                     T t[2], jp[6];
-                    backsub_obs<T, FACT>(P, o, __ldg(P.pm_cam + o), t, jp);
+                    backsub_obs<T>(P, o, __ldg(P.pm_cam + o), t, jp);
 #pragma unroll
                     for (int k = 0; k < 3; ++k) a[k] += jp[k] * t[0] + jp[3 + k] * t[1];
                 }
@@ -1905,8 +1736,8 @@ __global__ void __launch_bounds__(kBlock) backsub_kernel(Prob P, double *partial
                 if (base + lane < m) {
                     const int64_t o = (int64_t)o0 + base + lane;
                     T t[2], jp[6];
-                    backsub_obs<T, FACT>(P, o, __ldg(P.pm_cam + o), t, jp);
-                    ldec += backsub_dec<T, FACT>(P, o, t, jp, dp);
+                    backsub_obs<T>(P, o, __ldg(P.pm_cam + o), t, jp);
+                    ldec += backsub_dec<T>(P, o, t, jp, dp);
                 }
             }
         }
@@ -1915,18 +1746,172 @@ __global__ void __launch_bounds__(kBlock) backsub_kernel(Prob P, double *partial
     if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
+// The same over the slices of the factored form: t and u as in the PCG point
+// pass from the rows of dc; the second sweep over the lane's observations
+// recomputes t, adds Jp dp = D R dp (R from the quaternion) and the residual
+// e = f d p - u, and sums the model decrease -W (e.d + |d|^2 / 2), one FP64
+// addition per observation.  SMEM: the CTA forms the rows of dc in shared memory.
+template <bool SMEM>
+__global__ void __launch_bounds__(1024, 1) backsub_slices_kernel(Prob P, double *partial) {
+    __shared__ double sb[32];
+    if (P.st->done) return;
+    extern __shared__ __align__(16) float s_rows[];
+    if (SMEM) {
+        for (int cam = threadIdx.x; cam < P.nc; cam += blockDim.x) {
+            float v[9], r[kRowG];
+#pragma unroll
+            for (int j = 0; j < 9; ++j) v[j] = (float)P.x[(int64_t)cam * kVec + j];
+            fact_row(P, cam, v, r);
+            float4 *dst = (float4 *)(s_rows + cam * kRowS);
+#pragma unroll
+            for (int i = 0; i < kRowG / 4; ++i) dst[i] = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+        }
+        __syncthreads();
+    }
+    const float *ps = SMEM ? s_rows : nullptr, *rows = (const float *)P.pT;
+    const float *__restrict__ Ci = (const float *)P.Cinv;
+    const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+    const unsigned full = 0xffffffffu;
+    double ldec = 0.0;
+    for (int w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < P.n_slices; w += gridDim.x * nwarp) {
+        const int4 sl = __ldg(P.slice + w);
+        const int K = sl.w & 0xffff, lg = sl.w >> 16, in = lane >> lg;
+        const bool act = in < (sl.y & 0xff);
+        const int s = sl.x + (act ? in : 0);
+        float a[3];
+        fact_slice_sum(P, ps, rows, (int64_t)sl.z + lane, K, a);
+        for (int d = 1; d < (1 << lg); d <<= 1) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) a[q] += __shfl_xor_sync(full, a[q], d);
+        }
+        const int64_t pt = __ldg(P.sp_pt + s);
+        if (P.has_fixed && P.pt_fixed[pt]) a[0] = a[1] = a[2] = 0.f;
+        float ci[6], dp[3];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) ci[q] = __ldg(Ci + (int64_t)q * P.np_pad + s);
+        apply_sym3(ci, (float)P.w[3 * pt] - a[0], (float)P.w[3 * pt + 1] - a[1], (float)P.w[3 * pt + 2] - a[2], dp);
+        if (act && (lane & ((1 << lg) - 1)) == 0) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                P.dp[3 * pt + k] = (double)dp[k];
+                P.pts_new[3 * pt + k] = P.pts[3 * pt + k] + (double)dp[k];
+            }
+        }
+        const bool fixed = P.has_fixed && P.pt_fixed[pt];
+        const float f0 = fixed ? 0.f : dp[0], f1 = fixed ? 0.f : dp[1], f2 = fixed ? 0.f : dp[2];
+        for (int k = 0; k < K; ++k) {
+            const int64_t slot = (int64_t)sl.z + 32 * k + lane;
+            const FactStream st = load_stream(P, slot);
+            if (st.cam < 0) continue;
+            const float px = st.px, py = st.py, iz = st.iz, W = st.W;
+            const float2 uv = __ldg(P.sl_uv32 + slot);
+            const CamRow r = load_row(ps, rows, st.cam);
+            FactObs o = fact_obs(px, py, iz, r);
+            const float c0 = r.q2 * f2 - r.q3 * f1, c1 = r.q3 * f0 - r.q1 * f2, c2 = r.q1 * f1 - r.q2 * f0;
+            o.w0 += iz * (f0 + r.q0 * c0 + (r.q2 * c2 - r.q3 * c1));
+            o.w1 += iz * (f1 + r.q0 * c1 + (r.q3 * c0 - r.q1 * c2));
+            o.w2 += iz * (f2 + r.q0 * c2 + (r.q1 * c1 - r.q2 * c0));
+            float d0, d1;
+            fact_t(o, px, py, d0, d1);
+            const float r2 = px * px + py * py, fd = r.f * (1.f + r2 * (r.k1 + r.k2 * r2));
+            const float e0 = fd * px - uv.x, e1 = fd * py - uv.y;
+            ldec -= (double)(W * (d0 * (e0 + 0.5f * d0) + d1 * (e1 + 0.5f * d1)));
+        }
+    }
+    const double s = block_sum(ldec, sb);
+    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+}
+
+// FP64 form over slices (block-owned layout): u = H alpha + g sigma as in the
+// PCG; with delta = alpha + dp the model term of an observation is
+// |d|^2 = delta^T H delta + 2 sigma g.delta + sigma^2 W r2, and
+// -sum e~.d = v.dc + w.dp, the gradient against the step.
+__global__ void __launch_bounds__(512, 1) backsub_slices64_kernel(Prob P, double *partial) {
+    __shared__ double sb[32];
+    if (P.st->done) return;
+    extern __shared__ __align__(16) double s_rows64[];
+    for (int e = threadIdx.x; e < 10 * P.nc; e += blockDim.x) {
+        const int cam = e / 10, q = e - 10 * cam, g0 = q < 3 ? 0 : (q < 6 ? 3 : 6);
+        double r;
+        if (q == 9) {
+            r = __ldg((const double *)P.camtab + (int64_t)cam * kCamTab + 24);
+        } else {
+            const double *ct = P.ctr64 + (int64_t)cam * kCtr + 3 * g0 + (q - g0), *v = P.x + (int64_t)cam * kVec + g0;
+            r = fma(ct[0], v[0], fma(ct[3], v[1], ct[6] * v[2]));
+        }
+        s_rows64[cam * kRowD + q] = r;
+    }
+    __syncthreads();
+    const double *__restrict__ Ci = (const double *)P.Cinv;
+    const int lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
+    const unsigned full = 0xffffffffu;
+    double ldec = 0.0;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 9 * (int64_t)P.nc; t += (int64_t)gridDim.x * blockDim.x)
+        ldec = fma(P.v[t], P.x[t / 9 * kVec + t % 9], ldec);
+    for (int w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < P.n_slices; w += gridDim.x * nwarp) {
+        const int4 sl = __ldg(P.slice + w);
+        const int K = sl.w & 0xffff, lg = sl.w >> 16, in = lane >> lg;
+        const bool act = in < (sl.y & 0xff);
+        const int s = sl.x + (act ? in : 0);
+        const double X[3] = {__ldg(P.sp_X64 + 4 * (int64_t)s), __ldg(P.sp_X64 + 4 * (int64_t)s + 1),
+                             __ldg(P.sp_X64 + 4 * (int64_t)s + 2)};
+        double a[3] = {0.0, 0.0, 0.0};
+        for (int k = 0; k < K; ++k) {
+            const HgObs o = load_hg(P, (int64_t)sl.z + 32 * k + lane);
+            if (o.cam >= 0) hg_u(P, o, s_rows64 + o.cam * kRowD, X, a);
+        }
+        for (int d = 1; d < (1 << lg); d <<= 1) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) a[q] += __shfl_xor_sync(full, a[q], d);
+        }
+        const int64_t pt = __ldg(P.sp_pt + s);
+        if (P.has_fixed && P.pt_fixed[pt]) a[0] = a[1] = a[2] = 0.0;
+        double ci[6], dp[3];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) ci[q] = __ldg(Ci + (int64_t)q * P.np_pad + s);
+        const double w0 = P.w[3 * pt], w1 = P.w[3 * pt + 1], w2 = P.w[3 * pt + 2];
+        apply_sym3(ci, w0 - a[0], w1 - a[1], w2 - a[2], dp);
+        if (P.has_fixed && P.pt_fixed[pt]) dp[0] = dp[1] = dp[2] = 0.0;
+        if (act && (lane & ((1 << lg) - 1)) == 0) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                P.dp[3 * pt + k] = dp[k];
+                P.pts_new[3 * pt + k] = P.pts[3 * pt + k] + dp[k];
+            }
+            ldec += w0 * dp[0] + w1 * dp[1] + w2 * dp[2];
+        }
+        for (int k = 0; k < K; ++k) {
+            const int64_t slot = (int64_t)sl.z + 32 * k + lane;
+            const HgObs o = load_hg(P, slot);
+            if (o.cam < 0) continue;
+            const double *r = s_rows64 + o.cam * kRowD;
+            double al[3];
+            hg_alpha(P, r, o.cam, X, al);
+            const double sg = fma(o.v[9], fma(o.v[9], r[8], r[7]), r[6]);
+            const double d0 = al[0] + dp[0], d1 = al[1] + dp[1], d2 = al[2] + dp[2];
+            const double h0 = fma(o.v[0], d0, fma(o.v[1], d1, fma(o.v[2], d2, 2.0 * sg * o.v[6])));
+            const double h1 = fma(o.v[1], d0, fma(o.v[3], d1, fma(o.v[4], d2, 2.0 * sg * o.v[7])));
+            const double h2 = fma(o.v[2], d0, fma(o.v[4], d1, fma(o.v[5], d2, 2.0 * sg * o.v[8])));
+            const double wr = P.sl_w64 ? __ldg(P.sl_w64 + slot) * o.v[9] : o.v[9];
+            ldec -= 0.5 * fma(d0, h0, fma(d1, h1, fma(d2, h2, sg * sg * wr)));
+        }
+    }
+    const double s = block_sum(ldec, sb);
+    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+}
+
 // Camera rows (with the constants) of the PCG solution dc, for the factored
-// back-substitution; one thread per camera.
+// back-substitution of problems whose rows do not fit in shared memory.
 __global__ void fact_rows_kernel(Prob P, const double *__restrict__ x, float *__restrict__ rows) {
     if (P.st->done) return;
     for (int cam = blockIdx.x * blockDim.x + threadIdx.x; cam < P.nc; cam += gridDim.x * blockDim.x) {
-        float v[9], r[kRow];
+        float v[9], r[kRowG];
 #pragma unroll
         for (int j = 0; j < 9; ++j) v[j] = (float)x[(int64_t)cam * kVec + j];
-        fact_row((const float *)P.camtab + (int64_t)cam * kCamTab, v, true, r);
-        float4 *dst = (float4 *)(rows + (int64_t)cam * kRow);
+        fact_row(P, cam, v, r);
+        float4 *dst = (float4 *)(rows + (int64_t)cam * kRowG);
 #pragma unroll
-        for (int i = 0; i < kRow / 4; ++i) dst[i] = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+        for (int i = 0; i < kRowG / 4; ++i) dst[i] = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
     }
 }
 
@@ -1975,38 +1960,24 @@ cudaError_t launch_damp(const Prob &P, int damping, int precond, const int32_t *
 // search direction (nc x 9) when it also fits; otherwise the point pass
 // gathers p from global memory and an extra barrier is needed.
 void plan_pcg_smem(Prob &P) {
+    if (P.own) return;  // planned with the blocks (sell.cu)
     const int w = P.fp32 ? 4 : 8;
-    const int per_cam = P.fact ? kRow : 9;  // the factored form stages a kRow-float row per camera
+    const int per_cam = P.fact ? kRowS : 9;  // the factored form stages a row per camera
     const int64_t budget = 227 * 1024 - 12 * 1024;
-    const int64_t slots = (int64_t)P.pcg_max_cta_chunks * 9 * 8;
+    const int64_t slots = (int64_t)(P.fact ? P.pcg_max_cta_cams + 32 : P.pcg_max_cta_chunks) * 9 * 8;
     const int64_t psb = (((int64_t)P.nc * per_cam * w) + 127) & ~(int64_t)127;
     P.pcg_use_ps = (psb + slots <= budget) ? 1 : 0;
     P.pcg_ps_bytes = P.pcg_use_ps ? (int)psb : 0;
-    // the staged point pass of the factored form, when the camera rows do not fit
-    // in shared memory (their gather from L2 then sits on the direct pass's
-    // critical path), with as many stages (2..kMaxStages) as fit.  Where the rows
-    // fit, the direct pass is faster (Venice-shaped problem: 109 us per PCG
-    // iteration against 134 with two stages, 152 with three stages and the rows
-    // in L2, and 147 with a per-warp cp.async prefetch of the next chunk);
-    // Final-shaped: 1,318 against 1,475 us with two stages
-    const int64_t base = ((P.pcg_ps_bytes + slots) + 127) & ~(int64_t)127;
-    const bool ranges_ok = 6 * (int64_t)P.np + 64 < (int64_t)INT32_MAX && (int64_t)P.n + 64 < (int64_t)INT32_MAX;
-    int64_t stages = P.fact && !P.pcg_use_ps && P.n_tiles > 0 && ranges_ok ? (budget - base) / kStageBytes : 0;
-    if (stages > kMaxStages) stages = kMaxStages;
-    if (stages < 2) stages = 0;
-    P.pcg_stages = (int)stages;
-    P.pcg_stage_off = (int)base;
-    P.pcg_smem = stages ? (int)(base + stages * kStageBytes) : (int)(P.pcg_ps_bytes + slots);
+    P.pcg_smem = (int)(P.pcg_ps_bytes + slots);
 }
 
 int pcg_block(const Prob &P) { return P.fp32 ? PcgBlock<float>::value : PcgBlock<double>::value; }
 
 template <bool SR>
 static const void *pcg_fn_v(const Prob &P) {
-    if (!P.fp32) return (const void *)pcg_kernel<double, true, false, SR>;
-    if (P.autodiff) return (const void *)pcg_kernel<float, true, false, SR>;
-    return P.pcg_stages ? (const void *)pcg_kernel<float, false, true, SR>
-                        : (const void *)pcg_kernel<float, false, false, SR>;
+    if (P.own) return P.fp32 ? (const void *)pcg_own_kernel<float, SR> : (const void *)pcg_own_kernel<double, SR>;
+    if (!P.fp32) return (const void *)pcg_kernel<double, true, SR>;
+    return P.autodiff ? (const void *)pcg_kernel<float, true, SR> : (const void *)pcg_kernel<float, false, SR>;
 }
 static const void *pcg_fn(const Prob &P, int variant = MBA_PCG_STANDARD) {
     return variant == MBA_PCG_SINGLE_REDUCTION ? pcg_fn_v<true>(P) : pcg_fn_v<false>(P);
@@ -2040,8 +2011,7 @@ cudaError_t launch_pcg(const Prob &P, int mode, int max_iter, double tol, long l
     // the barrier targets count arrivals from zero in every launch
     cudaError_t e = cudaMemsetAsync(&P.st->barrier, 0, sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    // the shared-memory plan differs between problems (stages, search direction),
-    // so the kernel's dynamic shared-memory limit is set for this launch
+    // the shared-memory plan differs between problems, so the kernel's dynamic shared-memory limit is set for this launch
     e = cudaFuncSetAttribute(pcg_fn(P, variant), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     Prob Pc = P;
@@ -2051,12 +2021,26 @@ cudaError_t launch_pcg(const Prob &P, int mode, int max_iter, double tol, long l
 
 cudaError_t launch_backsub(const Prob &P, double *partial, int nb, cudaStream_t s) {
     if (P.fact) {
-        fact_rows_kernel<<<(P.nc + 127) / 128, 128, 0, s>>>(P, P.x, (float *)P.pT);
-        backsub_kernel<float, true><<<nb, kBlock, 0, s>>>(P, partial);
+        const int smem = P.nc * kRowS * 4;
+        const SliceGrid g = slice_grid(P);
+        nb = g.ctas;
+        if (smem <= 220 * 1024) {
+            cudaFuncSetAttribute(backsub_slices_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            backsub_slices_kernel<true><<<g.ctas, g.threads, smem, s>>>(P, partial);
+        } else {
+            fact_rows_kernel<<<(P.nc + 127) / 128, 128, 0, s>>>(P, P.x, (float *)P.pT);
+            backsub_slices_kernel<false><<<g.ctas, g.threads, 0, s>>>(P, partial);
+        }
+    } else if (P.own) {
+        const int smem = P.nc * kRowD * 8;  // fits: the block-owned product holds the same rows
+        const SliceGrid g = slice_grid(P, 512);
+        nb = g.ctas;
+        cudaFuncSetAttribute(backsub_slices64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        backsub_slices64_kernel<<<g.ctas, g.threads, smem, s>>>(P, partial);
     } else if (P.fp32) {
-        backsub_kernel<float, false><<<nb, kBlock, 0, s>>>(P, partial);
+        backsub_kernel<float><<<nb, kBlock, 0, s>>>(P, partial);
     } else {
-        backsub_kernel<double, false><<<nb, kBlock, 0, s>>>(P, partial);
+        backsub_kernel<double><<<nb, kBlock, 0, s>>>(P, partial);
     }
     ldec_final_kernel<<<1, kBlock, 0, s>>>(partial, nb, P.st);
     cams_new_kernel<<<(P.nc * 9 + kBlock - 1) / kBlock, kBlock, 0, s>>>(P);
