@@ -27,8 +27,18 @@
 // The IRLS weight W multiplies the products once (W Jp^T Jc p, W Jp b), which
 // equals the sqrt(W) scaling of both factors.
 //
-// Summation orders are fixed by the launch schedule (threads per CTA), so a
-// schedule gives the same bits on every run.
+// Few windows.  With fewer windows than SMs one CTA per window leaves most of the
+// GPU idle, and an FP64 window is bound by its SM's FP64 pipe.  The automatic
+// schedule then gives each window a thread-block cluster of 2 to 16 CTAs (the
+// CL instances): observations, points and the blocks and rows of S~ are divided
+// over the ranks, the camera-side state is kept in every rank's shared memory
+// and the ranks exchange sums, B~^-1 blocks and the rows of q = S~ p through
+// distributed shared memory.  Every rank runs the same scalar recurrences on the
+// same values, so the ranks take the same decisions and meet at the same
+// cluster barriers.
+//
+// Summation orders are fixed by the launch schedule (threads per CTA, cluster
+// size), so a schedule gives the same bits on every run.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -64,6 +74,7 @@ struct BatchOpts {
 
 struct BatchArgs {
     int32_t nw, ncmax, loss, s_smem;  // s_smem: explicit S~ held in shared memory
+    int32_t srows, pad;       // cluster form: rows of S~ a rank holds in shared memory (0: none)
     double delta;
     const WinDesc *desc;
     const int32_t *order;     // claim order (windows by decreasing observation count)
@@ -115,7 +126,48 @@ struct WinMem {
     T *rT;  // r rounded to T, the preconditioner's input (FP64: r itself)
     T *S;  // explicit S~ in shared memory (NULL: the CTA's global scratch)
     int32_t *cptr, *wf, *wl, *wcam0;
+    // cluster form: rank and size, this rank's rows of S~ (NULL: read from the
+    // scratch), their stride, two exchange buffers of scalars
+    int32_t rank, csz, slot_id, ldS;
+    T *Srow;
+    double *xch;
 };
+
+// ---------------------------------------------------------------------------
+// thread-block cluster helpers (CL instances)
+// ---------------------------------------------------------------------------
+constexpr int kMaxCluster = 16;
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t peer_addr(const void *p, int rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ double ld_peer(const double *p, int rank) {
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(peer_addr(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ int ld_peer(const int32_t *p, int rank) {
+    int v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(peer_addr(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_peer(double *p, int rank, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(peer_addr(p, rank)), "d"(v) : "memory");
+}
+__device__ __forceinline__ void st_peer(float *p, int rank, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_addr(p, rank)), "f"(v) : "memory");
+}
+// every thread of every CTA of the cluster; orders global and shared memory
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <bool CL>
+__device__ __forceinline__ void win_sync() {
+    if constexpr (CL) cluster_barrier();
+    else __syncthreads();
+}
 
 // Pairs staged per warp while a Schur block is formed, and the stride of one
 // staged pair (Jc~ of the first observation, F = G Jc~ of the second; padded).
@@ -161,7 +213,28 @@ __host__ __device__ inline size_t win_carve(unsigned char *base, int ncmax, int 
     m.wcam0 = (int32_t *)take(4 * (size_t)nwarp);
     m.BinvT = (T *)take(sizeof(T) * 45 * (size_t)ncmax);
     m.S = svals > 0 ? (T *)take(sizeof(T) * (size_t)svals) : nullptr;
+    m.rank = 0;
+    m.csz = 1;
+    m.slot_id = 0;
+    m.ldS = 0;
+    m.Srow = nullptr;
+    m.xch = nullptr;
     return (size_t)off;
+}
+
+// Stride of a cluster rank's rows of S~: 8 mod 32, so that the four rows a warp
+// reads at a time (eight lanes each) start in different banks.
+__host__ __device__ inline int srow_ld(int m9) { return (m9 + 23) / 32 * 32 + 8; }
+// The cluster form's additions: the exchange buffers and, if rows > 0, this
+// rank's rows of S~.
+template <typename T>
+__host__ __device__ inline size_t cluster_carve(unsigned char *base, size_t off, int ncmax, int rows, WinMem<T> &m) {
+    m.xch = (double *)(base + off);
+    off += sizeof(double) * 2 * kMaxCluster;
+    m.ldS = srow_ld(9 * ncmax);
+    m.Srow = rows > 0 ? (T *)(base + off) : nullptr;
+    off += sizeof(T) * (size_t)rows * m.ldS;
+    return off;
 }
 
 // Per-window control state (shared, written by thread 0 between barriers).
@@ -217,6 +290,19 @@ __device__ __forceinline__ double2 cta_sum2(double a, double b, double *sb) {
     }
     __syncthreads();
     return make_double2(sb[2 * NT], sb[2 * NT + 1]);
+}
+
+// Sum over the cluster's ranks of one value per CTA (the same in its threads),
+// added in rank order by every rank.  `turn` alternates between the two exchange
+// buffers: a rank can be one barrier ahead of another, not two.
+__device__ __forceinline__ double cluster_sum(double v, double *xch, int rank, int csz, int &turn) {
+    double *buf = xch + kMaxCluster * (turn & 1);
+    turn += 1;
+    if (threadIdx.x < (unsigned)csz) st_peer(buf + rank, (int)threadIdx.x, v);
+    cluster_barrier();
+    double s = 0.0;
+    for (int r = 0; r < csz; ++r) s += buf[r];
+    return s;
 }
 
 // The same sum, with fin(x, y) run by thread 0 on the result before the
@@ -501,15 +587,16 @@ __device__ __forceinline__ void load_rec(const BatchArgs &A, const WinDesc &d, i
 // Linearisation over the window's warp chunks: e, Jp and W per observation; per point
 // C = sum W Jp^T Jp and w = -sum W Jp^T e by a segmented scan (whole points per
 // chunk) or a warp sum (one long-track point); the point-major X record and W.
-template <typename T, int NT>
+template <typename T, int NT, bool CL>
 __device__ void lin_points(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d) {
     constexpr int NW = NT / 32;
+    const int rk = CL ? M.rank : 0, cs = CL ? M.csz : 1;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned full = 0xffffffffu;
     T *Xw = (T *)A.Xw;
     T *Wpm = (T *)A.Wpm;
     const T delta = (T)A.delta;
-    for (int c = d.wch0 + wid; c < d.wch0 + d.nwch; c += NW) {
+    for (int c = d.wch0 + wid + NW * rk; c < d.wch0 + d.nwch; c += NW * cs) {
         const int2 c0 = __ldg(A.wchunk + c), c1 = __ldg(A.wchunk + c + 1);
         const int o0 = c0.y, m = c1.y - c0.y;
         const bool longp = m > 32;
@@ -569,11 +656,12 @@ __device__ void lin_points(const BatchArgs &A, const WinMem<T> &M, const WinDesc
 
 // Right-hand side pass, per observation (no segments): s_k = W Jp b_j with
 // b_j = C~_j^-1 wvec_j, into camera-major order.
-template <typename T, int NT>
+template <typename T, int NT, bool CL>
 __device__ void rhs_points(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, const double *wvec) {
     using T2 = typename V2<T>::type;
     T2 *cms = (T2 *)A.cms;
-    for (int k = threadIdx.x; k < d.n; k += NT) {
+    const int rk = CL ? M.rank : 0, cs = CL ? M.csz : 1;
+    for (int k = threadIdx.x + NT * rk; k < d.n; k += NT * cs) {
         PmRec<T> r;
         load_rec<T>(A, d, d.obs0 + k, r);
         const int pt = d.pt0 + (r.key >> 6);
@@ -727,14 +815,15 @@ __device__ void iter_points(const BatchArgs &A, const WinMem<T> &M, const WinDes
 // d_k = Jc x + Jp dp_j.  Forward solve: candidate points and this thread's
 // share of the model decrease sum_k W (-e.d - |d|^2/2).  Adjoint: W d_k per
 // observation in input order.
-template <typename T, int NT>
+template <typename T, int NT, bool CL>
 __device__ double back_points(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, const double *wvec,
                               bool adj) {
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned full = 0xffffffffu;
+    const int rk = CL ? M.rank : 0, cs = CL ? M.csz : 1;
     double ldec = 0.0;
-    for (int c = d.wch0 + wid; c < d.wch0 + d.nwch; c += NW) {
+    for (int c = d.wch0 + wid + NW * rk; c < d.wch0 + d.nwch; c += NW * cs) {
         const int2 c0 = __ldg(A.wchunk + c), c1 = __ldg(A.wchunk + c + 1);
         const int o0 = c0.y, m = c1.y - c0.y;
         // first sweep: u sums (segmented for whole-point chunks, warp-wide for a long track)
@@ -819,13 +908,15 @@ __device__ double back_points(const BatchArgs &A, const WinMem<T> &M, const WinD
 // sum goes to slot (w + camera), a slot no other segment uses.  LIN: the 45
 // entries of B = sum W Jc^T Jc and v = -sum W Jc^T e (54 per slot);
 // otherwise sum Jc^T s (9 per slot).
-template <typename T, int NT, bool LIN>
+template <typename T, int NT, bool LIN, bool CL>
 __device__ void camera_pass(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, bool wj = false) {
     using T2 = typename V2<T>::type;
     constexpr int NW = NT / 32;
     constexpr int K = LIN ? 54 : 9;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int lo = (int)(((int64_t)wid * d.n) / NW), hi = (int)(((int64_t)(wid + 1) * d.n) / NW);
+    // the warps of all ranks divide the window's observations
+    const int gw = wid + (CL ? NW * M.rank : 0), nwt = NW * (CL ? M.csz : 1);
+    const int lo = (int)(((int64_t)gw * d.n) / nwt), hi = (int)(((int64_t)(gw + 1) * d.n) / nwt);
     if (lo >= hi) return;
     T *cmX = (T *)A.cmX;
     const T2 *cms = (const T2 *)A.cms;
@@ -902,10 +993,16 @@ __device__ void camera_pass(const BatchArgs &A, const WinMem<T> &M, const WinDes
 }
 
 // Sum of camera i's segment slots (stride K), in warp order.
+// CL: warp w of the window is warp w mod NW of rank w / NW, whose slots are read
+// through distributed shared memory.
+template <int NW, bool CL>
 __device__ __forceinline__ double slot_sum(const double *slot, const int32_t *wf, const int32_t *wl, int i, int K,
                                            int q) {
     double s = 0.0;
-    for (int w = wf[i]; w <= wl[i]; ++w) s += slot[(w + i) * K + q];
+    for (int w = wf[i]; w <= wl[i]; ++w) {
+        if constexpr (CL) s += ld_peer(slot + ((w % NW) + i) * K + q, w / NW);
+        else s += slot[(w + i) * K + q];
+    }
     return s;
 }
 
@@ -947,29 +1044,59 @@ __device__ __forceinline__ double2 precond(const WinMem<T> &M, int nc) {
     return make_double2(rr, rz);
 }
 
-template <typename T, int NT>
+template <typename T, int NT, bool CL>
 __device__ void linearize(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, bool xs) {
     for (int t = threadIdx.x; t < d.nc * kCamTab; t += NT) {
         const int i = t / kCamTab, q = t - kCamTab * (t / kCamTab);
         M.tabT[i * kTabS + q] = (T)M.tab64[t];
     }
     __syncthreads();
-    lin_points<T, NT>(A, M, d);
+    lin_points<T, NT, CL>(A, M, d);
     __syncthreads();
-    camera_pass<T, NT, true>(A, M, d, xs);
-    __syncthreads();
+    camera_pass<T, NT, true, CL>(A, M, d, xs);
+    win_sync<CL>();
     for (int t = threadIdx.x; t < d.nc * 54; t += NT) {
         const int i = t / 54, q = t - 54 * (t / 54);
-        const double s = slot_sum(M.slot, M.wf, M.wl, i, 54, q);
+        const double s = slot_sum<NT / 32, CL>(M.slot, M.wf, M.wl, i, 54, q);
         if (q < 45) M.Hpp[45 * i + q] = s;
         else M.v[9 * i + (q - 45)] = s;
     }
-    __syncthreads();
+    win_sync<CL>();
 }
 
 // B~ = B + mu D and its inverse (Cholesky, FP64, packed), C~^-1 per point (adjugate, FP64 -> T).
-template <typename T, int NT>
+// CL: the ranks divide the cameras, one warp each (warp_spd_inverse9), and send
+// every B~^-1 to all ranks; they divide the points as well, and a failure
+// anywhere reaches every rank.
+template <typename T, int NT, bool CL>
 __device__ void damp(const BatchArgs &A, const WinMem<T> &M, WinState &S, const WinDesc &d, double mu, int damping) {
+    constexpr int NW = NT / 32;
+    if constexpr (CL) {
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        double *As = M.slot + (size_t)wid * 256, *Ys = As + 81, *il = Ys + 81;  // the slots are free here
+        for (int i = wid + NW * M.rank; i < d.nc; i += NW * M.csz) {
+            __syncwarp();
+            for (int e = lane; e < 81; e += 32) {
+                const int a = e / 9, b = e - 9 * (e / 9);
+                double v = M.Hpp[45 * i + sym9(a, b)];
+                if (a == b) v += mu * damp_term_b(damping, v);
+                As[e] = v;
+            }
+            __syncwarp();
+            if (warp_spd_inverse9(As, Ys, il, (double *)nullptr)) {
+                for (int e = lane; e < 45; e += 32) {  // entry (r, c), r <= c, of L^-T L^-1
+                    int r = 0, f = e;
+                    while (f >= 9 - r) f -= 9 - r, ++r;
+                    const int c = r + f;
+                    double v = 0.0;
+                    for (int k = c; k < 9; ++k) v += Ys[k * 9 + r] * Ys[k * 9 + c];
+                    for (int k = 0; k < M.csz; ++k) st_peer(M.BinvT + 45 * i + e, k, (T)v);
+                }
+            } else if (lane == 0) {
+                S.blockfail = 1;
+            }
+        }
+    } else
     for (int i = threadIdx.x; i < d.nc; i += NT) {
         double L[81];
         for (int a = 0; a < 9; ++a)
@@ -1013,7 +1140,7 @@ __device__ void damp(const BatchArgs &A, const WinMem<T> &M, WinState &S, const 
         }
     }
     T *Ci = (T *)A.Cinv;
-    for (int j = threadIdx.x; j < d.np; j += NT) {
+    for (int j = threadIdx.x + (CL ? NT * M.rank : 0); j < d.np; j += NT * (CL ? M.csz : 1)) {
         const int64_t pt = d.pt0 + j;
         const double *h = A.Hll + 6 * pt;
         const double a00 = h[0] + mu * damp_term_b(damping, h[0]), a01 = h[1], a02 = h[2];
@@ -1032,6 +1159,13 @@ __device__ void damp(const BatchArgs &A, const WinMem<T> &M, WinState &S, const 
         Ci[6 * pt + 3] = (T)((a00 * a22 - a02 * a02) * id);
         Ci[6 * pt + 4] = (T)((a02 * a01 - a00 * a12) * id);
         Ci[6 * pt + 5] = (T)((a00 * a11 - a01 * a01) * id);
+    }
+    if constexpr (CL) {
+        cluster_barrier();
+        int f = 0;
+        for (int r = 0; r < M.csz; ++r) f |= ld_peer(&S.blockfail, r);
+        cluster_barrier();
+        if (threadIdx.x == 0) S.blockfail = f;
     }
 }
 
@@ -1070,19 +1204,19 @@ __device__ __forceinline__ void ld24<double>(const double *p, double *o) {
     }
 }
 
-template <typename T, int NT>
+template <typename T, int NT, bool CL>
 __device__ void s_build(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, double mu, int damping) {
     constexpr int NW = NT / 32;
     constexpr int SP = Stage<T>::pairs, SS = Stage<T>::stride;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nc = d.nc, nb = nc * (nc + 1) / 2;
-    T *S = M.S ? M.S : (T *)A.S + A.smax * (int64_t)blockIdx.x;
+    T *S = M.S ? M.S : (T *)A.S + A.smax * (int64_t)(CL ? M.slot_id : blockIdx.x);
     T *st = M.stage + wid * SP * SS;
     const T *Jcm = (const T *)A.Jcm;
     const T *Ci = (const T *)A.Cinv;
     const int a = lane / 3, b0 = 3 * (lane - 3 * (lane / 3));
     int bi = 0, bk = 0, bcur = 0;  // (i, k) of block bcur, advanced incrementally
-    for (int blk = wid; blk < nb; blk += NW) {
+    for (int blk = wid + (CL ? NW * M.rank : 0); blk < nb; blk += NW * (CL ? M.csz : 1)) {
         while (bcur < blk) {
             ++bk;
             if (bk == nc) {
@@ -1143,6 +1277,20 @@ __device__ void s_build(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d
             }
         }
     }
+    if constexpr (CL) {
+        // this rank's rows of the symmetric S~, from the blocks all ranks formed
+        cluster_barrier();
+        if (M.Srow) {
+            const int m9 = 9 * nc, per = (m9 + M.csz - 1) / M.csz, r0 = per * M.rank, rows = min(per, m9 - r0);
+            const T *Sg = (const T *)A.S + A.smax * (int64_t)M.slot_id;
+            for (int e = threadIdx.x; e < rows * m9; e += NT) {
+                const int rr = e / m9, c = e - rr * m9, r = r0 + rr;
+                const int i = r / 9, a2 = r - 9 * i, k = c / 9, b2 = c - 9 * k;
+                M.Srow[rr * M.ldS + c] = i <= k ? __ldcg(Sg + 81 * (int64_t)blk_index(i, k, nc) + 9 * a2 + b2)
+                                                : __ldcg(Sg + 81 * (int64_t)blk_index(k, i, nc) + 9 * b2 + a2);
+            }
+        }
+    }
 }
 
 // q = S~ p (p given in M.pv as T) into M.q.
@@ -1171,12 +1319,52 @@ __device__ void s_matvec(const BatchArgs &A, const WinMem<T> &M, const WinDesc &
     }
 }
 
+// Cluster form: this rank's rows of q = S~ p, eight lanes per row, sent to every
+// rank's q.  Ends with the cluster barrier that completes q everywhere; `q` has
+// to alternate between two buffers (a rank may still read the previous one).
+template <typename T, int NT>
+__device__ void s_matvec_cluster(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, double *q) {
+    const int nc = d.nc, m9 = 9 * nc, per = (m9 + M.csz - 1) / M.csz, r0 = per * M.rank;
+    const int rows = min(per, m9 - r0), g = threadIdx.x & 7;
+    const T *pT = M.pv;
+    const T *Sg = (const T *)A.S + A.smax * (int64_t)M.slot_id;
+    for (int b0 = 0; b0 < rows; b0 += NT / 8) {
+        const int rr = b0 + (threadIdx.x >> 3);
+        T a0 = T(0), a1 = T(0);
+        if (rr < rows) {
+            if (M.Srow) {
+                const T *Sr = M.Srow + rr * M.ldS;
+                int c = g;
+                for (; c + 8 < m9; c += 16) {
+                    a0 += Sr[c] * pT[c];
+                    a1 += Sr[c + 8] * pT[c + 8];
+                }
+                if (c < m9) a0 += Sr[c] * pT[c];
+            } else {
+                const int r = r0 + rr, i = r / 9, a = r - 9 * i;
+                for (int k = g; k < nc; k += 8) {
+                    const T *Sb = Sg + 81 * (int64_t)(k < i ? blk_index(k, i, nc) : blk_index(i, k, nc)) + (k < i ? a : 9 * a);
+                    const int st = k < i ? 9 : 1;
+#pragma unroll
+                    for (int b = 0; b < 9; ++b) a0 += __ldcg(Sb + st * b) * pT[9 * k + b];
+                }
+            }
+        }
+        T v = a0 + a1;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (rr < rows)
+            for (int k = g; k < M.csz; k += 8) st_peer(q + r0 + rr, k, (double)v);
+    }
+    cluster_barrier();
+}
+
 // Schur-Jacobi preconditioner (solver variant) from the explicit S~: the
 // inverse (Cholesky, FP64) of each diagonal block replaces B~_i^-1; a block that
 // is not positive definite keeps B~_i^-1.  One thread per camera.
-template <typename T, int NT>
+template <typename T, int NT, bool CL>
 __device__ void sj_from_s(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d) {
-    const T *S = M.S ? M.S : (const T *)A.S + A.smax * (int64_t)blockIdx.x;
+    const T *S = M.S ? M.S : (const T *)A.S + A.smax * (int64_t)(CL ? M.slot_id : blockIdx.x);
     for (int i = threadIdx.x; i < d.nc; i += NT) {
         const T *Sb = S + 81 * (int64_t)blk_index(i, i, d.nc);
         double L[81], il[9];
@@ -1262,7 +1450,7 @@ __device__ __noinline__ int pcg_single_reduction(const BatchArgs &A, const WinMe
             __syncthreads();
             iter_points<T, NT>(A, M, d);
             __syncthreads();
-            camera_pass<T, NT, false>(A, M, d);
+            camera_pass<T, NT, false, false>(A, M, d);
             __syncthreads();
             for (int t = threadIdx.x; t < m9; t += NT) {
                 const int i = t / 9, a = t - 9 * (t / 9);
@@ -1272,7 +1460,7 @@ __device__ __noinline__ int pcg_single_reduction(const BatchArgs &A, const WinMe
 #pragma unroll
                 for (int b = 0; b < 9; ++b) bu = fma(Hi[sym9(a, b)], ui[b], bu);
                 bu = fma(mu * damp_term_b(damping, Hi[sym9(a, a)]), ui[a], bu);
-                const double w = bu - slot_sum(M.slot, M.wf, M.wl, i, 9, a);
+                const double w = bu - slot_sum<NT / 32, false>(M.slot, M.wf, M.wl, i, 9, a);
                 M.q[t] = w;
                 wu = fma(M.z[t], w, wu);
             }
@@ -1320,22 +1508,23 @@ __device__ __noinline__ int pcg_single_reduction(const BatchArgs &A, const WinMe
     return n;
 }
 
-template <typename T, int NT>
+template <typename T, int NT, bool CL>
 __device__ int pcg(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, const double *vvec, const double *wvec,
                    double mu, int damping, int max_iter, double tol, bool xs, double *g0, bool sr) {
     const int m9 = 9 * d.nc;
-    rhs_points<T, NT>(A, M, d, wvec);
-    __syncthreads();
-    camera_pass<T, NT, false>(A, M, d);
-    __syncthreads();
+    rhs_points<T, NT, CL>(A, M, d, wvec);
+    win_sync<CL>();
+    camera_pass<T, NT, false, CL>(A, M, d);
+    win_sync<CL>();
     for (int t = threadIdx.x; t < m9; t += NT) {
         const int i = t / 9, a = t - 9 * (t / 9);
-        const double rv = vvec[t] - slot_sum(M.slot, M.wf, M.wl, i, 9, a);
+        const double rv = vvec[t] - slot_sum<NT / 32, CL>(M.slot, M.wf, M.wl, i, 9, a);
         M.r[t] = rv;
         M.rT[t] = (T)rv;
         M.x[t] = 0.0;
     }
-    __syncthreads();
+    win_sync<CL>();  // CL: every rank has read the slots
+    if constexpr (!CL)
     if (sr) return pcg_single_reduction<T, NT>(A, M, d, mu, damping, max_iter, tol, xs, g0);
     // scalar recurrences in thread 0 (see cta_sum2f): sc[0] holds beta or alpha,
     // *go the continue flag
@@ -1363,23 +1552,25 @@ __device__ int pcg(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, con
         for (;;) {
             const double beta = sc[0];
             double pq = 0.0;
-            if (xs) {
+            double *qv = (CL && (n & 1)) ? M.sv : M.q;
+            if (CL || xs) {
                 for (int t = threadIdx.x; t < m9; t += NT) {
                     const double pn = n == 0 ? M.z[t] : fma(beta, M.p[t], M.z[t]);
                     M.p[t] = pn;
                     M.pv[t] = (T)pn;
                 }
                 __syncthreads();
-                s_matvec<T, NT>(A, M, d);
-                for (int t = threadIdx.x; t < m9; t += NT) pq = fma(M.p[t], M.q[t], pq);
-            } else {
+                if constexpr (CL) s_matvec_cluster<T, NT>(A, M, d, qv);
+                else s_matvec<T, NT>(A, M, d);
+                for (int t = threadIdx.x; t < m9; t += NT) pq = fma(M.p[t], qv[t], pq);
+            } else if constexpr (!CL) {
             for (int t = threadIdx.x; t < m9; t += NT) M.p[t] = n == 0 ? M.z[t] : fma(beta, M.p[t], M.z[t]);
             __syncthreads();
             make_pv<T, NT>(M, M.p, d.nc);
             __syncthreads();
             iter_points<T, NT>(A, M, d);
             __syncthreads();
-            camera_pass<T, NT, false>(A, M, d);
+            camera_pass<T, NT, false, false>(A, M, d);
             __syncthreads();
             for (int t = threadIdx.x; t < m9; t += NT) {
                 const int i = t / 9, a = t - 9 * (t / 9);
@@ -1389,7 +1580,7 @@ __device__ int pcg(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, con
 #pragma unroll
                 for (int b = 0; b < 9; ++b) bp = fma(Hi[sym9(a, b)], pi_[b], bp);
                 bp = fma(mu * damp_term_b(damping, Hi[sym9(a, a)]), pi_[a], bp);
-                const double q = bp - slot_sum(M.slot, M.wf, M.wl, i, 9, a);
+                const double q = bp - slot_sum<NT / 32, CL>(M.slot, M.wf, M.wl, i, 9, a);
                 M.q[t] = q;
                 pq = fma(M.p[t], q, pq);
             }
@@ -1403,7 +1594,7 @@ __device__ int pcg(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, con
             const double alpha = sc[0];
             for (int t = threadIdx.x; t < m9; t += NT) {
                 M.x[t] = fma(alpha, M.p[t], M.x[t]);
-                const double rv = fma(-alpha, M.q[t], M.r[t]);
+                const double rv = fma(-alpha, qv[t], M.r[t]);
                 M.r[t] = rv;
                 M.rT[t] = (T)rv;
             }
@@ -1424,10 +1615,10 @@ __device__ int pcg(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, con
 }
 
 // F = 1/2 sum rho(|e|^2) in FP64 with the FP64 camera table in M.tab64.
-template <typename T, int NT>
+template <typename T, int NT, bool CL>
 __device__ double cost(const BatchArgs &A, const WinMem<T> &M, const WinDesc &d, const double *pts) {
     double acc = 0.0;
-    for (int k = threadIdx.x; k < d.n; k += NT) {
+    for (int k = threadIdx.x + (CL ? NT * M.rank : 0); k < d.n; k += NT * (CL ? M.csz : 1)) {
         const int o = d.obs0 + k;
         const int2 pc = __ldg(A.pm_pc + o);
         const double2 uv = __ldg(A.pm_uv + o);
@@ -1448,23 +1639,21 @@ __device__ __forceinline__ void tables64(const WinMem<T> &M, const double *cams,
 }
 
 // Warp ownership of the camera-major observations of a window.
-template <int NT>
-__device__ __forceinline__ int warp_lo(int w, int n) {
-    return (int)(((int64_t)w * n) / (NT / 32));
-}
-template <int NT>
-__device__ int owner_warp(int r, int n) {
-    constexpr int NW = NT / 32;
+__device__ __forceinline__ int warp_lo(int w, int n, int NW) { return (int)(((int64_t)w * n) / NW); }
+__device__ int owner_warp(int r, int n, int NW) {
     int w = (int)(((int64_t)r * NW) / n);
     if (w > NW - 1) w = NW - 1;
-    while (w + 1 < NW && warp_lo<NT>(w + 1, n) <= r) ++w;
-    while (w > 0 && warp_lo<NT>(w, n) > r) --w;
+    while (w + 1 < NW && warp_lo(w + 1, n, NW) <= r) ++w;
+    while (w > 0 && warp_lo(w, n, NW) > r) --w;
     return w;
 }
 
-template <typename T, int NT>
+template <typename T, int NT, bool CL>
 __device__ __forceinline__ void solve_window(const BatchArgs &A, const BatchOpts &O, const WinMem<T> &M, WinState &S, int wi) {
     constexpr int NW = NT / 32;
+    const int rk = CL ? M.rank : 0, cs = CL ? M.csz : 1, first = NT * rk, step = NT * cs;
+    int turn = 0;  // exchange buffer of cluster_sum
+    (void)turn;
     const WinDesc d = A.desc[wi];
     const int tid = threadIdx.x, m9 = 9 * d.nc;
     for (int t = tid; t < m9; t += NT) M.cams[t] = A.cams[9 * (int64_t)d.cam0 + t];
@@ -1487,11 +1676,11 @@ __device__ __forceinline__ void solve_window(const BatchArgs &A, const BatchOpts
     }
     __syncthreads();
     for (int i = tid; i < d.nc; i += NT) {
-        M.wf[i] = owner_warp<NT>(M.cptr[i], d.n);
-        M.wl[i] = owner_warp<NT>(M.cptr[i + 1] - 1, d.n);
+        M.wf[i] = owner_warp(M.cptr[i], d.n, NW * cs);
+        M.wl[i] = owner_warp(M.cptr[i + 1] - 1, d.n, NW * cs);
     }
     if (tid < NW) {
-        const int lo = warp_lo<NT>(tid, d.n);
+        const int lo = warp_lo(tid + NW * rk, d.n, NW * cs);
         int c = 0;
         while (c + 1 < d.nc && M.cptr[c + 1] <= lo) ++c;
         M.wcam0[tid] = c;
@@ -1499,7 +1688,8 @@ __device__ __forceinline__ void solve_window(const BatchArgs &A, const BatchOpts
     tables64<T, NT>(M, M.cams, d.nc);
     __syncthreads();
     {
-        const double F = cost<T, NT>(A, M, d, A.pts);
+        double F = cost<T, NT, CL>(A, M, d, A.pts);
+        if constexpr (CL) F = cluster_sum(F, M.xch, rk, cs, turn);
         if (tid == 0) {
             S.F = F;
             S.F0 = F;
@@ -1509,11 +1699,11 @@ __device__ __forceinline__ void solve_window(const BatchArgs &A, const BatchOpts
     for (int it = 0; it < O.max_iter; ++it) {
         if (S.done) break;
         if (S.relin) {
-            linearize<T, NT>(A, M, d, O.explicit_schur != 0);
+            linearize<T, NT, CL>(A, M, d, O.explicit_schur != 0);
             if (tid == 0) S.relin = 0;
         }
         const double mu = 1.0 / S.radius;
-        damp<T, NT>(A, M, S, d, mu, O.damping);
+        damp<T, NT, CL>(A, M, S, d, mu, O.damping);
         __syncthreads();
         if (S.blockfail) {  // no step: the iteration counts as rejected (the rule of lm.cu)
             __syncthreads();
@@ -1530,24 +1720,26 @@ __device__ __forceinline__ void solve_window(const BatchArgs &A, const BatchOpts
         }
         if (S.status != MBA_OK) break;
         if (O.explicit_schur) {
-            s_build<T, NT>(A, M, d, mu, O.damping);
+            s_build<T, NT, CL>(A, M, d, mu, O.damping);
             __syncthreads();
             if (O.precond == MBA_PRECOND_SCHUR_JACOBI) {
-                sj_from_s<T, NT>(A, M, d);
+                sj_from_s<T, NT, CL>(A, M, d);
                 __syncthreads();
             }
         }
-        const int np_ = pcg<T, NT>(A, M, d, M.v, A.wv, mu, O.damping, O.pcg_max_iter, O.pcg_tol,
+        const int np_ = pcg<T, NT, CL>(A, M, d, M.v, A.wv, mu, O.damping, O.pcg_max_iter, O.pcg_tol,
                                    O.explicit_schur != 0, O.forcing ? &S.g0 : nullptr, O.pcg_variant != 0);
         make_pv<T, NT>(M, M.x, d.nc);
         __syncthreads();
-        double ld = back_points<T, NT>(A, M, d, A.wv, false);
+        double ld = back_points<T, NT, CL>(A, M, d, A.wv, false);
         ld = cta_sum2<NT>(ld, 0.0, M.sb).x;
+        if constexpr (CL) ld = cluster_sum(ld, M.xch, rk, cs, turn);  // and every candidate point is written
         for (int t = tid; t < m9; t += NT) M.camn[t] = M.cams[t] + M.x[t];
         __syncthreads();
         tables64<T, NT>(M, M.camn, d.nc);
         __syncthreads();
-        const double Fn = cost<T, NT>(A, M, d, A.pts_new);
+        double Fn = cost<T, NT, CL>(A, M, d, A.pts_new);
+        if constexpr (CL) Fn = cluster_sum(Fn, M.xch, rk, cs, turn);
         if (tid == 0) {
             // trust-region rule of lm.cu
             const double F = S.F, L = ld;
@@ -1577,10 +1769,10 @@ __device__ __forceinline__ void solve_window(const BatchArgs &A, const BatchOpts
         __syncthreads();
         if (S.accept) {
             for (int t = tid; t < m9; t += NT) M.cams[t] = M.camn[t];
-            for (int t = tid; t < 3 * d.np; t += NT)
+            for (int t = tid + first; t < 3 * d.np; t += step)
                 A.pts[3 * (int64_t)d.pt0 + t] = A.pts_new[3 * (int64_t)d.pt0 + t];
         }
-        __syncthreads();
+        win_sync<CL>();
     }
     // adjoint at the solution (mba_adjoint): v = M^-1 gbar, dL/du_k = W_k J_k v, dL/dx0 = mu D v
     if (O.adjoint) {
@@ -1588,36 +1780,36 @@ __device__ __forceinline__ void solve_window(const BatchArgs &A, const BatchOpts
             tables64<T, NT>(M, M.cams, d.nc);
             __syncthreads();
             if (S.relin) {
-                linearize<T, NT>(A, M, d, O.explicit_schur != 0);
+                linearize<T, NT, CL>(A, M, d, O.explicit_schur != 0);
                 if (tid == 0) S.relin = 0;
             }
             const double mu = O.adj_mu >= 0.0 ? O.adj_mu : S.mu_acc;
-            damp<T, NT>(A, M, S, d, mu, O.damping);
+            damp<T, NT, CL>(A, M, S, d, mu, O.damping);
             __syncthreads();
             if (tid == 0 && S.blockfail) S.status = MBA_ERR_NONFINITE;
             __syncthreads();
             if (S.status == MBA_OK) {
                 if (O.explicit_schur) {
-                    s_build<T, NT>(A, M, d, mu, O.damping);
+                    s_build<T, NT, CL>(A, M, d, mu, O.damping);
                     __syncthreads();
                     if (O.precond == MBA_PRECOND_SCHUR_JACOBI) {
-                        sj_from_s<T, NT>(A, M, d);
+                        sj_from_s<T, NT, CL>(A, M, d);
                         __syncthreads();
                     }
                 }
-                const int na = pcg<T, NT>(A, M, d, A.gbar_c + 9 * (int64_t)d.cam0, A.gbar_p, mu, O.damping,
+                const int na = pcg<T, NT, CL>(A, M, d, A.gbar_c + 9 * (int64_t)d.cam0, A.gbar_p, mu, O.damping,
                                           O.adj_pcg_max, O.adj_pcg_tol, O.explicit_schur != 0, nullptr,
                                           O.pcg_variant != 0);
                 make_pv<T, NT>(M, M.x, d.nc);
                 __syncthreads();
-                back_points<T, NT>(A, M, d, A.gbar_p, true);
-                __syncthreads();
-                for (int t = tid; t < m9; t += NT) {
+                back_points<T, NT, CL>(A, M, d, A.gbar_p, true);
+                win_sync<CL>();
+                for (int t = tid + first; t < m9; t += step) {
                     const int i = t / 9, a = t - 9 * (t / 9);
                     A.grad_c0[9 * (int64_t)d.cam0 + t] =
                         mu * damp_term_b(O.damping, M.Hpp[45 * i + sym9(a, a)]) * M.x[t];
                 }
-                for (int t = tid; t < 3 * d.np; t += NT) {
+                for (int t = tid + first; t < 3 * d.np; t += step) {
                     const int64_t j = d.pt0 + t / 3;
                     const int a = t - 3 * (t / 3);
                     A.grad_p0[3 * j + a] =
@@ -1627,28 +1819,28 @@ __device__ __forceinline__ void solve_window(const BatchArgs &A, const BatchOpts
             }
         } else if (S.status == MBA_OK) {
             // no accepted step: x* = x0 for any nearby input
-            for (int k = tid; k < d.n; k += NT) {
+            for (int k = tid + first; k < d.n; k += step) {
                 const int64_t o = __ldg(A.pm_orig + d.obs0 + k);
                 A.grad_obs[2 * o] = 0.0;
                 A.grad_obs[2 * o + 1] = 0.0;
             }
-            for (int t = tid; t < m9; t += NT) A.grad_c0[9 * (int64_t)d.cam0 + t] = A.gbar_c[9 * (int64_t)d.cam0 + t];
-            for (int t = tid; t < 3 * d.np; t += NT)
+            for (int t = tid + first; t < m9; t += step) A.grad_c0[9 * (int64_t)d.cam0 + t] = A.gbar_c[9 * (int64_t)d.cam0 + t];
+            for (int t = tid + first; t < 3 * d.np; t += step)
                 A.grad_p0[3 * (int64_t)d.pt0 + t] = A.gbar_p[3 * (int64_t)d.pt0 + t];
         }
         __syncthreads();
         if (S.status != MBA_OK) {
-            for (int k = tid; k < d.n; k += NT) {
+            for (int k = tid + first; k < d.n; k += step) {
                 const int64_t o = __ldg(A.pm_orig + d.obs0 + k);
                 A.grad_obs[2 * o] = 0.0;
                 A.grad_obs[2 * o + 1] = 0.0;
             }
-            for (int t = tid; t < m9; t += NT) A.grad_c0[9 * (int64_t)d.cam0 + t] = 0.0;
-            for (int t = tid; t < 3 * d.np; t += NT) A.grad_p0[3 * (int64_t)d.pt0 + t] = 0.0;
+            for (int t = tid + first; t < m9; t += step) A.grad_c0[9 * (int64_t)d.cam0 + t] = 0.0;
+            for (int t = tid + first; t < 3 * d.np; t += step) A.grad_p0[3 * (int64_t)d.pt0 + t] = 0.0;
         }
     }
-    for (int t = tid; t < m9; t += NT) A.cams[9 * (int64_t)d.cam0 + t] = M.cams[t];
-    if (tid == 0) {
+    for (int t = tid + first; t < m9; t += step) A.cams[9 * (int64_t)d.cam0 + t] = M.cams[t];
+    if (tid == 0 && rk == 0) {
         mba_window_summary o;
         o.iterations = S.iter;
         o.accepted = S.acc_total;
@@ -1662,13 +1854,41 @@ __device__ __forceinline__ void solve_window(const BatchArgs &A, const BatchOpts
         o.pad = 0;
         A.out[wi] = o;
     }
-    __syncthreads();
+    win_sync<CL>();
 }
 
 __device__ __forceinline__ unsigned long long global_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
+}
+
+// One cluster per window (clusters and CTAs of a cluster: see the top).
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT, 1) batch_cluster_kernel(BatchArgs A) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ WinState S;
+    WinMem<T> M;
+    const size_t off = win_carve<T>(smem_raw, A.ncmax, NT / 32, 0, M);
+    uint32_t rank, size;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
+    cluster_carve<T>(smem_raw, off, A.ncmax, A.srows, M);
+    M.rank = (int)rank;
+    M.csz = (int)size;
+    M.slot_id = (int)(blockIdx.x / size);
+    const BatchOpts O = *A.opts;
+    for (;;) {
+        if (threadIdx.x == 0 && rank == 0) S.win = atomicAdd(A.counter, 1);
+        cluster_barrier();
+        const int k = ld_peer(&S.win, 0);
+        cluster_barrier();
+        if (k >= A.nw) break;  // no rank touches another's memory after the barrier above
+        const int wi = __ldg(A.order + k);
+        const unsigned long long t0 = global_ns();
+        solve_window<T, NT, true>(A, O, M, S, wi);  // ends with a cluster barrier
+        if (threadIdx.x == 0 && rank == 0) A.win_ns[wi] = global_ns() - t0;
+    }
 }
 
 template <typename T, int NT, int MINB>
@@ -1686,7 +1906,7 @@ __global__ void __launch_bounds__(NT, MINB) batch_kernel(BatchArgs A) {
         if (k >= A.nw) break;
         const int wi = __ldg(A.order + k);
         const unsigned long long t0 = global_ns();
-        solve_window<T, NT>(A, O, M, S, wi);  // ends with a block barrier
+        solve_window<T, NT, false>(A, O, M, S, wi);  // ends with a block barrier
         if (threadIdx.x == 0) A.win_ns[wi] = global_ns() - t0;
     }
 }
@@ -1868,6 +2088,17 @@ const void *kernel_ptr(bool fp32, int nt, int cps) {
     return cps >= 3 ? (const void *)batch_kernel<double, 256, 3> : (const void *)batch_kernel<double, 256, 2>;
 }
 
+// Cluster instances: 256 threads, one CTA per SM.
+const void *cluster_kernel_ptr(bool fp32) {
+    return fp32 ? (const void *)batch_cluster_kernel<float, 256> : (const void *)batch_cluster_kernel<double, 256>;
+}
+size_t cluster_smem(bool fp32, int ncmax, int rows) {
+    WinMem<float> mf;
+    WinMem<double> md;
+    return fp32 ? cluster_carve<float>(nullptr, win_carve<float>(nullptr, ncmax, 8, 0, mf), ncmax, rows, mf)
+                : cluster_carve<double>(nullptr, win_carve<double>(nullptr, ncmax, 8, 0, md), ncmax, rows, md);
+}
+
 // Dynamic shared memory of a launch; svals > 0 also holds S~ (svals values of T).
 size_t kernel_smem(bool fp32, int nt, int ncmax, int64_t svals) {
     if (fp32) return nt == 256 ? smem_bytes<float, 256>(ncmax, svals) : smem_bytes<float, 512>(ncmax, svals);
@@ -1902,6 +2133,8 @@ struct mba_batch {
     int schur = 0;                  // schedule: 1 implicit, 2 explicit Schur product
     int sms = 0;
     int nt = 0, cps = 0;            // schedule in use
+    bool automatic = true;          // threads and CTAs per SM were left to the library
+    int g_cl = 0;                   // cluster size the graph was captured with (1: none)
     cudaGraphExec_t gexec = nullptr;
     int g_nt = 0, g_grid = 0, g_cps = 0;  // schedule the graph was captured with
     bool g_ssm = false;
@@ -1959,25 +2192,94 @@ bool s_in_smem(const mba_batch *b) {
     return b->schur == 2 && b->explicit_ok && max_ctas_per_sm(b, b->nt, b->cps, true) >= b->cps;
 }
 
-mba_status build_graph(mba_batch *b) {
+// Cluster size of the automatic schedule: the largest of 16, 8, 4 for which
+// every window has its cluster at once, one CTA per SM; two CTAs per window up to
+// one window per SM (clusters then claim the windows longest-first, so the
+// longest window no longer sets the time alone); 1 (no clusters) with more
+// windows than that, for the implicit product and for the single-reduction PCG.  Eight FP64 windows of 5 to 30 cameras with the adjoint: 7.2 ms with 16 CTAs
+// each, 41.3 ms with one.
+int cluster_size(const mba_batch *b, const BatchOpts &o, int *rows, size_t *smem, int *clusters_out) {
+    *rows = 0;
+    *clusters_out = 0;
+    *smem = 0;
+    if (!b->automatic || !b->explicit_ok || !o.explicit_schur || o.pcg_variant != MBA_PCG_STANDARD) return 1;
+    const void *k = cluster_kernel_ptr(b->fp32);
+    int optin = 0, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    const size_t limit = (size_t)optin - 2048;  // static shared memory
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    for (int c = kMaxCluster; c >= 2; c /= 2) {
+        if (c > 2 ? (int64_t)b->nw * c > b->sms : b->nw > b->sms) continue;
+        int r = (9 * b->ncmax + c - 1) / c;
+        if (cluster_smem(b->fp32, b->ncmax, r) > limit) r = 0;
+        const size_t sm = cluster_smem(b->fp32, b->ncmax, r);
+        if (sm > limit) return 1;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) break;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = c;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)(b->nw * c));
+        cfg.blockDim = dim3(256);
+        cfg.dynamicSmemBytes = sm;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, k, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        if (c > 2 ? clusters < b->nw : clusters < 1) continue;
+        *clusters_out = clusters < b->nw ? clusters : b->nw;
+        *rows = r;
+        *smem = sm;
+        return c;
+    }
+    cudaGetLastError();
+    return 1;
+}
+
+mba_status build_graph(mba_batch *b, const BatchOpts &o) {
+    int srows = 0;
+    size_t csm = 0;
+    int nclus = 0;
+    const int cl = cluster_size(b, o, &srows, &csm, &nclus);
     const int grid_full = b->sms * b->cps;
     const int grid = grid_full < b->nw ? grid_full : b->nw;
     const bool ssm = s_in_smem(b);
-    if (b->gexec && b->g_nt == b->nt && b->g_grid == grid && b->g_cps == b->cps && b->g_ssm == ssm) return MBA_OK;
+    if (b->gexec && b->g_nt == b->nt && b->g_grid == grid && b->g_cps == b->cps && b->g_ssm == ssm && b->g_cl == cl)
+        return MBA_OK;
     if (b->gexec) {
         cudaGraphExecDestroy(b->gexec);
         b->gexec = nullptr;
     }
-    const void *k = kernel_ptr(b->fp32, b->nt, b->cps);
-    const size_t sm = kernel_smem(b->fp32, b->nt, b->ncmax, ssm ? b->A.smax : 0);
+    const void *k = cl > 1 ? cluster_kernel_ptr(b->fp32) : kernel_ptr(b->fp32, b->nt, b->cps);
+    const size_t sm = cl > 1 ? csm : kernel_smem(b->fp32, b->nt, b->ncmax, ssm ? b->A.smax : 0);
     BCK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     cudaGraph_t g = nullptr;
     BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e1 = cudaMemsetAsync(b->counter, 0, sizeof(int32_t), b->stream);
     BatchArgs args = b->A;
-    args.s_smem = ssm ? 1 : 0;
+    args.s_smem = cl == 1 && ssm ? 1 : 0;
+    args.srows = srows;
     void *kargs[] = {(void *)&args};
-    cudaError_t e2 = cudaLaunchKernel(k, dim3(grid), dim3(b->nt), kargs, sm, b->stream);
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = cl > 1 ? dim3((unsigned)(nclus * cl)) : dim3(grid);
+    cfg.blockDim = cl > 1 ? dim3(256) : dim3(b->nt);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = b->stream;
+    cfg.attrs = at;
+    cfg.numAttrs = cl > 1 ? 1 : 0;
+    cudaError_t e2 = cudaLaunchKernelExC(&cfg, k, kargs);
     cudaError_t e3 = cudaStreamEndCapture(b->stream, &g);
     if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -1994,6 +2296,7 @@ mba_status build_graph(mba_batch *b) {
     b->g_grid = grid;
     b->g_cps = b->cps;
     b->g_ssm = ssm;
+    b->g_cl = cl;
     return MBA_OK;
 }
 
@@ -2360,6 +2663,7 @@ mba_status mba_batch_set_schedule(mba_batch *b, const mba_batch_schedule *sc) {
     b->nt = nt;
     b->cps = cps;
     b->schur = schur;
+    b->automatic = sc->threads_per_cta == 0 && sc->ctas_per_sm == 0;
     return MBA_OK;
 }
 
@@ -2411,7 +2715,7 @@ mba_status mba_batch_solve(mba_batch *b, const mba_solver_options *opt, const mb
         BCK(cudaMemcpyAsync(b->gbar_c, adj->grad_cameras, 72 * (size_t)b->nc, cudaMemcpyHostToDevice, s));
         BCK(cudaMemcpyAsync(b->gbar_p, adj->grad_points, 24 * (size_t)b->np, cudaMemcpyHostToDevice, s));
     }
-    mba_status st = build_graph(b);
+    mba_status st = build_graph(b, bo);
     if (st != MBA_OK) return st;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ms) {
@@ -2476,6 +2780,51 @@ mba_status mba_batch_autotune(mba_batch *b, const mba_solver_options *opt, mba_b
         if (st != MBA_OK && st != MBA_ERR_NONFINITE) return st;
     }
     const int nts[2] = {256, 512};
+    const bool auto0 = b->automatic;
+    bool bauto = false;
+    // one timed solve; false on an error (in *err)
+    auto timed = [&](mba_status *err, double *t) -> bool {
+        mba_status st = mba_batch_solve(b, opt, nullptr, nullptr, t);
+        if (st != MBA_OK && st != MBA_ERR_NONFINITE) {
+            *err = st;
+            return false;
+        }
+        if (cudaMemcpyAsync(b->A.cams, b->cams_bak, 72 * (size_t)b->nc, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+            cudaMemcpyAsync(b->A.pts, b->pts_bak, 24 * (size_t)b->np, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess) {
+            *err = api_fail(MBA_ERR_CUDA, "autotune: restoring the parameters");
+            return false;
+        }
+        return true;
+    };
+    auto restore = [&]() {
+        b->nt = nt0;
+        b->cps = cps0;
+        b->schur = sc0;
+        b->automatic = auto0;
+    };
+    mba_status err = MBA_OK;
+    // the automatic schedule where it gives each window a cluster, then every
+    // combination of threads, CTAs per SM and Schur form
+    if (b->explicit_ok) {
+        b->nt = 256;
+        b->cps = 1;
+        b->schur = 2;
+        b->automatic = true;
+        double t = 0.0;
+        if (!timed(&err, &t)) {
+            restore();
+            return err;
+        }
+        if (b->g_cl > 1) {
+            best = t;
+            bnt = 256;
+            bcps = 1;
+            bsc = 2;
+            bauto = true;
+        }
+    }
+    b->automatic = false;
     for (int sch = b->explicit_ok ? 2 : 1; sch >= 1; --sch)
     for (int a = 0; a < 2; ++a) {
         for (int c = 1; c <= kMaxCtasPerSm; ++c) {
@@ -2484,27 +2833,23 @@ mba_status mba_batch_autotune(mba_batch *b, const mba_solver_options *opt, mba_b
             b->cps = c;
             b->schur = sch;
             double t = 0.0;
-            mba_status st = mba_batch_solve(b, opt, nullptr, nullptr, &t);
-            BCK(cudaMemcpyAsync(b->A.cams, b->cams_bak, 72 * (size_t)b->nc, cudaMemcpyDeviceToDevice, s));
-            BCK(cudaMemcpyAsync(b->A.pts, b->pts_bak, 24 * (size_t)b->np, cudaMemcpyDeviceToDevice, s));
-            BCK(cudaStreamSynchronize(s));
-            if (st != MBA_OK && st != MBA_ERR_NONFINITE) {
-                b->nt = nt0;
-                b->cps = cps0;
-                b->schur = sc0;
-                return st;
+            if (!timed(&err, &t)) {
+                restore();
+                return err;
             }
             if (best < 0.0 || t < best) {
                 best = t;
                 bnt = nts[a];
                 bcps = c;
                 bsc = sch;
+                bauto = false;
             }
         }
     }
     b->nt = bnt;
     b->cps = bcps;
     b->schur = bsc;
+    b->automatic = bauto;
     if (chosen) {
         chosen->threads_per_cta = bnt;
         chosen->ctas_per_sm = bcps;

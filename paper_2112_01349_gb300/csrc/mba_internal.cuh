@@ -417,6 +417,68 @@ template <typename T> __device__ __forceinline__ void stcg(T *p, T v) { __stcg(p
 // to cover the latency of HBM.
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
+// Warp-collective inverse of a symmetric positive definite 9x9 matrix in FP64.
+// A (shared memory, 81 doubles, both triangles set) is overwritten by its
+// lower Cholesky factor (right-looking: lane-parallel column scaling and
+// trailing update), Y (shared, 81) receives L^-1 by forward substitution, one
+// column per lane, and inv (global, row-major) = L^-T L^-1.  Returns false on
+// every lane, writing nothing, if a pivot is not positive.  The chains are
+// short (about 9 steps per column) where one thread per matrix would run
+// hundreds of dependent FP64 operations.
+__device__ inline bool warp_spd_inverse9(double *A, double *Y, double *il, double *inv) {
+    const int lane = threadIdx.x & 31;
+    // this lane's lower-triangle entries (r >= c) of the trailing updates
+    int e_r[2], e_c[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int e = lane + 32 * h;
+        int r = 0;
+        while (r < 9 && (r + 1) * (r + 2) / 2 <= e) ++r;
+        e_r[h] = r;
+        e_c[h] = e - r * (r + 1) / 2;
+    }
+    for (int j = 0; j < 9; ++j) {
+        __syncwarp();
+        const double d = A[j * 9 + j];
+        if (!(d > 0.0) || !isfinite(d)) return false;
+        const double l = sqrt(d), ilj = 1.0 / l;
+        __syncwarp();
+        if (lane == 0) {
+            A[j * 9 + j] = l;
+            il[j] = ilj;
+        }
+        if (lane > j && lane < 9) A[lane * 9 + j] *= ilj;
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = e_r[h], c = e_c[h];
+            if (lane + 32 * h < 45 && c > j) A[r * 9 + c] -= A[r * 9 + j] * A[c * 9 + j];
+        }
+    }
+    __syncwarp();
+    if (lane < 9) {  // column `lane` of L^-1 (rows >= lane)
+        const int c = lane;
+        for (int r = 0; r < 9; ++r) {
+            if (r < c) {
+                Y[r * 9 + c] = 0.0;
+                continue;
+            }
+            double s = r == c ? 1.0 : 0.0;
+            for (int k = c; k < r; ++k) s -= A[r * 9 + k] * Y[k * 9 + c];
+            Y[r * 9 + c] = s * il[r];
+        }
+    }
+    __syncwarp();
+    if (!inv) return true;  // the caller forms what it needs of L^-T L^-1 from Y
+    for (int e = lane; e < 81; e += 32) {
+        const int r = e / 9, c = e - 9 * (e / 9), k0 = r > c ? r : c;
+        double s = 0.0;
+        for (int k = k0; k < 9; ++k) s += Y[k * 9 + r] * Y[k * 9 + c];
+        inv[e] = s;
+    }
+    return true;
+}
+
 // Block-wide sum of one double per thread in a fixed tree order (shuffles in
 // each warp, then across the warp sums in warp 0); result valid in thread 0.
 // sbuf holds one double per warp (up to 32).
