@@ -257,6 +257,7 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
         P.sp_pt = P.sorted ? c.take<int32_t>((size_t)np) : nullptr;
         P.sl_cam = P.sorted ? c.take<int32_t>(slots) : nullptr;
         P.cm_sp = P.sorted ? c.take<int32_t>((size_t)n) : nullptr;
+        P.sl_uv = P.sorted ? c.take<double2>(slots) : nullptr;
         P.sl_uv32 = fact ? c.take<float2>(slots) : nullptr;
         P.sl_px = fact ? c.take<float4>(slots) : nullptr;
         P.sl_w = fact && lossy ? c.take<float>(slots) : nullptr;
@@ -264,7 +265,6 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
         P.camstat = fact ? c.take<float>((size_t)kCamStat * nc) : nullptr;
         P.ctr = fact ? c.take<float>((size_t)kCtr * nc) : nullptr;
         const bool own64 = P.own && !P.fp32;
-        P.sl_uv = own64 ? c.take<double2>(slots) : nullptr;
         P.sl_hg = own64 ? c.take<double2>(5 * slots) : nullptr;
         P.sl_w64 = own64 && lossy ? c.take<double>(slots) : nullptr;
         P.sp_X64 = own64 ? c.take<double>(4 * (size_t)np) : nullptr;

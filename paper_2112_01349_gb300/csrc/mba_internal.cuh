@@ -138,7 +138,7 @@ struct Prob {
     double2 *r_hg;          // FP64: [5][rslot_cap] pairs of H00 H01 H02 H11 H12 H22 g0 g1 g2 r2
     double2 *sl_hg;         // FP64: [5][slot_cap] the same in slice order
     double *sl_w64;         // FP64: [slot_cap] IRLS weight (null without a loss)
-    double2 *sl_uv;         // FP64: [slot_cap] pixels
+    double2 *sl_uv;         // [slots] pixels in FP64 (the cost; the FP64 linearisation)
     double *sp_X64, *sp_b64;  // FP64: [np][4] sorted point order
     double *ctr64;          // FP64: [nc][kCtr] row transform
     void *c_part;           // [n_vblk][nc][kPartF / kPartD] T

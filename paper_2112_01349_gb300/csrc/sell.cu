@@ -61,8 +61,8 @@ __global__ void fill_slots_kernel(Prob P, const int32_t *__restrict__ pt_sp, con
             c.y + (int64_t)sl * 32 * c.w + 32 * (k >> c.z) + ((q - sl * per) << c.z) + (k & ((1 << c.z) - 1));
         P.sl_cam[slot] = P.pm_cam[o];
         const double2 uv = P.pm_uv[o];
+        P.sl_uv[slot] = uv;
         if (P.sl_uv32) P.sl_uv32[slot] = make_float2((float)uv.x, (float)uv.y);
-        else P.sl_uv[slot] = uv;
     }
 }
 
