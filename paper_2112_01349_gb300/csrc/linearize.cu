@@ -33,21 +33,13 @@ inline unsigned grid_for(int64_t n, int per = kBlock) {
 // (1, 0, 0; k1, f, 0; k2, 0, f)^T for f, k1, k2 (the Jacobian of f d(r^2) is
 // d, f r^2, f r^4 = the row (1, k1, k2) / (0, f, 0) / (0, 0, f) applied to
 // (1, r^2, r^4)).
-__device__ __forceinline__ void factored_camera(const double *row, float *stat, float *ctr) {
-    const double w0 = row[25], w1 = row[26], w2 = row[27];
-    const double th = sqrt(w0 * w0 + w1 * w1 + w2 * w2), root2 = 1.4142135623730951;
-    double sh = 0.0, ch = 1.0, k = 0.5;
-    if (row[24] == 0.0) {
-        sincos(0.5 * th, &sh, &ch);
-        k = sh / th;
-    }
+__device__ __forceinline__ void factored_camera(const double *row, const double *quat, float *stat, float *ctr) {
+    const double root2 = 1.4142135623730951;
     stat[0] = (float)row[21];
     stat[1] = (float)row[22];
     stat[2] = (float)row[23];
-    stat[3] = (float)(root2 * ch);
-    stat[4] = (float)(root2 * k * w0);
-    stat[5] = (float)(root2 * k * w1);
-    stat[6] = (float)(root2 * k * w2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) stat[3 + q] = (float)(root2 * quat[q]);
     stat[7] = (float)row[18];
     stat[8] = (float)row[19];
     stat[9] = (float)row[20];
@@ -87,7 +79,8 @@ __global__ void camera_table_kernel(const double *__restrict__ cams, int32_t nc,
     if (gate == 2 && st->done) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
         double row[kCamTab];
-        camera_table_row(cams + 9 * (int64_t)i, row);
+        double quat[4];
+        camera_table_row(cams + 9 * (int64_t)i, row, quat);
         if (tab)
 #pragma unroll
             for (int q = 0; q < kCamTab; ++q) tab[(int64_t)i * kCamTab + q] = (T)row[q];
@@ -95,7 +88,7 @@ __global__ void camera_table_kernel(const double *__restrict__ cams, int32_t nc,
 #pragma unroll
             for (int q = 0; q < kCamTab; ++q) tab64[(int64_t)i * kCamTab + q] = row[q];
         if (ctr64) own_camera(row, ctr64 + (int64_t)i * kCtr);
-        if (ctr) factored_camera(row, stat + (int64_t)i * kCamStat, ctr + (int64_t)i * kCtr);
+        if (ctr) factored_camera(row, quat, stat + (int64_t)i * kCamStat, ctr + (int64_t)i * kCtr);
         if (tabff) {  // R, t, f, k1, k2 as float-float
 #pragma unroll
             for (int q = 0; q < 9; ++q) {
@@ -493,7 +486,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) lin_camera_ker
             pa = pb;
             pb = pc;
             T e[2], Jc[18], Jp[6], pz[3];
-            edge_eval<T, AD, true, false>(ctab, X0, X1, X2, u0, u1, e, Jc, Jp, AD ? nullptr : pz);
+            edge_eval<T, AD, true, false>(ctab, X0, X1, X2, u0, u1, e, Jc, Jp, FACT ? pz : nullptr);
             zero_fixed_columns<T>(P, cam, pt, Jc, (T *)nullptr);
             T rho, W;
             loss_weight<T>(P.loss, delta, e[0] * e[0] + e[1] * e[1], &rho, &W);
@@ -515,14 +508,6 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) lin_camera_ker
                 const int64_t o = P.own ? (int64_t)P.cm2r[s] : (int64_t)s;
                 (P.own ? P.r_rx : P.RXcm)[o] = rx;
                 if (P.loss != MBA_LOSS_NONE) (P.own ? P.r_w : P.cm_w)[o] = W;
-            }
-            if constexpr (sizeof(T) == 8 && !AD) {
-                if (P.own) {
-                    T h[6];
-#pragma unroll
-                    for (int r = 0; r < 6; ++r) h[r] = W * Jp[r];
-                    store_hg(P.r_hg + P.cm2r[s], P.rslot_cap, h, Jp, pz);
-                }
             }
             int idx = 0;
 #pragma unroll
@@ -547,6 +532,216 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) lin_camera_ker
         P.cpart[54 * (int64_t)c + lane] = mine0;
         if (lane < 22) P.cpart[54 * (int64_t)c + 32 + lane] = mine1;
     }
+}
+
+// ---------------------------------------------------------------------------
+// Camera blocks of the block-owned FP64 form.  In the basis of the product's raw
+// sums a residual row is (X x jp, jp, p (1, r2, r2^2)), jp a row of Jp, and
+// Jc = ctr applied to it, so B = ctr (sum W raw^T raw) ctr^T per camera.  The sum
+// has 44 distinct entries: H = W Jp^T Jp (6), X x H (9), X x H x X (6), g and
+// X x g with g = W Jp^T p (9 each, times 1, r2, r2^2), W r2 (1 .. r2^4) (5); with v's
+// nine, 53 sums of about 130 FP64 instructions where J^T W J from the nine
+// columns takes 170 beside forming them.  The 53 lane sums of a chunk are reduced
+// by exchanging halves, 62 additions instead of 5 x 54.
+// Both matter because the FP64 pipe bounds the kernel: 5.0M observations
+// 3.34 -> 1.86 ms.
+// ---------------------------------------------------------------------------
+constexpr int kRawSums = 53;
+__device__ __forceinline__ int raw_index(int a, int b) {  // raw components a <= b of 0..8 (rotation, translation, intrinsics)
+    const int ga = a / 3, gb = b / 3, i = a - 3 * ga, k = b - 3 * gb;
+    if (ga == 0) return gb == 0 ? 15 + sym3(i, k) : (gb == 1 ? 6 + 3 * i + k : 30 + 3 * k + i);
+    if (ga == 1) return gb == 1 ? sym3(i, k) : 21 + 3 * k + i;
+    return 39 + i + k;
+}
+
+// A chunk of a camera on the first-order rotation branch (its rotation columns
+// are not of that form): the 54 sums of the final basis.
+__device__ __noinline__ void lin_camera64_small(const Prob &P, int cam, const double *ctab, int b0, int b1, double *out) {
+    const int lane = threadIdx.x & 31;
+    for (int q0 = 0; q0 < 54; q0 += 9) {
+        double acc[9];
+        for (int q = 0; q < 9; ++q) acc[q] = 0.0;
+        for (int s = b0 + lane; s < b1; s += 32) {
+            const int64_t pt = P.cm_pt[s];
+            const double2 uv = P.cm_uv[s];
+            double e[2], Jc[18], Jp[6], rho, W;
+            project<double, true>(ctab, P.pts[3 * pt], P.pts[3 * pt + 1], P.pts[3 * pt + 2], uv.x, uv.y, e, Jc, Jp);
+            loss_weight<double>(P.loss, P.delta, e[0] * e[0] + e[1] * e[1], &rho, &W);
+            int idx = 0;
+            for (int a = 0; a < 9; ++a)
+                for (int b = a; b < 9; ++b, ++idx)
+                    if (idx >= q0 && idx < q0 + 9) acc[idx - q0] += W * (Jc[a] * Jc[b] + Jc[9 + a] * Jc[9 + b]);
+            for (int a = 0; a < 9; ++a)
+                if (q0 == 45) acc[a] -= W * (Jc[a] * e[0] + Jc[9 + a] * e[1]);
+        }
+        for (int q = 0; q < 9; ++q) {
+            double v = acc[q];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) out[q0 + q] = v;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kBlock, 1) lin_camera64_kernel(Prob P, int force) {
+    if (!force && (P.st->done || !P.st->relin)) return;
+    __shared__ double ctabs[kWarps][kCamTab];
+    const double *__restrict__ camtab = (const double *)P.camtab;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double *ctab = ctabs[wid];
+    for (int c = blockIdx.x * kWarps + wid; c < P.n_cchunks; c += gridDim.x * kWarps) {
+        const int cam = P.cchunk_cam[c];
+        const int b0 = P.cchunk_beg[c], b1 = P.cchunk_beg[c + 1];
+        __syncwarp();
+        if (lane < kCamTab) ctab[lane] = camtab[(int64_t)cam * kCamTab + lane];
+        __syncwarp();
+        const bool small = __double2hiint(ctab[24]) != 0;
+        double acc[64];
+#pragma unroll
+        for (int q = 0; q < 64; ++q) acc[q] = 0.0;
+        int s = b0 + lane;
+        int pn = s < b1 ? __ldg(P.cm_sp + s) : 0;
+        for (; s < b1; s += 32) {
+            const int64_t pt = pn;
+            if (s + 32 < b1) pn = __ldg(P.cm_sp + s + 32);
+            const double2 xa = __ldg((const double2 *)(P.sp_X64 + 4 * pt)), uv = __ldg(P.cm_uv + s);
+            const double X0 = xa.x, X1 = xa.y, X2 = __ldg(P.sp_X64 + 4 * pt + 2);
+            double e[2], Jc[18], Jp[6], pz[3];
+            project<double, true>(ctab, X0, X1, X2, uv.x, uv.y, e, Jc, Jp, pz);
+            double h[6], W = 1.0;
+            if (P.loss != MBA_LOSS_NONE) {
+                double rho;
+                loss_weight<double>(P.loss, P.delta, e[0] * e[0] + e[1] * e[1], &rho, &W);
+#pragma unroll
+                for (int q = 0; q < 6; ++q) h[q] = W * Jp[q];
+            } else {
+#pragma unroll
+                for (int q = 0; q < 6; ++q) h[q] = Jp[q];
+            }
+            const double r2 = fma(pz[0], pz[0], pz[1] * pz[1]);
+            const double H[6] = {fma(h[0], Jp[0], h[3] * Jp[3]), fma(h[0], Jp[1], h[3] * Jp[4]), fma(h[0], Jp[2], h[3] * Jp[5]),
+                                 fma(h[1], Jp[1], h[4] * Jp[4]), fma(h[1], Jp[2], h[4] * Jp[5]), fma(h[2], Jp[2], h[5] * Jp[5])};
+            const double g[3] = {fma(h[0], pz[0], h[3] * pz[1]), fma(h[1], pz[0], h[4] * pz[1]), fma(h[2], pz[0], h[5] * pz[1])};
+            {
+                double2 *o = P.r_hg + P.cm2r[s];
+                const int64_t st = P.rslot_cap;
+                o[0] = make_double2(H[0], H[1]);
+                o[st] = make_double2(H[2], H[3]);
+                o[2 * st] = make_double2(H[4], H[5]);
+                o[3 * st] = make_double2(g[0], g[1]);
+                o[4 * st] = make_double2(g[2], r2);
+            }
+            if (small) continue;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) acc[q] += H[q];
+            // U = X x H (column k), then U x X
+            double U[3][3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const double h0 = H[k], h1 = H[k == 0 ? 1 : 2 + k], h2 = H[k == 0 ? 2 : 3 + k];
+                U[0][k] = fma(X1, h2, -X2 * h1);
+                U[1][k] = fma(X2, h0, -X0 * h2);
+                U[2][k] = fma(X0, h1, -X1 * h0);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) acc[6 + 3 * i + k] += U[i][k];
+            }
+            acc[15] = fma(X1, U[0][2], fma(-X2, U[0][1], acc[15]));
+            acc[16] = fma(X2, U[0][0], fma(-X0, U[0][2], acc[16]));
+            acc[17] = fma(X0, U[0][1], fma(-X1, U[0][0], acc[17]));
+            acc[18] = fma(X2, U[1][0], fma(-X0, U[1][2], acc[18]));
+            acc[19] = fma(X0, U[1][1], fma(-X1, U[1][0], acc[19]));
+            acc[20] = fma(X0, U[2][1], fma(-X1, U[2][0], acc[20]));
+            const double xg[3] = {fma(X1, g[2], -X2 * g[1]), fma(X2, g[0], -X0 * g[2]), fma(X0, g[1], -X1 * g[0])};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const double a1 = r2 * g[k], c1 = r2 * xg[k];
+                acc[21 + k] += g[k];
+                acc[24 + k] += a1;
+                acc[27 + k] = fma(r2, a1, acc[27 + k]);
+                acc[30 + k] += xg[k];
+                acc[33 + k] += c1;
+                acc[36 + k] = fma(r2, c1, acc[36 + k]);
+            }
+            const double q0 = P.loss != MBA_LOSS_NONE ? W * r2 : r2, q1 = q0 * r2, q2 = q1 * r2, q3 = q2 * r2;
+            acc[39] += q0;
+            acc[40] += q1;
+            acc[41] += q2;
+            acc[42] += q3;
+            acc[43] = fma(q3, r2, acc[43]);
+            const double y0 = fma(h[0], e[0], h[3] * e[1]), y1 = fma(h[1], e[0], h[4] * e[1]),
+                         y2 = fma(h[2], e[0], h[5] * e[1]);
+            acc[44] -= y0;
+            acc[45] -= y1;
+            acc[46] -= y2;
+            acc[47] = fma(-X1, y2, fma(X2, y1, acc[47]));
+            acc[48] = fma(-X2, y0, fma(X0, y2, acc[48]));
+            acc[49] = fma(-X0, y1, fma(X1, y0, acc[49]));
+            double t = fma(pz[0], e[0], pz[1] * e[1]);
+            if (P.loss != MBA_LOSS_NONE) t *= W;
+            const double t1 = r2 * t;
+            acc[50] -= t;
+            acc[51] -= t1;
+            acc[52] = fma(-r2, t1, acc[52]);
+        }
+        __syncwarp();
+        double *out = P.cpart + 54 * (int64_t)c;
+        if (small) {
+            lin_camera64_small(P, cam, ctab, b0, b1, out);
+            continue;
+        }
+#pragma unroll
+        for (int w = 32; w >= 2; w >>= 1) {
+            const bool up = lane & (w >> 1);
+#pragma unroll
+            for (int q = 0; q < w; ++q) {
+                const double send = up ? acc[q] : acc[q + w], keep = up ? acc[q + w] : acc[q];
+                acc[q] = keep + __shfl_xor_sync(full, send, w >> 1);
+            }
+        }
+        const int idx = 2 * lane;  // bit 4 chose 32, ..., bit 0 chose 2
+        if (idx < kRawSums) out[idx] = acc[0];
+        if (idx + 1 < kRawSums) out[idx + 1] = acc[1];
+    }
+}
+
+// One camera per 64 threads: the chunk sums in order, then B = ctr raw ctr^T and
+// v = ctr raw (or the sums themselves for first-order cameras).
+__global__ void __launch_bounds__(64) cam_finalize64_kernel(Prob P, const int32_t *__restrict__ cfirst, int force) {
+    if (!force && (P.st->done || !P.st->relin)) return;
+    __shared__ double raw[54], ct[27];
+    const int i = blockIdx.x, t = threadIdx.x;
+    const bool small = ((const double *)P.camtab)[(int64_t)i * kCamTab + 24] != 0.0;
+    const bool fixed = P.has_fixed && P.cam_fixed[i];  // its Jacobian columns are zero
+    if (t < 54) {
+        double s = 0.0;
+        if (t < kRawSums || small)
+            for (int c = cfirst[i]; c < cfirst[i + 1]; ++c) s += P.cpart[54 * (int64_t)c + t];
+        raw[t] = fixed ? 0.0 : s;
+    }
+    if (t < 27) ct[t] = P.ctr64[(int64_t)i * kCtr + t];
+    __syncthreads();
+    if (t >= 54) return;
+    double r = 0.0;
+    if (small) {
+        r = raw[t];
+    } else if (t < 45) {
+        int a = 0, f = t;
+        while (f >= 9 - a) f -= 9 - a, ++a;
+        const int b = a + f, ga = a / 3 * 3, gb = b / 3 * 3;
+        for (int k = 0; k < 3; ++k) {
+            double m = 0.0;
+            for (int l = 0; l < 3; ++l) {
+                const int p = ga + k, q = gb + l;
+                m = fma(raw[p <= q ? raw_index(p, q) : raw_index(q, p)], ct[3 * b + l], m);
+            }
+            r = fma(ct[3 * a + k], m, r);
+        }
+    } else {
+        const int a = t - 45, g = a / 3, at = g == 0 ? 47 : (g == 1 ? 44 : 50);
+        for (int k = 0; k < 3; ++k) r = fma(ct[3 * a + k], raw[at + k], r);
+    }
+    if (t < 45) P.Hpp[45 * (int64_t)i + t] = r;
+    else P.v[9 * (int64_t)i + (t - 45)] = r;
 }
 
 __global__ void cam_finalize_kernel(Prob P, const int32_t *__restrict__ cfirst, int force) {
@@ -763,6 +958,10 @@ static void launch_lin_pair(const Prob &P, int force, cudaStream_t s) {
     }
     int nbc = (P.n_cchunks + kWarps - 1) / kWarps;
     if (nbc > 152 * 16) nbc = 152 * 16;
+    if (sizeof(T) == 8 && !AD && P.own) {
+        lin_camera64_kernel<<<nbc < 1 ? 1 : nbc, kBlock, 0, s>>>(P, force);
+        return;
+    }
     lin_camera_kernel<T, AD><<<nbc < 1 ? 1 : nbc, kBlock, 0, s>>>(P, force);
 }
 
@@ -778,7 +977,8 @@ cudaError_t launch_linearize_impl(const Prob &P, const int32_t *cfirst, int forc
         if (P.autodiff) launch_lin_pair<double, true>(P, force, s);
         else launch_lin_pair<double, false>(P, force, s);
     }
-    cam_finalize_kernel<<<grid_for((int64_t)P.nc * 54), kBlock, 0, s>>>(P, cfirst, force);
+    if (!P.fp32 && P.own) cam_finalize64_kernel<<<P.nc, 64, 0, s>>>(P, cfirst, force);
+    else cam_finalize_kernel<<<grid_for((int64_t)P.nc * 54), kBlock, 0, s>>>(P, cfirst, force);
     return cudaGetLastError();
 }
 

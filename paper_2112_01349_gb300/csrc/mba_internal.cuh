@@ -207,21 +207,32 @@ __host__ __device__ __forceinline__ int sym3(int a, int b) {
 // Table row: R[9] M[9] t[3] f k1 k2 small w[3] (w: the raw angle-axis, read by
 // the dual-number path, which evaluates the edge functor from the parameters).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void camera_table_row(const double *c, double *o) {
+// quat (optional): the unit quaternion of the rotation.
+__device__ __forceinline__ void camera_table_row(const double *c, double *o, double *quat = nullptr) {
     const double w0 = c[0], w1 = c[1], w2 = c[2];
     const double th2 = w0 * w0 + w1 * w1 + w2 * w2;
     double R[9], M[9];
     double small;
     if (th2 > DBL_EPSILON) {
         const double th = sqrt(th2);
-        double s, co;
-        sincos(th, &s, &co);
-        const double k0 = w0 / th, k1 = w1 / th, k2 = w2 / th;
-        const double oc = 1.0 - co;
+        // one sine and cosine, of the half angle: sin = 2 sh ch, 1 - cos = 2 sh^2
+        // (the quaternion of the factored form is (ch, sh k))
+        double sh, ch;
+        sincos(0.5 * th, &sh, &ch);
+        const double ith = 1.0 / th;
+        const double k0 = w0 * ith, k1 = w1 * ith, k2 = w2 * ith;
+        const double s = 2.0 * sh * ch, oc = 2.0 * sh * sh, co = 1.0 - oc;
+        if (quat) {
+            quat[0] = ch;
+            quat[1] = sh * k0;
+            quat[2] = sh * k1;
+            quat[3] = sh * k2;
+        }
         R[0] = co + oc * k0 * k0;      R[1] = -s * k2 + oc * k0 * k1; R[2] = s * k1 + oc * k0 * k2;
         R[3] = s * k2 + oc * k1 * k0;  R[4] = co + oc * k1 * k1;      R[5] = -s * k0 + oc * k1 * k2;
         R[6] = -s * k1 + oc * k2 * k0; R[7] = s * k0 + oc * k2 * k1;  R[8] = co + oc * k2 * k2;
         // (R^T - I) [w]_x, then add w w^T and divide by th^2
+        const double ith2 = ith * ith;
         const double A[9] = {R[0] - 1.0, R[3], R[6], R[1], R[4] - 1.0, R[7], R[2], R[5], R[8] - 1.0};
         const double W[9] = {0.0, -w2, w1, w2, 0.0, -w0, -w1, w0, 0.0};
         const double wv[3] = {w0, w1, w2};
@@ -230,7 +241,7 @@ __device__ __forceinline__ void camera_table_row(const double *c, double *o) {
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 double acc = A[i * 3 + 0] * W[0 * 3 + j] + A[i * 3 + 1] * W[1 * 3 + j] + A[i * 3 + 2] * W[2 * 3 + j];
-                M[i * 3 + j] = (acc + wv[i] * wv[j]) / th2;
+                M[i * 3 + j] = (acc + wv[i] * wv[j]) * ith2;
             }
         small = 0.0;
     } else {
@@ -240,6 +251,12 @@ __device__ __forceinline__ void camera_table_row(const double *c, double *o) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) M[i] = (i % 4 == 0) ? 1.0 : 0.0;
         small = 1.0;
+        if (quat) {
+            quat[0] = 1.0;
+            quat[1] = 0.5 * w0;
+            quat[2] = 0.5 * w1;
+            quat[3] = 0.5 * w2;
+        }
     }
 #pragma unroll
     for (int i = 0; i < 9; ++i) { o[i] = R[i]; o[9 + i] = M[i]; }
@@ -520,14 +537,16 @@ __device__ __forceinline__ bool grid_barrier(DevState *st, uint32_t &epoch, long
             unsigned int seen;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(ctr) : "memory");
             if ((int)(seen - target) >= 0) break;
-            int e;
-            asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(e) : "l"(&st->err) : "memory");
-            if (e != 0 || ++polls > limit) {
+            // another CTA's error is looked for now and then: the load would double
+            // the time of a poll
+            int e = 0;
+            if ((++polls & 63) == 0)
+                asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(e) : "l"(&st->err) : "memory");
+            if (e != 0 || polls > limit) {
                 atomicCAS(&st->err, 0, (int)MBA_ERR_TIMEOUT);
                 ok = 0;
                 break;
             }
-            __nanosleep(16);
         }
         s_ok = ok;
     }
