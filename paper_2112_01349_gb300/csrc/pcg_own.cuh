@@ -376,20 +376,35 @@ __device__ __forceinline__ double own_dot_sum(const double *dots, int n) {
     return x;
 }
 
+// The owner's vectors, nine values per camera of the CTA, in shared memory for
+// the whole launch: only z's rows and the partial sums travel.
+struct OwnVec {
+    double *x, *r, *z, *p, *q, *s;
+};
+
 // Owner's part of a product: the cameras [cb, cb + m) of this CTA.  Groups of
 // kGroup blocks' partials are added in T, the groups in FP64, in block order;
 // then one warp per camera, 27 lanes: lane 9 t + a holds component a and a third
-// t of every 9-term row product.  Modes as camera_pass; leaves the dot products
-// in dots (three arrays of 9 m).
+// t of every 9-term row product (the row is loaded before the partials, so that
+// its latency overlaps theirs).  Modes as camera_pass; leaves the dot products in
+// dots (three arrays of 9 m).
 constexpr int kGroup = 16;
 template <typename T, int MODE>
-__device__ void own_finalize(const Prob &P, int cb, int m, double *gsum, double *dots, const double *p_prev,
-                             double *p_cur, double beta, bool first) {
+__device__ void own_finalize(const Prob &P, int cb, int m, const OwnVec &V, double *gsum, double *dots, double beta,
+                             bool first) {
     constexpr int PS = OwnShape<T>::part;
     const T *part = (const T *)P.c_part;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const unsigned full = 0xffffffffu;
     const int ng = (P.n_vblk + kGroup - 1) / kGroup, m9 = 9 * m;
+    const int th = lane < 27 ? lane / 9 : 0, a = lane < 27 ? lane - 9 * th : 0;
+    const double *Mat = MODE == CAM_RHS ? P.Binv : P.Bd;
+    const int64_t mo = a * 9 + 3 * th;
+    double r0 = 0.0, r1 = 0.0, r2 = 0.0;
+    if (wid < m) {
+        const double *M = Mat + 81 * (int64_t)(cb + wid) + mo;
+        r0 = __ldg(M), r1 = __ldg(M + 1), r2 = __ldg(M + 2);
+    }
     for (int t = threadIdx.x; t < m9 * ng; t += blockDim.x) {
         const int g = t / m9, r = t - g * m9, c = r / 9, q = r - 9 * c;
         T v[kGroup];
@@ -405,20 +420,19 @@ __device__ void own_finalize(const Prob &P, int cb, int m, double *gsum, double 
         gsum[t] = (double)v[0];
     }
     __syncthreads();
-    const int th = lane < 27 ? lane / 9 : 0, a = lane < 27 ? lane - 9 * th : 0;
     for (int c = wid; c < m; c += nwarp) {
-        const int cam = cb + c;
-        const int64_t vo = (int64_t)cam * kVec + a;
-        // loads first: this third of the lane's row of B~ (or B~^-1), the vectors
-        const double *M = (MODE == CAM_RHS ? P.Binv : P.Bd) + 81 * (int64_t)cam + a * 9 + 3 * th;
-        const double r0 = __ldg(M), r1 = __ldg(M + 1), r2 = __ldg(M + 2);
-        double pv = 0.0, rv = 0.0;
+        const int cam = cb + c, vo = 9 * c + a;
+        if (c != wid) {
+            const double *M = Mat + 81 * (int64_t)cam + mo;
+            r0 = __ldg(M), r1 = __ldg(M + 1), r2 = __ldg(M + 2);
+        }
+        double pv = 0.0;
         if (MODE == CAM_RHS) pv = P.v[9 * (int64_t)cam + a];
-        else if (MODE == CAM_MATVEC) pv = P.p[vo];
-        else if (MODE == CAM_SR) pv = ldcg(P.z + vo), rv = ldcg(P.r + vo);
-        else pv = first ? ldcg(P.z + vo) : fma(beta, ldcg(p_prev + vo), ldcg(P.z + vo));
+        else if (MODE == CAM_MATVEC) pv = P.p[(int64_t)cam * kVec + a];
+        else if (MODE == CAM_SR) pv = V.z[vo];
+        else pv = first ? V.z[vo] : fma(beta, V.p[vo], V.z[vo]);
         double s = 0.0;
-        for (int g = th; g < ng; g += 3) s += gsum[g * m9 + 9 * c + a];
+        for (int g = th; g < ng; g += 3) s += gsum[g * m9 + vo];
         s = sum_thirds(s, a);
         const int g0 = a < 3 ? 0 : (a < 6 ? 3 : 6);
         double cs = 0.0;
@@ -438,25 +452,29 @@ __device__ void own_finalize(const Prob &P, int cb, int m, double *gsum, double 
         if (MODE == CAM_RHS) {
             const T row = own_row_lane(P, cam, (T)y, 0, a);
             if (lane < 9) {
-                stcg(P.g + vo, x);
-                stcg(P.x + vo, 0.0);
-                stcg(P.r + vo, x);
-                stcg(P.z + vo, y);
-                stcg((T *)P.zT + vo, row);
-                dots[9 * c + a] = x * x;
-                dots[m9 + 9 * c + a] = x * y;
+                stcg(P.g + (int64_t)cam * kVec + a, x);
+                stcg((T *)P.zT + (int64_t)cam * kVec + a, row);
+                V.x[vo] = 0.0;
+                V.r[vo] = x;
+                V.z[vo] = y;
+                dots[vo] = x * x;
+                dots[m9 + vo] = x * y;
             }
         } else {
             const double q = y - cs;
             if (lane < 9) {
-                stcg(P.q + vo, q);
-                if (MODE == CAM_ITER) stcg(p_cur + vo, pv);
-                if (MODE == CAM_SR) {
-                    dots[9 * c + a] = rv * rv;
-                    dots[m9 + 9 * c + a] = rv * pv;
-                    dots[2 * m9 + 9 * c + a] = q * pv;
+                if (MODE == CAM_MATVEC) {
+                    stcg(P.q + (int64_t)cam * kVec + a, q);
+                } else if (MODE == CAM_SR) {
+                    const double rv = V.r[vo];
+                    V.q[vo] = q;
+                    dots[vo] = rv * rv;
+                    dots[m9 + vo] = rv * pv;
+                    dots[2 * m9 + vo] = q * pv;
                 } else {
-                    dots[9 * c + a] = pv * q;
+                    V.q[vo] = q;
+                    V.p[vo] = pv;
+                    dots[vo] = pv * q;
                 }
             }
         }
@@ -465,11 +483,11 @@ __device__ void own_finalize(const Prob &P, int cb, int m, double *gsum, double 
 }
 
 // z = B~^-1 r of one camera by its warp (27 lanes), r in every lane's component.
-__device__ __forceinline__ double own_precond(const double *Mrow, double rv, int th, int a) {
+__device__ __forceinline__ double own_precond(const double *b, double rv, int th, int a) {
     const unsigned full = 0xffffffffu;
-    double z = __ldg(Mrow) * __shfl_sync(full, rv, 3 * th);
-    z = fma(__ldg(Mrow + 1), __shfl_sync(full, rv, 3 * th + 1), z);
-    z = fma(__ldg(Mrow + 2), __shfl_sync(full, rv, 3 * th + 2), z);
+    double z = b[0] * __shfl_sync(full, rv, 3 * th);
+    z = fma(b[1], __shfl_sync(full, rv, 3 * th + 1), z);
+    z = fma(b[2], __shfl_sync(full, rv, 3 * th + 2), z);
     return sum_thirds(z, a);
 }
 
@@ -515,12 +533,20 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
         }
     };
     const int th = lane < 27 ? lane / 9 : 0, a = lane < 27 ? lane - 9 * th : 0;
+    double *vec = dots + 3 * m9;
+    const OwnVec V = {vec, vec + m9, vec + 2 * m9, vec + 3 * m9, vec + 4 * m9, vec + 5 * m9};
+    // this lane's third of its row of B~^-1 for the warp's first camera (or c)
+    auto load_binv = [&](int c, double *b) {
+        const double *B = P.Binv + 81 * (int64_t)(cb + c) + a * 9 + 3 * th;
+        b[0] = __ldg(B), b[1] = __ldg(B + 1), b[2] = __ldg(B + 2);
+    };
+    double binv[3] = {0.0, 0.0, 0.0};
 
     if (mode == PCG_MATVEC) {
         // p given in P.p (FP64): q = B~ p - E C~^-1 E^T p
         own_stage(P, rows, 0.0, true, P.p);
         product(std::false_type{});
-        if (barrier()) own_finalize<T, CAM_MATVEC>(P, cb, m, gsum, dots, nullptr, nullptr, 0.0, true);
+        if (barrier()) own_finalize<T, CAM_MATVEC>(P, cb, m, V, gsum, dots, 0.0, true);
         return;
     }
 
@@ -530,7 +556,7 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
     product(std::true_type{});
     ok = barrier();
     if (ok) {
-        own_finalize<T, CAM_RHS>(P, cb, m, gsum, dots, nullptr, nullptr, 0.0, true);
+        own_finalize<T, CAM_RHS>(P, cb, m, V, gsum, dots, 0.0, true);
         if (mode == PCG_RHS_ONLY) return;
         publish(2, part_rr, part_rho, nullptr);
         ok = barrier();
@@ -545,7 +571,8 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
             own_stage(P, rows, 0.0, true, nullptr);
             product(std::false_type{});
             if (!(ok = barrier())) break;
-            own_finalize<T, CAM_SR>(P, cb, m, gsum, dots, nullptr, nullptr, 0.0, false);
+            if (wid < m) load_binv(wid, binv);
+            own_finalize<T, CAM_SR>(P, cb, m, V, gsum, dots, 0.0, false);
             publish(3, part_rr, part_rho, part_pq);
             if (!(ok = barrier())) break;
             const double2 rz = sum_parts2(part_rr, part_rho, G);
@@ -582,22 +609,23 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
             const double alpha = s_alpha, beta = s_beta;
             const bool last = n + 1 >= max_iter;  // the step cap ends the solve after this update
             for (int c = wid; c < m; c += nwarp) {
-                const int64_t vo = (int64_t)(cb + c) * kVec + a;
-                const double u = ldcg(P.z + vo), w = ldcg(P.q + vo);
-                const double pn = n == 0 ? u : fma(beta, ldcg(P.p + vo), u);
-                const double sn = n == 0 ? w : fma(beta, ldcg(P.p2 + vo), w);
-                const double rv = fma(-alpha, sn, ldcg(P.r + vo)), xv = fma(alpha, pn, ldcg(P.x + vo));
-                const double z = own_precond(P.Binv + 81 * (int64_t)(cb + c) + a * 9 + 3 * th, rv, th, a);
+                const int vo = 9 * c + a;
+                if (c != wid) load_binv(c, binv);
+                const double u = V.z[vo], w = V.q[vo];
+                const double pn = n == 0 ? u : fma(beta, V.p[vo], u);
+                const double sn = n == 0 ? w : fma(beta, V.s[vo], w);
+                const double rv = fma(-alpha, sn, V.r[vo]), xv = fma(alpha, pn, V.x[vo]);
+                const double z = own_precond(binv, rv, th, a);
                 const T row = own_row_lane(P, cb + c, (T)z, 0, a);
                 __syncwarp();
                 if (lane < 9) {
-                    stcg(P.p + vo, pn);
-                    stcg(P.p2 + vo, sn);
-                    stcg(P.x + vo, xv);
-                    stcg(P.r + vo, rv);
-                    stcg(P.z + vo, z);
-                    stcg((T *)P.zT + vo, row);
-                    dots[9 * c + a] = rv * rv;
+                    V.p[vo] = pn;
+                    V.s[vo] = sn;
+                    V.x[vo] = xv;
+                    V.r[vo] = rv;
+                    V.z[vo] = z;
+                    stcg((T *)P.zT + (int64_t)(cb + c) * kVec + a, row);
+                    dots[vo] = rv * rv;
                 }
             }
             ++n;
@@ -624,8 +652,8 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
                 }
                 s_r0 = r0;
                 s_rho = s0.y;
-                s_rn = r0;
-                s_stop = t * r0;
+                s_rn = s0.x;
+                s_stop = (t * r0) * (t * r0);
                 s_go = (r0 > 0.0 && isfinite(s0.y)) ? 1 : 0;
                 s_beta = 0.0;
             }
@@ -634,13 +662,12 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
         if (ok && s_go) {
             for (;;) {
                 const double beta = s_beta;
-                double *p_cur = (n & 1) ? P.p2 : P.p;
-                const double *p_prev = (n & 1) ? P.p : P.p2;
                 own_stage(P, rows, beta, n == 0, nullptr);
                 product(std::false_type{});
                 if (!(ok = barrier())) break;
-                own_finalize<T, CAM_ITER>(P, cb, m, gsum, dots, p_prev, p_cur, beta, n == 0);
+                own_finalize<T, CAM_ITER>(P, cb, m, V, gsum, dots, beta, n == 0);
                 publish(1, part_pq, nullptr, nullptr);
+                if (wid < m) load_binv(wid, binv);
                 if (!(ok = barrier())) break;
                 const double pq = sum_parts(part_pq, G);
                 if (threadIdx.x == 0) {
@@ -653,19 +680,19 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
                 const double alpha = s_alpha;
                 // x += alpha p; r -= alpha q; z = B~^-1 r, one warp per camera
                 for (int c = wid; c < m; c += nwarp) {
-                    const int64_t vo = (int64_t)(cb + c) * kVec + a;
-                    const double xv = fma(alpha, ldcg(p_cur + vo), ldcg(P.x + vo));
-                    const double rv = fma(-alpha, ldcg(P.q + vo), ldcg(P.r + vo));
-                    const double z = own_precond(P.Binv + 81 * (int64_t)(cb + c) + a * 9 + 3 * th, rv, th, a);
+                    const int vo = 9 * c + a;
+                    if (c != wid) load_binv(c, binv);
+                    const double xv = fma(alpha, V.p[vo], V.x[vo]), rv = fma(-alpha, V.q[vo], V.r[vo]);
+                    const double z = own_precond(binv, rv, th, a);
                     const T row = own_row_lane(P, cb + c, (T)z, 0, a);
                     __syncwarp();
                     if (lane < 9) {
-                        stcg(P.x + vo, xv);
-                        stcg(P.r + vo, rv);
-                        stcg(P.z + vo, z);
-                        stcg((T *)P.zT + vo, row);
-                        dots[9 * c + a] = rv * rv;
-                        dots[m9 + 9 * c + a] = rv * z;
+                        V.x[vo] = xv;
+                        V.r[vo] = rv;
+                        V.z[vo] = z;
+                        stcg((T *)P.zT + (int64_t)(cb + c) * kVec + a, row);
+                        dots[vo] = rv * rv;
+                        dots[m9 + vo] = rv * z;
                     }
                 }
                 __syncthreads();
@@ -674,10 +701,11 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
                 ++n;
                 const double2 sums = sum_parts2(part_rho, part_rr, G);
                 if (threadIdx.x == 0) {
-                    const double rho_prev = s_rho, rho = sums.x, rn = sqrt(sums.y);
+                    // |r| <= t |r0| as squares: a root less on every iteration's scalar chain
+                    const double rho_prev = s_rho, rho = sums.x;
                     s_rho = rho;
-                    s_rn = rn;
-                    const bool go = !(rn <= s_stop || n >= max_iter) && isfinite(rho);
+                    s_rn = sums.y;
+                    const bool go = !(sums.y <= s_stop || n >= max_iter) && isfinite(rho);
                     s_go = go ? 1 : 0;
                     s_beta = go ? rho / rho_prev : 0.0;
                 }
@@ -687,9 +715,13 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
         }
     }
     if (!ok) atomicCAS(&st->err, 0, (int)MBA_ERR_TIMEOUT);
+    __syncthreads();
+    if (ok)
+        for (int t = threadIdx.x; t < m9; t += blockDim.x) P.x[(int64_t)(cb + t / 9) * kVec + t % 9] = V.x[t];
     if (ok && blockIdx.x == 0 && threadIdx.x == 0) {
         st->pcg_iters = n;
-        st->pcg_rel_res = s_r0 > 0.0 ? s_rn / s_r0 : 0.0;
+        const double rn = SR ? s_rn : sqrt(s_rn);  // the standard loop keeps the square
+        st->pcg_rel_res = s_r0 > 0.0 ? rn / s_r0 : 0.0;
         if (forcing && !(s_g0 > 0.0)) st->g0 = s_r0;
     }
 }

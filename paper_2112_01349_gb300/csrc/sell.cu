@@ -143,7 +143,7 @@ cudaError_t build_slices(Prob &P, int grid, int max_track, void *tmp, size_t tmp
     if (P.own) {
         const int64_t rows = ((int64_t)P.nc * (P.fp32 ? kRowS * 4 : kRowD * 8) + 127) / 128 * 128;
         const int64_t cams = (P.nc + grid - 1) / grid;  // cameras of an owner, at most
-        const int64_t dots = 27 * cams * 8;
+        const int64_t dots = (3 + 6) * 9 * cams * 8;  // dot products and the owner's six vectors
         std::vector<int32_t> used;
         P.own = 0;
         for (int m = 1; m <= 4 && !P.own; ++m) {
