@@ -80,7 +80,7 @@ __global__ void camera_table_kernel(const double *__restrict__ cams, int32_t nc,
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
         double row[kCamTab];
         double quat[4];
-        camera_table_row(cams + 9 * (int64_t)i, row, quat);
+        camera_table_row<true>(cams + 9 * (int64_t)i, row, quat);
         if (tab)
 #pragma unroll
             for (int q = 0; q < kCamTab; ++q) tab[(int64_t)i * kCamTab + q] = (T)row[q];
