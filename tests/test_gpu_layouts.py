@@ -74,6 +74,21 @@ def test_product_and_step(mba, shape, precision, tol, loss):
     rel_close(so["final_cost"], rl["final_cost"], 1e-6 if precision == "fp64" else 1e-4, "final cost")
 
 
+@pytest.mark.parametrize("jacobian", ["analytic", "autodiff"])
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-6), ("fp32", 2e-3)])
+@pytest.mark.parametrize("per_camera", [31, 32, 33, 255, 256, 257, 513])
+def test_schur_jacobi_chunk_edges(mba, per_camera, precision, tol, jacobian):
+    """The Schur-Jacobi blocks of cameras with observations around a warp and
+    around a chunk of 256.  Tolerances: those of a step of a few PCG iterations."""
+    sc = make_scene(2, per_camera, track=("fixed", 2), sigma=0.5, seed=11)
+    with mba.Problem(*_args(sc), precision=precision, jacobian=jacobian) as pr:
+        st = pr.step(0.1, pcg_max_iter=4, pcg_rel_tol=0.0, preconditioner="schur_jacobi")
+    rs = oracle.step(*_args(sc), 0.1, pcg_max=4, pcg_tol=0.0, precond="schur_jacobi")
+    for a in range(9):
+        rel_close(st["dc"][:, a], rs["dc"].reshape(-1, 9)[:, a], tol, f"dc[{a}]")
+    rel_close(st["dp"], rs["dp"].reshape(-1, 3), tol, "dp")
+
+
 @pytest.mark.parametrize("precision,tol", [("fp64", 1e-9), ("fp32", 1e-4)])
 @pytest.mark.parametrize("shape", ["cams-127", "rows-in-L2"])
 def test_first_order_rotations_and_fixed_nodes(mba, shape, precision, tol):
