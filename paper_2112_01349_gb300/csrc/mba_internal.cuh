@@ -276,6 +276,24 @@ __device__ __forceinline__ void camera_table_row(const double *c, double *o, dou
 __device__ __forceinline__ float rcp_rn(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double rcp_rn(double x) { return __drcp_rn(x); }
 
+// 1 / x: the hardware seed (20 bits) and two Newton-Raphson steps, four FP64
+// instructions where the correctly rounded reciprocal takes about twice that.
+// A seed of zero or infinity (x infinite, zero, subnormal) is the result itself;
+// the test is on its upper word, in integers, off the FP64 pipe.
+__device__ __forceinline__ bool seed_ok(double r) {
+    return (unsigned)((__double2hiint(r) & 0x7fffffff) - 1) < 0x7fefffffu;
+}
+
+__device__ __forceinline__ double fast_rcp(double x) {
+    double r0;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(x));
+    double e = fma(-x, r0, 1.0);
+    double r = fma(r0, e, r0);
+    e = fma(-x, r, 1.0);
+    r = fma(r, e, r);
+    return seed_ok(r0) ? r : r0;
+}
+
 // Residual e = pi(c, X) - u and, if JAC, the analytic Jacobians Jc (2x9, row
 // major: w, t, f, k1, k2) and Jp (2x3) by the chain rule, in precision T.
 // pz (optional): the normalised point p = (px, py) and 1 / P_z.
