@@ -22,7 +22,7 @@ constexpr int kRowS = 20;            // the same in shared memory: 80-byte rows 
                                      // random rows into eight different bank groups (a 64-byte stride has two)
 constexpr int kRowD = 10;            // doubles per camera row of the block-owned FP64 product (m, a', v_f, v_a, v_b, flag)
 constexpr int kPartF = 12, kPartD = 10;  // stride of a camera's nine partial sums (FP32, FP64), for 16-byte stores
-constexpr int kOwnSmem = 218 * 1024; // dynamic shared memory the block-owned PCG kernel may use
+constexpr int kOwnSmem = 225 * 1024; // dynamic shared memory the block-owned PCG kernel may use
 constexpr int kMaxParts = 16;        // parts a camera's run may be split into
 constexpr int kCtr = 28;             // stride of a camera's 9 x 3 row transform (27 values)
 constexpr int kCamStat = 12;         // per camera: f, k1, k2, the quaternion of R times sqrt 2 (w, x, y, z), t (3), pad

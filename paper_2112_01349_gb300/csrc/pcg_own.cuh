@@ -234,15 +234,35 @@ __device__ void own_points(const Prob &P, const T *rows, float *bs, int blk, int
     }
 }
 
+// The layout words of a warp's first run slice: loaded before the barrier that
+// publishes b, so that their latency overlaps it.
+struct RunBegin {
+    int j, j0, j1;
+    int2 rs, ln;
+};
+__device__ __forceinline__ RunBegin own_cameras_begin(const Prob &P, int blk) {
+    RunBegin rb;
+    rb.j0 = __ldg(P.blk_rslice + blk);
+    rb.j1 = __ldg(P.blk_rslice + blk + 1);
+    rb.j = rb.j0 + (threadIdx.x >> 5);
+    rb.rs = rb.ln = make_int2(0, 0);
+    if (rb.j < rb.j1) {
+        rb.rs = __ldg(P.rslice + rb.j);
+        rb.ln = __ldg(P.rlane + 32 * (int64_t)rb.j + (threadIdx.x & 31));
+    }
+    return rb;
+}
+
 // Camera pass of one block: every run's nine raw sums into the block's partials.
-__device__ void own_cameras(const Prob &P, const float *rows, const float *bs, int blk, int *next) {
+__device__ void own_cameras(const Prob &P, const float *rows, const float *bs, int *next, const RunBegin &rb) {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    const int j0 = __ldg(P.blk_rslice + blk), j1 = __ldg(P.blk_rslice + blk + 1), pb = P.own_pb;
+    const int j1 = rb.j1, pb = P.own_pb;
     int jn = 0;
-    for (int j = j0 + (threadIdx.x >> 5); j < j1; j = jn) {
-        jn = j0 + claim(next);
-        const int2 rs = __ldg(P.rslice + j), ln = __ldg(P.rlane + 32 * (int64_t)j + lane);
+    int2 rs = rb.rs, ln = rb.ln;
+    for (int j = rb.j; j < j1; j = jn) {
+        jn = rb.j0 + claim(next);
+        if (j != rb.j) rs = __ldg(P.rslice + j), ln = __ldg(P.rlane + 32 * (int64_t)j + lane);
         // the warp's next slice goes to L2 while this one is worked
         const int2 nx = __ldg(P.rslice + (jn < j1 ? jn : j));
         const int64_t pf = nx.x;
@@ -301,14 +321,15 @@ struct RunObs {
         load_hg(P.r_hg + slot, P.rslot_cap, h);
     }
 };
-__device__ void own_cameras(const Prob &P, const double *rows, const float *, int blk, int *next) {
+__device__ void own_cameras(const Prob &P, const double *rows, const float *, int *next, const RunBegin &rb) {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
-    const int j0 = __ldg(P.blk_rslice + blk), j1 = __ldg(P.blk_rslice + blk + 1);
+    const int j1 = rb.j1;
     int jn = 0;
-    for (int j = j0 + (threadIdx.x >> 5); j < j1; j = jn) {
-        jn = j0 + claim(next);
-        const int2 rs = __ldg(P.rslice + j), ln = __ldg(P.rlane + 32 * (int64_t)j + lane);
+    int2 rs = rb.rs, ln = rb.ln;
+    for (int j = rb.j; j < j1; j = jn) {
+        jn = rb.j0 + claim(next);
+        if (j != rb.j) rs = __ldg(P.rslice + j), ln = __ldg(P.rlane + 32 * (int64_t)j + lane);
         const int cam = ln.x < 0 ? 0 : ln.x;
         const bool small = row_small(rows[cam * kRowD + 9]);
         double acc[10];
@@ -517,9 +538,10 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
     auto product = [&](auto rhs) {
         for (int blk = blockIdx.x; blk < P.nblk; blk += G) {
             own_points<T, decltype(rhs)::value>(P, rows, bs, blk, s_next);
+            const RunBegin rb = own_cameras_begin(P, blk);
             __syncthreads();
             if (threadIdx.x == 0) s_next[0] = nwarp;
-            own_cameras(P, rows, bs, blk, s_next + 1);
+            own_cameras(P, rows, bs, s_next + 1, rb);
             __syncthreads();
             if (threadIdx.x == 0) s_next[1] = nwarp;
         }
