@@ -243,9 +243,9 @@ def mba_evaluate(h, residuals=True, jacobians=True):
     info = mba_problem_info(h)
     n = info["n"]
     cost = C.c_double()
-    e = np.zeros((n, 2)) if residuals else None
-    jc = np.zeros((n, 2, 9)) if jacobians else None
-    jp = np.zeros((n, 2, 3)) if jacobians else None
+    e = np.empty((n, 2)) if residuals else None
+    jc = np.empty((n, 2, 9)) if jacobians else None
+    jp = np.empty((n, 2, 3)) if jacobians else None
     f = lambda a: None if a is None else a.ctypes.data_as(C.c_void_p)  # noqa: E731
     _check(load().mba_evaluate(h, C.byref(cost), f(e), f(jc), f(jp)))
     return cost.value, e, jc, jp
@@ -289,8 +289,8 @@ def mba_solve(h, trace_capacity=0, **opts):
 
 def mba_get_parameters(h, cameras=None, points=None):
     info = mba_problem_info(h)
-    cams = np.zeros((info["nc"], 9)) if cameras is None else cameras
-    pts = np.zeros((info["np"], 3)) if points is None else points
+    cams = np.empty((info["nc"], 9)) if cameras is None else cameras
+    pts = np.empty((info["np"], 3)) if points is None else points
     pc, _ = _ptr(cams, np.float64)
     pp, _ = _ptr(pts, np.float64)
     _check(load().mba_get_parameters(h, pc, pp))
@@ -310,8 +310,8 @@ def mba_reset(h):
 def mba_get_ordering(h):
     info = mba_problem_info(h)
     n, nc, np_ = info["n"], info["nc"], info["np"]
-    pt_perm, pt_ptr = np.zeros(n, np.int32), np.zeros(np_ + 1, np.int32)
-    cam_perm, cam_ptr = np.zeros(n, np.int32), np.zeros(nc + 1, np.int32)
+    pt_perm, pt_ptr = np.empty(n, np.int32), np.empty(np_ + 1, np.int32)
+    cam_perm, cam_ptr = np.empty(n, np.int32), np.empty(nc + 1, np.int32)
     f = lambda a: a.ctypes.data_as(C.c_void_p)  # noqa: E731
     _check(load().mba_get_ordering(h, f(pt_perm), f(pt_ptr), f(cam_perm), f(cam_ptr)))
     return pt_perm, pt_ptr, cam_perm, cam_ptr
@@ -320,9 +320,9 @@ def mba_get_ordering(h):
 def mba_linear_system(h, mu, damping="diag"):
     info = mba_problem_info(h)
     nc, np_ = info["nc"], info["np"]
-    Hpp, v = np.zeros((nc, 9, 9)), np.zeros((nc, 9))
-    Hll, w = np.zeros((np_, 3, 3)), np.zeros((np_, 3))
-    rhs = np.zeros((nc, 9))
+    Hpp, v = np.empty((nc, 9, 9)), np.empty((nc, 9))
+    Hll, w = np.empty((np_, 3, 3)), np.empty((np_, 3))
+    rhs = np.empty((nc, 9))
     f = lambda a: a.ctypes.data_as(C.c_void_p)  # noqa: E731
     _check(load().mba_linear_system(h, float(mu), DAMPING[damping], f(Hpp), f(v), f(Hll), f(w), f(rhs)))
     return dict(Hpp=Hpp, v=v, Hll=Hll, w=w, rhs=rhs)
@@ -331,7 +331,7 @@ def mba_linear_system(h, mu, damping="diag"):
 def mba_schur_matvec(h, mu, x, damping="diag"):
     info = mba_problem_info(h)
     xx = np.ascontiguousarray(x, dtype=np.float64).reshape(info["nc"], 9)
-    y = np.zeros_like(xx)
+    y = np.empty_like(xx)
     _check(load().mba_schur_matvec(h, float(mu), DAMPING[damping], xx.ctypes.data_as(C.c_void_p),
                                    y.ctypes.data_as(C.c_void_p)))
     return y
@@ -340,7 +340,7 @@ def mba_schur_matvec(h, mu, x, damping="diag"):
 def mba_step(h, mu, **opts):
     info = mba_problem_info(h)
     o = solver_options(**opts)
-    dc, dp = np.zeros((info["nc"], 9)), np.zeros((info["np"], 3))
+    dc, dp = np.empty((info["nc"], 9)), np.empty((info["np"], 3))
     it, md = C.c_int32(), C.c_double()
     _check(load().mba_step(h, float(mu), C.byref(o), dc.ctypes.data_as(C.c_void_p), dp.ctypes.data_as(C.c_void_p),
                            C.byref(it), C.byref(md)))
@@ -354,8 +354,8 @@ def mba_adjoint(h, grad_cameras, grad_points, mu=-1.0, **opts):
     o = solver_options(**opts)
     gc = np.ascontiguousarray(grad_cameras, dtype=np.float64).reshape(info["nc"], 9)
     gp = np.ascontiguousarray(grad_points, dtype=np.float64).reshape(info["np"], 3)
-    go = np.zeros((info["n"], 2))
-    gc0, gp0 = np.zeros((info["nc"], 9)), np.zeros((info["np"], 3))
+    go = np.empty((info["n"], 2))
+    gc0, gp0 = np.empty((info["nc"], 9)), np.empty((info["np"], 3))
     it = C.c_int32()
     f = lambda a: a.ctypes.data_as(C.c_void_p)  # noqa: E731
     _check(load().mba_adjoint(h, C.byref(o), float(mu), f(gc), f(gp), f(go), f(gc0), f(gp0), C.byref(it)))
@@ -521,8 +521,10 @@ def mba_batch_autotune(h, **opts):
 
 
 def _summaries(arr):
+    # through a structured view: one conversion per field instead of one per window and field
+    view = np.frombuffer(arr, dtype=np.dtype(WindowSummary))
     names = [f[0] for f in WindowSummary._fields_ if f[0] != "pad"]
-    return [{k: getattr(s, k) for k in names} for s in arr]
+    return [dict(zip(names, row)) for row in zip(*(view[k].tolist() for k in names))]
 
 
 def mba_batch_solve(h, grad_cameras=None, grad_points=None, adjoint_pcg_max_iter=500, adjoint_pcg_rel_tol=1e-12,
@@ -551,7 +553,7 @@ def mba_batch_solve(h, grad_cameras=None, grad_points=None, adjoint_pcg_max_iter
 
 def mba_batch_get_parameters(h):
     info = mba_batch_info(h)
-    cams, pts = np.zeros((info["nc"], 9)), np.zeros((info["np"], 3))
+    cams, pts = np.empty((info["nc"], 9)), np.empty((info["np"], 3))
     _check(load().mba_batch_get_parameters(h, _vp(cams), _vp(pts)))
     return cams, pts
 
@@ -569,7 +571,7 @@ def mba_batch_reset(h):
 
 def mba_batch_get_gradients(h):
     info = mba_batch_info(h)
-    go, gc, gp = np.zeros((info["n"], 2)), np.zeros((info["nc"], 9)), np.zeros((info["np"], 3))
+    go, gc, gp = np.empty((info["n"], 2)), np.empty((info["nc"], 9)), np.empty((info["np"], 3))
     _check(load().mba_batch_get_gradients(h, _vp(go), _vp(gc), _vp(gp)))
     return dict(grad_obs=go, grad_init_cam=gc, grad_init_pt=gp)
 
@@ -625,8 +627,8 @@ def _bal_read_text(path):
     bpath = os.fsencode(path)
     nc, np_, n = C.c_int32(), C.c_int32(), C.c_int64()
     _check(lib.mba_bal_read(bpath, C.byref(nc), C.byref(np_), C.byref(n), None, None, None, None, None))
-    cams, pts = np.zeros((nc.value, 9)), np.zeros((np_.value, 3))
-    obs = np.zeros((n.value, 2))
+    cams, pts = np.empty((nc.value, 9)), np.empty((np_.value, 3))
+    obs = np.empty((n.value, 2))
     ci, pi = np.zeros(n.value, np.int32), np.zeros(n.value, np.int32)
     _check(lib.mba_bal_read(bpath, C.byref(nc), C.byref(np_), C.byref(n), _vp(cams), _vp(pts), _vp(obs), _vp(ci),
                             _vp(pi)))
