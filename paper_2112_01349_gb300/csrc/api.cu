@@ -771,11 +771,12 @@ mba_status mba_solve(mba_problem *pr, const mba_solver_options *opt, mba_summary
     CK(rec(ne > 0 ? ne - 1 : 0));
     // state_init, camera table, 2 cost kernels; per iteration: camera table, 3
     // linearisation, 2 damping, PCG, 3 back-substitution, camera table, 2 cost,
-    // LM update, accept; the FP32 forms add their point copy and, where the
+    // LM update, accept; the FP32 forms and the block-owned FP64
+    // one add their point copy and, where the
     // factored form's camera rows do not fit in shared memory, the rows of dc, the
     // float-float cost its point copy before each cost, the Schur-Jacobi
     // preconditioner two damping kernels
-    const int fact = (P.fp32 ? 1 : 0) + (P.fact && P.nc * kRowS * 4 > 220 * 1024 ? 1 : 0), ffc = ff ? 1 : 0;
+    const int fact = (P.fp32 || P.own ? 1 : 0) + (P.fact && P.nc * kRowS * 4 > 220 * 1024 ? 1 : 0), ffc = ff ? 1 : 0;
     const int launches =
         4 + ffc + (15 + fact + ffc + (o.preconditioner == MBA_PRECOND_SCHUR_JACOBI ? 2 : 0)) * o.max_iter;
     DevState hs;
