@@ -66,6 +66,84 @@ __global__ void fill_runs_kernel(Prob P, const int32_t *__restrict__ ord, const 
     }
 }
 
+// part of a run of l observations: those k with k mod parts equal to it
+__device__ __forceinline__ int part_len(int l, int parts, int part) { return (l + parts - 1 - part) / parts; }
+
+// One CTA per block: its (camera, part) pairs by decreasing length, then index
+// (bitonic sort of m = 2^k keys in shared memory); info: its slices and rounds.
+__global__ void __launch_bounds__(512) sort_runs_kernel(const int32_t *__restrict__ len, int nc, int parts, int lg,
+                                                        int m, unsigned long long *__restrict__ sorted, int2 *info) {
+    extern __shared__ unsigned long long key[];
+    __shared__ int s_used, s_rounds;
+    const int items = nc * parts, per = 32 >> lg;
+    const int32_t *l = len + (int64_t)blockIdx.x * nc;
+    if (threadIdx.x == 0) s_used = 0, s_rounds = 0;
+    for (int i = threadIdx.x; i < m; i += blockDim.x)
+        key[i] = i < items ? ((unsigned long long)(unsigned)~part_len(l[i / parts], parts, i % parts) << 32) | (unsigned)i
+                           : ~0ull;
+    for (int k = 2; k <= m; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            __syncthreads();
+            for (int t = threadIdx.x; t < m / 2; t += blockDim.x) {
+                const int i = 2 * t - (t & (j - 1)), o = i + j;
+                const unsigned long long a = key[i], b = key[o];
+                if ((a > b) == ((i & k) == 0)) key[i] = b, key[o] = a;
+            }
+        }
+    __syncthreads();
+    int used = 0, rounds = 0;
+    for (int i = threadIdx.x; i < items; i += blockDim.x) {
+        const unsigned long long a = key[i];
+        const int n = (int)~(unsigned)(a >> 32);
+        sorted[(int64_t)blockIdx.x * items + i] = a;
+        if (n > 0) {
+            ++used;
+            if (i % per == 0) rounds += (n + (1 << lg) - 1) >> lg;
+        }
+    }
+    atomicAdd(&s_used, used);
+    atomicAdd(&s_rounds, rounds);
+    __syncthreads();
+    if (threadIdx.x == 0) info[blockIdx.x] = make_int2((s_used + per - 1) / per, s_rounds);
+}
+
+// The run slices of a block (from slice first[b], round round0[b]): first slot and
+// rounds, the (camera, row of the partial sums) of every lane, and the first slot
+// of every (camera, part).
+constexpr int kBlockSlices = 256;
+__global__ void __launch_bounds__(256) run_slices_kernel(Prob P, const unsigned long long *__restrict__ sorted,
+                                                         const int32_t *__restrict__ round0, int parts, int lg,
+                                                         int32_t *__restrict__ base) {
+    __shared__ int s_start[kBlockSlices + 1];
+    const int b = blockIdx.x, items = P.nc * parts, per = 32 >> lg, G = 1 << lg;
+    const int first = P.blk_rslice[b], nsl = P.blk_rslice[b + 1] - first;
+    const unsigned long long *key = sorted + (int64_t)b * items;
+    for (int j = threadIdx.x; j < nsl; j += blockDim.x)
+        s_start[j] = ((int)~(unsigned)(key[j * per] >> 32) + G - 1) >> lg;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int r = round0[b];
+        for (int j = 0; j < nsl; ++j) {
+            const int K = s_start[j];
+            P.rslice[first + j] = make_int2(32 * r, K);
+            s_start[j] = r;
+            r += K;
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 32 * nsl; i += blockDim.x) {
+        const int j = i >> 5, lane = i & 31, q = j * per + (lane >> lg);
+        int2 ln = make_int2(-1, 0);
+        const unsigned long long a = q < items ? key[q] : ~0ull;
+        if ((int)~(unsigned)(a >> 32) > 0) {
+            const int it = (int)(a & 0xffffffffu), cam = it / parts, part = it % parts;
+            ln = make_int2(cam, b * parts + part);
+            if ((lane & (G - 1)) == 0) base[((int64_t)b * P.nc + cam) * parts + part] = 32 * s_start[j] + lane;
+        }
+        P.rlane[32 * (int64_t)first + i] = ln;
+    }
+}
+
 inline unsigned grid_for(int64_t n) {
     int64_t g = (n + kBlock - 1) / kBlock;
     if (g > 152 * 16) g = 152 * 16;
@@ -90,7 +168,8 @@ bool own_wanted(const Prob &P, int grid) {
 
 size_t own_tmp_bytes(const Prob &P, int64_t nblk) {
     return al256(8 * (size_t)P.np) + 3 * al256(4 * (size_t)P.n) + 2 * al256(4 * ((size_t)nblk * P.nc + 2)) +
-           al256(4 * (size_t)nblk * P.nc * (P.nc < 128 ? kMaxParts : 1)) + 4 * (size_t)exclusive_scan_tmp_ints(nblk * P.nc + 2) + 1024 +
+           al256(4 * (size_t)nblk * P.nc * (P.nc < 128 ? kMaxParts : 1)) +
+           al256(8 * (size_t)nblk * P.nc * (P.nc < 128 ? kMaxParts : 1)) + 2 * al256(8 * (size_t)nblk) + 4 * (size_t)exclusive_scan_tmp_ints(nblk * P.nc + 2) + 1024 +
            stable_sort_tmp_bytes(P.n, (int32_t)nblk + 1);
 }
 
@@ -109,21 +188,21 @@ cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void **pool, size_t 
             *run = (int32_t *)take(4 * (size_t)P.n);
     int32_t *count = (int32_t *)take(4 * ((size_t)nruns + 2)), *run_ptr = (int32_t *)take(4 * ((size_t)nruns + 2));
     int32_t *base_d = (int32_t *)take(4 * (size_t)nruns * (P.nc < 128 ? kMaxParts : 1));
+    auto *sorted = (unsigned long long *)take(8 * (size_t)nruns * (P.nc < 128 ? kMaxParts : 1));
+    int2 *info_d = (int2 *)take(8 * (size_t)nblk);
+    int32_t *round0_d = (int32_t *)take(4 * (size_t)nblk);
     int32_t *scan_tmp = (int32_t *)take(4 * (size_t)exclusive_scan_tmp_ints(nruns + 2));
     const size_t sort_bytes = stable_sort_tmp_bytes(P.n, (int32_t)nblk + 1);
 
     point_blocks_kernel<<<grid_for(P.n_slices), kBlock, 0, s>>>(P.slice, P.n_slices, P.nblk, sp_bl);
     obs_block_kernel<<<grid_for(P.n), kBlock, 0, s>>>(P.cm_sp, sp_bl, P.n, key);
-    cudaError_t e = stable_sort_by_key(key, P.n, (int32_t)nblk, ord, run_ptr, t, sort_bytes, s);  // run_ptr: unused here
+    cudaError_t e = stable_sort_by_key(key, P.n, (int32_t)nblk, ord, nullptr, t, sort_bytes, s);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(count, 0, 4 * ((size_t)nruns + 2), s);
     if (e != cudaSuccess) return e;
     run_key_kernel<<<grid_for(P.n), kBlock, 0, s>>>(ord, key, P.cam_ptr, P.nc, P.n, run, count);
     e = exclusive_scan_i32(count, run_ptr, nruns + 1, scan_tmp, s);
     if (e != cudaSuccess) return e;
-    std::vector<int32_t> len((size_t)nruns);
-    e = cudaMemcpyAsync(len.data(), count, 4 * (size_t)nruns, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
 
     // few cameras: split their runs until a block has work for a few hundred lanes
@@ -142,44 +221,30 @@ cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void **pool, size_t 
     while (lg < 3 && (2 << lg) <= mean / parts &&
            (items_blk << (lg + 1)) <= (P.fp32 ? 4096 : (lg == 0 ? 1024 : 256)))
         ++lg;
-    const int G = 1 << lg, per = 32 / G;
 
-    std::vector<int32_t> base((size_t)nruns * parts, 0), blk((size_t)nblk + 1);
-    std::vector<int2> rs, lanes;
+    // sort on the device, offsets of the blocks here, then the slices on the device:
+    // laid out on the host (counts read back, tables of 32 lanes a slice sent), the
+    // creation of 1.0M points and 5.0M observations took 8.6 ms instead of 3.5, of
+    // 50k points and 250k observations 1.77 instead of 1.01
+    int m = 2;
+    while (m < items_blk) m *= 2;
+    if (m > 4096) return cudaErrorInvalidValue;
+    sort_runs_kernel<<<(unsigned)nblk, 512, 8 * (size_t)m, s>>>(count, P.nc, parts, lg, m, sorted, info_d);
+    std::vector<int2> info((size_t)nblk);
+    e = cudaMemcpyAsync(info.data(), info_d, 8 * (size_t)nblk, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return e;
+    std::vector<int32_t> blk((size_t)nblk + 1), round0((size_t)nblk);
     int64_t slots = 0;
-    std::vector<int32_t> order, bucket;
+    blk[0] = 0;
     for (int64_t b = 0; b < nblk; ++b) {
-        blk[b] = (int32_t)rs.size();
-        // the block's (camera, part) pairs by decreasing length: counting sort
-        const int32_t *l = len.data() + b * P.nc;
-        const int64_t items = (int64_t)P.nc * parts;
-        auto part_len = [&](int64_t it) { return (int32_t)((l[it / parts] + parts - 1 - it % parts) / parts); };
-        int32_t longest = 0;
-        for (int32_t c = 0; c < P.nc; ++c) longest = std::max(longest, (l[c] + parts - 1) / parts);
-        bucket.assign((size_t)longest + 2, 0);
-        for (int64_t it = 0; it < items; ++it) bucket[(size_t)(longest - part_len(it)) + 1]++;
-        for (size_t k = 1; k < bucket.size(); ++k) bucket[k] += bucket[k - 1];
-        const int32_t used = bucket[(size_t)longest];  // those of length >= 1
-        order.resize((size_t)items);
-        for (int64_t it = 0; it < items; ++it) order[(size_t)bucket[(size_t)(longest - part_len(it))]++] = (int32_t)it;
-        for (int32_t q0 = 0; q0 < used; q0 += per) {
-            const int K = (part_len(order[q0]) + G - 1) >> lg;
-            rs.push_back(make_int2((int32_t)slots, K));
-            for (int j = 0; j < per; ++j) {
-                const int32_t q = q0 + j;
-                int2 ln = make_int2(-1, 0);
-                if (q < used) {
-                    const int64_t it = order[q], cam = it / parts, part = it % parts;
-                    base[(size_t)((b * P.nc + cam) * parts + part)] = (int32_t)slots + j * G;
-                    ln = make_int2((int32_t)cam, (int32_t)(b * parts + part));
-                }
-                for (int g = 0; g < G; ++g) lanes.push_back(ln);
-            }
-            slots += 32 * (int64_t)K;
-        }
+        if (info[b].x > kBlockSlices) return cudaErrorInvalidValue;
+        blk[b + 1] = blk[b] + info[b].x;
+        round0[b] = (int32_t)(slots / 32);
+        slots += 32 * (int64_t)info[b].y;
         if (slots > 2000000000ll) return cudaErrorInvalidValue;
     }
-    blk[nblk] = (int32_t)rs.size();
+    const size_t nrs = (size_t)blk[nblk];
     P.r_lg = lg;
     P.rslot_cap = (slots + 31) / 32 * 32;
 
@@ -194,8 +259,8 @@ cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void **pool, size_t 
             off += al256(bytes ? bytes : 1);
             return p;
         };
-        P.rslice = (int2 *)arr(8 * rs.size());
-        P.rlane = (int2 *)arr(8 * lanes.size());
+        P.rslice = (int2 *)arr(8 * nrs);
+        P.rlane = (int2 *)arr(32 * 8 * nrs);
         P.blk_rslice = (int32_t *)arr(4 * blk.size());
         P.cm2r = (int32_t *)arr(4 * (size_t)P.n);
         P.c_part = arr(part_vals * (P.fp32 ? 4 : 8));
@@ -214,14 +279,13 @@ cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void **pool, size_t 
             if (e != cudaSuccess) return e;
         }
     }
-    e = cudaMemcpyAsync(P.rslice, rs.data(), 8 * rs.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(P.rlane, lanes.data(), 8 * lanes.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(P.blk_rslice, blk.data(), 4 * blk.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(base_d, base.data(), 4 * base.size(), cudaMemcpyHostToDevice, s);
+    e = cudaMemcpyAsync(P.blk_rslice, blk.data(), 4 * blk.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(round0_d, round0.data(), 4 * round0.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(P.c_part, 0, part_vals * (P.fp32 ? 4 : 8), s);
     if (e == cudaSuccess)
         e = P.fp32 ? cudaMemsetAsync(P.r_pt16, 0xff, 2 * ns, s) : cudaMemsetAsync(P.r_pt, 0xff, 4 * ns, s);
     if (e != cudaSuccess) return e;
+    run_slices_kernel<<<(unsigned)nblk, 256, 0, s>>>(P, sorted, round0_d, parts, lg, base_d);
     fill_runs_kernel<<<grid_for(P.n), kBlock, 0, s>>>(P, ord, run, run_ptr, base_d, parts, lg, sp_bl);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host vectors go out of scope

@@ -183,6 +183,22 @@ __global__ void iota_copy_kernel(const int32_t *kin, int64_t n, int32_t *kout, i
     }
 }
 
+// Few keys (track lengths, cameras): counted in shared memory, since a handful of
+// hot counters would serialise the whole grid's atomics (1.0M track lengths:
+// 0.6 ms), then one atomic per block and key.
+constexpr int32_t kHistKeys = 4096;
+__global__ void __launch_bounds__(kBlock) count_keys_smem_kernel(const int32_t *keys, int64_t n, int32_t nkeys,
+                                                                 int32_t *cnt) {
+    __shared__ int32_t h[kHistKeys];
+    for (int32_t q = threadIdx.x; q < nkeys; q += blockDim.x) h[q] = 0;
+    __syncthreads();
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+        atomicAdd(&h[keys[k]], 1);
+    __syncthreads();
+    for (int32_t q = threadIdx.x; q < nkeys; q += blockDim.x)
+        if (h[q]) atomicAdd(&cnt[q], h[q]);
+}
+
 __global__ void count_keys_kernel(const int32_t *keys, int64_t n, int32_t *cnt) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
         atomicAdd(&cnt[keys[k]], 1);
@@ -246,9 +262,15 @@ cudaError_t stable_sort_by_key(const int32_t *keys_in, int64_t n, int32_t nkeys,
         cudaError_t e = cudaMemcpyAsync(perm_out, vcur, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s);
         if (e != cudaSuccess) return e;
     }
+    if (!ptr_out) return cudaGetLastError();
     cudaError_t e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (nkeys + 1), s);
     if (e != cudaSuccess) return e;
-    count_keys_kernel<<<grid_for(n), kBlock, 0, s>>>(keys_in, n, cnt);
+    if (nkeys <= kHistKeys) {
+        const unsigned g = grid_for(n);
+        count_keys_smem_kernel<<<g < 152 * 4 ? g : 152 * 4, kBlock, 0, s>>>(keys_in, n, nkeys, cnt);
+    } else {
+        count_keys_kernel<<<grid_for(n), kBlock, 0, s>>>(keys_in, n, cnt);
+    }
     return exclusive_scan(cnt, ptr_out, (int64_t)nkeys + 1, stmp, s);
 }
 
