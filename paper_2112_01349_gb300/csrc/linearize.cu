@@ -70,7 +70,9 @@ __device__ __forceinline__ void own_camera(const double *row, double *ctr) {
     for (int q = 0; q < 9; ++q) ctr[18 + q] = in[q];
 }
 
-template <typename T>
+// HALF: from the half angle, where the analytic products (block-owned, gathered)
+// read the table; dual numbers and a stored FP64 Jacobian keep the full angle.
+template <typename T, bool HALF>
 __global__ void camera_table_kernel(const double *__restrict__ cams, int32_t nc, T *__restrict__ tab,
                                     double *__restrict__ tab64, float2 *__restrict__ tabff,
                                     float *__restrict__ stat, float *__restrict__ ctr, double *__restrict__ ctr64,
@@ -80,15 +82,15 @@ __global__ void camera_table_kernel(const double *__restrict__ cams, int32_t nc,
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
         double row[kCamTab];
         double quat[4];
-        camera_table_row<true>(cams + 9 * (int64_t)i, row, quat);
+        camera_table_row<HALF>(cams + 9 * (int64_t)i, row, quat);
         if (tab)
 #pragma unroll
             for (int q = 0; q < kCamTab; ++q) tab[(int64_t)i * kCamTab + q] = (T)row[q];
+        if (ctr64) own_camera(row, ctr64 + (int64_t)i * kCtr);
+        if (ctr) factored_camera(row, quat, stat + (int64_t)i * kCamStat, ctr + (int64_t)i * kCtr);
         if (tab64)
 #pragma unroll
             for (int q = 0; q < kCamTab; ++q) tab64[(int64_t)i * kCamTab + q] = row[q];
-        if (ctr64) own_camera(row, ctr64 + (int64_t)i * kCtr);
-        if (ctr) factored_camera(row, quat, stat + (int64_t)i * kCamStat, ctr + (int64_t)i * kCtr);
         if (tabff) {  // R, t, f, k1, k2 as float-float
 #pragma unroll
             for (int q = 0; q < 9; ++q) {
@@ -1009,31 +1011,27 @@ __global__ void __launch_bounds__(kBlock) evaluate_slice_kernel(Prob P, const in
 
 int cost_grid(const Prob &P) { return (int)grid_for(P.n); }
 
-cudaError_t launch_camera_tables(const Prob &P, const double *cams, bool for_lin, cudaStream_t s) {
+template <typename T>
+static cudaError_t launch_table(const Prob &P, const double *cams, T *tab, double *tab64, float2 *tabff, float *stat,
+                                float *ctr, double *ctr64, int gate, cudaStream_t s) {
     const unsigned g = grid_for(P.nc, 128);
-    if (for_lin) {
-        if (P.fp32)
-            camera_table_kernel<float><<<g, 128, 0, s>>>(cams, P.nc, (float *)P.camtab, nullptr, nullptr, P.camstat,
-                                                         P.ctr, nullptr, P.st, 1);
-        else
-            camera_table_kernel<double><<<g, 128, 0, s>>>(cams, P.nc, (double *)P.camtab, nullptr, nullptr, nullptr,
-                                                          nullptr, P.ctr64, P.st, 1);
-    } else {
-        camera_table_kernel<double><<<g, 128, 0, s>>>(cams, P.nc, nullptr, P.camtab64, P.camff, nullptr, nullptr,
-                                                      nullptr, P.st, 2);
-    }
+    if (P.own || P.fact)
+        camera_table_kernel<T, true><<<g, 128, 0, s>>>(cams, P.nc, tab, tab64, tabff, stat, ctr, ctr64, P.st, gate);
+    else
+        camera_table_kernel<T, false><<<g, 128, 0, s>>>(cams, P.nc, tab, tab64, tabff, stat, ctr, ctr64, P.st, gate);
     return cudaGetLastError();
 }
 
+cudaError_t launch_camera_tables(const Prob &P, const double *cams, bool for_lin, cudaStream_t s) {
+    if (!for_lin)
+        return launch_table<double>(P, cams, nullptr, P.camtab64, P.camff, nullptr, nullptr, nullptr, 2, s);
+    if (P.fp32) return launch_table(P, cams, (float *)P.camtab, nullptr, nullptr, P.camstat, P.ctr, nullptr, 1, s);
+    return launch_table(P, cams, (double *)P.camtab, nullptr, nullptr, nullptr, nullptr, P.ctr64, 1, s);
+}
+
 cudaError_t launch_camera_tables_forced(const Prob &P, const double *cams, cudaStream_t s) {
-    const unsigned g = grid_for(P.nc, 128);
-    if (P.fp32)
-        camera_table_kernel<float><<<g, 128, 0, s>>>(cams, P.nc, (float *)P.camtab, P.camtab64, P.camff, P.camstat,
-                                                     P.ctr, nullptr, P.st, 0);
-    else
-        camera_table_kernel<double><<<g, 128, 0, s>>>(cams, P.nc, (double *)P.camtab, P.camtab64, nullptr, nullptr,
-                                                      nullptr, P.ctr64, P.st, 0);
-    return cudaGetLastError();
+    if (P.fp32) return launch_table(P, cams, (float *)P.camtab, P.camtab64, P.camff, P.camstat, P.ctr, nullptr, 0, s);
+    return launch_table(P, cams, (double *)P.camtab, P.camtab64, nullptr, nullptr, nullptr, P.ctr64, 0, s);
 }
 
 cudaError_t launch_split_observations(const Prob &P, cudaStream_t s) {

@@ -208,7 +208,7 @@ __host__ __device__ __forceinline__ int sym3(int a, int b) {
 // the dual-number path, which evaluates the edge functor from the parameters).
 // ---------------------------------------------------------------------------
 // HALF: one sine and cosine, of the half angle, and reciprocals instead of
-// divides (11.5 -> 9 us for 200 cameras); its quaternion goes to quat.
+// divides (11.5 -> 9 us for 200 cameras); the rotation's quaternion goes to quat.
 template <bool HALF = false>
 __device__ __forceinline__ void camera_table_row(const double *c, double *o, double *quat = nullptr) {
     const double w0 = c[0], w1 = c[1], w2 = c[2];

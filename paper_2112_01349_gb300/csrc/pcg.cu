@@ -86,7 +86,7 @@ __global__ void damp_points_kernel(Prob P, int damping) {
             atomicExch(&st->blockfail, 1);
             continue;
         }
-        const double id = fast_rcp(det);
+        const double id = sorted ? fast_rcp(det) : 1.0 / det;
         Ci[base] = (T)(c00 * id);
         Ci[base + step] = (T)(c01 * id);
         Ci[base + 2 * step] = (T)(c02 * id);
