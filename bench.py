@@ -75,12 +75,12 @@ def pcg_bytes_per_iter(sc, w: int) -> float:
 
 
 def pcg_streamed_bytes_per_iter(sc) -> float:
-    """Bytes the factored FP32 Schur product streams per PCG iteration: per
-    observation (px, py, 1/P_z) 12, W Jp 24, camera index 4, position of s 4,
-    s written 8 in the point pass and (RX, 1/P_z) 16, s 8 in the camera pass;
-    per point C~^-1 (6 floats) and a CSR offset; per camera B~ and B~^-1 (81
-    doubles each) and six FP64 vectors of stride 12."""
-    return sc.n * 76 + sc.np_ * 28 + sc.nc * (2 * 81 * 8 + 6 * 12 * 8)
+    """Bytes the block-owned FP32 Schur product streams per PCG iteration: per
+    observation (camera, px, py, 1/P_z) 16 on the point side and (RX, 1/P_z) 16
+    and a point index 2 on the camera side; per point C~^-1 (6 floats); per camera
+    B~ and B~^-1 (81 doubles each) and six FP64 vectors of stride 12.  The blocks'
+    partial sums (48 B per block and camera, written and read) stay in L2."""
+    return sc.n * 34 + sc.np_ * 24 + sc.nc * (2 * 81 * 8 + 6 * 12 * 8)
 
 
 def lin_bytes_per_obs(sc, w: int) -> float:
@@ -128,12 +128,11 @@ def batch_flops(ws, summaries, schur: str) -> float:
 # and FP64.  Traffic grows with the observation count, so a launch moves this
 # many bytes per observation per pass; None once the kernel has changed since
 # the capture.  The last full-size capture gave 61.3 B (FP32-mixed) and 431.1 B
-# (FP64); both kernels have changed since (the FP32 one loads its B~ rows
-# earlier, the FP64 one runs fewer scan levels), so no figure is claimed.
+# (FP64), for kernels that the block-owned one has replaced, so no figure is
+# claimed.
 PCG_TRAFFIC_B_PER_OBS_PASS = {}
-PCG_TRAFFIC_NOTE = ("null: the kernel changed after the last full-size DRAM capture (61.3 B per observation per "
-                    "pass FP32-mixed, 431.1 B FP64); the FP32 change loads the same rows earlier, the FP64 one "
-                    "runs fewer FP64 scan levels; not re-taken")
+PCG_TRAFFIC_NOTE = ("null: the kernel was replaced after the last full-size DRAM capture (61.3 B per observation per "
+                    "pass FP32-mixed, 431.1 B FP64); not re-taken")
 
 
 def oracle_sample_time(threads: int, scale: float) -> dict:
@@ -704,9 +703,9 @@ def main():
         "warmup": args.warmup, "ms_per_step": a32["ms_per_step"], "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32+f64 (FP32-mixed)", "data": "synthetic",
         "config": {"workload": workload_desc(sc), "precision": "fp32-mixed (FP64 accept/reject cost)",
-                   "l2": "inputs larger than L2 (per PCG pass: 0.38 GB streamed FP32, 1.7 GB FP64)",
+                   "l2": "inputs larger than L2 (per PCG pass: 0.2 GB streamed FP32, 0.84 GB FP64)",
                    "parallelism": "replicas" if world > 1 else "1 GPU"},
-        "roofline": {"kernel": "pcg_kernel (persistent PCG, implicit Schur product)", "bound": "hbm",
+        "roofline": {"kernel": "pcg_own_kernel (persistent PCG, block-owned implicit Schur product)", "bound": "hbm",
                      "achieved": a32["gbs"], "peak": hbm_peak, "unit": "GB/s", "frac": a32["gbs"] / hbm_peak,
                      "peak_kind": peak_kind, "traffic": a32["traffic_per_launch"],
                      "traffic_unit": "bytes per launch (ncu dram__bytes_read+write per observation per pass of a "
@@ -715,8 +714,8 @@ def main():
                      "algorithmic": "per PCG iteration 100 B per observation (stored Jacobian + camera index), "
                                     "72 B per point, 576 B per camera",
                      "streamed_gbs": a32["streamed_gbs"], "streamed_frac": a32["streamed_gbs"] / hbm_peak,
-                     "streamed": "bytes the factored FP32 product actually streams: 76 B per observation per "
-                                 "iteration, 28 B per point, 1.9 KB per camera",
+                     "streamed": "bytes the factored FP32 product actually streams: 34 B per observation per "
+                                 "iteration, 24 B per point, 1.9 KB per camera",
                      "dram_gbs": a32["dram_gbs"],
                      "dram_frac": None if a32["dram_gbs"] is None else a32["dram_gbs"] / hbm_peak,
                      "traffic_note": PCG_TRAFFIC_NOTE if a32["traffic_per_launch"] is None else None,
@@ -724,7 +723,7 @@ def main():
                      "pcg_iters_per_solve": a32["pcg_iters"] / max(1, len(s32)),
                      "other_kernels": {
                          "pcg_single_reduction_fp32": None if not variants else {
-                             "kernel": "pcg_kernel, single-reduction (Chronopoulos-Gear) instance",
+                             "kernel": "pcg_own_kernel, single-reduction (Chronopoulos-Gear) instance",
                              "bound": "hbm", "unit": "GB/s",
                              "us_per_pcg_iter": variants["single_reduction_pcg"]["us_per_pcg_iter"],
                              "achieved": pcg_bytes_per_iter(sc, 4) / (variants["single_reduction_pcg"]["us_per_pcg_iter"]
