@@ -917,7 +917,12 @@ __device__ void camera_pass(const BatchArgs &A, const WinMem<T> &M, const WinDes
     // the warps of all ranks divide the window's observations
     const int gw = wid + (CL ? NW * M.rank : 0), nwt = NW * (CL ? M.csz : 1);
     const int lo = (int)(((int64_t)gw * d.n) / nwt), hi = (int)(((int64_t)(gw + 1) * d.n) / nwt);
-    if (lo >= hi) return;
+    if (lo >= hi) {
+        // no observations (fewer than warps): the camera around position lo may add
+        // this warp's slot, between those of the warps before and after it
+        for (int q = lane; q < K; q += 32) M.slot[(wid + M.wcam0[wid]) * K + q] = 0.0;
+        return;
+    }
     T *cmX = (T *)A.cmX;
     const T2 *cms = (const T2 *)A.cms;
     const T delta = (T)A.delta;

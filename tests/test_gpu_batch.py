@@ -318,3 +318,44 @@ def test_measured_order_changes_no_result(mba):
     assert [x["final_cost"] for x in r1["summaries"]] == [x["final_cost"] for x in r2["summaries"]]
     np.testing.assert_array_equal(p1[0], p2[0])
     np.testing.assert_array_equal(p1[1], p2[1])
+
+
+# fewer observations than the warps of a window's thread-block cluster (128, 64, 32
+# and 16 warps for batches of one to nine, up to 19, up to 38 and more windows), so
+# that some warps own no observation: (cameras, points), every camera sees every point
+FEW = [(6, 7), (5, 20), (4, 30), (5, 10), (8, 8), (7, 3), (10, 2), (6, 21)]
+
+
+@pytest.mark.parametrize("loss", ["none", "huber"])
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-6), ("fp32", 3e-3)])
+@pytest.mark.parametrize("count", [1, 3, 8, 15, 30, 50])
+def test_windows_of_few_observations(mba, count, precision, tol, loss):
+    """Windows of 20 to 126 observations against the oracle, forward and adjoint,
+    and bit for bit on repeat.  Tolerances: those of parameters and adjoints
+    elsewhere in this file."""
+    ws = [make_scene(*FEW[w % len(FEW)], track=("fixed", FEW[w % len(FEW)][0]), sigma=1.0, seed=300 + w)
+          for w in range(count)]
+    opts = dict(max_iter=3, pcg_max_iter=15, pcg_rel_tol=1e-10, initial_radius=10.0)
+    rng = np.random.default_rng(count)
+    with mba.Batch(_tuples(ws), precision=precision, loss=loss, huber_delta=2.0 if loss == "huber" else 0.0) as b:
+        gc, gp = rng.normal(size=(b.info["nc"], 9)), rng.normal(size=(b.info["np"], 3))
+        runs = []
+        for _ in range(2):
+            b.reset()
+            r = b.solve(gc, gp, adjoint_pcg_max_iter=200, adjoint_pcg_rel_tol=1e-12, adjoint_mu=0.3, **opts)
+            runs.append((*b.parameters(), *b.gradients().values()))
+        for a, c in zip(*runs):
+            np.testing.assert_array_equal(a, c)
+        co, po, oo = b.offsets
+    cams, pts, go, gc0, gp0 = runs[0]
+    for w, s in enumerate(ws):
+        c, p, o = slice(co[w], co[w + 1]), slice(po[w], po[w + 1]), slice(oo[w], oo[w + 1])
+        ref = _oracle_solve(s, loss=loss, delta=2.0, max_iter=3, pcg_max=15, initial_radius=10.0)
+        assert r["summaries"][w]["status"] == 0
+        rel_close(cams[c], ref["cameras"], tol, f"window {w} cameras")
+        rel_close(pts[p], ref["points"], tol, f"window {w} points")
+        adj = oracle.adjoint(cams[c], pts[p], s.observations, s.cam_idx, s.pt_idx, 0.3, gc[c], gp[p], loss=loss,
+                             delta=2.0, pcg_max=200, pcg_tol=1e-12)
+        rel_close(go[o], adj["grad_obs"], tol, f"window {w} observation gradient")
+        rel_close(gc0[c], adj["grad_c0"], tol, f"window {w} camera gradient")
+        rel_close(gp0[p], adj["grad_p0"], tol, f"window {w} point gradient")
