@@ -502,6 +502,10 @@ __device__ void point_pass(const Prob &P, const T *ps, const T *pT, typename V2<
 // first nine are linear in v, so row(z) + beta row(p) is the row of z + beta p.
 // ---------------------------------------------------------------------------
 
+// A fixed camera's Jacobian columns are zero, so its rows are, whatever the
+// vector holds there: zero in a solve, but the upstream gradient's part in an adjoint.
+__device__ __forceinline__ bool fixed_camera(const Prob &P, int cam) { return P.has_fixed && P.cam_fixed[cam]; }
+
 // Warp-collective (all 32 lanes call it): lanes 9s..9s+8 hold the nine
 // components of camera `cam` (lane s of the three-camera group); returns the
 // lane's component of the camera's row.
@@ -520,7 +524,7 @@ __device__ __forceinline__ float fact_row_lane(const Prob &P, int cam, double va
         const float *t = P.camstat + (int64_t)cam * kCamStat + 7;
         r -= n1 * __ldg(t + b2) - n2 * __ldg(t + b1);
     }
-    return r;
+    return fixed_camera(P, cam) ? 0.f : r;
 }
 
 // The whole row of one camera by one thread.
@@ -539,6 +543,9 @@ __device__ __forceinline__ void fact_row(const Prob &P, int cam, const float *v,
     r[3] -= r[1] * t2 - r[2] * t1;
     r[4] -= r[2] * t0 - r[0] * t2;
     r[5] -= r[0] * t1 - r[1] * t0;
+    if (fixed_camera(P, cam))
+#pragma unroll
+        for (int q = 0; q < 9; ++q) r[q] = 0.f;
 #pragma unroll
     for (int q = 0; q < 7; ++q) r[9 + q] = st[q];
 }
@@ -694,6 +701,7 @@ __device__ void point_pass_fact_rhs(const Prob &P) {
 #pragma unroll
         for (int q = 0; q < 6; ++q) ci[q] = __ldg(Ci + (int64_t)q * P.np_pad + s);
         apply_sym3(ci, (float)P.w[3 * pt], (float)P.w[3 * pt + 1], (float)P.w[3 * pt + 2], b);
+        if (P.has_fixed && P.pt_fixed[pt]) b[0] = b[1] = b[2] = 0.f;  // its Jacobian columns are zero
         P.sp_b[s] = make_float4(b[0], b[1], b[2], 0.f);
     }
 }
@@ -1067,9 +1075,8 @@ __device__ void stage_p(const Prob &P, T *ps, const double *p_prev, const T *pT_
         } else {
             for (int cam = threadIdx.x; cam < P.nc; cam += blockDim.x) {
                 float v[9], r[kRowG];
-                const bool fixed = P.has_fixed && P.cam_fixed[cam];  // its Jacobian columns are zero
 #pragma unroll
-                for (int j = 0; j < 9; ++j) v[j] = fixed ? 0.f : (float)src_given[(int64_t)cam * kVec + j];
+                for (int j = 0; j < 9; ++j) v[j] = (float)src_given[(int64_t)cam * kVec + j];
                 fact_row(P, cam, v, r);
                 float4 *dst = (float4 *)(ps + cam * kRowS);
 #pragma unroll
@@ -1297,10 +1304,7 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
                 if (!given) stcg(p_cur + vo, pn);
                 if (!FACT) stcg(pT + vo, (T)pn);
             }
-            if constexpr (FACT) {
-                const bool fixed = given && act && P.has_fixed && P.cam_fixed[cam];
-                store_row(act ? cam : 0, act, fixed ? 0.0 : pn, nullptr, (float *)pT);
-            }
+            if constexpr (FACT) store_row(act ? cam : 0, act, pn, nullptr, (float *)pT);
         }
     };
 
@@ -1811,7 +1815,7 @@ __global__ void __launch_bounds__(512, 1) backsub_slices64_kernel(Prob P, double
             r = __ldg((const double *)P.camtab + (int64_t)cam * kCamTab + 24);
         } else {
             const double *ct = P.ctr64 + (int64_t)cam * kCtr + 3 * g0 + (q - g0), *v = P.x + (int64_t)cam * kVec + g0;
-            r = fma(ct[0], v[0], fma(ct[3], v[1], ct[6] * v[2]));
+            r = fixed_camera(P, cam) ? 0.0 : fma(ct[0], v[0], fma(ct[3], v[1], ct[6] * v[2]));
         }
         s_rows64[cam * kRowD + q] = r;
     }
@@ -1845,7 +1849,6 @@ __global__ void __launch_bounds__(512, 1) backsub_slices64_kernel(Prob P, double
         for (int q = 0; q < 6; ++q) ci[q] = __ldg(Ci + (int64_t)q * P.np_pad + s);
         const double w0 = P.w[3 * pt], w1 = P.w[3 * pt + 1], w2 = P.w[3 * pt + 2];
         apply_sym3(ci, w0 - a[0], w1 - a[1], w2 - a[2], dp);
-        if (P.has_fixed && P.pt_fixed[pt]) dp[0] = dp[1] = dp[2] = 0.0;
         if (act && (lane & ((1 << lg) - 1)) == 0) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
@@ -1854,6 +1857,7 @@ __global__ void __launch_bounds__(512, 1) backsub_slices64_kernel(Prob P, double
             }
             ldec += w0 * dp[0] + w1 * dp[1] + w2 * dp[2];
         }
+        if (P.has_fixed && P.pt_fixed[pt]) dp[0] = dp[1] = dp[2] = 0.0;  // moves no pixel
         for (int k = 0; k < K; ++k) {
             const int64_t slot = (int64_t)sl.z + 32 * k + lane;
             const HgObs o = load_hg(P, slot);

@@ -41,7 +41,7 @@ __device__ __forceinline__ double own_row_lane(const Prob &P, int cam, double v,
     double r = 0.0;
 #pragma unroll
     for (int i = 0; i < 3; ++i) r = fma(__ldg(ct + 3 * i), __shfl_sync(0xffffffffu, v, (at + i) & 31), r);
-    return r;
+    return fixed_camera(P, cam) ? 0.0 : r;
 }
 
 // Camera rows in shared memory: row(z) + beta row(previous p) (first: row(z) and
@@ -60,7 +60,7 @@ __device__ void own_stage(const Prob &P, double *rows, double beta, bool first, 
     if (given) {
         for (int cam = threadIdx.x; cam < P.nc; cam += blockDim.x) {
             const double *ct = P.ctr64 + (int64_t)cam * kCtr, *v = given + (int64_t)cam * kVec;
-            const bool fixed = P.has_fixed && P.cam_fixed[cam];  // its Jacobian columns are zero
+            const bool fixed = fixed_camera(P, cam);
             for (int g = 0; g < 3; ++g)
                 for (int b = 0; b < 3; ++b) {
                     double x = 0.0;
@@ -83,8 +83,9 @@ __device__ void own_stage(const Prob &P, double *rows, double beta, bool first, 
     __syncthreads();
 }
 
-// b of the slice's points: a summed over the point's lanes, b = C~^-1 a (a = 0
-// for fixed points), written by the first lane of each point.
+// b of the slice's points: a summed over the point's lanes, b = C~^-1 a (zero for
+// fixed points, also where the right-hand side of an adjoint has an entry
+// there), written by the first lane of each point.
 template <typename T>
 __device__ __forceinline__ void own_store_b(const Prob &P, int s, int loc, const T *b, float *bs) {
     if constexpr (sizeof(T) == 4) {
@@ -224,7 +225,7 @@ __device__ void own_points(const Prob &P, const T *rows, float *bs, int blk, int
             }
         }
         if (in < count && (RHS || (lane & ((1 << lg) - 1)) == 0)) {
-            if (!RHS && P.has_fixed && P.pt_fixed[P.sp_pt[s]]) a[0] = a[1] = a[2] = T(0);
+            if (P.has_fixed && P.pt_fixed[P.sp_pt[s]]) a[0] = a[1] = a[2] = T(0);
             apply_sym3(ci, a[0], a[1], a[2], b);
             own_store_b<T>(P, s, (sl.y >> 8) + in, b, bs);
         }
@@ -463,7 +464,7 @@ __device__ void own_finalize(const Prob &P, int cb, int m, const OwnVec &V, doub
             if constexpr (sizeof(T) == 4) cs = fma((double)__ldg(P.ctr + (int64_t)cam * kCtr + 3 * a + b), raw, cs);
             else cs = fma(__ldg(P.ctr64 + (int64_t)cam * kCtr + 3 * a + b), raw, cs);
         }
-        if (P.has_fixed && P.cam_fixed[cam]) cs = 0.0;  // its Jacobian columns are zero
+        if (fixed_camera(P, cam)) cs = 0.0;
         // the vector of the row product: g = v - c (right-hand side) or p
         const double x = MODE == CAM_RHS ? pv - cs : pv;
         double y = r0 * __shfl_sync(full, x, 3 * th);

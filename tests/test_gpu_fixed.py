@@ -127,3 +127,58 @@ def test_graph_fixed_nodes_equal_the_array_masks(mba):
     assert s1["final_cost"] == s2["final_cost"]
     np.testing.assert_array_equal(c1, c2)
     np.testing.assert_array_equal(p1, p2)
+
+
+def _damped_solve(sc, cf, pf, mu, gc, gp, loss):
+    """v = M^-1 gbar with M = J^T W J + mu D over all parameters, the Jacobian's
+    columns of fixed nodes zero, by conjugate gradients on D^-1/2 M D^-1/2 (its
+    spectrum lies in [mu, mu + track length + 9]): W J v, mu D v."""
+    import scipy.sparse as sp
+    from scipy.sparse.linalg import LinearOperator, cg
+
+    _, _, Jc, Jp, W = oracle.evaluate(sc.cameras, sc.points, sc.observations, sc.cam_idx, sc.pt_idx, loss=loss,
+                                      delta=2.0)
+    Jc, Jp = Jc * ~cf[sc.cam_idx][:, None, None], Jp * ~pf[sc.pt_idx][:, None, None]
+    row = np.repeat(np.arange(2 * sc.n), 12).reshape(sc.n, 2, 12)
+    col = np.concatenate([9 * sc.cam_idx[:, None].astype(np.int64) + np.arange(9),
+                          9 * sc.nc + 3 * sc.pt_idx[:, None].astype(np.int64) + np.arange(3)], 1)
+    col = np.repeat(col[:, None, :], 2, 1)
+    m = 9 * sc.nc + 3 * sc.np_
+    J = sp.csr_matrix((np.concatenate([Jc, Jp], 2).ravel(), (row.ravel(), col.ravel())), shape=(2 * sc.n, m))
+    w2 = np.repeat(W, 2)
+    D = np.clip(np.asarray(J.multiply(J).T @ w2).ravel(), 1e-6, 1e32)
+    s = 1 / np.sqrt(D)
+    op = LinearOperator((m, m), matvec=lambda x: s * (J.T @ (w2 * (J @ (s * x)))) + mu * x)
+    g = np.concatenate([gc.ravel(), gp.ravel()])
+    # fixed nodes stand alone: M = mu D there
+    free = ~np.concatenate([np.repeat(cf, 9), np.repeat(pf, 3)])
+    x, info = cg(op, np.where(free, s * g, 0.0), rtol=1e-13, maxiter=5000)
+    assert info == 0
+    v = s * x
+    x0 = np.where(free, mu * D * v, g)
+    return (w2 * (J @ v)).reshape(sc.n, 2), x0[:9 * sc.nc].reshape(-1, 9), x0[9 * sc.nc:].reshape(-1, 3)
+
+
+# the block-owned products, the gathered FP32 and the stored FP64 one, dual numbers
+@pytest.mark.parametrize("variant", ["standard", "single_reduction"])
+@pytest.mark.parametrize("nc,npts,precision,jacobian,loss", [
+    (12, 300, "fp64", "analytic", "none"), (12, 300, "fp32", "analytic", "none"), (140, 9000, "fp64", "analytic", "huber"),
+    (140, 9000, "fp32", "analytic", "huber"), (2500, 6000, "fp32", "analytic", "none"),
+    (2500, 6000, "fp64", "analytic", "none"), (12, 300, "fp32", "autodiff", "none")])
+def test_adjoint_with_fixed_nodes(mba, nc, npts, precision, jacobian, loss, variant):
+    """The upstream gradient reaches fixed nodes too: they take it as it is
+    (mu D v = gbar) and pass nothing on to the others."""
+    sc = make_scene(nc, npts, track=("geom", 0.25), sigma=1.0, seed=77)
+    rng = np.random.default_rng(8)
+    cf, pf = rng.random(nc) < 0.25, rng.random(npts) < 0.25
+    gc, gp = rng.normal(size=(nc, 9)), rng.normal(size=(npts, 3))
+    mu = 0.3
+    with mba.Problem(sc.cameras, sc.points, sc.observations, sc.cam_idx, sc.pt_idx, precision=precision,
+                     jacobian=jacobian, loss=loss, huber_delta=2.0 if loss == "huber" else 0.0) as pr:
+        pr.set_fixed(cf, pf)
+        r = pr.adjoint(gc, gp, mu=mu, pcg_max_iter=1000, pcg_rel_tol=1e-14, pcg_variant=variant)
+    go, gc0, gp0 = _damped_solve(sc, cf, pf, mu, gc, gp, loss)
+    tol = 1e-7 if precision == "fp64" else 2e-3
+    rel_close(r["grad_obs"], go, tol, "grad_obs")
+    rel_close(r["grad_init_cam"], gc0, tol, "grad_init_cam")
+    rel_close(r["grad_init_pt"], gp0, tol, "grad_init_pt")
