@@ -591,7 +591,7 @@ def main():
 
         def batch_e2e():
             h = mba.mba_batch_create(co, po, oo, hb[0], hb[1], hb[2], hb[3], hb[4], precision="fp32", stream=stream)
-            mba.mba_batch_set_schedule(h, tune["threads_per_cta"], tune["ctas_per_sm"])
+            mba.mba_batch_set_schedule(h, tune["threads_per_cta"], tune["ctas_per_sm"], tune["schur"], tune["clusters"])
             mba.mba_batch_solve(h, gcb, gpb, adjoint_pcg_max_iter=500, adjoint_pcg_rel_tol=1e-10, **bopts)
             cv = mba.mba_batch_get_parameters(h)
             g = mba.mba_batch_get_gradients(h)
@@ -615,7 +615,7 @@ def main():
             "window_lm_iterations_per_s": sum(x["iterations"] for x in sm_b) / (t_full / 1e3),
             "pcg_iters_forward": pcg_b, "pcg_iters_adjoint": adj_b,
             "schedule": {"threads_per_cta": tune["threads_per_cta"], "ctas_per_sm": tune["ctas_per_sm"],
-                         "schur": tune["schur"], "autotune_ms": tune["ms"]},
+                         "schur": tune["schur"], "clusters": tune["clusters"], "autotune_ms": tune["ms"]},
             "launch": "one CUDA graph replay (claim-counter reset + one persistent kernel)",
             "gpu_launches": 1,
             "roofline": {"kernel": "batch_kernel (persistent, one window per CTA)", "bound": "alu",

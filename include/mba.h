@@ -357,13 +357,20 @@ typedef struct {
  * ctas_per_sm: resident windows per SM (1..4, capped by occupancy); schur: how
  * the PCG forms S p (Alg. 3): 1 = implicit (two passes over the observations
  * per iteration), 2 = explicit (S formed once per damped solve as 9x9 blocks,
- * then a dense product per iteration).  Zero fields choose automatically.  The
+ * then a dense product per iteration).  Zero fields choose automatically.
+ * clusters: 1 = a batch of fewer windows than the GPU has SMs gives each window a
+ * thread-block cluster of 256-thread CTAs where the explicit product and the
+ * standard PCG run (threads_per_cta and ctas_per_sm then hold for the other
+ * solves); 0 = never, unless threads_per_cta and ctas_per_sm are both zero.
+ * mba_batch_get_schedule and mba_batch_autotune fill every field: the schedule
+ * they give, set on a batch of the same windows, repeats its results.  The
  * schedule changes the rounding inside a window (results agree to rounding),
  * never the method; a given schedule gives the same bits on every run. */
 typedef struct {
     int32_t threads_per_cta;
     int32_t ctas_per_sm;
     int32_t schur;
+    int32_t clusters;
 } mba_batch_schedule;
 
 /* Upstream gradient for the adjoint of every window (same form as

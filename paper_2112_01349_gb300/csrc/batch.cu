@@ -2138,7 +2138,7 @@ struct mba_batch {
     int schur = 0;                  // schedule: 1 implicit, 2 explicit Schur product
     int sms = 0;
     int nt = 0, cps = 0;            // schedule in use
-    bool automatic = true;          // threads and CTAs per SM were left to the library
+    bool clusters = true;           // a cluster per window where the windows are few
     int g_cl = 0;                   // cluster size the graph was captured with (1: none)
     cudaGraphExec_t gexec = nullptr;
     int g_nt = 0, g_grid = 0, g_cps = 0;  // schedule the graph was captured with
@@ -2207,7 +2207,7 @@ int cluster_size(const mba_batch *b, const BatchOpts &o, int *rows, size_t *smem
     *rows = 0;
     *clusters_out = 0;
     *smem = 0;
-    if (!b->automatic || !b->explicit_ok || !o.explicit_schur || o.pcg_variant != MBA_PCG_STANDARD) return 1;
+    if (!b->clusters || !b->explicit_ok || !o.explicit_schur || o.pcg_variant != MBA_PCG_STANDARD) return 1;
     const void *k = cluster_kernel_ptr(b->fp32);
     int optin = 0, dev = 0;
     cudaGetDevice(&dev);
@@ -2663,12 +2663,13 @@ mba_status mba_batch_info(const mba_batch *b, int32_t *n_windows, int64_t *n_cam
 mba_status mba_batch_set_schedule(mba_batch *b, const mba_batch_schedule *sc) {
     if (!b || !sc) return api_fail(MBA_ERR_INVALID_ARG, "NULL argument");
     int nt = 0, cps = 0, schur = 0;
+    if (sc->clusters != 0 && sc->clusters != 1) return api_fail(MBA_ERR_INVALID_ARG, "clusters must be 0 or 1");
     mba_status st = resolve_schedule(b, sc->threads_per_cta, sc->ctas_per_sm, sc->schur, &nt, &cps, &schur);
     if (st != MBA_OK) return st;
     b->nt = nt;
     b->cps = cps;
     b->schur = schur;
-    b->automatic = sc->threads_per_cta == 0 && sc->ctas_per_sm == 0;
+    b->clusters = sc->clusters || (sc->threads_per_cta == 0 && sc->ctas_per_sm == 0);
     return MBA_OK;
 }
 
@@ -2677,6 +2678,7 @@ mba_status mba_batch_get_schedule(const mba_batch *b, mba_batch_schedule *sc) {
     sc->threads_per_cta = b->nt;
     sc->ctas_per_sm = b->cps;
     sc->schur = b->schur;
+    sc->clusters = b->clusters ? 1 : 0;
     return MBA_OK;
 }
 
@@ -2785,8 +2787,8 @@ mba_status mba_batch_autotune(mba_batch *b, const mba_solver_options *opt, mba_b
         if (st != MBA_OK && st != MBA_ERR_NONFINITE) return st;
     }
     const int nts[2] = {256, 512};
-    const bool auto0 = b->automatic;
-    bool bauto = false;
+    const bool clus0 = b->clusters;
+    bool bclus = false;
     // one timed solve; false on an error (in *err)
     auto timed = [&](mba_status *err, double *t) -> bool {
         mba_status st = mba_batch_solve(b, opt, nullptr, nullptr, t);
@@ -2806,7 +2808,7 @@ mba_status mba_batch_autotune(mba_batch *b, const mba_solver_options *opt, mba_b
         b->nt = nt0;
         b->cps = cps0;
         b->schur = sc0;
-        b->automatic = auto0;
+        b->clusters = clus0;
     };
     mba_status err = MBA_OK;
     // the automatic schedule where it gives each window a cluster, then every
@@ -2815,7 +2817,7 @@ mba_status mba_batch_autotune(mba_batch *b, const mba_solver_options *opt, mba_b
         b->nt = 256;
         b->cps = 1;
         b->schur = 2;
-        b->automatic = true;
+        b->clusters = true;
         double t = 0.0;
         if (!timed(&err, &t)) {
             restore();
@@ -2826,10 +2828,10 @@ mba_status mba_batch_autotune(mba_batch *b, const mba_solver_options *opt, mba_b
             bnt = 256;
             bcps = 1;
             bsc = 2;
-            bauto = true;
+            bclus = true;
         }
     }
-    b->automatic = false;
+    b->clusters = false;
     for (int sch = b->explicit_ok ? 2 : 1; sch >= 1; --sch)
     for (int a = 0; a < 2; ++a) {
         for (int c = 1; c <= kMaxCtasPerSm; ++c) {
@@ -2847,18 +2849,19 @@ mba_status mba_batch_autotune(mba_batch *b, const mba_solver_options *opt, mba_b
                 bnt = nts[a];
                 bcps = c;
                 bsc = sch;
-                bauto = false;
+                bclus = false;
             }
         }
     }
     b->nt = bnt;
     b->cps = bcps;
     b->schur = bsc;
-    b->automatic = bauto;
+    b->clusters = bclus;
     if (chosen) {
         chosen->threads_per_cta = bnt;
         chosen->ctas_per_sm = bcps;
         chosen->schur = bsc;
+        chosen->clusters = bclus ? 1 : 0;
     }
     if (ms_best) *ms_best = best;
     return MBA_OK;

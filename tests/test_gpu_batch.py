@@ -359,3 +359,28 @@ def test_windows_of_few_observations(mba, count, precision, tol, loss):
         rel_close(go[o], adj["grad_obs"], tol, f"window {w} observation gradient")
         rel_close(gc0[c], adj["grad_c0"], tol, f"window {w} camera gradient")
         rel_close(gp0[p], adj["grad_p0"], tol, f"window {w} point gradient")
+
+
+def test_a_schedule_can_be_applied_again(mba):
+    """set_schedule(schedule()) and set_schedule(autotune()) repeat the bits of the
+    batch that they were read from, in a new batch of the same windows."""
+    ws = make_windows(3, seed=21)
+    opts = dict(max_iter=3, pcg_max_iter=30, pcg_rel_tol=1e-10)
+
+    def solve(b):
+        b.reset()
+        b.solve(**opts)
+        return b.parameters()
+
+    with mba.Batch(_tuples(ws), precision="fp64") as b:
+        first = solve(b)
+        kept = b.schedule()
+        tuned = b.autotune(**opts)
+        tuned.pop("ms")
+        best = solve(b)
+        assert b.schedule() == tuned
+    for schedule, want in ((kept, first), (tuned, best)):
+        with mba.Batch(_tuples(ws), precision="fp64") as b:
+            b.set_schedule(**schedule)
+            for got, ref in zip(solve(b), want):
+                np.testing.assert_array_equal(got, ref)
