@@ -5,6 +5,8 @@
 #include <cstdio>
 #include <cstring>
 #include <atomic>
+#include <mutex>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -57,6 +59,23 @@ bool over_memory_limit(size_t bytes) {
 mba_status api_fail(mba_status st, const char *msg) {
     g_err = msg ? msg : "";
     return st;
+}
+
+cudaError_t allow_smem(const void *fn) {
+    static std::mutex mu;
+    static std::set<std::pair<int, const void *>> done;
+    int dev = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done.count({dev, fn})) return cudaSuccess;
+    cudaFuncAttributes at;
+    e = cudaFuncGetAttributes(&at, fn);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes);
+    if (e == cudaSuccess) done.insert({dev, fn});
+    return e;
 }
 }  // namespace mba
 

@@ -2165,7 +2165,7 @@ int max_ctas_per_sm(const mba_batch *b, int nt, int cps, bool s_smem = false) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (sm > (size_t)optin) return 0;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) return 0;
+    if (allow_smem(k) != cudaSuccess) return 0;
     int blocks = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k, nt, sm) != cudaSuccess) return 0;
     return blocks;
@@ -2213,7 +2213,7 @@ int cluster_size(const mba_batch *b, const BatchOpts &o, int *rows, size_t *smem
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     const size_t limit = (size_t)optin - 2048;  // static shared memory
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess || allow_smem(k) != cudaSuccess) {
         cudaGetLastError();
         return 1;
     }
@@ -2223,7 +2223,6 @@ int cluster_size(const mba_batch *b, const BatchOpts &o, int *rows, size_t *smem
         if (cluster_smem(b->fp32, b->ncmax, r) > limit) r = 0;
         const size_t sm = cluster_smem(b->fp32, b->ncmax, r);
         if (sm > limit) return 1;
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) break;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -2265,7 +2264,7 @@ mba_status build_graph(mba_batch *b, const BatchOpts &o) {
     }
     const void *k = cl > 1 ? cluster_kernel_ptr(b->fp32) : kernel_ptr(b->fp32, b->nt, b->cps);
     const size_t sm = cl > 1 ? csm : kernel_smem(b->fp32, b->nt, b->ncmax, ssm ? b->A.smax : 0);
-    BCK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    BCK(allow_smem(k));
     cudaGraph_t g = nullptr;
     BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e1 = cudaMemsetAsync(b->counter, 0, sizeof(int32_t), b->stream);

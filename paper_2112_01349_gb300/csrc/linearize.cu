@@ -1042,13 +1042,13 @@ cudaError_t launch_split_observations(const Prob &P, cudaStream_t s) {
 }
 
 template <typename T, bool AD>
-static void launch_lin_pair(const Prob &P, int force, cudaStream_t s) {
+static cudaError_t launch_lin_pair(const Prob &P, int force, cudaStream_t s) {
     if (!AD && P.n_slices > 0) {
         // one CTA per SM, with as many warps as there are slices for it
         const int smem = P.nc * (sizeof(T) == 4 ? kRowS * 4 : 15 * 8);
         const SliceGrid g = slice_grid(P, sizeof(T) == 4 ? 1024 : 512);
         if (smem <= 220 * 1024) {
-            cudaFuncSetAttribute(lin_slices_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (cudaError_t e = allow_smem((const void *)lin_slices_kernel<T, true>)) return e;
             lin_slices_kernel<T, true><<<g.ctas, g.threads, smem, s>>>(P, force);
         } else {
             lin_slices_kernel<T, false><<<g.ctas, g.threads, 0, s>>>(P, force);
@@ -1067,20 +1067,21 @@ static void launch_lin_pair(const Prob &P, int force, cudaStream_t s) {
         if (!AD && P.own) lin_camera64_kernel<<<nb, kBlock, 0, s>>>(P, force);
         else lin_camera_kernel<T, AD><<<nb, kBlock, 0, s>>>(P, force);
     }
+    return cudaGetLastError();
 }
 
 cudaError_t launch_linearize_impl(const Prob &P, const int32_t *cfirst, int force, cudaStream_t s) {
+    cudaError_t e;
     if (P.fp32) {
         point_table_kernel<<<grid_for(P.np), kBlock, 0, s>>>(P.pts, P.fact ? P.sp_pt : nullptr, P.np,
                                                              P.fact ? P.sp_X : P.pts32, P.st, force ? 0 : 1);
-        if (P.autodiff) launch_lin_pair<float, true>(P, force, s);
-        else launch_lin_pair<float, false>(P, force, s);
+        e = P.autodiff ? launch_lin_pair<float, true>(P, force, s) : launch_lin_pair<float, false>(P, force, s);
     } else {
         if (P.own)
             point_table64_kernel<<<grid_for(P.np), kBlock, 0, s>>>(P.pts, P.sp_pt, P.np, P.sp_X64, P.st, force ? 0 : 1);
-        if (P.autodiff) launch_lin_pair<double, true>(P, force, s);
-        else launch_lin_pair<double, false>(P, force, s);
+        e = P.autodiff ? launch_lin_pair<double, true>(P, force, s) : launch_lin_pair<double, false>(P, force, s);
     }
+    if (e != cudaSuccess) return e;
     if (P.fact) cam_finalize_raw_kernel<float><<<P.nc, 64, 0, s>>>(P, cfirst, force);
     else if (P.own) cam_finalize_raw_kernel<double><<<P.nc, 64, 0, s>>>(P, cfirst, force);
     else cam_finalize_kernel<<<grid_for((int64_t)P.nc * 54), kBlock, 0, s>>>(P, cfirst, force);
@@ -1100,7 +1101,7 @@ cudaError_t launch_cost_impl(const Prob &P, const double *pts, double *partial, 
         const int smem = P.nc * 15 * 8;
         SliceGrid g = slice_grid(P, 512);
         if (smem <= 220 * 1024) {
-            cudaFuncSetAttribute(cost_slices_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (cudaError_t e = allow_smem((const void *)cost_slices_kernel<true>)) return e;
             cost_slices_kernel<true><<<g.ctas, g.threads, smem, s>>>(P, pts, partial, gate);
         } else {
             g.ctas *= 2;

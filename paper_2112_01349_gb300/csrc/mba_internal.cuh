@@ -649,6 +649,12 @@ mba_status api_fail(mba_status st, const char *msg);
 // mba_set_device_memory_limit
 bool over_memory_limit(size_t bytes);
 
+// api.cu: lets launches of fn take as much dynamic shared memory as a CTA can have.
+// Done once per device and kernel: the limit belongs to the kernel, not to a
+// launch, so a size set per problem could be lowered by another thread before
+// this thread's launch.
+cudaError_t allow_smem(const void *fn);
+
 // lm.cu
 cudaError_t launch_state_init(const Prob &P, double radius, double mu_override, int keep_cost, cudaStream_t s);
 cudaError_t launch_lm_update(const Prob &P, const mba_solver_options &o, cudaStream_t s);

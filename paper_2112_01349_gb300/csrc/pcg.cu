@@ -1964,7 +1964,7 @@ static const void *pcg_fn(const Prob &P, int variant = MBA_PCG_STANDARD) {
 
 static int resident(const void *fn, int block, size_t smem) {
     int blocks = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    if (allow_smem(fn) != cudaSuccess) return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, block, smem) != cudaSuccess) return 0;
     return blocks;
 }
@@ -1990,8 +1990,7 @@ cudaError_t launch_pcg(const Prob &P, int mode, int max_iter, double tol, long l
     // the barrier targets count arrivals from zero in every launch
     cudaError_t e = cudaMemsetAsync(&P.st->barrier, 0, sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    // the shared-memory plan differs between problems, so the kernel's dynamic shared-memory limit is set for this launch
-    e = cudaFuncSetAttribute(pcg_fn(P, variant), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(pcg_fn(P, variant));
     if (e != cudaSuccess) return e;
     Prob Pc = P;
     void *args[] = {(void *)&Pc, (void *)&mode, (void *)&max_iter, (void *)&tol, (void *)&spin_limit, (void *)&forcing};
@@ -2004,7 +2003,7 @@ cudaError_t launch_backsub(const Prob &P, double *partial, int nb, cudaStream_t 
         const SliceGrid g = slice_grid(P);
         nb = g.ctas;
         if (smem <= 220 * 1024) {
-            cudaFuncSetAttribute(backsub_slices_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (cudaError_t e = allow_smem((const void *)backsub_slices_kernel<true>)) return e;
             backsub_slices_kernel<true><<<g.ctas, g.threads, smem, s>>>(P, partial);
         } else {
             fact_rows_kernel<<<(P.nc + 127) / 128, 128, 0, s>>>(P, P.x, (float *)P.pT);
@@ -2014,7 +2013,7 @@ cudaError_t launch_backsub(const Prob &P, double *partial, int nb, cudaStream_t 
         const int smem = P.nc * kRowD * 8;  // fits: the block-owned product holds the same rows
         const SliceGrid g = slice_grid(P, 512);
         nb = g.ctas;
-        cudaFuncSetAttribute(backsub_slices64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (cudaError_t e = allow_smem((const void *)backsub_slices64_kernel)) return e;
         backsub_slices64_kernel<<<g.ctas, g.threads, smem, s>>>(P, partial);
     } else if (P.fp32) {
         backsub_kernel<float><<<nb, kBlock, 0, s>>>(P, partial);

@@ -74,3 +74,37 @@ def test_invalid_solver_options_are_rejected(mba, bad):
         # the handle is still usable afterwards
         assert pr.solve(max_iter=2, pcg_max_iter=10)["status"] == 0
     assert np.isfinite(sc.cameras).all()
+
+
+def test_problems_of_different_sizes_in_two_threads(mba):
+    """Separate handles are independent: two threads, each with its own problem
+    (few and many cameras, so the kernels' shared memory differs), get what they
+    get alone."""
+    import threading
+
+    shapes = {"few": (12, 400), "many": (1500, 8000)}
+    out, errors = {}, []
+
+    def work(name, rounds):
+        try:
+            sc = make_scene(*shapes[name], sigma=0.5, seed=54)
+            for precision in ("fp32", "fp64"):
+                with mba.Problem(sc.cameras, sc.points, sc.observations, sc.cam_idx, sc.pt_idx, precision=precision) as pr:
+                    got = []
+                    for _ in range(rounds):
+                        pr.reset()
+                        got.append(pr.solve(max_iter=3, pcg_max_iter=5, initial_radius=10.0)["final_cost"])
+                assert len(set(got)) == 1
+                out.setdefault((name, precision), set()).add(got[0])
+        except Exception as e:  # noqa: BLE001 - reported by the main thread
+            errors.append((name, repr(e)))
+
+    for name in shapes:
+        work(name, 1)
+    threads = [threading.Thread(target=work, args=(name, 300)) for name in shapes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    assert all(len(v) == 1 for v in out.values()), out
