@@ -24,6 +24,8 @@ constexpr int kRowD = 10;            // doubles per camera row of the block-owne
 constexpr int kPartF = 12, kPartD = 10;  // stride of a camera's nine partial sums (FP32, FP64), for 16-byte stores
 constexpr int kOwnSmem = 225 * 1024; // dynamic shared memory the block-owned PCG kernel may use
 constexpr int kMaxParts = 16;        // parts a camera's run may be split into
+constexpr int kRunRounds = 32;       // rounds of a run slice, at most, unless its runs have a warp each
+constexpr int kRunLg = 28, kRunMask = (1 << kRunLg) - 1;  // a run slice's word: rounds | log2 of the lanes per run << kRunLg
 constexpr int kCtr = 28;             // stride of a camera's 9 x 3 row transform (27 values)
 constexpr int kCamStat = 12;         // per camera: f, k1, k2, the quaternion of R times sqrt 2 (w, x, y, z), t (3), pad
 constexpr int kCamChunk = 256;       // observations per camera-major chunk (at least)
@@ -125,11 +127,11 @@ struct Prob {
     int32_t own, nblk, n_vblk;  // blocks; rows of partial sums (blocks x parts)
     int32_t own_pb;         // points of a block, at most (the stride of b in shared memory)
     int32_t own_off_b, own_off_dots;  // byte offsets in the kernel's dynamic shared memory
-    int32_t r_lg;           // log2 of the lanes per run
+    int32_t long_runs;      // 1: some slice has more than kRunRounds rounds
     int64_t rslot_cap;
-    int2 *rslice;           // per run slice: (first slot, rounds)
+    int2 *rslice;           // per run slice: (first slot, rounds | log2 of the lanes per run << kRunLg)
     int2 *rlane;            // [run slices][32]: (camera or -1, row of the partial sums)
-    int32_t *blk_rslice;    // nblk + 1
+    int4 *blk_run;          // per block: its first run slice, the first of at most kRunRounds rounds, its end
     int32_t *cm2r;          // camera-major position -> run slot
     float4 *r_rx;           // FP32: [run slots] (R X, 1 / P_z)
     uint16_t *r_pt16;       // FP32: the point's index in its block, 0xffff in padding

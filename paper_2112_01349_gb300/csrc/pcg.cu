@@ -1954,7 +1954,8 @@ int pcg_block(const Prob &P) { return P.fp32 ? PcgBlock<float>::value : PcgBlock
 
 template <bool SR>
 static const void *pcg_fn_v(const Prob &P) {
-    if (P.own) return P.fp32 ? (const void *)pcg_own_kernel<float, SR> : (const void *)pcg_own_kernel<double, SR>;
+    if (P.own && !P.fp32) return (const void *)pcg_own_kernel<double, SR, false>;
+    if (P.own) return P.long_runs ? (const void *)pcg_own_kernel<float, SR, true> : (const void *)pcg_own_kernel<float, SR, false>;
     if (!P.fp32) return (const void *)pcg_kernel<double, true, SR>;
     return P.autodiff ? (const void *)pcg_kernel<float, true, SR> : (const void *)pcg_kernel<float, false, SR>;
 }

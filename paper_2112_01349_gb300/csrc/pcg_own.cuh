@@ -238,13 +238,14 @@ __device__ void own_points(const Prob &P, const T *rows, float *bs, int blk, int
 // The layout words of a warp's first run slice: loaded before the barrier that
 // publishes b, so that their latency overlaps it.
 struct RunBegin {
-    int j, j0, j1;
+    int j, j0, j1;  // the warp's slice; the block's first (FP32: after the long runs) and end
     int2 rs, ln;
 };
+template <typename T>
 __device__ __forceinline__ RunBegin own_cameras_begin(const Prob &P, int blk) {
     RunBegin rb;
-    rb.j0 = __ldg(P.blk_rslice + blk);
-    rb.j1 = __ldg(P.blk_rslice + blk + 1);
+    const int4 b = __ldg(P.blk_run + blk);
+    rb.j0 = sizeof(T) == 4 ? b.y : b.x, rb.j1 = b.z;
     rb.j = rb.j0 + (threadIdx.x >> 5);
     rb.rs = rb.ln = make_int2(0, 0);
     if (rb.j < rb.j1) {
@@ -254,10 +255,72 @@ __device__ __forceinline__ RunBegin own_cameras_begin(const Prob &P, int blk) {
     return rb;
 }
 
+// The sums over a run's G lanes into the block's row of the partials, or onto what
+// the run's earlier rounds left there.
+__device__ __forceinline__ void own_store_sums(const Prob &P, int2 ln, int G, bool add, float *acc) {
+    for (int d = 1; d < G; d <<= 1) {
+#pragma unroll
+        for (int a = 0; a < 9; ++a) acc[a] += __shfl_xor_sync(0xffffffffu, acc[a], d);
+    }
+    if (ln.x < 0 || (threadIdx.x & (G - 1))) return;
+    float4 *o = (float4 *)((float *)P.c_part + ((int64_t)ln.y * P.nc + ln.x) * kPartF);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        float4 v = make_float4(acc[4 * a], acc[4 * a + 1], acc[4 * a + 2], acc[4 * a + 3]);
+        if (add) {
+            const float4 u = __ldcg(o + a);
+            v = make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w);
+        }
+        __stcg(o + a, v);
+    }
+}
+__device__ __forceinline__ CamConst own_cam_const(const float *rows, int cam) {
+    const float *row = rows + (cam < 0 ? 0 : cam) * kRowS;
+    const float4 c = ((const float4 *)row)[2], q = ((const float4 *)row)[3];
+    const float2 t = ((const float2 *)row)[8];
+    CamConst ct;
+    ct.f = c.y, ct.k1 = c.z, ct.k2 = c.w, ct.t0 = t.x, ct.t1 = t.y;
+    ct.q0 = q.x, ct.q1 = q.y, ct.q2 = q.z, ct.q3 = q.w;
+    return ct;
+}
+
+// Runs of more than kRunRounds rounds (a warp each): that many rounds at a time,
+// added up in the block's row, so that no FP32 sum grows longer.  In kernel
+// instances of its own (LONG): its registers cost the others 2 % of an iteration.
+__device__ __forceinline__ void own_long_runs(const Prob &P, const float *rows, const float *bs, int blk) {
+    const int lane = threadIdx.x & 31, pb = P.own_pb;
+    const int4 b = __ldg(P.blk_run + blk);
+    for (int j = b.x + (threadIdx.x >> 5); j < b.y; j += blockDim.x >> 5) {
+        const int2 rs = __ldg(P.rslice + j), ln = __ldg(P.rlane + 32 * (int64_t)j + lane);
+        const int K = rs.y & kRunMask;
+#pragma unroll 1
+        for (int k0 = 0; k0 < K; k0 += kRunRounds) {
+            const CamConst ct = own_cam_const(rows, ln.x);
+            float acc[12];
+#pragma unroll
+            for (int a = 0; a < 12; ++a) acc[a] = 0.f;
+            const int k1 = min(K, k0 + kRunRounds);
+#pragma unroll 1
+            for (int k = k0; k < k1; ++k) {
+                const int64_t slot = (int64_t)rs.x + 32 * k + lane;
+                const int p = __ldg(P.r_pt16 + slot);
+                if (p != 0xffff)
+                    fact_camera_obs(ct, __ldg(P.r_rx + slot), make_float4(bs[p], bs[pb + p], bs[2 * pb + p], 0.f),
+                                    P.r_w ? __ldg(P.r_w + slot) : 1.f, acc);
+            }
+            own_store_sums(P, ln, 32, k0 > 0, acc);
+        }
+    }
+}
+
 // Camera pass of one block: every run's nine raw sums into the block's partials.
-__device__ void own_cameras(const Prob &P, const float *rows, const float *bs, int *next, const RunBegin &rb) {
+// LONG: some blocks have runs of more than kRunRounds rounds.  600 cameras, 500k observations, one camera with 5 % of them, against as many
+// lanes for every run: FP64 338 -> 102 us per PCG iteration, FP32 35 -> 28; with
+// 25 %, 745 -> 93 and 57 -> 26.
+template <bool LONG>
+__device__ void own_cameras(const Prob &P, const float *rows, const float *bs, int *next, const RunBegin &rb, int blk) {
     const int lane = threadIdx.x & 31;
-    const unsigned full = 0xffffffffu;
+    if constexpr (LONG) own_long_runs(P, rows, bs, blk);
     const int j1 = rb.j1, pb = P.own_pb;
     int jn = 0;
     int2 rs = rb.rs, ln = rb.ln;
@@ -267,26 +330,19 @@ __device__ void own_cameras(const Prob &P, const float *rows, const float *bs, i
         // the warp's next slice goes to L2 while this one is worked
         const int2 nx = __ldg(P.rslice + (jn < j1 ? jn : j));
         const int64_t pf = nx.x;
-        const int pk = nx.y;
+        const int pk = nx.y & kRunMask, K = rs.y & kRunMask;
         int64_t slot = (int64_t)rs.x + lane;
         float4 Xn = __ldg(P.r_rx + slot);
         int pn = __ldg(P.r_pt16 + slot);
-        CamConst ct;
-        {
-            const float *row = rows + (ln.x < 0 ? 0 : ln.x) * kRowS;
-            const float4 c = ((const float4 *)row)[2], q = ((const float4 *)row)[3];
-            const float2 t = ((const float2 *)row)[8];
-            ct.f = c.y, ct.k1 = c.z, ct.k2 = c.w, ct.t0 = t.x, ct.t1 = t.y;
-            ct.q0 = q.x, ct.q1 = q.y, ct.q2 = q.z, ct.q3 = q.w;
-        }
+        const CamConst ct = own_cam_const(rows, ln.x);
         float acc[12];
 #pragma unroll
         for (int a = 0; a < 12; ++a) acc[a] = 0.f;
-        for (int k = 0; k < rs.y; ++k, slot += 32) {
+        for (int k = 0; k < K; ++k, slot += 32) {
             const float4 X = Xn;
             const int p = pn;
             prefetch_l2(P.r_rx + pf + 32 * (k < pk ? k : 0) + lane);
-            if (k + 1 < rs.y) {
+            if (k + 1 < K) {
                 Xn = __ldg(P.r_rx + slot + 32);
                 pn = __ldg(P.r_pt16 + slot + 32);
             }
@@ -294,16 +350,7 @@ __device__ void own_cameras(const Prob &P, const float *rows, const float *bs, i
                 fact_camera_obs(ct, X, make_float4(bs[p], bs[pb + p], bs[2 * pb + p], 0.f),
                                 P.r_w ? __ldg(P.r_w + slot) : 1.f, acc);
         }
-        for (int d = 1; d < (1 << P.r_lg); d <<= 1) {
-#pragma unroll
-            for (int a = 0; a < 9; ++a) acc[a] += __shfl_xor_sync(full, acc[a], d);
-        }
-        if (ln.x >= 0 && (lane & ((1 << P.r_lg) - 1)) == 0) {
-            float4 *o = (float4 *)((float *)P.c_part + ((int64_t)ln.y * P.nc + ln.x) * kPartF);
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-                __stcg(o + a, make_float4(acc[4 * a], acc[4 * a + 1], acc[4 * a + 2], acc[4 * a + 3]));
-        }
+        own_store_sums(P, ln, 1 << (rs.y >> kRunLg), false, acc);
     }
 }
 // One observation of an FP64 run: H, g, r2 and its point's X and b (b written by
@@ -322,7 +369,8 @@ struct RunObs {
         load_hg(P.r_hg + slot, P.rslot_cap, h);
     }
 };
-__device__ void own_cameras(const Prob &P, const double *rows, const float *, int *next, const RunBegin &rb) {
+template <bool LONG>
+__device__ void own_cameras(const Prob &P, const double *rows, const float *, int *next, const RunBegin &rb, int) {
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
     const int j1 = rb.j1;
@@ -338,15 +386,16 @@ __device__ void own_cameras(const Prob &P, const double *rows, const float *, in
         for (int a = 0; a < 10; ++a) acc[a] = 0.0;
         // the next round's values are in flight while one is worked, the point
         // index another round ahead
+        const int K = rs.y & kRunMask;
         int64_t slot = (int64_t)rs.x + lane;
         RunObs nxt;
         nxt.load(P, __ldg(P.r_pt + slot), slot);
-        int p2 = rs.y > 1 ? __ldg(P.r_pt + slot + 32) : -1;
-        for (int k = 0; k < rs.y; ++k, slot += 32) {
+        int p2 = K > 1 ? __ldg(P.r_pt + slot + 32) : -1;
+        for (int k = 0; k < K; ++k, slot += 32) {
             const RunObs c = nxt;
-            if (k + 1 < rs.y) {
+            if (k + 1 < K) {
                 nxt.load(P, p2, slot + 32);
-                p2 = k + 2 < rs.y ? __ldg(P.r_pt + slot + 64) : -1;
+                p2 = k + 2 < K ? __ldg(P.r_pt + slot + 64) : -1;
             }
             if (c.p < 0) continue;
             const double *h = c.h;
@@ -369,11 +418,12 @@ __device__ void own_cameras(const Prob &P, const double *rows, const float *, in
             acc[1] = fma(c.X2, v0, fma(-c.X0, v2, acc[1]));
             acc[2] = fma(c.X0, v1, fma(-c.X1, v0, acc[2]));
         }
-        for (int d = 1; d < (1 << P.r_lg); d <<= 1) {
+        const int G = 1 << (rs.y >> kRunLg);
+        for (int d = 1; d < G; d <<= 1) {
 #pragma unroll
             for (int a = 0; a < 9; ++a) acc[a] += __shfl_xor_sync(full, acc[a], d);
         }
-        if (ln.x >= 0 && (lane & ((1 << P.r_lg) - 1)) == 0) {
+        if (ln.x >= 0 && (lane & (G - 1)) == 0) {
             double2 *o = (double2 *)((double *)P.c_part + ((int64_t)ln.y * P.nc + ln.x) * kPartD);
 #pragma unroll
             for (int a = 0; a < 5; ++a) __stcg(o + a, make_double2(acc[2 * a], acc[2 * a + 1]));
@@ -521,7 +571,7 @@ __device__ __forceinline__ double own_precond(const double *b, double rv, int th
 // (barriers and dependent sums).  FP64, 5.0M observations 747 -> 449 us (point side
 // 179, camera side 224: the FP64 pipe), 780k 156 -> 105, 250k 63 -> 53, 10k
 // 37 -> 18.6.
-template <typename T, bool SR>
+template <typename T, bool SR, bool LONG>
 __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
     pcg_own_kernel(Prob P, int mode, int max_iter, double tol, long long spin, int forcing) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -547,10 +597,10 @@ __global__ void __launch_bounds__(PcgBlock<T>::value, 1)
     auto product = [&](auto rhs) {
         for (int blk = blockIdx.x; blk < P.nblk; blk += G) {
             own_points<T, decltype(rhs)::value>(P, rows, bs, blk, s_next);
-            const RunBegin rb = own_cameras_begin(P, blk);
+            const RunBegin rb = own_cameras_begin<T>(P, blk);
             __syncthreads();
             if (threadIdx.x == 0) s_next[0] = nwarp;
-            own_cameras(P, rows, bs, s_next + 1, rb);
+            own_cameras<LONG>(P, rows, bs, s_next + 1, rb, blk);
             __syncthreads();
             if (threadIdx.x == 0) s_next[1] = nwarp;
         }

@@ -147,3 +147,40 @@ def test_clusters_agree_with_one_cta_per_window(mba, count, cams, precision, tol
     rel_close(p1[1], p2[1], tol, "points")
     for k in ("grad_obs", "grad_init_cam", "grad_init_pt"):
         rel_close(g1[k], g2[k], 100 * tol if precision == "fp64" else 3e-2, k)
+
+
+@pytest.mark.parametrize("loss", ["none", "huber"])
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-9), ("fp32", 1e-4)])
+@pytest.mark.parametrize("nc,npts", [(40, 9000), (300, 60_000), (300, 200_000)])
+def test_a_camera_that_sees_every_point(mba, nc, npts, precision, tol, loss):
+    """One camera with far longer runs than the others: a warp per run, and (FP32)
+    runs of more than 32 rounds.  The layout does not grow with the longest run: a
+    block pads one slice of 32 slots to at most 32 rounds (84 bytes per slot in
+    FP64, 152 blocks).  Tolerances as above."""
+    plain = make_scene(nc, npts, track=("fixed", 2), sigma=0.5, seed=9)
+    # the first observation of every point not yet seen by camera 0 moves there
+    cam = plain.cam_idx.copy()
+    _, first = np.unique(plain.pt_idx, return_index=True)
+    seen = np.zeros(npts, bool)
+    seen[plain.pt_idx[cam == 0]] = True
+    move = first[~seen]
+    cam[move] = 0
+    assert np.bincount(cam, minlength=nc).min() > 0
+    true = oracle.evaluate(plain.cameras_true, plain.points_true, np.zeros((plain.n, 2)), cam, plain.pt_idx,
+                           jacobians=False)[1]
+    uv = true + np.random.default_rng(4).normal(size=true.shape)
+    args = (plain.cameras, plain.points, uv, cam, plain.pt_idx)
+    x = np.random.default_rng(5).normal(size=(nc, 9))
+    opts = dict(precision=precision, loss=loss, huber_delta=2.0 if loss == "huber" else 0.0)
+    with mba.Problem(*_args(plain), **opts) as pr:
+        size = pr.info["device_bytes"]
+    with mba.Problem(*args, **opts) as pr:
+        assert pr.info["device_bytes"] < 1.1 * size + 152 * 32 * 32 * 84
+        y = pr.schur_matvec(0.1, x)
+        st = pr.step(0.1, pcg_max_iter=6, pcg_rel_tol=0.0)
+    rel_close(y, oracle.schur(*args, 0.1, x=x.reshape(-1), loss=loss, delta=2.0)["y"].reshape(-1, 9), tol, "S x")
+    rs = oracle.step(*args, 0.1, pcg_max=6, pcg_tol=0.0, loss=loss, delta=2.0)
+    stol = 1e-6 if precision == "fp64" else 2e-3
+    for a in range(9):
+        rel_close(st["dc"][:, a], rs["dc"].reshape(-1, 9)[:, a], stol, f"dc[{a}]")
+    rel_close(st["dp"], rs["dp"].reshape(-1, 3), stol, "dp")
