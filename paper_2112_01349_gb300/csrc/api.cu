@@ -84,8 +84,7 @@ struct mba_problem {
     cudaStream_t stream = nullptr;
     void *pool = nullptr;
     size_t pool_bytes = 0;
-    void *pool2 = nullptr;          // arrays whose layout depends on the sorted observations
-    size_t pool2_bytes = 0;
+    char *late = nullptr;           // arrays whose layout depends on the sorted observations
     int32_t *cfirst = nullptr;      // per camera first chunk (device)
     int32_t *orig_cam = nullptr, *orig_pt = nullptr;
     double2 *orig_uv = nullptr;
@@ -153,7 +152,6 @@ void mba_problem_destroy(mba_problem *pr) {
     if (!pr) return;
     if (pr->stream) cudaStreamSynchronize(pr->stream);
     if (pr->pool) cudaFree(pr->pool);
-    if (pr->pool2) cudaFree(pr->pool2);
     delete pr;
 }
 
@@ -215,6 +213,7 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
     const bool stored = !P.fact && !P.own;  // the PCG reads a stored Jacobian
     const int red_len = 3 * 8192;
     const int64_t stage = n < kEvalSlice ? n : kEvalSlice;
+    const size_t late_bytes = own_pool_bytes(P, sms);
 
     auto layout = [&](Carve &c) {
         P.cams = c.take<double>(9 * (size_t)nc);
@@ -305,6 +304,7 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
         P.st = c.take<DevState>(1);
         pr->trace_dev = c.take<mba_iteration>(kTraceCap);
         pr->eval_stage = c.take<double>(26 * (size_t)stage);
+        pr->late = c.take<char>(late_bytes);
     };
     Carve sizing;
     layout(sizing);
@@ -312,13 +312,11 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
     P.red_len = red_len;
     // scratch of the sorts; the sliced order reuses it once the observations are sorted
     size_t sort_tmp = std::max(stable_sort_tmp_bytes(n, np > nc ? np : nc), sell_tmp_bytes(np));
-    if (P.own) sort_tmp = std::max(sort_tmp, own_tmp_bytes(P, 4 * (int64_t)sms));
+    if (P.own) sort_tmp = std::max(sort_tmp, own_tmp_bytes(P, sms));
     sort_tmp = al(sort_tmp);  // the observations follow it
     const size_t setup_bytes = sort_tmp + al(sizeof(double) * 2 * (size_t)n) + 256;
-    // the second pool's size is known after the sorts: about its share per observation here
-    const size_t later = P.own ? (P.fp32 ? 24 : 92) * (size_t)n : (P.fact ? 20 * (size_t)n + 16 * (size_t)np : 0);
-    if (mba::over_memory_limit(pr->pool_bytes + later + setup_bytes)) {
-        const size_t need = pr->pool_bytes + later + setup_bytes;
+    if (mba::over_memory_limit(pr->pool_bytes + setup_bytes)) {
+        const size_t need = pr->pool_bytes + setup_bytes;
         delete pr;
         return fail(MBA_ERR_OOM, "device memory limit: creation needs " + std::to_string(need) + " bytes");
     }
@@ -396,30 +394,9 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
     // padding slots are never written: camera -1, all bits set
     if (P.sl_px) CKC(cudaMemsetAsync(P.sl_px, 0xff, sizeof(float4) * (size_t)P.nslots, s));
     if (!P.own && !P.fact && P.sorted) return cleanup_fail(MBA_ERR_INVALID_ARG, "internal: block-owned layout");
-    if (P.own) {
-        const cudaError_t e = build_own(P, tmp, sort_tmp, &pr->pool2, &pr->pool2_bytes, s);
-        if (e == cudaErrorMemoryAllocation) {
-            cudaGetLastError();
-            return cleanup_fail(MBA_ERR_OOM, "device memory for " + std::to_string(pr->pool2_bytes) + " bytes of run layout");
-        }
-        CKC(e);
-    } else if (P.fact) {  // the gathered product's arrays
-        const bool lossy = o.loss != MBA_LOSS_NONE;
-        auto layout2 = [&](Carve &c) {
-            P.RXcm = c.take<float4>((size_t)n);
-            P.sp_b = c.take<float4>((size_t)np);
-            P.cm_w = lossy ? c.take<float>((size_t)n) : nullptr;
-        };
-        Carve size2, real2;
-        layout2(size2);
-        pr->pool2_bytes = size2.off;
-        if (mba::over_memory_limit(pr->pool_bytes + size2.off) || cudaMalloc(&pr->pool2, size2.off) != cudaSuccess) {
-            cudaGetLastError();
-            return cleanup_fail(MBA_ERR_OOM, "device memory for " + std::to_string(size2.off) + " bytes");
-        }
-        real2.base = (char *)pr->pool2;
-        layout2(real2);
-    }
+    int32_t *run_flag = flags + 3;
+    if (P.own) CKC(build_own(P, tmp, sort_tmp, pr->late, late_bytes, run_flag, s));
+    else if (P.fact) gathered_arrays(P, pr->late);
 
     // PCG camera partition: one group of whole cameras per CTA (one CTA per SM),
     // cut at the camera boundaries nearest to equal observation counts; then
@@ -502,7 +479,10 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
     CKC(cudaMemsetAsync(P.st, 0, sizeof(DevState), s));
     if (P.J) CKC(cudaMemsetAsync(P.J, 0, 24 * (size_t)P.npad * w, s));
     if (P.res) CKC(cudaMemsetAsync(P.res, 0, 2 * (size_t)P.npad * w, s));
+    if (P.own) CKC(cudaMemcpyAsync(hflags, run_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     CKC(cudaStreamSynchronize(s));
+    if (P.own && (hflags[0] & 2)) return cleanup_fail(MBA_ERR_INVALID_ARG, "internal: run layout");
+    P.long_runs = P.own ? hflags[0] & 1 : 0;
     cudaFree(tmp);
 #undef CKC
     plan_pcg_smem(P);
@@ -526,7 +506,7 @@ mba_status mba_problem_info(const mba_problem *pr, int32_t *nc, int32_t *np, int
     if (nc) *nc = pr->P.nc;
     if (np) *np = pr->P.np;
     if (n) *n = pr->P.n;
-    if (bytes) *bytes = pr->pool_bytes + pr->pool2_bytes;
+    if (bytes) *bytes = pr->pool_bytes;
     return MBA_OK;
 }
 

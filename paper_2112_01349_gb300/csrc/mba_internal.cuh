@@ -24,6 +24,7 @@ constexpr int kRowD = 10;            // doubles per camera row of the block-owne
 constexpr int kPartF = 12, kPartD = 10;  // stride of a camera's nine partial sums (FP32, FP64), for 16-byte stores
 constexpr int kOwnSmem = 225 * 1024; // dynamic shared memory the block-owned PCG kernel may use
 constexpr int kMaxParts = 16;        // parts a camera's run may be split into
+constexpr int kMaxBlocks = 4;        // blocks per CTA
 constexpr int kRunRounds = 32;       // rounds of a run slice, at most, unless its runs have a warp each
 constexpr int kRunLg = 28, kRunMask = (1 << kRunLg) - 1;  // a run slice's word: rounds | log2 of the lanes per run << kRunLg
 constexpr int kCtr = 28;             // stride of a camera's 9 x 3 row transform (27 values)
@@ -600,10 +601,14 @@ cudaError_t build_pm2cm(Prob &P, int32_t *tmp_n, cudaStream_t s);
 int64_t sell_slot_bound(int64_t n, int32_t np);
 int64_t sell_slice_bound(int64_t n, int32_t np);
 size_t sell_tmp_bytes(int32_t np);
+int64_t sell_block_points(int64_t n, int32_t np, int64_t nblk);
 // own.cu: the block-owned layout
 bool own_wanted(const Prob &P, int grid);
-size_t own_tmp_bytes(const Prob &P, int64_t nblk);
-cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void **pool, size_t *pool_bytes, cudaStream_t s);
+bool own_fits(Prob &P, int grid, int m, int64_t pb);
+size_t own_pool_bytes(const Prob &P, int grid);
+size_t own_tmp_bytes(const Prob &P, int grid);
+size_t gathered_arrays(Prob &P, char *base);
+cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void *pool, size_t pool_bytes, int32_t *flag, cudaStream_t s);
 // launch shape of a kernel that works whole slices per warp, one CTA per SM
 struct SliceGrid {
     int ctas, threads;

@@ -11,14 +11,12 @@
 // owner adds in block order.  Cameras with long runs (few cameras) are split
 // into parts, each with its own row.
 //
-// G is one number for most slices (lg in build_own).  A slice whose first (longest) run
+// G is one number for most slices (OwnPlan).  A slice whose first (longest) run
 // would take more than kRunRounds rounds takes more lanes per run, up to a whole
 // warp: a camera that sees far more points than the others would otherwise pad
 // its 32 / G - 1 neighbours to its own length and keep one warp busy long after
-// the others.  600 cameras, 500k observations, 5 % of them in one camera:
-// see own_cameras for the times.
+// the others (see own_cameras for the times).
 #include <algorithm>
-#include <vector>
 
 #include "mba_internal.cuh"
 
@@ -61,7 +59,8 @@ __global__ void run_key_kernel(const int32_t *__restrict__ ord, const int32_t *_
 
 __global__ void fill_runs_kernel(Prob P, const int32_t *__restrict__ ord, const int32_t *__restrict__ run,
                                  const int32_t *__restrict__ run_ptr, const int2 *__restrict__ base, int parts,
-                                 const int2 *__restrict__ sp_bl) {
+                                 const int2 *__restrict__ sp_bl, const int32_t *__restrict__ flag) {
+    if (*flag & 2) return;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < P.n; t += (int64_t)gridDim.x * blockDim.x) {
         const int s = ord[t], r = run[t], k = (int)(t - run_ptr[r]);
         const int part = k % parts, kk = k / parts;
@@ -152,8 +151,9 @@ constexpr int kBlockSlices = 4096;  // a block has no more (camera, part) pairs
 __global__ void __launch_bounds__(256) run_slices_kernel(Prob P, const unsigned long long *__restrict__ sorted,
                                                          const int2 *__restrict__ cut,
                                                          const int32_t *__restrict__ round0, int parts,
-                                                         int2 *__restrict__ base) {
+                                                         int2 *__restrict__ base, const int32_t *__restrict__ flag) {
     __shared__ int s_start[kBlockSlices];
+    if (*flag & 2) return;
     const int b = blockIdx.x, items = P.nc * parts;
     const int first = P.blk_run[b].x, nsl = P.blk_run[b].z - first;
     const unsigned long long *key = sorted + (int64_t)b * items;
@@ -194,7 +194,134 @@ inline unsigned grid_for(int64_t n) {
 
 size_t al256(size_t v) { return (v + 255) & ~size_t(255); }
 
+// First slice and round of every block (one CTA, any number of blocks).  flag: bit 0
+// some slice has more than kRunRounds rounds, bit 1 the arrays are too small (their
+// size is a bound, so this does not happen; nothing is written then).
+__global__ void __launch_bounds__(1024) run_offsets_kernel(const int4 *__restrict__ info, int nblk, int64_t cap_slices,
+                                                           int64_t cap_slots, int4 *__restrict__ blk_run,
+                                                           int32_t *__restrict__ round0, int32_t *flag) {
+    __shared__ int2 s[1024];
+    __shared__ int s_long;
+    const int t = threadIdx.x;
+    if (t == 0) s_long = 0;
+    int2 carry = make_int2(0, 0);
+    for (int b0 = 0; b0 < nblk; b0 += 1024) {
+        const int4 v = b0 + t < nblk ? info[b0 + t] : make_int4(0, 0, 0, 0);
+        __syncthreads();
+        s[t] = make_int2(v.x, v.y);
+        if (v.z > 0) s_long = 1;
+        for (int d = 1; d < 1024; d <<= 1) {
+            __syncthreads();
+            const int2 a = s[t], b = t >= d ? s[t - d] : make_int2(0, 0);
+            __syncthreads();
+            s[t] = make_int2(a.x + b.x, a.y + b.y);
+        }
+        __syncthreads();
+        const int first = carry.x + s[t].x - v.x;
+        if (b0 + t < nblk) {
+            blk_run[b0 + t] = make_int4(first, first + v.z, first + v.x, 0);
+            round0[b0 + t] = carry.y + s[t].y - v.y;
+        }
+        carry.x += s[1023].x;
+        carry.y += s[1023].y;
+    }
+    __syncthreads();
+    if (t == 0) *flag = s_long | (carry.x > cap_slices || 32ll * carry.y > cap_slots ? 2 : 0);
+}
+
+// How the runs of nblk blocks are laid out, and how large that can get.
+struct OwnPlan {
+    int64_t nblk;
+    int parts, lg;           // parts of a camera's run, log2 of the lanes per run
+    int64_t slices, slots;   // run slices and slots, at most
+};
+OwnPlan own_plan(const Prob &P, int64_t nblk) {
+    OwnPlan pl{};
+    pl.nblk = nblk;
+    // few cameras: split their runs until a block has work for a few hundred lanes
+    const double mean = (double)P.n / ((double)nblk * P.nc);
+    pl.parts = 1;
+    while (pl.parts < kMaxParts && (int64_t)P.nc * pl.parts < 128 && mean / pl.parts > 16.0) pl.parts *= 2;
+    // lanes per run, no more than the mean run fills.  FP32: a few rounds of the
+    // CTA's warps.  FP64: two where the runs then still fit its 512 lanes twice,
+    // more only to give the FP64 pipe a handful of warps (the reduction of nine
+    // values over a run's lanes takes a third of a round's pipe time per level)
+    const int64_t items = (int64_t)P.nc * pl.parts;
+    while (pl.lg < 3 && (2 << pl.lg) <= mean / pl.parts &&
+           (items << (pl.lg + 1)) <= (P.fp32 ? 4096 : (pl.lg == 0 ? 1024 : 256)))
+        ++pl.lg;
+    // Slots.  A slice that follows one with as many lanes per run takes, per run, no
+    // more than a run of the slice before it, rounded up to G: together n and the
+    // rounding.  A slice whose runs have a warp each pads only to 32.  That leaves
+    // the first slice of each number of lanes in a block, at most kRunRounds rounds;
+    // one with 2^c lanes, more than usual, holds a run of more than kRunRounds 2^(c-1).
+    const int64_t G = int64_t(1) << pl.lg, per = 32 / G, n = P.n;
+    const int64_t used = items * nblk < n ? items * nblk : n, longs = n / (kRunRounds * G);
+    const int64_t usual = used / per + nblk;  // slices of the usual number of lanes
+    pl.slices = usual + longs;
+    pl.slots = n + (G - 1) * per * usual + 31 * longs + std::min<int64_t>(32 * kRunRounds * nblk, 32 * (n / G + nblk));
+    for (int c = pl.lg + 1; c < 5; ++c)
+        pl.slots += 32 * kRunRounds * std::min<int64_t>(nblk, n / (kRunRounds << (c - 1)));
+    pl.slots = (pl.slots + 31) / 32 * 32;
+    return pl;
+}
+
+// The arrays of a plan in a piece of memory (base NULL: only their size).
+size_t own_arrays(Prob &P, const OwnPlan &pl, char *base) {
+    size_t off = 0;
+    auto arr = [&](size_t bytes) -> void * {
+        void *p = base ? base + off : nullptr;
+        off += al256(bytes ? bytes : 1);
+        return p;
+    };
+    const size_t ns = (size_t)pl.slots;
+    P.rslot_cap = pl.slots;
+    P.rslice = (int2 *)arr(8 * (size_t)pl.slices);
+    P.rlane = (int2 *)arr(32 * 8 * (size_t)pl.slices);
+    P.blk_run = (int4 *)arr(16 * (size_t)pl.nblk);
+    P.cm2r = (int32_t *)arr(4 * (size_t)P.n);
+    P.c_part = arr((size_t)pl.nblk * pl.parts * P.nc * (P.fp32 ? kPartF * 4 : kPartD * 8));
+    if (P.fp32) {
+        P.r_rx = (float4 *)arr(16 * ns);
+        P.r_pt16 = (uint16_t *)arr(2 * ns);
+        P.r_w = P.loss != MBA_LOSS_NONE ? (float *)arr(4 * ns) : nullptr;
+    } else {
+        P.r_pt = (int32_t *)arr(4 * ns);
+        P.r_hg = (double2 *)arr(80 * ns);
+    }
+    return off;
+}
+
+// Blocks per CTA with which b of a block's points is sure to fit in shared memory,
+// kMaxBlocks if none is (FP64 keeps b in global memory: one block per CTA fits).
+int own_blocks(const Prob &P, int grid) {
+    int m = 1;
+    Prob Q = P;
+    while (m < kMaxBlocks && !own_fits(Q, grid, m, sell_block_points(P.n, P.np, (int64_t)grid * m))) ++m;
+    return m;
+}
+
 }  // namespace
+
+// Shared memory of the block-owned PCG kernel with m blocks per CTA of at most pb
+// points: camera rows; b of a block's points (FP32) or the owner's group sums over
+// all blocks; dot products and the owner's six vectors.
+bool own_fits(Prob &P, int grid, int m, int64_t pb) {
+    const int64_t rows = ((int64_t)P.nc * (P.fp32 ? kRowS * 4 : kRowD * 8) + 127) / 128 * 128;
+    const int64_t cams = (P.nc + grid - 1) / grid;  // cameras of an owner, at most
+    const int64_t dots = (3 + 6) * 9 * cams * 8;
+    const int64_t vblk = (int64_t)grid * m * (P.nc >= 128 ? 1 : kMaxParts);
+    int64_t region = (vblk + 7) / 8 * 9 * cams * 8;
+    if (P.fp32 && pb * 12 > region) region = pb * 12;
+    region = (region + 127) / 128 * 128;
+    if (rows + region + dots > kOwnSmem || (P.fp32 && pb > 65000)) return false;
+    P.nblk = grid * m;
+    P.own_pb = (int32_t)pb;
+    P.own_off_b = (int32_t)rows;
+    P.own_off_dots = (int32_t)(rows + region);
+    P.pcg_smem = (int32_t)(rows + region + dots);
+    return true;
+}
 
 // The block-owned product is used where the camera rows leave room in shared
 // memory and where the runs are long enough that the partial sums (written and
@@ -205,19 +332,58 @@ constexpr int64_t kSmallParts = 16 << 20;
 bool own_wanted(const Prob &P, int grid) {
     const int64_t rows = (int64_t)P.nc * (P.fp32 ? kRowS * 4 : kRowD * 8);
     const int64_t parts = (int64_t)grid * P.nc * (P.fp32 ? kPartF * 4 : kPartD * 8);
-    return rows + 40 * 1024 <= kOwnSmem && ((double)P.n >= kMinRun * (double)grid * P.nc || parts <= kSmallParts);
+    if (rows + 40 * 1024 > kOwnSmem || ((double)P.n < kMinRun * (double)grid * P.nc && parts > kSmallParts)) return false;
+    Prob Q = P;
+    if (!P.fp32 && !own_fits(Q, grid, 1, 0)) return false;  // no other form to fall back to
+    for (int m = 1; m <= kMaxBlocks; ++m)
+        if (own_plan(P, (int64_t)grid * m).slots >= (int64_t(1) << 31) - 64) return false;
+    return true;
 }
 
-size_t own_tmp_bytes(const Prob &P, int64_t nblk) {
+// Memory of the layout, whatever the slices turn out to be: the largest over the
+// numbers of blocks that may be taken and, where none is sure to fit (FP32), the
+// gathered product's arrays.
+size_t own_pool_bytes(const Prob &P, int grid) {
+    Prob Q = P;
+    if (!P.own) return P.fact ? gathered_arrays(Q, nullptr) : 0;
+    const int most = P.fp32 ? own_blocks(P, grid) : 1;
+    size_t bytes = 0;
+    for (int m = 1; m <= most; ++m) bytes = std::max(bytes, own_arrays(Q, own_plan(P, (int64_t)grid * m), nullptr));
+    if (P.fp32 && most == kMaxBlocks) bytes = std::max(bytes, gathered_arrays(Q, nullptr));
+    return bytes;
+}
+
+// The gathered FP32 product's arrays in a piece of memory (base NULL: only their size).
+size_t gathered_arrays(Prob &P, char *base) {
+    size_t off = 0;
+    auto arr = [&](size_t bytes) -> void * {
+        void *p = base ? base + off : nullptr;
+        off += al256(bytes);
+        return p;
+    };
+    P.RXcm = (float4 *)arr(16 * (size_t)P.n);
+    P.sp_b = (float4 *)arr(16 * (size_t)P.np);
+    P.cm_w = P.loss != MBA_LOSS_NONE ? (float *)arr(4 * (size_t)P.n) : nullptr;
+    return off;
+}
+
+size_t own_tmp_bytes(const Prob &P, int grid) {
+    const int64_t nblk = (int64_t)grid * (P.fp32 ? own_blocks(P, grid) : 1);
     return al256(8 * (size_t)P.np) + 3 * al256(4 * (size_t)P.n) + 2 * al256(4 * ((size_t)nblk * P.nc + 2)) +
-           3 * al256(8 * (size_t)nblk * P.nc * (P.nc < 128 ? kMaxParts : 1)) + 2 * al256(16 * (size_t)nblk) + 4 * (size_t)exclusive_scan_tmp_ints(nblk * P.nc + 2) + 1024 +
+           3 * al256(8 * (size_t)nblk * P.nc * (P.nc < 128 ? kMaxParts : 1)) + al256(16 * (size_t)nblk) +
+           al256(4 * (size_t)nblk) + al256(4 * (size_t)exclusive_scan_tmp_ints(nblk * P.nc + 2)) +
            stable_sort_tmp_bytes(P.n, (int32_t)nblk + 1);
 }
 
-// Builds the run layout; allocates its arrays (OwnArrays, freed with the problem).
-cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void **pool, size_t *pool_bytes, cudaStream_t s) {
+// Builds the run layout in `pool` (own_pool_bytes), on the device alone: with its
+// sizes read back and its arrays allocated here, the creation of 2,000 points took
+// 0.83 instead of 0.76 ms, of 50k points (FP32) 1.12 instead of 0.99.  *flag: see
+// run_offsets_kernel.
+cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void *pool, size_t pool_bytes, int32_t *flag, cudaStream_t s) {
+    const OwnPlan pl = own_plan(P, P.nblk);
     const int64_t nblk = P.nblk, nruns = nblk * P.nc;
-    if (tmp_bytes < own_tmp_bytes(P, nblk)) return cudaErrorInvalidValue;
+    if (own_arrays(P, pl, (char *)pool) > pool_bytes) return cudaErrorInvalidValue;
+    P.n_vblk = (int32_t)(nblk * pl.parts);
     char *t = (char *)tmp;
     auto take = [&](size_t bytes) {
         char *p = t;
@@ -235,6 +401,7 @@ cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void **pool, size_t 
     int32_t *round0_d = (int32_t *)take(4 * (size_t)nblk);
     int32_t *scan_tmp = (int32_t *)take(4 * (size_t)exclusive_scan_tmp_ints(nruns + 2));
     const size_t sort_bytes = stable_sort_tmp_bytes(P.n, (int32_t)nblk + 1);
+    if ((size_t)(t - (char *)tmp) + sort_bytes > tmp_bytes) return cudaErrorInvalidValue;
 
     point_blocks_kernel<<<grid_for(P.n_slices), kBlock, 0, s>>>(P.slice, P.n_slices, P.nblk, sp_bl);
     obs_block_kernel<<<grid_for(P.n), kBlock, 0, s>>>(P.cm_sp, sp_bl, P.n, key);
@@ -245,92 +412,19 @@ cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void **pool, size_t 
     run_key_kernel<<<grid_for(P.n), kBlock, 0, s>>>(ord, key, P.cam_ptr, P.nc, P.n, run, count);
     e = exclusive_scan_i32(count, run_ptr, nruns + 1, scan_tmp, s);
     if (e != cudaSuccess) return e;
-
-    // few cameras: split their runs until a block has work for a few hundred lanes
-    const double mean = (double)P.n / (double)nruns;
-    int parts = 1;
-    while (parts < kMaxParts && (int64_t)P.nc * parts < 128 && mean / parts > 16.0) parts *= 2;
-    P.n_vblk = (int32_t)(nblk * parts);
-    // shared memory: camera rows, b of a block's points (FP32) or the owner's
-    // group sums over them, dot products
-    // lanes per run, no more than the mean run fills.  FP32: a few rounds of the
-    // CTA's warps.  FP64: two where the runs then still fit its 512 lanes twice,
-    // more only to give the FP64 pipe a handful of warps (the reduction of nine
-    // values over a run's lanes takes a third of a round's pipe time per level)
-    int lg = 0;
-    const int64_t items_blk = (int64_t)P.nc * parts;
-    while (lg < 3 && (2 << lg) <= mean / parts &&
-           (items_blk << (lg + 1)) <= (P.fp32 ? 4096 : (lg == 0 ? 1024 : 256)))
-        ++lg;
-
-    // sort on the device, offsets of the blocks here, then the slices on the device:
-    // laid out on the host (counts read back, tables of 32 lanes a slice sent), the
-    // creation of 1.0M points and 5.0M observations took 8.6 ms instead of 3.5, of
-    // 50k points and 250k observations 1.77 instead of 1.01
     int m = 2;
-    while (m < items_blk) m *= 2;
-    if (m > 4096) return cudaErrorInvalidValue;
-    sort_runs_kernel<<<(unsigned)nblk, 512, 8 * (size_t)m, s>>>(count, P.nc, parts, lg, m, sorted, cut, info_d);
-    std::vector<int4> info((size_t)nblk);
-    e = cudaMemcpyAsync(info.data(), info_d, 16 * (size_t)nblk, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return e;
-    std::vector<int4> blk((size_t)nblk);
-    std::vector<int32_t> round0((size_t)nblk);
-    int64_t slots = 0;
-    int32_t nrs = 0;
-    for (int64_t b = 0; b < nblk; ++b) {
-        blk[b] = make_int4(nrs, nrs + info[b].z, nrs + info[b].x, 0);
-        nrs += info[b].x;
-        if (info[b].z > 0) P.long_runs = 1;
-        round0[b] = (int32_t)(slots / 32);
-        slots += 32 * (int64_t)info[b].y;
-        if (slots > 2000000000ll) return cudaErrorInvalidValue;
-    }
-    P.rslot_cap = (slots + 31) / 32 * 32;
-
-    // arrays
-    const bool loss = P.loss != MBA_LOSS_NONE;
-    const size_t ns = (size_t)P.rslot_cap, part_vals = (size_t)P.n_vblk * P.nc * (P.fp32 ? kPartF : kPartD);
-    for (int pass = 0; pass < 2; ++pass) {
-        char *q = (char *)*pool;
-        size_t off = 0;
-        auto arr = [&](size_t bytes) -> void * {
-            void *p = pass ? q + off : nullptr;
-            off += al256(bytes ? bytes : 1);
-            return p;
-        };
-        P.rslice = (int2 *)arr(8 * (size_t)nrs);
-        P.rlane = (int2 *)arr(32 * 8 * (size_t)nrs);
-        P.blk_run = (int4 *)arr(16 * blk.size());
-        P.cm2r = (int32_t *)arr(4 * (size_t)P.n);
-        P.c_part = arr(part_vals * (P.fp32 ? 4 : 8));
-        if (P.fp32) {
-            P.r_rx = (float4 *)arr(16 * ns);
-            P.r_pt16 = (uint16_t *)arr(2 * ns);
-            P.r_w = loss ? (float *)arr(4 * ns) : nullptr;
-        } else {
-            P.r_pt = (int32_t *)arr(4 * ns);
-            P.r_hg = (double2 *)arr(80 * ns);
-        }
-        if (pass == 0) {
-            *pool_bytes = off;
-            if (over_memory_limit(off)) return cudaErrorMemoryAllocation;
-            e = cudaMalloc(pool, off);
-            if (e != cudaSuccess) return e;
-        }
-    }
-    e = cudaMemcpyAsync(P.blk_run, blk.data(), 16 * blk.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(round0_d, round0.data(), 4 * round0.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(P.c_part, 0, part_vals * (P.fp32 ? 4 : 8), s);
+    while (m < P.nc * pl.parts) m *= 2;
+    if (m > kBlockSlices) return cudaErrorInvalidValue;
+    sort_runs_kernel<<<(unsigned)nblk, 512, 8 * (size_t)m, s>>>(count, P.nc, pl.parts, pl.lg, m, sorted, cut, info_d);
+    run_offsets_kernel<<<1, 1024, 0, s>>>(info_d, (int)nblk, pl.slices, pl.slots, P.blk_run, round0_d, flag);
+    e = cudaMemsetAsync(P.c_part, 0, (size_t)P.n_vblk * P.nc * (P.fp32 ? kPartF * 4 : kPartD * 8), s);
     if (e == cudaSuccess)
-        e = P.fp32 ? cudaMemsetAsync(P.r_pt16, 0xff, 2 * ns, s) : cudaMemsetAsync(P.r_pt, 0xff, 4 * ns, s);
+        e = P.fp32 ? cudaMemsetAsync(P.r_pt16, 0xff, 2 * (size_t)pl.slots, s)
+                   : cudaMemsetAsync(P.r_pt, 0xff, 4 * (size_t)pl.slots, s);
     if (e != cudaSuccess) return e;
-    run_slices_kernel<<<(unsigned)nblk, 256, 0, s>>>(P, sorted, cut, round0_d, parts, base_d);
-    fill_runs_kernel<<<grid_for(P.n), kBlock, 0, s>>>(P, ord, run, run_ptr, base_d, parts, sp_bl);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host vectors go out of scope
-    return e;
+    run_slices_kernel<<<(unsigned)nblk, 256, 0, s>>>(P, sorted, cut, round0_d, pl.parts, base_d, flag);
+    fill_runs_kernel<<<grid_for(P.n), kBlock, 0, s>>>(P, ord, run, run_ptr, base_d, pl.parts, sp_bl, flag);
+    return cudaGetLastError();
 }
 
 }  // namespace mba

@@ -314,9 +314,10 @@ __device__ __forceinline__ void own_long_runs(const Prob &P, const float *rows, 
 }
 
 // Camera pass of one block: every run's nine raw sums into the block's partials.
-// LONG: some blocks have runs of more than kRunRounds rounds.  600 cameras, 500k observations, one camera with 5 % of them, against as many
-// lanes for every run: FP64 338 -> 102 us per PCG iteration, FP32 35 -> 28; with
-// 25 %, 745 -> 93 and 57 -> 26.
+// LONG: some blocks have runs of more than kRunRounds rounds.  600 cameras, 500k
+// observations, one camera with 5 % of them, against as many lanes for every run:
+// FP64 338 -> 102 us per PCG iteration, FP32 35 -> 28; with 25 %, 745 -> 93 and
+// 57 -> 26.
 template <bool LONG>
 __device__ void own_cameras(const Prob &P, const float *rows, const float *bs, int *next, const RunBegin &rb, int blk) {
     const int lane = threadIdx.x & 31;

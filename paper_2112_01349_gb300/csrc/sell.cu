@@ -95,6 +95,15 @@ int64_t sell_slot_bound(int64_t n, int32_t np) {
 }
 int64_t sell_slice_bound(int64_t n, int32_t np) { return sell_slot_bound(n, np) / 32 + 1; }
 
+// Points of a block at most, slices dealt to nblk blocks in turn.  Full slices hold
+// more points the shorter their tracks are, so that a block's slices hold at most as
+// many as an equal share and one slice (32) more.  A class's last slice may be
+// partly empty, and a class of few points has its own number of lanes: up to 62
+// points per class that other blocks do not have.
+int64_t sell_block_points(int64_t n, int32_t np, int64_t nblk) {
+    return (np / nblk + 33 + 62 * class_bound(n) / nblk + 31) / 32 * 32;
+}
+
 // Scratch (tmp): the sort's, then keys and inverse (np each), the class offsets
 // (kMaxTrack + 2) and the class table (kMaxTrack + 1 int4).
 size_t sell_tmp_bytes(int32_t np) {
@@ -141,29 +150,18 @@ cudaError_t build_slices(Prob &P, int grid, int max_track, void *tmp, size_t tmp
     // block's points are numbered in slice order; as few blocks per CTA as let b of
     // a block's points fit in shared memory beside the camera rows (FP32)
     if (P.own) {
-        const int64_t rows = ((int64_t)P.nc * (P.fp32 ? kRowS * 4 : kRowD * 8) + 127) / 128 * 128;
-        const int64_t cams = (P.nc + grid - 1) / grid;  // cameras of an owner, at most
-        const int64_t dots = (3 + 6) * 9 * cams * 8;  // dot products and the owner's six vectors
         std::vector<int32_t> used;
         P.own = 0;
-        for (int m = 1; m <= 4 && !P.own; ++m) {
-            P.nblk = grid * m;
-            used.assign((size_t)P.nblk, 0);
-            for (size_t i = 0; i < slices.size(); ++i) used[i % P.nblk] += slices[i].y;
+        for (int m = 1; m <= kMaxBlocks && !P.own; ++m) {
+            used.assign((size_t)grid * m, 0);
+            for (size_t i = 0; i < slices.size(); ++i) used[i % used.size()] += slices[i].y;
             int32_t most = 0;
             for (int32_t u : used) most = u > most ? u : most;
-            P.own_pb = (most + 31) / 32 * 32;
-            const int64_t groups = ((int64_t)P.nblk * kMaxParts + 7) / 8 * 9 * cams * 8;  // with parts; see build_own
-            const int64_t groups1 = ((int64_t)P.nblk + 7) / 8 * 9 * cams * 8;
-            int64_t region = P.nc >= 128 ? groups1 : groups;
-            if (P.fp32 && (int64_t)P.own_pb * 12 > region) region = (int64_t)P.own_pb * 12;
-            region = (region + 127) / 128 * 128;
-            if (rows + region + dots > kOwnSmem || (P.fp32 && P.own_pb > 65000)) continue;
-            P.own = 1;
-            P.own_off_b = (int32_t)rows;
-            P.own_off_dots = (int32_t)(rows + region);
-            P.pcg_smem = (int32_t)(rows + region + dots);
+            P.own = own_fits(P, grid, m, (most + 31) / 32 * 32) ? 1 : 0;
         }
+    }
+    if (P.own) {
+        std::vector<int32_t> used;
         used.assign((size_t)P.nblk, 0);
         for (size_t i = 0; i < slices.size(); ++i) {
             const int32_t count = slices[i].y;

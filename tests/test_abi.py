@@ -51,3 +51,31 @@ def test_memory_limit_gives_oom_before_any_allocation():
     finally:
         mba.mba_set_device_memory_limit(0)
     assert np.isfinite(sc.cameras).all()
+
+
+def test_memory_limit_counts_everything_a_creation_allocates():
+    """Many cameras and few observations: most of the memory is the blocks'
+    partial sums, whose size follows from the shape and is part of the check."""
+    import re
+
+    from paper_2112_01349_gb300 import mba
+    from scenes import make_scene
+
+    sc = make_scene(2000, 14_000, track=("fixed", 2), seed=1)
+    args = (sc.cameras, sc.points, sc.observations, sc.cam_idx, sc.pt_idx)
+
+    def refusal(limit):
+        mba.mba_set_device_memory_limit(limit)
+        try:
+            mba.Problem(*args, precision="fp32").close()
+        except mba.MbaError as e:
+            return e.status, str(e)
+        finally:
+            mba.mba_set_device_memory_limit(0)
+        return 0, ""
+
+    status, text = refusal(1)
+    need = int(re.search(r"needs (\d+) bytes", text).group(1))
+    assert status == mba.MBA_ERR_OOM and need > 152 * 2000 * 48
+    assert refusal(need - 1) == (status, text)
+    assert "device memory limit" not in refusal(need)[1]

@@ -108,3 +108,36 @@ def test_problems_of_different_sizes_in_two_threads(mba):
         t.join()
     assert not errors, errors
     assert all(len(v) == 1 for v in out.values()), out
+
+
+@pytest.mark.parametrize("nc,npts,track,precision,loss,jacobian", [
+    (2000, 14_000, ("fixed", 2), "fp32", "none", "analytic"), (2000, 14_000, ("fixed", 2), "fp64", "huber", "analytic"),
+    (12, 9000, ("geom", 0.25), "fp32", "huber", "analytic"), (12, 9000, ("geom", 0.25), "fp64", "none", "analytic"),
+    (601, 20_000, ("lognormal", 6.5, 300), "fp32", "none", "analytic"), (2500, 9000, ("fixed", 4), "fp32", "huber", "analytic"),
+    (2500, 9000, ("fixed", 4), "fp64", "none", "analytic"), (40, 3000, ("fixed", 4), "fp32", "none", "autodiff")])
+def test_memory_cap_is_exact(mba, nc, npts, track, precision, loss, jacobian):
+    """The bytes that a refused creation names are enough, one byte less is
+    refused, and the handle takes no more than they say."""
+    import re
+
+    sc = make_scene(nc, npts, track=track, sigma=0.5, seed=55)
+
+    def create():
+        return mba.Problem(sc.cameras, sc.points, sc.observations, sc.cam_idx, sc.pt_idx, precision=precision,
+                           loss=loss, huber_delta=2.0 if loss == "huber" else 0.0, jacobian=jacobian)
+
+    try:
+        mba.mba_set_device_memory_limit(1)
+        with pytest.raises(mba.MbaError) as e:
+            create()
+        need = int(re.search(r"needs (\d+) bytes", str(e.value)).group(1))
+        mba.mba_set_device_memory_limit(need - 1)
+        with pytest.raises(mba.MbaError) as e:
+            create()
+        assert e.value.status == mba.MBA_ERR_OOM and "device memory limit" in str(e.value)
+        mba.mba_set_device_memory_limit(need)
+        with create() as pr:
+            assert pr.info["device_bytes"] < need
+            assert pr.solve(max_iter=2, pcg_max_iter=5)["status"] == 0
+    finally:
+        mba.mba_set_device_memory_limit(0)
