@@ -184,3 +184,25 @@ def test_a_camera_that_sees_every_point(mba, nc, npts, precision, tol, loss):
     for a in range(9):
         rel_close(st["dc"][:, a], rs["dc"].reshape(-1, 9)[:, a], stol, f"dc[{a}]")
     rel_close(st["dp"], rs["dp"].reshape(-1, 3), stol, "dp")
+
+
+# b of a CTA's points beside the camera rows in shared memory: two, three and four
+# blocks per CTA, two with split runs, and more points than four can hold (gathered)
+@pytest.mark.parametrize("nc,npts,track,loss", [(2000, 900_000, 2, "none"), (2000, 1_600_000, 2, "huber"),
+                                                (1824, 3_000_000, 1, "none"), (100, 3_000_000, 1, "huber"),
+                                                (2290, 480_000, 3, "huber")])
+def test_blocks_per_cta(mba, nc, npts, track, loss):
+    """Tolerances as above."""
+    sc = make_scene(nc, npts, track=("fixed", track), sigma=0.5, seed=12)
+    x = np.random.default_rng(5).normal(size=(nc, 9))
+    with mba.Problem(*_args(sc), precision="fp32", loss=loss, huber_delta=2.0 if loss == "huber" else 0.0) as pr:
+        y = pr.schur_matvec(0.1, x)
+        st = pr.step(0.1, pcg_max_iter=4, pcg_rel_tol=0.0)
+        f = pr.solve(max_iter=1, pcg_max_iter=4, initial_radius=10.0)["final_cost"]
+    rel_close(y, oracle.schur(*_args(sc), 0.1, x=x.reshape(-1), loss=loss, delta=2.0)["y"].reshape(-1, 9), 1e-4, "S x")
+    rs = oracle.step(*_args(sc), 0.1, pcg_max=4, pcg_tol=0.0, loss=loss, delta=2.0)
+    for a in range(9):
+        rel_close(st["dc"][:, a], rs["dc"].reshape(-1, 9)[:, a], 2e-3, f"dc[{a}]")
+    rel_close(st["dp"], rs["dp"].reshape(-1, 3), 2e-3, "dp")
+    ref = oracle.lm_solve(*_args(sc), max_iter=1, pcg_max=4, initial_radius=10.0, loss=loss, delta=2.0)
+    rel_close(f, ref["final_cost"], 1e-4, "final cost")
