@@ -284,6 +284,7 @@ mba_status mba_problem_create(const double *cameras, int32_t nc, const double *p
         P.ctr = fact ? c.take<float>((size_t)kCtr * nc) : nullptr;
         const bool own64 = P.own && !P.fp32;
         P.sl_hg = own64 ? c.take<double2>(5 * slots) : nullptr;
+        P.sl2r = own64 ? c.take<int32_t>(slots) : nullptr;
         P.sl_w64 = own64 && lossy ? c.take<double>(slots) : nullptr;
         P.sp_X64 = own64 ? c.take<double>(4 * (size_t)np) : nullptr;
         P.sp_b64 = own64 ? c.take<double>(4 * (size_t)np) : nullptr;

@@ -313,13 +313,20 @@ __global__ void __launch_bounds__(kBlock, 4) lin_point_kernel(Prob P, int force)
     }
 }
 
-// H = W Jp^T Jp, g = W Jp^T p and r2 of one observation (h = W Jp), as pairs.
-__device__ __forceinline__ void store_hg(double2 *o, int64_t st, const double *h, const double *Jp, const double *pz) {
-    o[0] = make_double2(h[0] * Jp[0] + h[3] * Jp[3], h[0] * Jp[1] + h[3] * Jp[4]);
-    o[st] = make_double2(h[0] * Jp[2] + h[3] * Jp[5], h[1] * Jp[1] + h[4] * Jp[4]);
-    o[2 * st] = make_double2(h[1] * Jp[2] + h[4] * Jp[5], h[2] * Jp[2] + h[5] * Jp[5]);
-    o[3 * st] = make_double2(h[0] * pz[0] + h[3] * pz[1], h[1] * pz[0] + h[4] * pz[1]);
-    o[4 * st] = make_double2(h[2] * pz[0] + h[5] * pz[1], pz[0] * pz[0] + pz[1] * pz[1]);
+// H = W Jp^T Jp, g = W Jp^T p and r2 of one observation (h = W Jp), as pairs, to its
+// places in the slices and in the runs.
+__device__ __forceinline__ void store_hg(const Prob &P, int64_t slot, const double *h, const double *Jp, const double *pz) {
+    const double2 v[5] = {make_double2(fma(h[0], Jp[0], h[3] * Jp[3]), fma(h[0], Jp[1], h[3] * Jp[4])),
+                          make_double2(fma(h[0], Jp[2], h[3] * Jp[5]), fma(h[1], Jp[1], h[4] * Jp[4])),
+                          make_double2(fma(h[1], Jp[2], h[4] * Jp[5]), fma(h[2], Jp[2], h[5] * Jp[5])),
+                          make_double2(fma(h[0], pz[0], h[3] * pz[1]), fma(h[1], pz[0], h[4] * pz[1])),
+                          make_double2(fma(h[2], pz[0], h[5] * pz[1]), fma(pz[0], pz[0], pz[1] * pz[1]))};
+    double2 *r = P.r_hg + __ldg(P.sl2r + slot);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        P.sl_hg[slot + q * P.slot_cap] = v[q];
+        r[q * P.rslot_cap] = v[q];
+    }
 }
 
 // Point-major linearisation of the factored form over slices: per observation
@@ -405,7 +412,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 1024 : 512, 1) lin_slices_ker
                 P.sl_px[slot] = make_float4(__int_as_float(cam), pz[0], pz[1], pz[2]);
                 if (P.sl_w) P.sl_w[slot] = W;
             } else {
-                store_hg(P.sl_hg + slot, P.slot_cap, h, Jp, pz);
+                store_hg(P, slot, h, Jp, pz);
                 if (P.sl_w64) P.sl_w64[slot] = W;
             }
             q[0] += h[0] * Jp[0] + h[3] * Jp[3];
@@ -517,16 +524,21 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 2 : 1) lin_camera_ker
 }
 
 // ---------------------------------------------------------------------------
-// Camera blocks of the block-owned FP64 form.  In the basis of the product's raw
-// sums a residual row is (X x jp, jp, p (1, r2, r2^2)), jp a row of Jp, and
-// Jc = ctr applied to it, so B = ctr (sum W raw^T raw) ctr^T per camera.  The sum
-// has 44 distinct entries: H = W Jp^T Jp (6), X x H (9), X x H x X (6), g and
-// X x g with g = W Jp^T p (9 each, times 1, r2, r2^2), W r2 (1 .. r2^4) (5); with v's
-// nine, 53 sums of about 130 FP64 instructions where J^T W J from the nine
-// columns takes 170 beside forming them.  The 53 lane sums of a chunk are reduced
-// by exchanging halves, 62 additions instead of 5 x 54.
-// Both matter because the FP64 pipe bounds the kernel: 5.0M observations
-// 3.34 -> 1.86 ms.
+// Camera blocks of the block-owned FP64 form.  In the camera frame a residual row of
+// the Jacobian is ctr applied to (Y x d, d, p (1, r2, r2^2)), d a row of D =
+// d(pixel)/dP and Y = R X, or X on the first-order rotation branch, where ctr has I
+// in place of R M.  So B = ctr (sum W raw^T raw) ctr^T per camera, and the sum has
+// 44 distinct entries: H = W D^T D (6), Y x H (9), Y x H x Y (6), g and Y x g with
+// g = W D^T p (9 each, times 1, r2, r2^2), W r2 (1 .. r2^4) (5); with v's nine, 53
+// sums of about 130 FP64 instructions where J^T W J from the nine columns takes 170
+// beside forming them.  The 53 lane sums of a chunk are reduced by exchanging
+// halves, 62 additions instead of 5 x 54.  Both matter because the FP64 pipe bounds
+// the kernel (nine columns: 3.34 ms for 5.0M observations).
+// The product's H and g are in the world frame, where these sums were before.  Rotated
+// to the camera frame, such sums lose the entries of the viewing direction, |p|^2 of
+// the others in H: an error of 3.0e-13 of S x (16 cameras, 2.0M observations)
+// instead of 4.7e-14.  They are left to the point side, which has them at hand: a
+// linearisation of 5.0M observations took 2.93 ms, now 2.86.
 // ---------------------------------------------------------------------------
 constexpr int kRawSums = 53;
 __device__ __forceinline__ int raw_index(int a, int b) {  // raw components a <= b of 0..8 (rotation, translation, intrinsics)
@@ -534,34 +546,6 @@ __device__ __forceinline__ int raw_index(int a, int b) {  // raw components a <=
     if (ga == 0) return gb == 0 ? 15 + sym3(i, k) : (gb == 1 ? 6 + 3 * i + k : 30 + 3 * k + i);
     if (ga == 1) return gb == 1 ? sym3(i, k) : 21 + 3 * k + i;
     return 39 + i + k;
-}
-
-// A chunk of a camera on the first-order rotation branch (its rotation columns
-// are not of that form): the 54 sums of the final basis.
-__device__ __noinline__ void lin_camera64_small(const Prob &P, int cam, const double *ctab, int b0, int b1, double *out) {
-    const int lane = threadIdx.x & 31;
-    for (int q0 = 0; q0 < 54; q0 += 9) {
-        double acc[9];
-        for (int q = 0; q < 9; ++q) acc[q] = 0.0;
-        for (int s = b0 + lane; s < b1; s += 32) {
-            const int64_t pt = P.cm_pt[s];
-            const double2 uv = P.cm_uv[s];
-            double e[2], Jc[18], Jp[6], rho, W;
-            project<double, true>(ctab, P.pts[3 * pt], P.pts[3 * pt + 1], P.pts[3 * pt + 2], uv.x, uv.y, e, Jc, Jp);
-            loss_weight<double>(P.loss, P.delta, e[0] * e[0] + e[1] * e[1], &rho, &W);
-            int idx = 0;
-            for (int a = 0; a < 9; ++a)
-                for (int b = a; b < 9; ++b, ++idx)
-                    if (idx >= q0 && idx < q0 + 9) acc[idx - q0] += W * (Jc[a] * Jc[b] + Jc[9 + a] * Jc[9 + b]);
-            for (int a = 0; a < 9; ++a)
-                if (q0 == 45) acc[a] -= W * (Jc[a] * e[0] + Jc[9 + a] * e[1]);
-        }
-        for (int q = 0; q < 9; ++q) {
-            double v = acc[q];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) out[q0 + q] = v;
-        }
-    }
 }
 
 __global__ void __launch_bounds__(kBlock, 1) lin_camera64_kernel(Prob P, int force) {
@@ -590,57 +574,62 @@ __global__ void __launch_bounds__(kBlock, 1) lin_camera64_kernel(Prob P, int for
             const double X0 = xa.x, X1 = xa.y, X2 = __ldg(P.sp_X64 + 4 * pt + 2);
             double e[2], Jc[18], Jp[6], pz[3];
             project<double, true>(ctab, X0, X1, X2, uv.x, uv.y, e, Jc, Jp, pz);
-            double h[6], W = 1.0;
+            double Y[3];  // R X as in project
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const double y = ctab[3 * k] * X0 + ctab[3 * k + 1] * X1 + ctab[3 * k + 2] * X2;
+                Y[k] = small ? (k == 0 ? X0 : (k == 1 ? X1 : X2)) : y;
+            }
+            double hd[4], W = 1.0;  // W D (its first two columns)
+            const double D[4] = {Jc[3], Jc[4], Jc[12], Jc[13]};
             if (P.loss != MBA_LOSS_NONE) {
                 double rho;
                 loss_weight<double>(P.loss, P.delta, e[0] * e[0] + e[1] * e[1], &rho, &W);
 #pragma unroll
-                for (int q = 0; q < 6; ++q) h[q] = W * Jp[q];
+                for (int q = 0; q < 4; ++q) hd[q] = W * D[q];
             } else {
 #pragma unroll
-                for (int q = 0; q < 6; ++q) h[q] = Jp[q];
+                for (int q = 0; q < 4; ++q) hd[q] = D[q];
             }
-            const double r2 = fma(pz[0], pz[0], pz[1] * pz[1]);
-            const double H[6] = {fma(h[0], Jp[0], h[3] * Jp[3]), fma(h[0], Jp[1], h[3] * Jp[4]), fma(h[0], Jp[2], h[3] * Jp[5]),
-                                 fma(h[1], Jp[1], h[4] * Jp[4]), fma(h[1], Jp[2], h[4] * Jp[5]), fma(h[2], Jp[2], h[5] * Jp[5])};
-            const double g[3] = {fma(h[0], pz[0], h[3] * pz[1]), fma(h[1], pz[0], h[4] * pz[1]), fma(h[2], pz[0], h[5] * pz[1])};
-            {
-                double2 *o = P.r_hg + P.cm2r[s];
-                const int64_t st = P.rslot_cap;
-                o[0] = make_double2(H[0], H[1]);
-                o[st] = make_double2(H[2], H[3]);
-                o[2 * st] = make_double2(H[4], H[5]);
-                o[3 * st] = make_double2(g[0], g[1]);
-                o[4 * st] = make_double2(g[2], r2);
-            }
-            if (small) continue;
+            const double px = pz[0], py = pz[1], r2 = fma(px, px, py * py);
+            // the third entries from the first two, D's third column being D_xy p
+            double H[6], g[3];
+            H[0] = fma(hd[0], D[0], hd[2] * D[2]);
+            H[1] = fma(hd[0], D[1], hd[2] * D[3]);
+            H[3] = fma(hd[1], D[1], hd[3] * D[3]);
+            H[2] = fma(px, H[0], py * H[1]);
+            H[4] = fma(px, H[1], py * H[3]);
+            H[5] = fma(px, H[2], py * H[4]);
+            g[0] = fma(hd[0], px, hd[2] * py);
+            g[1] = fma(hd[1], px, hd[3] * py);
+            g[2] = fma(px, g[0], py * g[1]);
 #pragma unroll
             for (int q = 0; q < 6; ++q) acc[q] += H[q];
-            // U = X x H (column k), then U x X
+            // U = Y x H (column k), then U x Y
             double U[3][3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const double h0 = H[k], h1 = H[k == 0 ? 1 : 2 + k], h2 = H[k == 0 ? 2 : 3 + k];
-                U[0][k] = fma(X1, h2, -X2 * h1);
-                U[1][k] = fma(X2, h0, -X0 * h2);
-                U[2][k] = fma(X0, h1, -X1 * h0);
+                U[0][k] = fma(Y[1], h2, -Y[2] * h1);
+                U[1][k] = fma(Y[2], h0, -Y[0] * h2);
+                U[2][k] = fma(Y[0], h1, -Y[1] * h0);
 #pragma unroll
                 for (int i = 0; i < 3; ++i) acc[6 + 3 * i + k] += U[i][k];
             }
-            acc[15] = fma(X1, U[0][2], fma(-X2, U[0][1], acc[15]));
-            acc[16] = fma(X2, U[0][0], fma(-X0, U[0][2], acc[16]));
-            acc[17] = fma(X0, U[0][1], fma(-X1, U[0][0], acc[17]));
-            acc[18] = fma(X2, U[1][0], fma(-X0, U[1][2], acc[18]));
-            acc[19] = fma(X0, U[1][1], fma(-X1, U[1][0], acc[19]));
-            acc[20] = fma(X0, U[2][1], fma(-X1, U[2][0], acc[20]));
-            const double xg[3] = {fma(X1, g[2], -X2 * g[1]), fma(X2, g[0], -X0 * g[2]), fma(X0, g[1], -X1 * g[0])};
+            acc[15] = fma(Y[1], U[0][2], fma(-Y[2], U[0][1], acc[15]));
+            acc[16] = fma(Y[2], U[0][0], fma(-Y[0], U[0][2], acc[16]));
+            acc[17] = fma(Y[0], U[0][1], fma(-Y[1], U[0][0], acc[17]));
+            acc[18] = fma(Y[2], U[1][0], fma(-Y[0], U[1][2], acc[18]));
+            acc[19] = fma(Y[0], U[1][1], fma(-Y[1], U[1][0], acc[19]));
+            acc[20] = fma(Y[0], U[2][1], fma(-Y[1], U[2][0], acc[20]));
+            const double yg[3] = {fma(Y[1], g[2], -Y[2] * g[1]), fma(Y[2], g[0], -Y[0] * g[2]), fma(Y[0], g[1], -Y[1] * g[0])};
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const double a1 = r2 * g[k], c1 = r2 * xg[k];
+                const double a1 = r2 * g[k], c1 = r2 * yg[k];
                 acc[21 + k] += g[k];
                 acc[24 + k] += a1;
                 acc[27 + k] = fma(r2, a1, acc[27 + k]);
-                acc[30 + k] += xg[k];
+                acc[30 + k] += yg[k];
                 acc[33 + k] += c1;
                 acc[36 + k] = fma(r2, c1, acc[36 + k]);
             }
@@ -650,15 +639,14 @@ __global__ void __launch_bounds__(kBlock, 1) lin_camera64_kernel(Prob P, int for
             acc[41] += q2;
             acc[42] += q3;
             acc[43] = fma(q3, r2, acc[43]);
-            const double y0 = fma(h[0], e[0], h[3] * e[1]), y1 = fma(h[1], e[0], h[4] * e[1]),
-                         y2 = fma(h[2], e[0], h[5] * e[1]);
+            const double y0 = fma(hd[0], e[0], hd[2] * e[1]), y1 = fma(hd[1], e[0], hd[3] * e[1]), y2 = fma(px, y0, py * y1);
             acc[44] -= y0;
             acc[45] -= y1;
             acc[46] -= y2;
-            acc[47] = fma(-X1, y2, fma(X2, y1, acc[47]));
-            acc[48] = fma(-X2, y0, fma(X0, y2, acc[48]));
-            acc[49] = fma(-X0, y1, fma(X1, y0, acc[49]));
-            double t = fma(pz[0], e[0], pz[1] * e[1]);
+            acc[47] = fma(-Y[1], y2, fma(Y[2], y1, acc[47]));
+            acc[48] = fma(-Y[2], y0, fma(Y[0], y2, acc[48]));
+            acc[49] = fma(-Y[0], y1, fma(Y[1], y0, acc[49]));
+            double t = fma(px, e[0], py * e[1]);
             if (P.loss != MBA_LOSS_NONE) t *= W;
             const double t1 = r2 * t;
             acc[50] -= t;
@@ -667,10 +655,6 @@ __global__ void __launch_bounds__(kBlock, 1) lin_camera64_kernel(Prob P, int for
         }
         __syncwarp();
         double *out = P.cpart + 54 * (int64_t)c;
-        if (small) {
-            lin_camera64_small(P, cam, ctab, b0, b1, out);
-            continue;
-        }
 #pragma unroll
         for (int w = 32; w >= 2; w >>= 1) {
             const bool up = lane & (w >> 1);
@@ -809,27 +793,35 @@ __global__ void __launch_bounds__(kBlock, 2) lin_camera32_kernel(Prob P, int for
 }
 
 // One camera per 64 threads: the chunk sums in order, then B = ctr raw ctr^T and
-// v = ctr raw (or the sums themselves for first-order cameras).
+// v = ctr raw, with ctr as in factored_camera (FP64: from the table row; I for R M on
+// the first-order branch, whose sums have X in place of R X).
 template <typename T>
 __global__ void __launch_bounds__(64) cam_finalize_raw_kernel(Prob P, const int32_t *__restrict__ cfirst, int force) {
     if (!force && (P.st->done || !P.st->relin)) return;
     __shared__ double raw[54], ct[27];
     const int i = blockIdx.x, t = threadIdx.x;
-    const bool small = sizeof(T) == 8 && ((const double *)P.camtab)[(int64_t)i * kCamTab + 24] != 0.0;
     const bool fixed = P.has_fixed && P.cam_fixed[i];  // its Jacobian columns are zero
-    if (t < 54) {
+    if (t < kRawSums) {
         double s = 0.0;
-        if (t < kRawSums || small)
-            for (int c = cfirst[i]; c < cfirst[i + 1]; ++c) s += P.cpart[54 * (int64_t)c + t];
+        for (int c = cfirst[i]; c < cfirst[i + 1]; ++c) s += P.cpart[54 * (int64_t)c + t];
         raw[t] = fixed ? 0.0 : s;
     }
-    if (t < 27) ct[t] = sizeof(T) == 8 ? P.ctr64[(int64_t)i * kCtr + t] : (double)P.ctr[(int64_t)i * kCtr + t];
+    if (t < 27) {
+        if constexpr (sizeof(T) == 4) {
+            ct[t] = (double)P.ctr[(int64_t)i * kCtr + t];
+        } else {
+            const double *row = (const double *)P.camtab + (int64_t)i * kCamTab;
+            const int g = t / 9, a = (t - 9 * g) / 3, b = t % 3;
+            const double rm = fma(row[3 * b], row[9 + a], fma(row[3 * b + 1], row[12 + a], row[3 * b + 2] * row[15 + a]));
+            const double f = row[21], kb = row[21 + b], unit = a == b ? 1.0 : 0.0;
+            const bool first_order = row[24] != 0.0;
+            ct[t] = g == 0 && !first_order ? rm : (g == 2 && a == b && a > 0 ? f : (g == 2 && a == 0 && b > 0 ? kb : unit));
+        }
+    }
     __syncthreads();
     if (t >= 54) return;
     double r = 0.0;
-    if (small) {
-        r = raw[t];
-    } else if (t < 45) {
+    if (t < 45) {
         int a = 0, f = t;
         while (f >= 9 - a) f -= 9 - a, ++a;
         const int b = a + f, ga = a / 3 * 3, gb = b / 3 * 3;

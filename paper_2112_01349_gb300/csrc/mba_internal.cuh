@@ -133,7 +133,8 @@ struct Prob {
     int2 *rslice;           // per run slice: (first slot, rounds | log2 of the lanes per run << kRunLg)
     int2 *rlane;            // [run slices][32]: (camera or -1, row of the partial sums)
     int4 *blk_run;          // per block: its first run slice, the first of at most kRunRounds rounds, its end
-    int32_t *cm2r;          // camera-major position -> run slot
+    int32_t *cm2r;          // FP32: camera-major position -> run slot
+    int32_t *sl2r;          // FP64: slot -> run slot
     float4 *r_rx;           // FP32: [run slots] (R X, 1 / P_z)
     uint16_t *r_pt16;       // FP32: the point's index in its block, 0xffff in padding
     float *r_w;             // FP32: IRLS weight (null without a loss)

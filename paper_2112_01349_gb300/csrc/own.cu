@@ -59,18 +59,27 @@ __global__ void run_key_kernel(const int32_t *__restrict__ ord, const int32_t *_
 
 __global__ void fill_runs_kernel(Prob P, const int32_t *__restrict__ ord, const int32_t *__restrict__ run,
                                  const int32_t *__restrict__ run_ptr, const int2 *__restrict__ base, int parts,
-                                 const int2 *__restrict__ sp_bl, const int32_t *__restrict__ flag) {
+                                 const int2 *__restrict__ sp_bl, int32_t *__restrict__ orig2r,
+                                 const int32_t *__restrict__ flag) {
     if (*flag & 2) return;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < P.n; t += (int64_t)gridDim.x * blockDim.x) {
         const int s = ord[t], r = run[t], k = (int)(t - run_ptr[r]);
         const int part = k % parts, kk = k / parts;
         const int2 at = base[(int64_t)r * parts + part];  // first slot, log2 G
         const int slot = at.x + 32 * (kk >> at.y) + (kk & ((1 << at.y) - 1));
-        P.cm2r[s] = slot;
+        if (P.fp32) P.cm2r[s] = slot;
+        else orig2r[P.cm_orig[s]] = slot;
         const int sp = P.cm_sp[s];
         if (P.r_pt16) P.r_pt16[slot] = (uint16_t)sp_bl[sp].y;
         else P.r_pt[slot] = sp;
     }
+}
+
+// slot -> observation in the input order (fill_slots_kernel) -> run slot
+__global__ void slot_runs_kernel(Prob P, const int32_t *__restrict__ orig2r, const int32_t *__restrict__ flag) {
+    if (*flag & 2) return;
+    for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < P.nslots; o += (int64_t)gridDim.x * blockDim.x)
+        if (P.sl_cam[o] >= 0) P.sl2r[o] = orig2r[P.sl2r[o]];
 }
 
 // part of a run of l observations: those k with k mod parts equal to it
@@ -279,7 +288,7 @@ size_t own_arrays(Prob &P, const OwnPlan &pl, char *base) {
     P.rslice = (int2 *)arr(8 * (size_t)pl.slices);
     P.rlane = (int2 *)arr(32 * 8 * (size_t)pl.slices);
     P.blk_run = (int4 *)arr(16 * (size_t)pl.nblk);
-    P.cm2r = (int32_t *)arr(4 * (size_t)P.n);
+    P.cm2r = P.fp32 ? (int32_t *)arr(4 * (size_t)P.n) : nullptr;
     P.c_part = arr((size_t)pl.nblk * pl.parts * P.nc * (P.fp32 ? kPartF * 4 : kPartD * 8));
     if (P.fp32) {
         P.r_rx = (float4 *)arr(16 * ns);
@@ -423,7 +432,8 @@ cudaError_t build_own(Prob &P, void *tmp, size_t tmp_bytes, void *pool, size_t p
                    : cudaMemsetAsync(P.r_pt, 0xff, 4 * (size_t)pl.slots, s);
     if (e != cudaSuccess) return e;
     run_slices_kernel<<<(unsigned)nblk, 256, 0, s>>>(P, sorted, cut, round0_d, pl.parts, base_d, flag);
-    fill_runs_kernel<<<grid_for(P.n), kBlock, 0, s>>>(P, ord, run, run_ptr, base_d, pl.parts, sp_bl, flag);
+    fill_runs_kernel<<<grid_for(P.n), kBlock, 0, s>>>(P, ord, run, run_ptr, base_d, pl.parts, sp_bl, key, flag);
+    if (!P.fp32) slot_runs_kernel<<<grid_for(P.nslots), kBlock, 0, s>>>(P, key, flag);
     return cudaGetLastError();
 }
 

@@ -62,6 +62,7 @@ __global__ void fill_slots_kernel(Prob P, const int32_t *__restrict__ pt_sp, con
         P.sl_cam[slot] = P.pm_cam[o];
         const double2 uv = P.pm_uv[o];
         P.sl_uv[slot] = uv;
+        if (P.sl2r) P.sl2r[slot] = P.pm_orig[o];  // until build_own
         if (P.sl_uv32) P.sl_uv32[slot] = make_float2((float)uv.x, (float)uv.y);
     }
 }

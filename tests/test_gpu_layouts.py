@@ -206,3 +206,24 @@ def test_blocks_per_cta(mba, nc, npts, track, loss):
     rel_close(st["dp"], rs["dp"].reshape(-1, 3), 2e-3, "dp")
     ref = oracle.lm_solve(*_args(sc), max_iter=1, pcg_max=4, initial_radius=10.0, loss=loss, delta=2.0)
     rel_close(f, ref["final_cost"], 1e-4, "final cost")
+
+
+@pytest.mark.parametrize("loss", ["none", "huber"])
+@pytest.mark.parametrize("nc,npts,first_order", [(16, 2000, False), (127, 5000, False), (127, 5000, True)])
+def test_camera_blocks_fp64(mba, nc, npts, first_order, loss):
+    """B of the block-owned FP64 form, entry by entry against the geometric mean of
+    its diagonal entries: a dozen roundings per observation, sums of at most 8 in a
+    lane, five levels of lanes and a few chunks, and two 3 x 3 transforms, here and
+    in the oracle: 100 units of 2^-53 at most."""
+    sc = make_scene(nc, npts, track=("fixed", 5), sigma=0.5, seed=13)
+    cams = sc.cameras.copy()
+    if first_order:
+        cams[::2, :3] = np.random.default_rng(1).normal(size=cams[::2, :3].shape) * 4e-9
+        cams[1::4, :3] = 0.0
+        cams[:, 3:6] = [0.0, 0.0, -8.0]
+    args = (cams, *_args(sc)[1:])
+    with mba.Problem(*args, precision="fp64", loss=loss, huber_delta=2.0 if loss == "huber" else 0.0) as pr:
+        got = pr.linear_system(0.1)["Hpp"]
+    ref = oracle.blocks(*args, loss=loss, delta=2.0)[0]
+    d = np.sqrt(np.einsum("iaa->ia", ref))
+    assert np.max(np.abs(got - ref) / (d[:, :, None] * d[:, None, :])) < 100 * 2.0**-53
