@@ -261,7 +261,9 @@ __device__ __forceinline__ void camera_table_row(const double *c, double *o, dou
         R[6] = -w1; R[7] = w0;  R[8] = 1.0;
 #pragma unroll
         for (int i = 0; i < 9; ++i) M[i] = (i % 4 == 0) ? 1.0 : 0.0;
-        small = 1.0;
+        // with w = 0 exactly (cameras that were never rotated) both branches agree: R =
+        // M = I, and the analytic products need no first-order terms
+        small = HALF && w0 == 0.0 && w1 == 0.0 && w2 == 0.0 ? 0.0 : 1.0;
         if (quat) {
             quat[0] = 1.0;
             quat[1] = 0.5 * w0;

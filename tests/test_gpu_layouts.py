@@ -227,3 +227,26 @@ def test_camera_blocks_fp64(mba, nc, npts, first_order, loss):
     ref = oracle.blocks(*args, loss=loss, delta=2.0)[0]
     d = np.sqrt(np.einsum("iaa->ia", ref))
     assert np.max(np.abs(got - ref) / (d[:, :, None] * d[:, None, :])) < 100 * 2.0**-53
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-9), ("fp32", 1e-4)])
+@pytest.mark.parametrize("nc,npts", [(2, 30), (127, 5000), (2500, 30_000)])
+def test_cameras_without_rotation(mba, nc, npts, precision, tol):
+    """All cameras at w = 0 exactly, where the first-order and the general branch of
+    the rotation agree: no first-order terms.  Tolerances as above."""
+    sc = make_scene(nc, npts, track=("fixed", min(nc, 5)), sigma=0.5, seed=14)
+    cams = sc.cameras.copy()
+    cams[:, :3] = 0.0
+    cams[:, 3:6] = [0.0, 0.0, -8.0]
+    args = (cams, *_args(sc)[1:])
+    x = np.random.default_rng(5).normal(size=(nc, 9))
+    with mba.Problem(*args, precision=precision) as pr:
+        _, e, jc, jp = pr.evaluate()
+        y = pr.schur_matvec(0.1, x)
+        st = pr.step(0.1, pcg_max_iter=6, pcg_rel_tol=0.0)
+    _, eo, jco, jpo, _ = oracle.evaluate(*args)
+    for got, ref in ((e, eo), (jc, jco), (jp, jpo)):
+        rel_close(got, ref, tol, "evaluate")
+    rel_close(y, oracle.schur(*args, 0.1, x=x.reshape(-1))["y"].reshape(-1, 9), tol, "S x")
+    rs = oracle.step(*args, 0.1, pcg_max=6, pcg_tol=0.0)
+    rel_close(st["dc"], rs["dc"].reshape(-1, 9), 1e-6 if precision == "fp64" else 2e-3, "dc")
