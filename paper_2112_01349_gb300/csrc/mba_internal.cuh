@@ -211,8 +211,18 @@ __host__ __device__ __forceinline__ int sym3(int a, int b) {
 // Table row: R[9] M[9] t[3] f k1 k2 small w[3] (w: the raw angle-axis, read by
 // the dual-number path, which evaluates the edge functor from the parameters).
 // ---------------------------------------------------------------------------
-// HALF: one sine and cosine, of the half angle, and reciprocals instead of
-// divides (11.5 -> 9 us for 200 cameras); the rotation's quaternion goes to quat.
+// HALF: one sine and cosine, of the half angle, and quotients as products with a
+// reciprocal and one step of iterative refinement (quotient), the same bits as
+// divides, which took 2 us more a table of 16 cameras (the step takes 0.3; without
+// it k and M were off in the last bit and v by twice as much); the rotation's
+// quaternion goes to quat.
+// a / b with ib = 1 / b correctly rounded: a product within a bit of it and its
+// residual, which leaves the correctly rounded quotient (Markstein, IBM J. Res. Dev.
+// 34, 1990) for quotients and residuals in the normal range.
+__device__ __forceinline__ double quotient(double a, double b, double ib) {
+    const double q = a * ib;
+    return fma(fma(-q, b, a), ib, q);
+}
 template <bool HALF = false>
 __device__ __forceinline__ void camera_table_row(const double *c, double *o, double *quat = nullptr) {
     const double w0 = c[0], w1 = c[1], w2 = c[2];
@@ -221,12 +231,13 @@ __device__ __forceinline__ void camera_table_row(const double *c, double *o, dou
     double small;
     if (th2 > DBL_EPSILON) {
         const double th = sqrt(th2);
-        double s, co, oc, k0, k1, k2, ith = 0.0;
+        double s, co, oc, k0, k1, k2, ith2 = 0.0;
         if (HALF) {  // sin = 2 sh ch, 1 - cos = 2 sh^2, quaternion (ch, sh k)
             double sh, ch;
             sincos(0.5 * th, &sh, &ch);
-            ith = 1.0 / th;
-            k0 = w0 * ith, k1 = w1 * ith, k2 = w2 * ith;
+            const double ith = 1.0 / th;
+            ith2 = 1.0 / th2;
+            k0 = quotient(w0, th, ith), k1 = quotient(w1, th, ith), k2 = quotient(w2, th, ith);
             s = 2.0 * sh * ch, oc = 2.0 * sh * sh, co = 1.0 - oc;
             if (quat) {
                 quat[0] = ch;
@@ -243,7 +254,6 @@ __device__ __forceinline__ void camera_table_row(const double *c, double *o, dou
         R[3] = s * k2 + oc * k1 * k0;  R[4] = co + oc * k1 * k1;      R[5] = -s * k0 + oc * k1 * k2;
         R[6] = -s * k1 + oc * k2 * k0; R[7] = s * k0 + oc * k2 * k1;  R[8] = co + oc * k2 * k2;
         // (R^T - I) [w]_x, then add w w^T and divide by th^2
-        const double ith2 = ith * ith;
         const double A[9] = {R[0] - 1.0, R[3], R[6], R[1], R[4] - 1.0, R[7], R[2], R[5], R[8] - 1.0};
         const double W[9] = {0.0, -w2, w1, w2, 0.0, -w0, -w1, w0, 0.0};
         const double wv[3] = {w0, w1, w2};
@@ -252,7 +262,8 @@ __device__ __forceinline__ void camera_table_row(const double *c, double *o, dou
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 double acc = A[i * 3 + 0] * W[0 * 3 + j] + A[i * 3 + 1] * W[1 * 3 + j] + A[i * 3 + 2] * W[2 * 3 + j];
-                M[i * 3 + j] = HALF ? (acc + wv[i] * wv[j]) * ith2 : (acc + wv[i] * wv[j]) / th2;
+                acc += wv[i] * wv[j];
+                M[i * 3 + j] = HALF ? quotient(acc, th2, ith2) : acc / th2;
             }
         small = 0.0;
     } else {
