@@ -874,20 +874,6 @@ __global__ void __launch_bounds__(kBlock) cost_partial_kernel(Prob P, const doub
     if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
-// sqrt(x) for positive x: the hardware seed of 1 / sqrt(x) and two
-// Newton-Raphson steps, then one on the root itself; infinity gives itself, and a
-// subnormal x, whose root is below 1.5e-154, gives itself as well.
-__device__ __forceinline__ double fast_sqrt(double x) {
-    double r0;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(x));
-    if (!seed_ok(r0)) return x;
-    const double h = 0.5 * x;
-    double r = fma(r0, fma(-h * r0, r0, 0.5), r0);
-    r = fma(r, fma(-h * r, r, 0.5), r);
-    const double q = x * r;
-    return fma(fma(-q, q, x), 0.5 * r, q);
-}
-
 // The same over slices (analytic problems): the point stays in registers over
 // its observations and the cameras' R, t, f, k1, k2 sit in shared memory (SMEM;
 // 15 doubles, an odd stride).  Bound by the FP64 pipe: 21 instructions and a

@@ -293,22 +293,39 @@ __device__ __forceinline__ void camera_table_row(const double *c, double *o, dou
 __device__ __forceinline__ float rcp_rn(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double rcp_rn(double x) { return __drcp_rn(x); }
 
-// 1 / x: the hardware seed (20 bits) and two Newton-Raphson steps, four FP64
-// instructions where the correctly rounded reciprocal takes about twice that.
-// A seed of zero or infinity (x infinite, zero, subnormal) is the result itself;
-// the test is on its upper word, in integers, off the FP64 pipe.
+// 1 / x: the hardware seed (20 bits) and two Newton-Raphson steps, which leave 40 and
+// 80 bits before the last rounding: within one unit in the last place of the
+// correctly rounded reciprocal.  Seeds of zero, infinity or NaN (x infinite, zero,
+// NaN, subnormal, or so large that 1 / x is subnormal) go the slow way; the test is on
+// the seed's upper word, in integers, off the FP64 pipe.
 __device__ __forceinline__ bool seed_ok(double r) {
     return (unsigned)((__double2hiint(r) & 0x7fffffff) - 1) < 0x7fefffffu;
 }
+__device__ __noinline__ inline double slow_rcp(double x) { return 1.0 / x; }
+__device__ __noinline__ inline double slow_sqrt(double x) { return sqrt(x); }
 
 __device__ __forceinline__ double fast_rcp(double x) {
     double r0;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(x));
+    if (!seed_ok(r0)) return slow_rcp(x);
     double e = fma(-x, r0, 1.0);
     double r = fma(r0, e, r0);
     e = fma(-x, r, 1.0);
-    r = fma(r, e, r);
-    return seed_ok(r0) ? r : r0;
+    return fma(r, e, r);
+}
+
+// sqrt(x): the hardware seed of 1 / sqrt(x) and two Newton-Raphson steps, then one on
+// the root itself: within one unit in the last place of the correctly rounded root.
+// x zero, negative, subnormal, infinite or NaN goes the slow way.
+__device__ __forceinline__ double fast_sqrt(double x) {
+    double r0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(x));
+    if (!seed_ok(r0)) return slow_sqrt(x);
+    const double h = 0.5 * x;
+    double r = fma(r0, fma(-h * r0, r0, 0.5), r0);
+    r = fma(r, fma(-h * r, r, 0.5), r);
+    const double q = x * r;
+    return fma(fma(-q, q, x), 0.5 * r, q);
 }
 
 // Residual e = pi(c, X) - u and, if JAC, the analytic Jacobians Jc (2x9, row

@@ -11,11 +11,13 @@ __global__ void eval(int what, int n, const double2 *in, double2 *out) {
     if (i >= n) return;
     const double a = in[i].x, b = in[i].y;
     if (what == 0) out[i] = make_double2(mba::quotient(a, b, 1.0 / b), a / b);
+    if (what == 1) out[i] = make_double2(mba::fast_rcp(a), 1.0 / a);
+    if (what == 2) out[i] = make_double2(mba::fast_sqrt(a), sqrt(a));
 }
 
 int main(int argc, char **argv) {
     if (argc < 2) return 2;
-    const int what = !strcmp(argv[1], "quotient") ? 0 : 2;
+    const int what = !strcmp(argv[1], "quotient") ? 0 : (!strcmp(argv[1], "rcp") ? 1 : 2);
     int n = 0;
     if (fread(&n, sizeof n, 1, stdin) != 1 || n < 1) return 2;
     std::vector<double2> v(n);

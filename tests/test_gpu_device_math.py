@@ -1,4 +1,5 @@
-"""FP64 arithmetic of the kernels against CUDA's own."""
+"""The FP64 reciprocal, root and quotient of the kernels against CUDA's own, over
+random mantissas and exponents and at the edges of the range."""
 import os
 import subprocess
 
@@ -8,6 +9,9 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+TINY, HUGE = np.finfo(float).tiny, np.finfo(float).max
+EDGES = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, -5e-324, 1e-310, TINY, -TINY, 2 * TINY, 2.0**1021,
+                  2.0**1022, 2.0**1022 * 1.5, -(2.0**1023), HUGE, -HUGE, 1.0, -1.0, 3.0])
 
 
 @pytest.fixture(scope="module")
@@ -34,7 +38,29 @@ def _random(n, low, high, seed):
     return np.ldexp(rng.uniform(1.0, 2.0, n), rng.integers(low, high, n)) * rng.choice([-1.0, 1.0], n)
 
 
+def _units(got, ref):
+    """Distance in units in the last place (same sign, finite)."""
+    return np.abs(got.view(np.int64) - ref.view(np.int64))
+
+
 def test_quotient_is_the_divide(run):
     a, b = _random(1 << 20, -300, 300, 1), np.abs(_random(1 << 20, -300, 300, 2))
     got, ref = run("quotient", a, b)
     np.testing.assert_array_equal(got, ref)
+
+
+@pytest.mark.parametrize("what", ["rcp", "sqrt"])
+def test_reciprocal_and_root(run, what):
+    """Within one unit in the last place (40- and 80-bit Newton iterates, rounded
+    once more), and CUDA's own result at the edges."""
+    x = _random(1 << 20, -1021, 1021, 3)
+    if what == "sqrt":
+        x = np.abs(x)
+    got, ref = run(what, x, x)
+    assert _units(got, ref).max() <= 1
+    got, ref = run(what, EDGES, EDGES)
+    exact = ~np.isin(np.abs(EDGES), [1.0, 3.0, TINY, 2 * TINY, 2.0**1021, 2.0**1022, 1.5 * 2.0**1022, 2.0**1023, HUGE])
+    np.testing.assert_array_equal(got[exact], ref[exact])
+    same = np.isfinite(ref)
+    assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(got[~same], ref[~same], equal_nan=True)
+    assert _units(got[same], ref[same]).max() <= 1
