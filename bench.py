@@ -84,10 +84,13 @@ def pcg_streamed_bytes_per_iter(sc) -> float:
 
 
 def lin_bytes_per_obs(sc, w: int) -> float:
-    """Algorithmic bytes of the residual + Jacobian + block step per observation:
-    pixels (2w), two indices (8), the point amortised over its track (3w/L) and
-    the Jacobian written (24w)."""
-    return (26.0 + 3.0 * sc.np_ / sc.n) * w + 8.0
+    """Bytes the linearisation moves per observation in the block-owned forms: camera
+    index, pixels and (FP64) run position on the point side, the product's data
+    written there (FP32: 16; FP64: 80 for the slices and 80 for the runs), point
+    index and pixels on the camera side and (FP32) 16 written into the runs; the
+    point and its blocks amortised over its track."""
+    per_obs, per_point = (4 + 8 + 16 + 4 + 8 + 16, 16 + 72) if w == 4 else (4 + 16 + 4 + 160 + 4 + 16, 32 + 72)
+    return per_obs + per_point * sc.np_ / sc.n
 
 
 # FP32 non-tensor peak derived from unit counts and clocks: 152 SMs x 128 FP32
@@ -123,16 +126,11 @@ def batch_flops(ws, summaries, schur: str) -> float:
 
 
 # DRAM bytes (ncu dram__bytes_read.sum + dram__bytes_write.sum) per observation
-# per pass of one pcg_kernel launch on the full Venice-shaped problem (30 PCG
+# per pass of one pcg_own_kernel launch on the full Venice-shaped problem (30 PCG
 # iterations plus the right-hand-side pass, 5,004,484 observations), FP32-mixed
-# and FP64.  Traffic grows with the observation count, so a launch moves this
-# many bytes per observation per pass; None once the kernel has changed since
-# the capture.  The last full-size capture gave 61.3 B (FP32-mixed) and 431.1 B
-# (FP64), for kernels that the block-owned one has replaced, so no figure is
-# claimed.
-PCG_TRAFFIC_B_PER_OBS_PASS = {}
-PCG_TRAFFIC_NOTE = ("null: the kernel was replaced after the last full-size DRAM capture (61.3 B per observation per "
-                    "pass FP32-mixed, 431.1 B FP64); not re-taken")
+# and FP64 (profiles/pcg_own_kernel_venice.md).  Traffic grows with the observation
+# count, so a launch moves this many bytes per observation per pass.
+PCG_TRAFFIC_B_PER_OBS_PASS = {4: 43.0, 8: 241.5}
 
 
 def oracle_sample_time(threads: int, scale: float) -> dict:
@@ -411,7 +409,7 @@ def main():
         passes = pcg_iters + launches  # the right-hand-side pass counts as one
         alg_bytes = passes * pcg_bytes_per_iter(sc, w)
         alg_flops = passes * pcg_flops_per_iter(sc)
-        traffic = PCG_TRAFFIC_B_PER_OBS_PASS.get(w)
+        traffic = PCG_TRAFFIC_B_PER_OBS_PASS[w]
         # linearisations: the first one, then one after every accepted step that
         # is not the solve's last iteration (a rejected step reuses the last one)
         lins = sum(1 + sum(t["accepted"] for t in s["trace"][:-1]) for s in sums)
@@ -419,9 +417,8 @@ def main():
         return dict(value=value, ms_per_step=ms / args.steps, pcg_ms=pcg_ms, pcg_iters=pcg_iters,
                     pcg_launches=launches, gbs=alg_bytes / (pcg_ms / 1e3) / 1e9,
                     streamed_gbs=passes * pcg_streamed_bytes_per_iter(sc) / (pcg_ms / 1e3) / 1e9,
-                    traffic_per_launch=None if traffic is None else traffic * sc.n * passes / launches,
-                    dram_gbs=None if traffic is None else traffic * sc.n * passes / (pcg_ms / 1e3) / 1e9,
-                    alg_bytes_per_launch=alg_bytes / launches,
+                    traffic_per_launch=traffic * sc.n * passes / launches,
+                    dram_gbs=traffic * sc.n * passes / (pcg_ms / 1e3) / 1e9,
                     tflops=alg_flops / (pcg_ms / 1e3) / 1e12,
                     us_per_pcg_iter=1e3 * pcg_ms / max(1, passes),
                     lin_ms_each=lin_ms / lins, lin_gbs=lins * sc.n * lin_bytes_per_obs(sc, w) / (lin_ms / 1e3) / 1e9,
@@ -655,7 +652,7 @@ def main():
             final[prec] = {"value": FINAL_LM_ITERS / (ms3 / 1e3), "unit": UNIT, "ms_per_solve": ms3,
                            "pcg_iters": s3["pcg_iters_total"], "accepted": s3["accepted"],
                            "us_per_pcg_iter": 1e3 * s3["ms_pcg"] / passes,
-                           "pcg_alg_gbs": passes * pcg_bytes_per_iter(sc3, w) / (s3["ms_pcg"] / 1e3) / 1e9,
+                           "pcg_stored_jacobian_gbs": passes * pcg_bytes_per_iter(sc3, w) / (s3["ms_pcg"] / 1e3) / 1e9,
                            "initial_cost": s3["initial_cost"], "final_cost": s3["final_cost"]}
         final["final_cost_rel_diff_fp32_vs_fp64"] = ((final["fp32"]["final_cost"] - final["fp64"]["final_cost"]) /
                                                      final["fp64"]["final_cost"])
@@ -706,19 +703,18 @@ def main():
                    "l2": "inputs larger than L2 (per PCG pass: 0.2 GB streamed FP32, 0.84 GB FP64)",
                    "parallelism": "replicas" if world > 1 else "1 GPU"},
         "roofline": {"kernel": "pcg_own_kernel (persistent PCG, block-owned implicit Schur product)", "bound": "hbm",
-                     "achieved": a32["gbs"], "peak": hbm_peak, "unit": "GB/s", "frac": a32["gbs"] / hbm_peak,
-                     "peak_kind": peak_kind, "traffic": a32["traffic_per_launch"],
+                     "achieved": a32["streamed_gbs"], "peak": hbm_peak, "unit": "GB/s",
+                     "frac": a32["streamed_gbs"] / hbm_peak, "peak_kind": peak_kind,
+                     "counted": "bytes the factored FP32 product streams: 34 B per observation per iteration, "
+                                "24 B per point, 1.9 KB per camera", "traffic": a32["traffic_per_launch"],
                      "traffic_unit": "bytes per launch (ncu dram__bytes_read+write per observation per pass of a "
                                      "full-size launch, times this run's observations and passes)",
-                     "algorithmic_bytes_per_launch": a32["alg_bytes_per_launch"],
-                     "algorithmic": "per PCG iteration 100 B per observation (stored Jacobian + camera index), "
-                                    "72 B per point, 576 B per camera",
-                     "streamed_gbs": a32["streamed_gbs"], "streamed_frac": a32["streamed_gbs"] / hbm_peak,
-                     "streamed": "bytes the factored FP32 product actually streams: 34 B per observation per "
-                                 "iteration, 24 B per point, 1.9 KB per camera",
+                     "stored_jacobian_gbs": a32["gbs"],
+                     "stored_jacobian": "the bytes a stored Jacobian would take instead (per PCG iteration 100 B per "
+                                        "observation, 72 B per point, 576 B per camera) over the same time: not "
+                                        "moved, for comparison with forms that store it",
                      "dram_gbs": a32["dram_gbs"],
-                     "dram_frac": None if a32["dram_gbs"] is None else a32["dram_gbs"] / hbm_peak,
-                     "traffic_note": PCG_TRAFFIC_NOTE if a32["traffic_per_launch"] is None else None,
+                     "dram_frac": a32["dram_gbs"] / hbm_peak,
                      "us_per_pcg_iter": a32["us_per_pcg_iter"], "share_of_solve": a32["pcg_share"],
                      "pcg_iters_per_solve": a32["pcg_iters"] / max(1, len(s32)),
                      "other_kernels": {
@@ -726,25 +722,25 @@ def main():
                              "kernel": "pcg_own_kernel, single-reduction (Chronopoulos-Gear) instance",
                              "bound": "hbm", "unit": "GB/s",
                              "us_per_pcg_iter": variants["single_reduction_pcg"]["us_per_pcg_iter"],
-                             "achieved": pcg_bytes_per_iter(sc, 4) / (variants["single_reduction_pcg"]["us_per_pcg_iter"]
-                                                                      / 1e6) / 1e9,
-                             "frac": pcg_bytes_per_iter(sc, 4) / (variants["single_reduction_pcg"]["us_per_pcg_iter"]
-                                                                  / 1e6) / 1e9 / hbm_peak,
-                             "note": "same algorithmic bytes per PCG iteration as the headline kernel; one global "
+                             "achieved": pcg_streamed_bytes_per_iter(sc) /
+                                         (variants["single_reduction_pcg"]["us_per_pcg_iter"] / 1e6) / 1e9,
+                             "frac": pcg_streamed_bytes_per_iter(sc) /
+                                     (variants["single_reduction_pcg"]["us_per_pcg_iter"] / 1e6) / 1e9 / hbm_peak,
+                             "note": "same bytes per PCG iteration as the headline kernel; one global "
                                      "reduction per PCG step instead of two (solver option, not the headline)"},
-                         "linearize_fp32": {"kernel": "lin_point + lin_camera + cam_finalize (+ camera table)",
+                         "linearize_fp32": {"kernel": "point_table + lin_slices + lin_camera32 + cam_finalize (+ camera table)",
                                             "bound": "hbm", "achieved": a32["lin_gbs"], "unit": "GB/s",
                                             "frac": a32["lin_gbs"] / hbm_peak,
                                             "ms_per_linearisation": a32["lin_ms_each"],
-                                            "algorithmic_bytes_per_obs": lin_bytes_per_obs(sc, 4)},
+                                            "bytes_per_obs": lin_bytes_per_obs(sc, 4)},
                          "linearize_fp64": {"achieved": a64["lin_gbs"], "unit": "GB/s",
                                             "frac": a64["lin_gbs"] / hbm_peak,
                                             "ms_per_linearisation": a64["lin_ms_each"],
-                                            "algorithmic_bytes_per_obs": lin_bytes_per_obs(sc, 8)},
+                                            "bytes_per_obs": lin_bytes_per_obs(sc, 8)},
                          "pcg_fp64": {"bound": "alu", "achieved": a64["tflops"], "peak": FP64_PEAK_TFLOPS,
                                       "unit": "TFLOP/s", "frac": a64["tflops"] / FP64_PEAK_TFLOPS,
                                       "peak_kind": "derived (152 SMs x 2 DFMA/clk x 2.07 GHz)",
-                                      "alg_gbs": a64["gbs"], "dram_gbs": a64["dram_gbs"],
+                                      "stored_jacobian_gbs": a64["gbs"], "dram_gbs": a64["dram_gbs"],
                                       "us_per_pcg_iter": a64["us_per_pcg_iter"]}}},
         "final_cost": a32["final_cost"], "accepted": a32["accepted"],
         "final_cost_rel_diff_vs_fp64": abs(a32["final_cost"] - a64["final_cost"]) / a64["final_cost"],

@@ -2197,12 +2197,13 @@ bool s_in_smem(const mba_batch *b) {
     return b->schur == 2 && b->explicit_ok && max_ctas_per_sm(b, b->nt, b->cps, true) >= b->cps;
 }
 
-// Cluster size of the automatic schedule: the largest of 16, 8, 4 for which
+// Cluster size where the schedule allows clusters: the largest of 16, 8, 4 for which
 // every window has its cluster at once, one CTA per SM; two CTAs per window up to
 // one window per SM (clusters then claim the windows longest-first, so the
 // longest window no longer sets the time alone); 1 (no clusters) with more
-// windows than that, for the implicit product and for the single-reduction PCG.  Eight FP64 windows of 5 to 30 cameras with the adjoint: 7.2 ms with 16 CTAs
-// each, 41.3 ms with one.
+// windows than that, for the implicit product and for the single-reduction PCG.
+// Eight FP64 windows of 5 to 30 cameras with the adjoint: 7.2 ms with 16 CTAs each,
+// 41.3 ms with one.
 int cluster_size(const mba_batch *b, const BatchOpts &o, int *rows, size_t *smem, int *clusters_out) {
     *rows = 0;
     *clusters_out = 0;
@@ -2213,7 +2214,8 @@ int cluster_size(const mba_batch *b, const BatchOpts &o, int *rows, size_t *smem
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     const size_t limit = (size_t)optin - 2048;  // static shared memory
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess || allow_smem(k) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        allow_smem(k) != cudaSuccess) {
         cudaGetLastError();
         return 1;
     }

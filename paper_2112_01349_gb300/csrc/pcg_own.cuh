@@ -566,10 +566,10 @@ __device__ __forceinline__ double own_precond(const double *b, double rv, int th
 
 // The whole solve in one cooperative launch, one CTA per SM.  Per iteration, against
 // the kernel with segmented scans and a scattered s (FP32) or a stored Jacobian
-// (FP64) that it replaced: FP32, 1,700 cameras and 5.0M observations 106 -> 75.4 us
+// (FP64) that it replaced: FP32, 1,700 cameras and 5.0M observations 106 -> 75.5 us
 // (point side 28.5, camera side 24.5: latency and issue; the streams alone take 30
 // at the measured 6.8 TB/s), 200 cameras and 250k observations 21.4 -> 19.1
-// (barriers and dependent sums).  FP64, 5.0M observations 747 -> 449 us (point side
+// (barriers and dependent sums).  FP64, 5.0M observations 747 -> 445 us (point side
 // 179, camera side 224: the FP64 pipe), 780k 156 -> 105, 250k 63 -> 53, 10k
 // 37 -> 18.6.
 template <typename T, bool SR, bool LONG>
