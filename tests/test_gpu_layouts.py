@@ -177,13 +177,14 @@ def test_a_camera_that_sees_every_point(mba, nc, npts, precision, tol, loss):
     with mba.Problem(*args, **opts) as pr:
         assert pr.info["device_bytes"] < 1.1 * size + 152 * 32 * 32 * 84
         y = pr.schur_matvec(0.1, x)
-        st = pr.step(0.1, pcg_max_iter=6, pcg_rel_tol=0.0)
+        steps = {v: pr.step(0.1, pcg_max_iter=6, pcg_rel_tol=0.0, pcg_variant=v) for v in ("standard", "single_reduction")}
     rel_close(y, oracle.schur(*args, 0.1, x=x.reshape(-1), loss=loss, delta=2.0)["y"].reshape(-1, 9), tol, "S x")
-    rs = oracle.step(*args, 0.1, pcg_max=6, pcg_tol=0.0, loss=loss, delta=2.0)
     stol = 1e-6 if precision == "fp64" else 2e-3
-    for a in range(9):
-        rel_close(st["dc"][:, a], rs["dc"].reshape(-1, 9)[:, a], stol, f"dc[{a}]")
-    rel_close(st["dp"], rs["dp"].reshape(-1, 3), stol, "dp")
+    for variant, st in steps.items():
+        rs = oracle.step(*args, 0.1, pcg_max=6, pcg_tol=0.0, loss=loss, delta=2.0, pcg_variant=variant)
+        for a in range(9):
+            rel_close(st["dc"][:, a], rs["dc"].reshape(-1, 9)[:, a], stol, f"{variant} dc[{a}]")
+        rel_close(st["dp"], rs["dp"].reshape(-1, 3), stol, f"{variant} dp")
 
 
 # b of a CTA's points beside the camera rows in shared memory: two, three and four
